@@ -297,9 +297,9 @@ class CircuitBench:
     def launches(self):
         """Library kernels per step: resident forward 1, resident backward 2
         (sweep + fixed-order dw sum); HBM-tiled: one launch per pass plus the
-        per-sample tables (circuits with x; the complex64 backward from a saved
-        state evaluates its own) and the partial sums (E; the per-sample
-        gradient terms, dx and dw); cluster forward 1, cluster backward 2."""
+        tables and the partial sums (E; the per-sample gradient terms, dx and dw,
+        which complex64 sums in one launch where a circuit has both); cluster
+        forward 1, cluster backward 2."""
         inf, nx, nw = self.info, self.w_.spec.num_x > 0, self.w_.spec.num_w > 0
         f = inf["fwd_passes"] + 1 + int(nx) if inf["fwd_path"] == 1 else 1
         if not self.w_.backward:

@@ -399,6 +399,17 @@ vqc_status upload(HostPlan& p) {
         s.dev_pass_accs = put(s.pass_accs.data(), s.pass_accs.size() * 4);
         s.dev_region_end = blob.size();
     }
+    for (auto& s : p.frames) {
+        s.dev_ops = put(s.ops.data(), s.ops.size() * sizeof(DOp));
+        s.dev_stages = put(s.stages.data(), s.stages.size() * sizeof(FStage));
+        s.dev_flips = put(s.flips.data(), s.flips.size() * sizeof(FFlip));
+        s.dev_fin = put(&s.fin, sizeof(FFinal));
+        // the passes copy their entries from the tables by slot
+        std::vector<int32_t> slots;
+        for (int32_t e : s.pass_entries) slots.push_back(p.entries[e].slot);
+        s.dev_pass_entries = put(slots.data(), slots.size() * 4);
+        s.dev_pass_accs = put(s.pass_accs.data(), s.pass_accs.size() * 4);
+    }
     size_t err_off = put(nullptr, 16);
     blob.resize(align256(blob.size()), 0);
     VQC_CUDA(cudaGetDevice(&p.device));
@@ -679,18 +690,17 @@ vqc_status run_cluster_backward(const HostPlan& p, int B, const void* x, const v
 
 // ---------------------------------------------------------------- HBM path
 struct PassGeo {
-    const Schedule* s = nullptr;
+    const FrameSchedule* s = nullptr;
     int K = 0, T = 0, S = 0, block = 0, grid = 0, wg = 1, ntiles = 1;
     long long nunits = 0;
     size_t smem = 0;
     int sm_sh = 0, sm_ps = 0, sm_psi = 0, sm_lam = 0, sm_acc = 0, sm_red = 0, sm_plan = 0,
-        sm_koff = 0;
-    bool plan_smem = false;
+        sm_tfl = 0, sm_koff = 0;
     const void* fn = nullptr;
 };
 
 vqc_status plan_hbm_uncached(const HostPlan& p, int mode, int B, PassGeo& L) {
-    L.s = find_hbm_schedule(p, mode);
+    L.s = find_frame(p, mode, VQC_PATH_HBM);
     if (!L.s) return fail(VQC_ERR_UNSUPPORTED, "no HBM-tiled schedule for this circuit");
     int dev = 0;
     VQC_CUDA(cudaGetDevice(&dev));
@@ -704,16 +714,21 @@ vqc_status plan_hbm_uncached(const HostPlan& p, int mode, int B, PassGeo& L) {
     L.T = 1 << (m - L.K);
     L.wg = L.T > 32 ? L.T / 32 : 1;
     L.ntiles = 1 << (p.n - m);
-    int ps_max = 0, sh_max = 0, acc_max = 0;
-    for (const DPass& ps : L.s->passes) {
+    int ps_max = 0, sh_max = 0, acc_max = 0, nst_max = 0, ops_max = 0;
+    for (const FPass& ps : L.s->passes) {
         ps_max = std::max(ps_max, ps.ps_count);
         sh_max = std::max(sh_max, ps.sh_count);
         acc_max = std::max(acc_max, ps.acc_count);
+        nst_max = std::max(nst_max, ps.stage_end - ps.stage_begin);
+        ops_max = std::max(ops_max, ps.op_end - ps.op_begin);
     }
     const size_t tdim = (size_t)1 << m;
     const size_t ew = dbl ? 8 : 32;   // reals per table entry
-    const size_t fixed = align16((size_t)sh_max * ew * rs) + 8 * 16 + 1024;   // + tile-copy offsets
-    const size_t per_tile = (size_t)ps_max * ew * rs + tdim * cs * (mode == 1 ? 2 : 1) +
+    const size_t apv = 16 / cs, nk = (tdim / apv + L.T - 1) / L.T;
+    const size_t prog = (size_t)nst_max * sizeof(FStage) + sizeof(FFinal) + (size_t)ops_max * sizeof(DOp) +
+                        (size_t)nst_max * L.s->nout * sizeof(FFlip);
+    const size_t fixed = align16((size_t)sh_max * ew * rs) + align16(prog) + align16(2 * nk * 8) + 8 * 16;
+    const size_t per_tile = (size_t)ps_max * ew * rs + tdim * cs * (mode == 1 ? 2 : 1) + (size_t)(nst_max + 1) * 8 +
                             (mode == 1 ? (size_t)acc_max * L.wg * 8 * rs : (size_t)L.wg * p.n * rs);
     int S = std::max(1, 128 / L.T);
     if ((size_t)di.smem_optin <= fixed + per_tile)
@@ -737,14 +752,9 @@ vqc_status plan_hbm_uncached(const HostPlan& p, int mode, int B, PassGeo& L) {
     L.sm_lam = take(mode == 1 ? (size_t)S * tdim * cs : 0);
     L.sm_acc = take(mode == 1 ? (size_t)S * acc_max * L.wg * 8 * rs : 0);
     L.sm_red = take(mode == 0 ? (size_t)S * L.wg * p.n * rs : 0);
-    {   // tile-copy offsets: one uint2 per vector round of a tile
-        const size_t apv = 16 / cs, nvec = tdim / apv;
-        L.sm_koff = take(((nvec + L.T - 1) / L.T) * 8);
-    }
-    const size_t plan_bytes = align16(p.dev_tab_end - p.dev_tab_begin) +
-                              (L.s->dev_region_end - L.s->dev_region_begin);
-    L.plan_smem = off + plan_bytes <= (size_t)di.smem_optin && plan_bytes <= 48 * 1024;
-    L.sm_plan = L.plan_smem ? take(plan_bytes) : 0;
+    L.sm_koff = take(2 * nk * 8);   // tile-copy offsets: one uint2 per vector round, read and written
+    L.sm_plan = take(prog);
+    L.sm_tfl = take((size_t)S * (nst_max + 1) * 8);
     L.smem = off;
     L.fn = p.dfloat ? pass_ptr_dd(mode, L.K, L.T >= 32)
            : (!dbl && mode == 0 && !p.has_ph2) ? pass_ptr_f32_fwd_nph(L.K, L.T >= 32)   // no phase cases
@@ -790,15 +800,20 @@ void forget_plan(const HostPlan* p) {
         it = it->first.plan == p ? g_cluster_cache.erase(it) : std::next(it);
 }
 
-// Workspace of the HBM path.  Forward: [control | working state | <Z> partials].
-// Backward: [control | psi | lam | gradient-term partials].
+// Workspace of the HBM path.  Forward: [control | working state | <Z> partials |
+// tables].  Backward: [control | psi | lam | rho sums | gradient terms | tables].
 struct HbmWs {
-    size_t state = 0, lam = 0, part = 0, terms = 0, ps = 0, total = 0;
+    size_t state = 0, lam = 0, part = 0, terms = 0, ps = 0, sh = 0, total = 0;
 };
 
+size_t hbm_state_bytes(const HostPlan& p, int B) {
+    return align256((size_t)B * ((size_t)1 << p.n) * (p.dtype == VQC_C128 ? 16 : 8));
+}
+
 HbmWs hbm_layout(const HostPlan& p, int mode, int B, int ntiles) {
-    const size_t rs = p.dtype == VQC_C128 ? 8 : 4, cs = 2 * rs;
-    const size_t sbytes = align256((size_t)B * ((size_t)1 << p.n) * cs);
+    const size_t rs = p.dtype == VQC_C128 ? 8 : 4;
+    const size_t sbytes = hbm_state_bytes(p, B);
+    const size_t entry = (p.dtype == VQC_C128 ? 8 : 32) * rs;
     HbmWs w;
     w.state = 256;
     if (mode == 0) {
@@ -810,56 +825,57 @@ HbmWs hbm_layout(const HostPlan& p, int mode, int B, int ntiles) {
         w.terms = w.part + align256((size_t)B * ntiles * std::max<size_t>(p.accs.size(), 1) * 4 * rs);
         w.ps = w.terms + align256((size_t)B * std::max<size_t>(p.term_src.size(), 1) * rs);
     }
-    // every sample's per-sample table entries [B][n_ps][entry words]
-    w.total = w.ps + align256((size_t)B * p.n_ps * (p.dtype == VQC_C128 ? 8 : 32) * rs);
+    // table entries: every sample's [B][n_ps], the shared ones [n_sh]
+    w.sh = w.ps + align256((size_t)B * p.n_ps * entry);
+    w.total = w.sh + align256((size_t)p.n_sh * entry);
     return w;
 }
 
-// Every sample's per-sample table entries into `out` (ps_tables), read by the
-// passes instead of evaluating them once per tile.
+// The call's table entries (run_tables), read by every pass.
 template <typename R>
-vqc_status launch_ps_tables(const HostPlan& p, int B, const void* x, const void* w, void* out,
-                            cudaStream_t stream) {
-    if (p.n_ps == 0) return VQC_OK;
+vqc_status launch_tables(const HostPlan& p, int B, const void* x, const void* w, void* out_ps, void* out_sh,
+                         cudaStream_t stream) {
+    if (p.n_ps + p.n_sh == 0) return VQC_OK;
     const char* base = static_cast<const char*>(p.dbuf);
     const DEntry* entries = reinterpret_cast<const DEntry*>(base + p.dev_entries);
     const int32_t* ps_list = reinterpret_cast<const int32_t*>(base + p.dev_ps_list);
+    const int32_t* sh_list = reinterpret_cast<const int32_t*>(base + p.dev_sh_list);
     const DConst* consts = reinterpret_cast<const DConst*>(base + p.dev_consts);
     const R* cang = reinterpret_cast<const R*>(base + p.dev_cang);
     const R* cmat = reinterpret_cast<const R*>(base + p.dev_cmat);
     const R* xr = static_cast<const R*>(x);
     const R* wr = static_cast<const R*>(w);
-    int Px = p.num_x, Bi = B, nps = p.n_ps;
-    void* args[] = {&entries, &ps_list, &consts, &cang, &cmat, &xr, &Px, &wr, &Bi, &nps, &out};
-    const int blocks = (int)std::min<long long>(4096, ((long long)B * nps + 255) / 256);
-    VQC_CUDA(launch(p.dfloat ? ps_tables_ptr_dd() : ps_tables_ptr(p.dtype == VQC_C128), dim3(std::max(blocks, 1)),
-                    dim3(256), args, 0, stream));
+    int Px = p.num_x, Bi = B, nps = p.n_ps, nsh = p.n_sh;
+    void* args[] = {&entries, &ps_list, &sh_list, &consts, &cang, &cmat, &xr, &Px, &wr, &Bi, &nps, &nsh, &out_ps, &out_sh};
+    const int blocks = (int)std::min<long long>(4096, ((long long)B * nps + nsh + 255) / 256);
+    VQC_CUDA(launch(p.dfloat ? run_tables_ptr_dd() : run_tables_ptr(p.dtype == VQC_C128), dim3(blocks), dim3(256),
+                    args, 0, stream));
     return VQC_OK;
 }
 
 template <typename R>
-void fill_pass_args(const HostPlan& p, const PassGeo& L, const DPass& ps, PArgs<R>& a) {
+void fill_pass_args(const HostPlan& p, const PassGeo& L, const FPass& ps, const void* ps_g, const void* sh_g,
+                    PArgs<R>& a) {
     const char* base = static_cast<const char*>(p.dbuf);
-    a.ops = reinterpret_cast<const DOp*>(base + L.s->dev_ops);
-    a.stages = reinterpret_cast<const DStage*>(base + L.s->dev_stages);
+    const FrameSchedule& s = *L.s;
+    const bool back = s.mode == 1;   // reads what the forward order writes
+    a.ops = reinterpret_cast<const DOp*>(base + s.dev_ops) + ps.op_begin;
+    a.stages = reinterpret_cast<const FStage*>(base + s.dev_stages) + ps.stage_begin;
+    a.flips = reinterpret_cast<const FFlip*>(base + s.dev_flips) + (size_t)ps.stage_begin * s.nout;
+    a.fin = &ps == &s.passes.back() ? reinterpret_cast<const FFinal*>(base + s.dev_fin) : nullptr;
     a.err = p.dev_error;
-    a.pass_entries = reinterpret_cast<const int32_t*>(base + L.s->dev_pass_entries);
-    a.pass_accs = reinterpret_cast<const int32_t*>(base + L.s->dev_pass_accs);
-    a.entries = reinterpret_cast<const DEntry*>(base + p.dev_entries);
-    a.consts = reinterpret_cast<const DConst*>(base + p.dev_consts);
-    a.cmat = reinterpret_cast<const R*>(base + p.dev_cmat);
-    a.cang = reinterpret_cast<const R*>(base + p.dev_cang);
-    a.accs = reinterpret_cast<const DAcc*>(base + p.dev_accs);
+    a.pass_entries = reinterpret_cast<const int32_t*>(base + s.dev_pass_entries);
+    a.pass_accs = reinterpret_cast<const int32_t*>(base + s.dev_pass_accs);
     a.n = p.n;
-    a.m = L.s->m;
-    a.K = L.K;
-    a.tbits = L.s->m - L.K;
+    a.m = s.m;
+    a.tbits = s.m - L.K;
     a.G = p.G_swz;
     a.S = L.S;
-    a.nout = p.n - L.s->m;
+    a.nout = s.nout;
     a.ntiles = L.ntiles;
-    a.stage_begin = ps.stage_begin;
-    a.stage_end = ps.stage_end;
+    a.nstages = ps.stage_end - ps.stage_begin;
+    a.nops = ps.op_end - ps.op_begin;
+    a.op_begin = ps.op_begin;
     a.ps_begin = ps.ps_begin;
     a.ps_count = ps.ps_count;
     a.sh_begin = ps.sh_begin;
@@ -868,28 +884,62 @@ void fill_pass_args(const HostPlan& p, const PassGeo& L, const DPass& ps, PArgs<
     a.acc_count = ps.acc_count;
     a.n_accs = (int)p.accs.size();
     a.n_ps = p.n_ps;
-    a.Px = p.num_x;
+    a.ps_g = ps_g;
+    a.sh_g = sh_g;
     a.nunits = L.nunits;
-    for (int i = 0; i < 24; ++i) {
-        a.tile_q[i] = ps.tile_q[i];
-        a.out_q[i] = ps.out_q[i];
+    for (int i = 0; i < kMaxTileBits; ++i) {
+        a.ga[i] = back ? ps.gout[i] : ps.gin[i];
+        a.sa[i] = back ? ps.gin[i] : ps.gout[i];
+        a.gs[i] = back ? ps.sout[i] : ps.sin[i];
+        a.ss[i] = back ? ps.sin[i] : ps.sout[i];
+    }
+    for (int i = 0; i < kMaxOuterBits; ++i) {
+        a.go[i] = back ? ps.oout[i] : ps.oin[i];
+        a.so[i] = back ? ps.oin[i] : ps.oout[i];
+        a.sosl[i] = back ? 0 : ps.oslot[i];
     }
     a.sm_sh = L.sm_sh; a.sm_ps = L.sm_ps; a.sm_psi = L.sm_psi; a.sm_lam = L.sm_lam;
     a.sm_acc = L.sm_acc; a.sm_red = L.sm_red; a.sm_koff = L.sm_koff;
-    a.plan = static_cast<const unsigned char*>(p.dbuf);
-    a.tab_off = (int)p.dev_tab_begin;
-    a.tab_bytes = (int)(p.dev_tab_end - p.dev_tab_begin);
-    a.sched_off = (int)L.s->dev_region_begin;
-    a.sched_bytes = (int)(L.s->dev_region_end - L.s->dev_region_begin);
-    a.sm_plan = L.sm_plan;
-    a.plan_smem = L.plan_smem ? 1 : 0;
+    a.sm_plan = L.sm_plan; a.sm_tfl = L.sm_tfl;
+}
+
+// The forward passes: psi0 (nullptr: |0...0>) -> out in logical order (nullptr:
+// not written), the state between passes in W (not out: the last pass writes
+// other addresses than it reads).  out_raw: double-float passes follow.
+template <typename R>
+vqc_status forward_passes(const HostPlan& p, const PassGeo& L, int B, const void* psi0, void* W, void* out,
+                          bool out_raw, R* E_part, const void* ps_g, const void* sh_g, cudaStream_t stream) {
+    using C = C2<R>;
+    const int np = (int)L.s->passes.size();
+    if (np == 1 && psi0 && out) {   // one pass from a caller's state into itself: through W
+        const size_t bytes = ((size_t)B << p.n) * sizeof(C);
+        const char *i = static_cast<const char*>(psi0), *o = static_cast<const char*>(out);
+        if (i < o + bytes && o < i + bytes) {
+            VQC_CUDA(cudaMemcpyAsync(W, psi0, bytes, cudaMemcpyDeviceToDevice, stream));
+            psi0 = W;
+        }
+    }
+    for (int i = 0; i < np; ++i) {
+        PArgs<R> a{};
+        fill_pass_args<R>(p, L, L.s->passes[i], ps_g, sh_g, a);
+        const bool last = i == np - 1;
+        a.B = B;
+        a.src_psi = static_cast<const C*>(i == 0 ? psi0 : W);
+        a.dst_psi = static_cast<C*>(last ? out : W);
+        a.E_part = last ? E_part : nullptr;
+        // double-float: raw pairs between passes, complex128 in and out
+        a.src_raw = i > 0;
+        a.dst_raw = !last || out_raw;
+        void* args[] = {&a};
+        VQC_CUDA(launch(L.fn, dim3(L.grid), dim3(L.block), args, L.smem, stream));
+    }
+    return VQC_OK;
 }
 
 template <typename R>
 vqc_status run_hbm_forward(const HostPlan& p, int B, const void* x, const void* w,
                            const void* psi0, void* E, void* state_out, void* ws, size_t ws_bytes,
-                           cudaStream_t stream, bool want_E) {
-    using C = C2<R>;
+                           cudaStream_t stream) {
     PassGeo L;
     vqc_status st = plan_hbm(p, 0, B, L);
     if (st != VQC_OK) return st;
@@ -898,40 +948,18 @@ vqc_status run_hbm_forward(const HostPlan& p, int B, const void* x, const void* 
         return fail(VQC_ERR_WORKSPACE, "forward workspace must be >= " + std::to_string(lay.total) +
                                            " bytes and 256-byte aligned");
     char* wsc = static_cast<char*>(ws);
-    C* W = state_out ? static_cast<C*>(state_out) : reinterpret_cast<C*>(wsc + lay.state);
     R* E_part = reinterpret_cast<R*>(wsc + lay.part);
-    void* ps_g = wsc + lay.ps;
-    st = launch_ps_tables<R>(p, B, x, w, ps_g, stream);
+    st = launch_tables<R>(p, B, x, w, wsc + lay.ps, wsc + lay.sh, stream);
     if (st != VQC_OK) return st;
-    const int np = (int)L.s->passes.size();
-    for (int i = 0; i < np; ++i) {
-        PArgs<R> a{};
-        fill_pass_args<R>(p, L, L.s->passes[i], a);
-        a.ps_g = ps_g;
-        a.B = B;
-        a.x = static_cast<const R*>(x);
-        a.w = static_cast<const R*>(w);
-        a.src_psi = i == 0 ? static_cast<const C*>(psi0) : W;
-        const bool last = i == np - 1;
-        a.dst_psi = (last && want_E && !state_out) ? nullptr : W;
-        a.E_part = (last && want_E) ? E_part : nullptr;
-        // double-float: raw pairs between passes, complex128 in and out (a
-        // pass reads its whole tile before writing it, so W may change format
-        // in place)
-        a.src_raw = i > 0;
-        a.dst_raw = !last;
-        void* args[] = {&a};
-        VQC_CUDA(launch(L.fn, dim3(L.grid), dim3(L.block), args, L.smem, stream));
-    }
-    if (want_E) {
-        const R* Ep = E_part;
-        R* Eo = static_cast<R*>(E);
-        int Bi = B, nt = L.ntiles, n = p.n;
-        void* args[] = {&Ep, &Bi, &nt, &n, &Eo};
-        const int blocks = (int)std::min<long long>(4096, ((long long)B * n + 255) / 256);
-        VQC_CUDA(launch(reduce_expz_ptr(p.dtype == VQC_C128), dim3(std::max(blocks, 1)),
-                                  dim3(256), args, 0, stream));
-    }
+    st = forward_passes<R>(p, L, B, psi0, wsc + lay.state, state_out, false, E_part, wsc + lay.ps, wsc + lay.sh,
+                           stream);
+    if (st != VQC_OK) return st;
+    const R* Ep = E_part;
+    R* Eo = static_cast<R*>(E);
+    int Bi = B, nt = L.ntiles, n = p.n;
+    void* args[] = {&Ep, &Bi, &nt, &n, &Eo};
+    const int blocks = (int)std::min<long long>(4096, ((long long)B * n + 255) / 256);
+    VQC_CUDA(launch(reduce_expz_ptr(p.dtype == VQC_C128), dim3(std::max(blocks, 1)), dim3(256), args, 0, stream));
     return VQC_OK;
 }
 
@@ -953,42 +981,25 @@ vqc_status run_hbm_backward(const HostPlan& p, int B, const void* x, const void*
     C* Lam = reinterpret_cast<C*>(wsc + lay.lam);
     R* rho = reinterpret_cast<R*>(wsc + lay.part);
     R* terms = reinterpret_cast<R*>(wsc + lay.terms);
-    void* ps_g = wsc + lay.ps;
-    if (p.dtype == VQC_C128 || !psi_final) {   // complex64 backward passes evaluate their own entries
-        st = launch_ps_tables<R>(p, B, x, w, ps_g, stream);
-        if (st != VQC_OK) return st;
-    }
+    const void *ps_g = wsc + lay.ps, *sh_g = wsc + lay.sh;
+    st = launch_tables<R>(p, B, x, w, wsc + lay.ps, wsc + lay.sh, stream);
+    if (st != VQC_OK) return st;
     const C* src0 = static_cast<const C*>(psi_final);
     if (!src0) {
-        // recompute the final state into Psi (the forward passes need no <Z>)
+        // recompute the final state into Psi (no <Z>); lam's region holds the
+        // state between these passes
         PassGeo Lf;
         st = plan_hbm(p, 0, B, Lf);
         if (st != VQC_OK) return st;
-        const int npf = (int)Lf.s->passes.size();
-        for (int i = 0; i < npf; ++i) {
-            PArgs<R> a{};
-            fill_pass_args<R>(p, Lf, Lf.s->passes[i], a);
-            a.ps_g = ps_g;
-            a.B = B;
-            a.x = static_cast<const R*>(x);
-            a.w = static_cast<const R*>(w);
-            a.src_psi = i == 0 ? static_cast<const C*>(psi0) : Psi;
-            a.dst_psi = Psi;
-            a.src_raw = i > 0;
-            a.dst_raw = 1;   // read only by the backward passes below
-            void* args[] = {&a};
-            VQC_CUDA(launch(Lf.fn, dim3(Lf.grid), dim3(Lf.block), args, Lf.smem, stream));
-        }
+        st = forward_passes<R>(p, Lf, B, psi0, Lam, Psi, true, static_cast<R*>(nullptr), ps_g, sh_g, stream);
+        if (st != VQC_OK) return st;
         src0 = Psi;
     }
     const int np = (int)L.s->passes.size();
     for (int i = np - 1; i >= 0; --i) {
         PArgs<R> a{};
-        fill_pass_args<R>(p, L, L.s->passes[i], a);
-        a.ps_g = ps_g;
+        fill_pass_args<R>(p, L, L.s->passes[i], ps_g, sh_g, a);
         a.B = B;
-        a.x = static_cast<const R*>(x);
-        a.w = static_cast<const R*>(w);
         a.gE = static_cast<const R*>(gE);
         const bool first = i == np - 1, last = i == 0;
         a.src_psi = first ? src0 : Psi;
@@ -1005,8 +1016,7 @@ vqc_status run_hbm_backward(const HostPlan& p, int B, const void* x, const void*
     const char* base = static_cast<const char*>(p.dbuf);
     const bool dbl = p.dtype == VQC_C128;
     int nt = (int)p.term_src.size();
-    const bool want = (dx && p.num_x > 0) || (dw && p.num_w > 0);
-    if (want && !p.accs.empty()) {   // per-sample gradient terms from the per-tile rho sums
+    if (((dx && p.num_x > 0) || (dw && p.num_w > 0)) && !p.accs.empty()) {   // per-sample gradient terms from the per-tile rho sums
         const R* r = rho;
         int Bi = B, ntl = L.ntiles, na = (int)p.accs.size(), Px = p.num_x;
         const DAcc* accs = reinterpret_cast<const DAcc*>(base + p.dev_accs);
@@ -1022,25 +1032,28 @@ vqc_status run_hbm_backward(const HostPlan& p, int B, const void* x, const void*
         VQC_CUDA(launch(p.dfloat ? reduce_terms_ptr_dd() : reduce_terms_ptr(dbl), dim3(std::max(blocks, 1)),
                         dim3(256), args, 0, stream));
     }
-    if (dx && p.num_x > 0) {
-        const R* t = terms;
-        int Bi = B, ntl = 1, Px = p.num_x;
-        const int32_t* ptr = reinterpret_cast<const int32_t*>(base + p.dev_xocc_ptr);
-        const int32_t* occ = reinterpret_cast<const int32_t*>(base + p.dev_xocc);
-        R* o = static_cast<R*>(dx);
-        void* args[] = {&t, &Bi, &ntl, &nt, &ptr, &occ, &Px, &o};
-        const int blocks = (int)std::min<long long>(4096, ((long long)B * Px + 255) / 256);
-        VQC_CUDA(launch(reduce_dx_ptr(dbl), dim3(std::max(blocks, 1)), dim3(256), args, 0,
-                                  stream));
+    const R* t = terms;
+    const int32_t* xptr = reinterpret_cast<const int32_t*>(base + p.dev_xocc_ptr);
+    const int32_t* xocc = reinterpret_cast<const int32_t*>(base + p.dev_xocc);
+    const int32_t* wptr = reinterpret_cast<const int32_t*>(base + p.dev_wocc_ptr);
+    const int32_t* wocc = reinterpret_cast<const int32_t*>(base + p.dev_wocc);
+    R *ox = static_cast<R*>(dx), *ow = static_cast<R*>(dw);
+    int Bi = B, Px = p.num_x, Pw = p.num_w;
+    const bool want_x = dx && Px > 0, want_w = dw && Pw > 0;
+    const int xblocks = (int)std::max<long long>(1, std::min<long long>(4096, ((long long)B * Px + 255) / 256));
+    if (!dbl && want_x && want_w) {
+        void* args[] = {&t, &Bi, &nt, &xptr, &xocc, &Px, &ox, &wptr, &wocc, &Pw, &ow};
+        VQC_CUDA(launch(reduce_grads_ptr(), dim3(Pw + xblocks), dim3(256), args, 0, stream));
+        return VQC_OK;
     }
-    if (dw && p.num_w > 0) {
-        const R* t = terms;
+    if (want_x) {
+        void* args[] = {&t, &Bi, &nt, &xptr, &xocc, &Px, &ox};
+        VQC_CUDA(launch(reduce_dx_ptr(dbl), dim3(xblocks), dim3(256), args, 0, stream));
+    }
+    if (want_w) {
         long long rows = B;
-        const int32_t* ptr = reinterpret_cast<const int32_t*>(base + p.dev_wocc_ptr);
-        const int32_t* occ = reinterpret_cast<const int32_t*>(base + p.dev_wocc);
-        R* o = static_cast<R*>(dw);
-        void* args[] = {&t, &rows, &nt, &ptr, &occ, &o};
-        VQC_CUDA(launch(reduce_dw_ptr(dbl), dim3(p.num_w), dim3(256), args, 0, stream));
+        void* args[] = {&t, &rows, &nt, &wptr, &wocc, &ow};
+        VQC_CUDA(launch(reduce_dw_ptr(dbl), dim3(Pw), dim3(256), args, 0, stream));
     }
     return VQC_OK;
 }
@@ -1049,12 +1062,12 @@ vqc_status run_hbm_backward(const HostPlan& p, int B, const void* x, const void*
 // ask for the HBM path), else the HBM path.
 bool use_hbm(const HostPlan& p, int mode, int B) {
     const char* f = std::getenv("VQC_FORCE_PATH");
-    if (f && std::string(f) == "hbm" && find_hbm_schedule(p, mode)) return true;
+    if (f && std::string(f) == "hbm" && find_frame(p, mode, VQC_PATH_HBM)) return true;
     Launch L;
     std::string saved = g_err;
     if (plan_launch(p, mode, B, L) == VQC_OK) return false;
     g_err = saved;
-    return find_hbm_schedule(p, mode) != nullptr;
+    return find_frame(p, mode, VQC_PATH_HBM) != nullptr;
 }
 
 // vqc_forward_backward on the resident path: one launch of the fused kernel,
@@ -1284,6 +1297,10 @@ size_t vqc_workspace_bytes(const vqc_plan* plan, int32_t batch, int32_t mode) {
                 need = std::max(need, bwd_workspace(p, L));
             }
         }
+        if (batch > 0 && !use_cluster(p, 1) && use_hbm(p, 1, batch)) {
+            // the final states in the backward's psi region, the forward's workspace behind them
+            need = std::max(need, hbm_state_bytes(p, batch) + vqc_workspace_bytes(plan, batch, 0));
+        }
         if (batch > 0 && use_cluster(p, 1)) {   // [either call's workspace | final states]
             const size_t cs = p.dtype == VQC_C128 ? 16 : 8;
             need = align256(need) + align256(((size_t)batch << p.n) * cs);
@@ -1380,9 +1397,9 @@ vqc_status vqc_forward(const vqc_plan* plan, int32_t batch, const void* x, const
         if (use_hbm(p, 0, batch)) {
             if (p.dtype == VQC_C64)
                 return run_hbm_forward<float>(p, batch, x, w, psi0, expz_out, state_out, workspace,
-                                              workspace_bytes, s, true);
+                                              workspace_bytes, s);
             return run_hbm_forward<double>(p, batch, x, w, psi0, expz_out, state_out, workspace,
-                                           workspace_bytes, s, true);
+                                           workspace_bytes, s);
         }
         if (p.dtype == VQC_C64)
             return run<float>(p, 0, batch, x, w, psi0, nullptr, nullptr, expz_out, state_out,
@@ -1496,9 +1513,8 @@ vqc_status vqc_forward_backward(const vqc_plan* plan, int32_t batch, const void*
         }
         // states beyond one SM: the forward (passes or cluster) leaves the final
         // states in the psi region of the backward's HBM layout, in this
-        // workspace, and the backward passes start from them (the forward's own
-        // working state is that region too, and its <Z> partials sit where the
-        // backward's lam goes: both are consumed before the backward starts)
+        // workspace, and the backward passes start from them; the forward's own
+        // workspace follows them, where the backward's lam goes later
         if (use_hbm(p, 1, batch)) {
             PassGeo Lb;
             st = plan_hbm(p, 1, batch, Lb);
@@ -1508,9 +1524,11 @@ vqc_status vqc_forward_backward(const vqc_plan* plan, int32_t batch, const void*
             if (!workspace || workspace_bytes < need || misaligned(workspace, 256))
                 return fail(VQC_ERR_WORKSPACE, "workspace must be >= " + std::to_string(need) +
                                                    " bytes and 256-byte aligned");
-            void* psi_final = static_cast<char*>(workspace) + lay.state;
-            st = vqc_forward(plan, batch, x, w, psi0, expz_out, psi_final, workspace, workspace_bytes,
-                             stream);
+            char* base = static_cast<char*>(workspace);
+            const size_t sbytes = hbm_state_bytes(p, batch);
+            void* psi_final = base + lay.state;
+            st = vqc_forward(plan, batch, x, w, psi0, expz_out, psi_final, base + sbytes,
+                             workspace_bytes - sbytes, stream);
             if (st != VQC_OK) return st;
             return vqc_backward(plan, batch, x, w, psi0, psi_final, grad_expz, grad_x, grad_w,
                                 workspace, workspace_bytes, stream);
@@ -1565,9 +1583,23 @@ vqc_status vqc_plan_info(const vqc_plan* plan, int32_t batch, vqc_plan_stats* ou
         const int K = choose_k(p, mode, B, sms);
         const bool clu = use_cluster(p, mode);
         const bool hbm = !clu && (ndev > 0 ? use_hbm(p, mode, B)
-                                           : (K == 0 && find_hbm_schedule(p, mode) != nullptr));
-        const Schedule* s = clu ? find_cluster_schedule(p, mode)
-                          : hbm ? find_hbm_schedule(p, mode) : (K ? find_schedule(p, mode, K) : nullptr);
+                                           : (K == 0 && find_frame(p, mode, VQC_PATH_HBM) != nullptr));
+        if (hbm) {
+            const FrameSchedule* s = find_frame(p, mode, VQC_PATH_HBM);
+            const int P = (int)s->passes.size();
+            *path = s->path;
+            *kk = s->K;
+            *ns = (int)s->stages.size();
+            *tq = s->m;
+            *np = P;
+            *tps = (1 << (s->m - s->K)) << (p.n - s->m);
+            // state traffic: forward reads and writes the state once per pass;
+            // the backward reads psi (and lam after the first pass) and writes
+            // both (except after the last pass)
+            *hb = mode == 0 ? 2.0 * P * sbytes : (4.0 * P - 3.0) * sbytes;
+            continue;
+        }
+        const Schedule* s = clu ? find_cluster_schedule(p, mode) : (K ? find_schedule(p, mode, K) : nullptr);
         if (!s) {
             *path = -1;
             continue;
@@ -1576,18 +1608,8 @@ vqc_status vqc_plan_info(const vqc_plan* plan, int32_t batch, vqc_plan_stats* ou
         *kk = s->K;
         *ns = (int)s->stages.size();
         *tq = s->m;
-        if (hbm) {
-            const int P = (int)s->passes.size();
-            *np = P;
-            *tps = (1 << (s->m - s->K)) << (p.n - s->m);
-            // state traffic: forward reads and writes the state once per pass;
-            // the backward reads psi (and lam after the first pass) and writes
-            // both (except after the last pass)
-            *hb = mode == 0 ? 2.0 * P * sbytes : (4.0 * P - 3.0) * sbytes;
-        } else {
-            *np = 1;
-            *tps = 1 << (p.n - s->K);
-        }
+        *np = 1;
+        *tps = 1 << (p.n - s->K);
     }
     g_err = saved;
     return VQC_OK;
@@ -1638,6 +1660,22 @@ vqc_status vqc_sync_check(void* stream) {
                         ((tripped & 2u) ? " HBM pass geometry" : "") +
                         ((tripped & 4u) ? " cluster geometry" : "") + " (the work was skipped)");
     return stage_error_check();   // vqc_stage_apply's tensor-core waits
+}
+
+// The frame schedules' records (frame.h), for the CPU tests; like vqc_plan_export.
+vqc_status vqc_frames_export(const vqc_plan* plan, void* buf, size_t* inout_bytes) {
+    if (!plan || !inout_bytes) return fail(VQC_ERR_INVALID_ARG, "NULL argument");
+    try {
+        std::vector<uint8_t> b = export_frames(plan->hp);
+        size_t cap = *inout_bytes;
+        *inout_bytes = b.size();
+        if (!buf) return VQC_OK;
+        if (cap < b.size()) return fail(VQC_ERR_INVALID_ARG, "buffer too small");
+        std::memcpy(buf, b.data(), b.size());
+        return VQC_OK;
+    } catch (...) {
+        return fail(VQC_ERR_OUT_OF_MEMORY, "export failed");
+    }
 }
 
 const char* vqc_last_error(void) { return g_err.c_str(); }

@@ -718,7 +718,21 @@ vqc_status compile_host(const vqc_gate* gates, int32_t G, int32_t n, int32_t nx,
         build_hbm_schedule(p, s);
         p.scheds.push_back(std::move(s));
     }
+    for (int mode = 0; mode < 2; ++mode) {
+        const Schedule* h = find_hbm_schedule(p, mode);
+        if (!h) continue;
+        int fm = std::min(frame_tile_qubits(mode, dtype), n - 1);
+        const int env_m = std::getenv("VQC_HBM_TILE_QUBITS") ? std::atoi(std::getenv("VQC_HBM_TILE_QUBITS")) : 0;
+        if (env_m > p.G_swz && env_m < n) fm = h->m;
+        p.frames.push_back(build_frame_schedule(p, mode, VQC_PATH_HBM, fm, h->K));
+    }
     return VQC_OK;
+}
+
+const FrameSchedule* find_frame(const HostPlan& p, int mode, int path, int K) {
+    for (const auto& s : p.frames)
+        if (s.mode == mode && s.path == path && (K == 0 || s.K == K)) return &s;
+    return nullptr;
 }
 
 const Schedule* find_schedule(const HostPlan& p, int mode, int K) {

@@ -7,6 +7,7 @@
 #include <string>
 #include <vector>
 
+#include "frame.h"
 #include "plan.h"
 #include "../../include/vqc.h"
 
@@ -61,6 +62,7 @@ struct HostPlan {
     int n_ps = 0, n_sh = 0;                // per-sample / shared table sizes
     int n_runs = 0;
     std::vector<Schedule> scheds;
+    std::vector<FrameSchedule> frames;     // what the HBM-tiled kernels run
     double fwd_flops = 0, bwd_flops = 0, recompute_flops = 0;
 
     // device copy
@@ -89,6 +91,12 @@ inline int hbm_k(int mode, int dtype) {
     return mode == 0 ? 4 : 3;
 }
 
+// Tile qubits of the frame schedules of the HBM passes.
+inline int frame_tile_qubits(int mode, int dtype) {
+    if (dtype == VQC_C64) return mode == 0 ? 13 : 12;
+    return mode == 0 ? 12 : 11;
+}
+
 // Maximum K per (mode, dtype) for register-resident blocks.
 inline int max_k(int mode, int dtype) {
     if (dtype == VQC_C64) return mode == 0 ? 5 : 4;
@@ -101,6 +109,7 @@ vqc_status compile_host(const vqc_gate* gates, int32_t G, int32_t n, int32_t nx,
 const Schedule* find_schedule(const HostPlan& p, int mode, int K);
 const Schedule* find_hbm_schedule(const HostPlan& p, int mode);
 const Schedule* find_cluster_schedule(const HostPlan& p, int mode);
+const FrameSchedule* find_frame(const HostPlan& p, int mode, int path, int K = 0);
 std::vector<uint8_t> export_plan(const HostPlan& p);
 
 }  // namespace vqc

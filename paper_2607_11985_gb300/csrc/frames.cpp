@@ -1,0 +1,812 @@
+// frames.cpp -- builds the frame schedules of frame.h from a plan's op list.
+#include <algorithm>
+#include <cstring>
+
+#include "engine.h"
+
+namespace vqc {
+namespace {
+
+bool odd(uint32_t v) { return (__builtin_popcount(v) & 1) != 0; }
+
+// An op in the storage frame: a run (direction d, selector r), or a diagonal op
+// on the parities r and r2.
+struct FOp {
+    bool run = false;
+    uint32_t d = 0, r = 0, r2 = 0;
+    int hop = -1;
+};
+
+bool commute(const FOp& a, const FOp& b) {
+    if (a.run && b.run) return !odd(a.r & b.d) && !odd(b.r & a.d);
+    if (a.run) return !odd(b.r & a.d) && !odd(b.r2 & a.d);
+    if (b.run) return !odd(a.r & b.d) && !odd(a.r2 & b.d);
+    return true;
+}
+
+// The subspace spanned by the vectors added so far.
+struct Span {
+    uint32_t piv[32] = {0};   // by highest set bit
+    int dim = 0;
+    uint32_t reduce(uint32_t v) const {
+        while (v) {
+            const int h = 31 - __builtin_clz(v);
+            if (!piv[h]) return v;
+            v ^= piv[h];
+        }
+        return 0;
+    }
+    bool add(uint32_t v) {
+        v = reduce(v);
+        if (!v) return false;
+        piv[31 - __builtin_clz(v)] = v;
+        ++dim;
+        return true;
+    }
+    std::vector<uint32_t> basis() const {
+        std::vector<uint32_t> b;
+        for (uint32_t v : piv)
+            if (v) b.push_back(v);
+        return b;
+    }
+};
+
+// Coordinates in a basis: coord(v) has bit i set when basis vector i is in v.
+struct Coords {
+    uint32_t piv[32] = {0}, comb[32] = {0};
+    explicit Coords(const std::vector<uint32_t>& b) {
+        for (size_t i = 0; i < b.size(); ++i) {
+            uint32_t v = b[i], c = 1u << i;
+            while (v) {
+                const int h = 31 - __builtin_clz(v);
+                if (!piv[h]) {
+                    piv[h] = v;
+                    comb[h] = c;
+                    break;
+                }
+                v ^= piv[h];
+                c ^= comb[h];
+            }
+        }
+    }
+    uint32_t operator()(uint32_t v) const {
+        uint32_t c = 0;
+        while (v) {
+            const int h = 31 - __builtin_clz(v);
+            c ^= comb[h];
+            v ^= piv[h];
+        }
+        return c;
+    }
+};
+
+// The vectors of span(vs) on which every functional of `sel` is even (a basis).
+std::vector<uint32_t> annihilated(std::vector<uint32_t> vs, const std::vector<uint32_t>& sel) {
+    for (uint32_t s : sel) {
+        int k = -1;
+        for (size_t i = 0; i < vs.size(); ++i)
+            if (odd(vs[i] & s)) {
+                if (k < 0) k = (int)i;
+                else vs[i] ^= vs[k];
+            }
+        if (k >= 0) vs.erase(vs.begin() + k);
+    }
+    return vs;
+}
+
+uint32_t image(const std::vector<uint32_t>& cols, uint32_t v) {   // XOR of cols[i] over v's bits
+    uint32_t r = 0;
+    for (size_t i = 0; i < cols.size(); ++i)
+        if ((v >> i) & 1) r ^= cols[i];
+    return r;
+}
+
+std::vector<uint32_t> inverse(std::vector<uint32_t> cols) {   // of an invertible matrix, as columns
+    const size_t n = cols.size();
+    std::vector<uint32_t> inv(n);
+    for (size_t i = 0; i < n; ++i) inv[i] = 1u << i;
+    for (size_t b = 0; b < n; ++b) {
+        size_t k = b;
+        while (!((cols[k] >> b) & 1)) ++k;
+        std::swap(cols[k], cols[b]);
+        std::swap(inv[k], inv[b]);
+        for (size_t j = 0; j < n; ++j)
+            if (j != b && ((cols[j] >> b) & 1)) {
+                cols[j] ^= cols[b];
+                inv[j] ^= inv[b];
+            }
+    }
+    return inv;
+}
+
+// Ops looked ahead of the first one that has to wait.  Beyond a few layers of
+// the widest circuit nothing can run early any more.
+constexpr size_t kLookahead = 160;
+// Table entries and accumulators of one pass: bounds its shared memory.
+constexpr int kMaxPassEntries = 96;
+
+struct StagePlan {
+    std::vector<int> ops;              // indices into the FOp list, time order
+    std::vector<uint32_t> D, R;        // directions and selectors of its runs, by local position
+    std::vector<uint32_t> sels;        // distinct selectors of its diagonal ops
+};
+
+// Cut a pass's ops into stages of at most K directions.
+std::vector<StagePlan> cut(const std::vector<FOp>& f, const std::vector<int>& ops, int K) {
+    std::vector<StagePlan> out;
+    std::vector<int> rem = ops;
+    do {   // an empty op list still gets one (empty) stage
+        StagePlan s;
+        std::vector<int> defer;
+        size_t i = 0;
+        for (; i < rem.size() && defer.size() <= kLookahead; ++i) {
+            const FOp& o = f[rem[i]];
+            bool ok = true;
+            for (int x : defer)
+                if (!commute(o, f[x])) { ok = false; break; }
+            if (ok && o.run) {
+                size_t j = 0;
+                while (j < s.D.size() && !(s.D[j] == o.d && s.R[j] == o.r)) ++j;
+                if (j == s.D.size()) {   // a new direction: dual to the others and to the parities
+                    ok = (int)s.D.size() < K;
+                    Span sp;
+                    for (uint32_t d : s.D) sp.add(d);
+                    ok = ok && sp.reduce(o.d) != 0;
+                    for (size_t k = 0; ok && k < s.D.size(); ++k)
+                        ok = !odd(s.R[k] & o.d) && !odd(o.r & s.D[k]);
+                    for (size_t k = 0; ok && k < s.sels.size(); ++k)
+                        ok = !odd(s.sels[k] & o.d) || s.sels[k] == o.r;
+                    if (ok) {
+                        s.D.push_back(o.d);
+                        s.R.push_back(o.r);
+                    }
+                }
+            } else if (ok) {
+                std::vector<uint32_t> add;
+                for (uint32_t r : {o.r, o.r2}) {   // a parity that a run changes is that run's own
+                    for (size_t k = 0; k < s.D.size(); ++k) ok = ok && (!odd(r & s.D[k]) || r == s.R[k]);
+                    if (std::find(s.sels.begin(), s.sels.end(), r) == s.sels.end()) add.push_back(r);
+                }
+                ok = ok && s.sels.size() + add.size() <= (size_t)kMaxSelectors;
+                if (ok) s.sels.insert(s.sels.end(), add.begin(), add.end());
+            }
+            (ok ? s.ops : defer).push_back(rem[i]);
+        }
+        defer.insert(defer.end(), rem.begin() + i, rem.end());
+        out.push_back(std::move(s));
+        rem.swap(defer);
+    } while (!rem.empty());
+    return out;
+}
+
+// Complete a stage's D to K vectors of the tile: every pad is even on the runs'
+// selectors, meets at most one diagonal selector, and no selector meets two of D.
+// False when the diagonal ops leave no such pads.
+bool pad(StagePlan& s, const std::vector<uint32_t>& V, int K) {
+    std::vector<uint32_t> A = annihilated(V, s.R);
+    std::vector<uint32_t> free = annihilated(A, s.sels);
+    // A's vectors dual to the diagonal selectors that D does not meet yet, then the free ones
+    std::vector<uint32_t> cand = free;
+    std::vector<uint32_t> rest = A;
+    for (size_t i = 0; i < s.sels.size(); ++i) {
+        int k = -1;
+        for (size_t j = 0; j < rest.size(); ++j)
+            if (odd(rest[j] & s.sels[i])) {
+                if (k < 0) k = (int)j;
+                else rest[j] ^= rest[k];
+            }
+        if (k < 0) continue;
+        uint32_t v = rest[k];
+        rest.erase(rest.begin() + k);
+        for (size_t l = i + 1; l < s.sels.size(); ++l)   // even on the later selectors if the rest allows it
+            if (odd(v & s.sels[l]))
+                for (uint32_t t : rest) {
+                    bool only = odd(t & s.sels[l]);
+                    for (size_t q = i + 1; only && q < l; ++q) only = !odd(t & s.sels[q]);
+                    if (only) { v ^= t; break; }
+                }
+        cand.push_back(v);
+    }
+    Span sp;
+    for (uint32_t d : s.D) sp.add(d);
+    for (uint32_t v : cand) {
+        if ((int)s.D.size() == K) break;
+        if (!sp.reduce(v)) continue;
+        bool ok = true;
+        int hits = 0;
+        for (uint32_t r : s.sels) {
+            if (!odd(r & v)) continue;
+            ++hits;
+            for (uint32_t d : s.D) ok = ok && !odd(r & d);
+        }
+        ok = ok && hits <= 1;
+        if (!ok) continue;
+        sp.add(v);
+        s.D.push_back(v);
+    }
+    return (int)s.D.size() == K;
+}
+
+struct PassPlan {
+    std::vector<int> ops;
+    std::vector<uint32_t> V;           // basis of the tile's subspace
+    std::vector<StagePlan> stages;
+};
+
+// A base vector of the stage moved along D so that every selector with a local
+// bit is even on it: the local bit alone is then the parity.
+uint32_t settle(const StagePlan& s, uint32_t v) {
+    const size_t nr = s.R.size();
+    for (size_t k = 0; k < nr; ++k)
+        if (odd(s.R[k] & v)) v ^= s.D[k];
+    for (uint32_t r : s.sels)
+        for (size_t k = nr; k < s.D.size(); ++k)
+            if (odd(r & s.D[k]) && odd(r & v)) v ^= s.D[k];
+    return v;
+}
+
+int rank_of(const std::vector<uint32_t>& v) {
+    Span s;
+    for (uint32_t x : v) s.add(x);
+    return s.dim;
+}
+
+struct Rng {   // small deterministic generator (xorshift32) for the swizzle search
+    uint32_t s = 2463534242u;
+    uint32_t next() {
+        s ^= s << 13;
+        s ^= s >> 17;
+        s ^= s << 5;
+        return s;
+    }
+};
+
+}  // namespace
+
+FrameSchedule build_frame_schedule(const HostPlan& p, int mode, int path, int m, int K) {
+    const int n = p.n, G = std::min(p.G_swz, m);
+    const bool tiled = path == VQC_PATH_HBM;
+    FrameSchedule S;
+    S.mode = mode;
+    S.K = K;
+    S.m = m;
+    S.path = path;
+    S.nout = n - m;
+    const int nout = n - m;
+
+    // the op list in the storage frame
+    std::vector<uint32_t> dir(n), sel(n);
+    for (int q = 0; q < n; ++q) dir[q] = sel[q] = 1u << q;
+    std::vector<FOp> f;
+    for (size_t i = 0; i < p.ops.size(); ++i) {
+        const HOp& o = p.ops[i];
+        if (o.type == OP_CX) {
+            sel[o.q1] ^= sel[o.q0];
+            dir[o.q0] ^= dir[o.q1];
+            continue;
+        }
+        FOp g;
+        g.hop = (int)i;
+        g.run = o.type == OP_M1;
+        g.r = sel[o.q0];
+        if (g.run) g.d = dir[o.q0];
+        else g.r2 = sel[o.q1];
+        f.push_back(g);
+    }
+
+    // ---- passes: each takes, in time order, every op that commutes with the ops
+    // it leaves behind while the tile has room for its direction.  At most m - G
+    // directions lie outside the previous tile (G shared ones carry the 128-byte
+    // lines); the last tile also holds the directions of the G lowest logical
+    // qubits, in whose order the final state is written.
+    std::vector<PassPlan> passes;
+    std::vector<int> rem(f.size());
+    for (size_t i = 0; i < f.size(); ++i) rem[i] = (int)i;
+    if (!tiled) {
+        PassPlan ps;
+        ps.ops = rem;
+        for (int q = 0; q < n; ++q) ps.V.push_back(1u << q);
+        passes.push_back(std::move(ps));
+    } else {
+        std::vector<uint32_t> prev, last_dirs(dir.begin(), dir.begin() + G);
+        // the forward's first tile holds the lines of the given state; the
+        // backward's first is its last to run and writes nothing
+        for (int i = 0; i < G; ++i) prev.push_back(1u << i);
+        bool shares = mode == 0;
+        for (;;) {
+            const int room = shares ? m - G : m;   // directions outside the previous tile
+            struct Try {
+                Span v, mod;                 // the tile; the previous tile plus the tile
+                std::vector<int> taken, left;
+                int fresh = 0;               // directions outside the previous tile
+                bool add(uint32_t d, int m, int room) {
+                    if (!v.reduce(d)) return true;
+                    const bool f = mod.reduce(d) != 0;
+                    if (v.dim >= m || (f && fresh >= room)) return false;
+                    v.add(d);
+                    if (f) { mod.add(d); ++fresh; }
+                    return true;
+                }
+            };
+            auto attempt = [&](const std::vector<uint32_t>& pre, Try& t) {
+                for (uint32_t d : prev) t.mod.add(d);
+                for (uint32_t d : pre)
+                    if (!t.add(d, m, room)) return false;
+                int entries = 0;
+                std::vector<char> have(p.entries.size(), 0);
+                size_t i = 0;
+                for (; i < rem.size() && t.left.size() <= kLookahead; ++i) {
+                    const FOp& o = f[rem[i]];
+                    bool ok = true;
+                    for (int x : t.left)
+                        if (!commute(o, f[x])) { ok = false; break; }
+                    const int e = p.ops[o.hop].entry;
+                    const bool newe = e >= 0 && !have[e];
+                    if (ok && newe) ok = entries < kMaxPassEntries;
+                    if (ok && o.run) ok = t.add(o.d, m, room);
+                    if (ok && newe) {
+                        have[e] = 1;
+                        ++entries;
+                    }
+                    (ok ? t.taken : t.left).push_back(rem[i]);
+                }
+                t.left.insert(t.left.end(), rem.begin() + i, rem.end());
+                return true;
+            };
+            Try fin, t;
+            const bool can_end = attempt(last_dirs, fin);
+            const bool end = can_end && fin.left.empty();
+            if (!end) {
+                attempt({}, t);
+                if (t.left.empty()) {
+                    if (can_end) {
+                        t = fin;
+                    } else {   // move towards the last tile
+                        for (uint32_t d : last_dirs) t.add(d, m, room);
+                    }
+                }
+            } else {
+                t = fin;
+            }
+            // fill up: G directions shared with the previous tile (its last-tile
+            // directions first), then unit vectors
+            {
+                std::vector<uint32_t> shared;
+                Span pv;
+                for (uint32_t d : prev) pv.add(d);
+                for (uint32_t d : last_dirs)
+                    if (!pv.reduce(d)) shared.push_back(d);
+                shared.insert(shared.end(), prev.begin(), prev.end());
+                for (uint32_t d : shared)
+                    if (t.v.dim - t.fresh < G) t.add(d, m, room);
+                for (int q = 0; q < n; ++q) t.add(1u << q, m, room);
+                for (uint32_t d : shared) t.add(d, m, room);
+            }
+            PassPlan ps;
+            ps.ops = t.taken;
+            ps.V = t.v.basis();
+            prev = ps.V;
+            shares = true;
+            passes.push_back(std::move(ps));
+            rem.swap(t.left);
+            if (end) break;
+        }
+    }
+    const int np = (int)passes.size();
+
+    // ---- stages of each pass; a stage whose diagonal ops leave no room for its
+    // pads gives its later diagonal ops to a stage of their own
+    for (PassPlan& ps : passes) {
+        std::vector<StagePlan> st = cut(f, ps.ops, K), out;
+        for (StagePlan& s : st) {
+            std::vector<StagePlan> work{s};
+            while (!work.empty()) {
+                StagePlan w = work.back();
+                work.pop_back();
+                StagePlan w0 = w;
+                if (pad(w, ps.V, K)) {
+                    out.push_back(std::move(w));
+                    continue;
+                }
+                // split in time order: the first half's ops, then the second's
+                std::vector<int> a(w0.ops.begin(), w0.ops.begin() + (w0.ops.size() + 1) / 2),
+                    b(w0.ops.begin() + (w0.ops.size() + 1) / 2, w0.ops.end());
+                std::vector<StagePlan> sb = cut(f, b, K), sa = cut(f, a, K);
+                for (size_t i = sb.size(); i-- > 0;) work.push_back(sb[i]);
+                for (size_t i = sa.size(); i-- > 0;) work.push_back(sa[i]);
+            }
+        }
+        ps.stages = std::move(out);
+    }
+
+    // ---- addresses, slots and records, in the order the passes run (the backward
+    // from the last).  A pass reads the state at the addresses M s; the forward
+    // starts at M = 1 (a state in logical order before the first gate) and writes
+    // logical order at its end, the backward starts there.
+    std::vector<uint32_t> M(n), Minv(n);   // columns: address of e_i; index vector of address bit i
+    for (int i = 0; i < n; ++i) {
+        M[i] = Minv[i] = 1u << i;
+        if (mode == 1) {
+            Minv[i] = dir[i];
+            M[i] = 0;
+            for (int j = 0; j < n; ++j) M[i] |= ((sel[j] >> i) & 1u) << j;
+        }
+    }
+    S.passes.resize(np);
+    S.fin = FFinal{};
+    Rng rng;
+    for (int step = 0; step < np; ++step) {
+        const int pi = mode == 0 ? step : np - 1 - step;
+        PassPlan& ps = passes[pi];
+        const bool last = pi == np - 1, end = step == np - 1;
+        FPass fp{};
+        // the tile's addresses as read: a reduced echelon basis with the G low units first
+        std::vector<uint32_t> gin, vin, opos, ovec;
+        auto echelon = [&](const std::vector<uint32_t>& addr, std::vector<uint32_t>& g) {
+            uint32_t lowm = (1u << G) - 1;
+            g.clear();
+            for (int i = 0; i < G; ++i) g.push_back(1u << i);
+            std::vector<uint32_t> r;
+            for (uint32_t a : addr) r.push_back(a & ~lowm);
+            Span sp;
+            for (uint32_t a : r) sp.add(a);
+            std::vector<uint32_t> b = sp.basis();   // ascending highest bit
+            for (size_t i = 0; i < b.size(); ++i)   // fully reduce
+                for (size_t j = 0; j < i; ++j) {
+                    const int h = 31 - __builtin_clz(b[j]);
+                    if ((b[i] >> h) & 1) b[i] ^= b[j];
+                }
+            g.insert(g.end(), b.begin(), b.end());
+        };
+        if (tiled) {
+            std::vector<uint32_t> addr;
+            for (uint32_t v : ps.V) addr.push_back(image(M, v));
+            echelon(addr, gin);
+        } else {
+            for (int i = 0; i < n; ++i) gin.push_back(1u << i);
+        }
+        uint32_t pivots = 0;
+        for (uint32_t g : gin) pivots |= 1u << (31 - __builtin_clz(g));
+        for (uint32_t g : gin) vin.push_back(image(Minv, g));
+        for (int b = 0; b < n; ++b)
+            if (!((pivots >> b) & 1)) {
+                opos.push_back(1u << b);
+                ovec.push_back(Minv[b]);
+            }
+        const Coords coord(vin);
+
+        // directions that the written lines will hold: ones that the next tile has
+        // too, at the forward's end the last logical ones
+        std::vector<uint32_t> line;
+        if (end) {
+            if (mode == 0) line.assign(dir.begin(), dir.begin() + G);
+        } else {
+            // V intersect V': vectors of V whose sum with V' vectors vanishes
+            const std::vector<uint32_t>&a = ps.V, &b = passes[pi + (mode == 0 ? 1 : -1)].V;
+            uint32_t piv[32] = {0}, ca[32] = {0};
+            auto ins = [&](uint32_t v, uint32_t c, bool fromb) {
+                while (v) {
+                    const int h = 31 - __builtin_clz(v);
+                    if (!piv[h]) {
+                        piv[h] = v;
+                        ca[h] = c;
+                        return;
+                    }
+                    v ^= piv[h];
+                    c ^= ca[h];
+                }
+                if (fromb && (int)line.size() < G) line.push_back(c);
+            };
+            // c: the part of the combination that comes from V
+            for (uint32_t v : a) ins(v, v, false);
+            for (uint32_t v : b) ins(v, 0, true);
+        }
+
+        // swizzle: slot bits 0..G-1 of tile bit i >= G also get column F[i]; a random
+        // choice whose lanes hit distinct banks in every stage and both copies
+        std::vector<uint32_t> F(m, 0);
+        const int tb = m - K, gl = std::min(G, tb);   // lanes that must differ in the low gl slot bits
+        auto slot_of = [&](uint32_t c) {
+            uint32_t s = c;
+            for (int i = G; i < m; ++i)
+                if ((c >> i) & 1) s ^= F[i];
+            return s;
+        };
+        auto bank = [&](uint32_t v) { return slot_of(coord(v)) & ((1u << G) - 1); };
+        // the stages' thread spaces: V's vectors even on the runs' selectors, without the pads
+        struct Threads {
+            std::vector<uint32_t> basis;
+        };
+        std::vector<Threads> th(ps.stages.size());
+        for (size_t si = 0; si < ps.stages.size(); ++si) {
+            const StagePlan& s = ps.stages[si];
+            Span sp;
+            for (uint32_t d : s.D) sp.add(d);
+            for (uint32_t v : annihilated(vin, s.R))
+                if (sp.add(v)) th[si].basis.push_back(settle(s, v));
+        }
+        const int vbits = p.dtype == VQC_C64 ? 1 : 0;   // bits inside a 16-byte vector of amplitudes
+        auto score = [&]() {
+            int bad = 0;
+            for (const Threads& t : th) {
+                std::vector<uint32_t> b;
+                for (uint32_t v : t.basis) b.push_back(bank(v) & ((1u << gl) - 1));
+                bad += gl - rank_of(b);
+            }
+            std::vector<uint32_t> b;
+            for (int i = vbits; i < std::min(m, G + vbits); ++i) b.push_back(bank(vin[i]));
+            bad += std::min((int)b.size(), G) - rank_of(b);
+            b.clear();
+            for (uint32_t v : line) b.push_back(bank(v));
+            if (!b.empty()) bad += 2 * std::max(0, G - vbits - rank_of(b));
+            return bad;
+        };
+        {
+            std::vector<uint32_t> best = F;
+            int best_bad = 1 << 20;
+            for (int trial = 0; trial < 256 && best_bad > 0; ++trial) {
+                for (int i = G; i < m; ++i)   // the first trial: the plain fold of the high bits
+                    F[i] = trial == 0 ? 1u << (i % G) : (rng.next() >> 8) & ((1u << G) - 1);
+                const int bad = score();
+                if (bad < best_bad) {
+                    best_bad = bad;
+                    best = F;
+                }
+            }
+            F = best;
+        }
+
+        // written order: the line's directions lowest, chosen so that the lanes that
+        // read the tile back differ in their banks
+        std::vector<uint32_t> gout, vout;
+        if (end && mode == 0 && tiled) {
+            std::vector<uint32_t> addr;
+            for (uint32_t v : ps.V) {
+                uint32_t a = 0;
+                for (int j = 0; j < n; ++j) a |= (uint32_t)odd(sel[j] & v) << j;
+                addr.push_back(a);
+            }
+            echelon(addr, gout);
+            for (uint32_t g : gout) vout.push_back(image(dir, g));
+        } else if (!tiled && mode == 0) {
+            gout = gin;
+            vout = dir;
+        } else if (end) {   // the backward's end: nothing is written
+            gout = gin;
+            vout = vin;
+        } else {
+            gout = gin;
+            std::vector<uint32_t> l = line, pickd;
+            Span bs;
+            if (vbits) {   // the vector's own bit: the one whose bank the others can spare
+                for (size_t i = 0; i < l.size(); ++i) {
+                    std::vector<uint32_t> b;
+                    for (size_t j = 0; j < l.size(); ++j)
+                        if (j != i) b.push_back(bank(l[j]));
+                    if (rank_of(b) == (int)l.size() - 1 || i + 1 == l.size()) {
+                        std::swap(l[0], l[i]);
+                        break;
+                    }
+                }
+            }
+            vout = l;
+            Span sp;
+            for (uint32_t v : vout) sp.add(v);
+            for (size_t i = vbits; i < vout.size(); ++i) bs.add(bank(vout[i]));
+            std::vector<uint32_t> others;
+            for (uint32_t v : vin)
+                if (sp.add(v)) others.push_back(v);
+            for (size_t i = 0; i < others.size(); ++i)
+                if (bs.reduce(bank(others[i]))) {
+                    std::swap(others[0], others[i]);
+                    break;
+                }
+            vout.insert(vout.end(), others.begin(), others.end());
+        }
+        if (end && mode == 0 && tiled && vbits) {   // the same for the final order's fifth bit
+            Span bs;
+            for (int i = 1; i < G; ++i) bs.add(bank(vout[i]));
+            for (int i = G; i < m; ++i)
+                if (bs.reduce(bank(vout[i]))) {
+                    std::swap(vout[G], vout[i]);
+                    std::swap(gout[G], gout[i]);
+                    break;
+                }
+        }
+        for (int i = 0; i < m; ++i) {   // in / out: before and after the pass in circuit order
+            (mode == 0 ? fp.gin : fp.gout)[i] = gin[i];
+            (mode == 0 ? fp.gout : fp.gin)[i] = gout[i];
+            (mode == 0 ? fp.sin : fp.sout)[i] = (int32_t)slot_of(coord(vin[i]));
+            (mode == 0 ? fp.sout : fp.sin)[i] = (int32_t)slot_of(coord(vout[i]));
+        }
+        for (int o = 0; o < nout; ++o) {
+            fp.oin[o] = fp.oout[o] = opos[o];
+            if (!(end && mode == 0)) continue;
+            // logical order: the tile's address with the line's bits (and its other
+            // pivots) zero, and the slot that amplitude is in
+            uint32_t a = 0;
+            for (int j = 0; j < n; ++j) a |= (uint32_t)odd(sel[j] & ovec[o]) << j;
+            for (int i = m - 1; i >= 0; --i)
+                if ((a >> (31 - __builtin_clz(gout[i]))) & 1) {
+                    a ^= gout[i];
+                    fp.oslot[o] ^= fp.sout[i];
+                }
+            fp.oout[o] = a;
+        }
+
+        // tables of the pass (the resident path keeps the plan's own slots)
+        std::vector<int> slot_id(p.entries.size(), -1), acc_id(p.accs.size(), -1);
+        if (tiled) {
+            fp.ps_begin = (int32_t)S.pass_entries.size();
+            for (int want = 1; want >= 0; --want) {
+                if (!want) fp.sh_begin = (int32_t)S.pass_entries.size();
+                for (int x : ps.ops) {
+                    const int e = p.ops[f[x].hop].entry;
+                    if (e < 0 || slot_id[e] >= 0 || p.entries[e].per_sample != want) continue;
+                    slot_id[e] = want ? fp.ps_count++ : fp.sh_count++;
+                    S.pass_entries.push_back(e);
+                }
+            }
+            fp.acc_begin = (int32_t)S.pass_accs.size();
+            for (int x : ps.ops) {
+                const int e = p.ops[f[x].hop].entry;
+                if (e < 0 || p.entries[e].acc == 0xffff || acc_id[p.entries[e].acc] >= 0) continue;
+                acc_id[p.entries[e].acc] = fp.acc_count++;
+                S.pass_accs.push_back(p.entries[e].acc);
+            }
+        } else {
+            for (size_t i = 0; i < p.entries.size(); ++i) slot_id[i] = p.entries[i].slot;
+            for (size_t i = 0; i < p.accs.size(); ++i) acc_id[i] = (int)i;
+        }
+
+        // stage records
+        fp.stage_begin = (int32_t)S.stages.size();
+        fp.op_begin = (int32_t)S.ops.size();
+        for (size_t si = 0; si < ps.stages.size(); ++si) {
+            const StagePlan& s = ps.stages[si];
+            FStage st{};
+            for (int k = 0; k < K; ++k) st.sigma[k] = (int32_t)slot_of(coord(s.D[k]));
+            // thread vectors: the first gl with independent banks
+            std::vector<uint32_t> tv, others;
+            Span bs;
+            for (uint32_t v : th[si].basis) {
+                if ((int)tv.size() < gl && bs.add(bank(v) & ((1u << gl) - 1))) tv.push_back(v);
+                else others.push_back(v);
+            }
+            tv.insert(tv.end(), others.begin(), others.end());
+            st.nthreadbits = (uint8_t)tv.size();
+            // parities outside the registers
+            std::vector<uint32_t> outside;
+            auto ref = [&](uint32_t r) -> uint8_t {
+                for (int k = 0; k < K; ++k)
+                    if (odd(r & s.D[k])) return (uint8_t)k;
+                size_t i = 0;
+                while (i < outside.size() && outside[i] != r) ++i;
+                if (i == outside.size()) outside.push_back(r);
+                return (uint8_t)(kRefPhys + i);
+            };
+            st.op_begin = (int32_t)S.ops.size();
+            std::vector<DOp> recs;
+            uint8_t pm = 0;
+            bool pure = true;
+            for (int x : s.ops) {
+                const FOp& o = f[x];
+                const HOp& h = p.ops[o.hop];
+                DOp d{};
+                if (h.entry >= 0) {
+                    const DEntry& e = p.entries[h.entry];
+                    d.slot = (uint16_t)slot_id[h.entry];
+                    d.flags = (uint8_t)((e.per_sample ? OPF_PER_SAMPLE : 0) |
+                                        (e.acc != 0xffff ? OPF_HAS_ACC : 0) | h.gen);
+                    d.aux = e.acc != 0xffff ? (uint16_t)acc_id[e.acc] : (uint16_t)0xffff;
+                }
+                if (o.run) {
+                    int k = 0;
+                    while (s.D[k] != o.d || s.R[k] != o.r) ++k;
+                    d.a = (uint8_t)k;
+                    d.code = (uint8_t)(DC_M1 + k);
+                    pure = pure && !((pm >> k) & 1);
+                    pm |= (uint8_t)(1u << k);
+                } else {
+                    pure = false;
+                    uint8_t ra = ref(o.r), rb = ref(o.r2);
+                    const bool la = ra < kRefPhys, lb = rb < kRefPhys;
+                    if (h.type == OP_CZ) {
+                        if (la && lb) {
+                            if (ra > rb) std::swap(ra, rb);
+                            d.code = (uint8_t)(DC_CZ_LL + cz_pair_index(ra, rb));
+                        } else if (la || lb) {
+                            if (!la) std::swap(ra, rb);
+                            d.code = (uint8_t)(DC_CZ_PL + ra);
+                        } else {
+                            d.code = DC_CZ_PP;
+                        }
+                    } else if (la && lb) {
+                        d.code = (uint8_t)(DC_PH2_LL + cz_pair_index(std::min(ra, rb), std::max(ra, rb)));
+                    } else if (la || lb) {
+                        d.code = (uint8_t)(DC_PH2_PL + (la ? ra : rb));
+                    } else {
+                        d.code = DC_PH2_PP;
+                    }
+                    d.a = ra;
+                    d.b = rb;
+                }
+                recs.push_back(d);
+            }
+            if (pure) std::sort(recs.begin(), recs.end(), [](const DOp& a, const DOp& b) { return a.a < b.a; });
+            S.ops.insert(S.ops.end(), recs.begin(), recs.end());
+            st.op_end = (int32_t)S.ops.size();
+            st.pure = pure ? 1 : 0;
+            st.pmask = pure ? pm : 0;
+            st.nsel = (uint8_t)outside.size();
+            auto word = [&](uint32_t v) {
+                uint32_t w = 0;
+                for (size_t i = 0; i < outside.size(); ++i) w |= (uint32_t)odd(outside[i] & v) << i;
+                return w;
+            };
+            for (size_t i = 0; i < tv.size(); ++i) {
+                st.tau[i] = (int32_t)slot_of(coord(tv[i]));
+                st.tmask[i] = word(tv[i]);
+            }
+            for (int o = 0; o < nout; ++o) {
+                const uint32_t v = settle(s, ovec[o]);
+                S.flips.push_back(FFlip{(int32_t)slot_of(coord(v ^ ovec[o])), word(v)});
+            }
+            S.stages.push_back(st);
+            if (last && si + 1 == ps.stages.size()) {
+                for (size_t i = 0; i < tv.size(); ++i)
+                    for (int j = 0; j < n; ++j)
+                        S.fin.tmask[i] |= (uint32_t)odd(sel[j] & tv[i]) << j;
+                for (int o = 0; o < nout; ++o)
+                    for (int j = 0; j < n; ++j)
+                        S.fin.omask[o] |= (uint32_t)odd(sel[j] & settle(s, ovec[o])) << j;
+                for (int j = 0; j < n; ++j)
+                    for (int k = 0; k < K; ++k) S.fin.lmask[j] |= (uint8_t)(odd(sel[j] & s.D[k]) << k);
+            }
+        }
+        fp.stage_end = (int32_t)S.stages.size();
+        fp.op_end = (int32_t)S.ops.size();
+        S.passes[pi] = fp;
+
+        // the frame after the pass: M' vout[i] = gin[i], M' = M on the outer vectors
+        if (!end) {
+            std::vector<uint32_t> Mi(n, 0);
+            for (int o = 0; o < nout; ++o) Mi[31 - __builtin_clz(opos[o])] = ovec[o];
+            for (int i = 0; i < m; ++i) {
+                const int h = 31 - __builtin_clz(gin[i]);
+                uint32_t v = vout[i];
+                for (int o = 0; o < nout; ++o)
+                    if (gin[i] & opos[o]) v ^= ovec[o];
+                Mi[h] = v;
+            }
+            Minv = Mi;
+            M = inverse(Minv);
+        }
+    }
+    return S;
+}
+
+std::vector<uint8_t> export_frames(const HostPlan& p) {
+    std::vector<uint8_t> out = {'V', 'Q', 'C', 'F'};
+    auto put = [&](const void* d, size_t bytes) {
+        const uint8_t* b = static_cast<const uint8_t*>(d);
+        out.insert(out.end(), b, b + bytes);
+    };
+    auto num = [&](int32_t v) { put(&v, 4); };
+    num((int32_t)p.frames.size());
+    for (const FrameSchedule& s : p.frames) {
+        for (int v : {s.mode, s.K, s.m, s.path, s.nout, (int)s.ops.size(), (int)s.stages.size(),
+                      (int)s.passes.size(), (int)s.pass_entries.size(), (int)s.pass_accs.size()})
+            num(v);
+        put(s.ops.data(), s.ops.size() * sizeof(DOp));
+        put(s.stages.data(), s.stages.size() * sizeof(FStage));
+        put(s.flips.data(), s.flips.size() * sizeof(FFlip));
+        put(s.passes.data(), s.passes.size() * sizeof(FPass));
+        put(s.pass_entries.data(), s.pass_entries.size() * 4);
+        put(s.pass_accs.data(), s.pass_accs.size() * 4);
+        put(&s.fin, sizeof(FFinal));
+    }
+    return out;
+}
+
+}  // namespace vqc

@@ -2,72 +2,64 @@
 // (paper, Sec. 3 "Complexity and Tradeoffs": the state, O(B 2^n), is the
 // memory wall; here it lives in HBM between passes).
 //
-// The compiler cuts the op list into passes.  A pass acts on tiles of m
-// qubits: the tile qubits always include the low qubits whose 2^G amplitudes
-// form one 128-byte chunk, so a tile is gathered from HBM as whole chunks.
-// One launch per pass: each CTA loads S tiles (the other n - m qubits fix the
-// tile), runs the pass's register-block stages on them in shared memory
-// exactly as the resident path does, and writes them back.  The forward's last
-// pass emits per-tile <Z> partials; the backward emits per-tile rho sums of
-// the pass's accumulators, which reduce_terms adds up per sample and turns into
-// gradient terms.  reduce_* kernels sum partials in a fixed order
-// (deterministic).
+// One launch per pass of a frame schedule (frame.h): each CTA gathers S tiles of
+// 2^m amplitudes, in whole 128-byte lines, into shared memory, runs the pass's
+// register-block stages there and writes the tiles back, in the order that gives
+// the next pass whole lines again.  The forward's last pass emits per-tile <Z>
+// partials; the backward emits per-tile rho sums of the pass's accumulators,
+// which reduce_terms adds up per sample and turns into gradient terms.  reduce_*
+// kernels sum partials in a fixed order (deterministic).
 #pragma once
 
-#include "sweep.cuh"
+#include "frame.cuh"
 
 namespace vqc {
 
 // R here is the storage real type (pass kernels take PArgs<St<R>>).
 template <typename R>
 struct PArgs {
-    const DOp* ops;
-    const DStage* stages;
-    const int32_t* pass_entries;
+    const DOp* ops;               // the pass's ops and stages
+    const FStage* stages;
+    const FFlip* flips;           // [stages][nout]
+    const FFinal* fin;            // last pass only (forward: <Z>; backward: lam = O psi)
+    const int32_t* pass_entries;  // table slots of the pass's entries
     const int32_t* pass_accs;
-    const DEntry* entries;
-    const DConst* consts;
-    const R* cmat;
-    const R* cang;
-    const DAcc* accs;
-    int n, m, K, tbits, G, S, nout, ntiles;
-    int stage_begin, stage_end;
-    int ps_begin, ps_count, sh_begin, sh_count, acc_begin, acc_count, n_accs, Px;
-    const void* ps_g;       // per-sample tables of every sample [B][n_ps][entry words] (ps_tables),
-                            // kernel real type (not read by the complex64 backward)
+    int n, m, tbits, G, S, nout, ntiles, nstages, nops, op_begin;
+    int ps_begin, ps_count, sh_begin, sh_count, acc_begin, acc_count, n_accs;
+    const void* ps_g;       // per-sample table entries [B][n_ps][entry words], kernel real type
+    const void* sh_g;       // shared table entries [n_sh][entry words] (both from run_tables)
     int n_ps;
     int B;
     long long nunits;
-    uint8_t tile_q[24], out_q[24];
-    const R* x;
-    const R* w;
+    uint32_t ga[kMaxTileBits], sa[kMaxTileBits];   // tile bit -> address, read and written order
+    int32_t gs[kMaxTileBits], ss[kMaxTileBits];    // tile bit -> slot, read and written order
+    uint32_t go[kMaxOuterBits], so[kMaxOuterBits]; // tile index bit -> address
+    int32_t sosl[kMaxOuterBits];                   // tile index bit -> slot, written order
     const R* gE;
     const C2<R>* src_psi;   // tiles are read from here (nullptr: start from |0...0>)
-    C2<R>* dst_psi;         // and written back here (nullptr: not written)
+    C2<R>* dst_psi;         // and written here (nullptr: not written)
     const C2<R>* src_lam;   // backward: lam tiles (nullptr: lam = O psi in the first stage)
     C2<R>* dst_lam;
     R* E_part;              // forward, last pass: [B * ntiles, n]
     R* rho;                 // backward: per-tile rho sums [B * ntiles][n_accs][4] (3 used)
     int sm_sh, sm_ps, sm_psi, sm_lam, sm_acc, sm_red;
-    const unsigned char* plan;   // plan regions copied to shared memory (see KArgs)
-    int tab_off, tab_bytes, sched_off, sched_bytes, sm_plan, plan_smem;
-    int sm_koff;                 // per-pass tile-copy offsets: [ceil(2^m / (APV * T))] uint2
-    unsigned* err;               // the plan's error word (launch self-check)
+    int sm_plan;            // copies of the pass's stages, ops, flips and fin
+    int sm_tfl;             // per tile: each stage's flip (uint2), then the logical parities
+    int sm_koff;            // tile-copy offsets per vector round, read order then written order: uint2
+    unsigned* err;          // the plan's error word (launch self-check)
     // double-float kernels only: src_psi / src_lam / dst_psi and dst_lam hold
     // raw (hi, lo) float pairs (workspace state passed between passes) rather
     // than complex128 values (caller buffers); ignored by other kernels
     int src_raw, lam_raw, dst_raw;
 };
 
-// Global amplitude index of tile-local index u (the low G tile bits are the
-// low G qubits; the rest follow tile_q).
-__device__ __forceinline__ uint32_t tile_global(uint32_t u, uint32_t tile_base, const uint8_t* tq,
-                                                int G) {
-    uint32_t g = tile_base | (u & ((1u << G) - 1u));
-    uint32_t hi = u >> G;
-    for (int i = G; hi; ++i, hi >>= 1)
-        if (hi & 1u) g |= 1u << tq[i];
-    return g;
+// XOR of cols[i] over the set bits of v.
+template <typename T, int N>
+__device__ __forceinline__ uint32_t xor_cols(const T (&cols)[N], uint32_t v) {
+    uint32_t r = 0;
+    for (int i = 0; v; ++i, v >>= 1)
+        if (v & 1u) r ^= (uint32_t)cols[i];
+    return r;
 }
 
 // 16-byte vectors of amplitudes, moved without taking register addresses.
@@ -111,47 +103,47 @@ template <typename R, bool RAW> struct VecSel { using t = Vec16<R>; };
 template <> struct VecSel<dd, true> { using t = Vec16Raw; };
 
 // Tile copies between HBM and shared memory.  A CTA-thread t moves vectors
-// v = t + k*T; the tile-local index of v splits into disjoint bit fields of t
-// and of k, and both the index deposit into global qubits and the swizzle are
-// linear in those fields, so each is a per-thread part XOR a per-k part
-// (tabulated once per pass in shared memory: koff[k] = (global, slot)).
+// v = t + k*T; address and slot of an amplitude are XOR-linear in its tile index,
+// so each is a per-thread part XOR a per-k part (tabulated once per pass in
+// shared memory: koff[k] = (address, slot)).  s1 is the slot offset of a
+// vector's second amplitude.
 template <typename R, bool RAW = false, int U = 8>
-__device__ __forceinline__ void tile_gather(C2<R>* sm, const SC2<R>* gs, uint32_t gt, uint32_t st,
-                                            const uint2* koff, int nk, int T, int t) {
+__device__ __forceinline__ void tile_gather(C2<R>* sm, const SC2<R>* gs, uint32_t gt, uint32_t st, uint32_t s1,
+                                            const uint2* koff, int nk) {
     using V = typename VecSel<R, RAW>::t;
     constexpr int APV = 16 / sizeof(C2<R>);
     int k = 0;
     for (; k + U <= nk; k += U) {
         V v[U];
 #pragma unroll
-        for (int j = 0; j < U; ++j) v[j].ld(gs + (gt | koff[k + j].x));
+        for (int j = 0; j < U; ++j) v[j].ld(gs + (gt ^ koff[k + j].x));
 #pragma unroll
         for (int j = 0; j < U; ++j) {
             const uint32_t sl = st ^ koff[k + j].y;
-#pragma unroll
-            for (int e = 0; e < APV; ++e) sm[sl ^ e] = v[j].a[e];
+            sm[sl] = v[j].a[0];
+            if constexpr (APV == 2) sm[sl ^ s1] = v[j].a[1];
         }
     }
     for (; k < nk; ++k) {
         V v;
-        v.ld(gs + (gt | koff[k].x));
+        v.ld(gs + (gt ^ koff[k].x));
         const uint32_t sl = st ^ koff[k].y;
-#pragma unroll
-        for (int e = 0; e < APV; ++e) sm[sl ^ e] = v.a[e];
+        sm[sl] = v.a[0];
+        if constexpr (APV == 2) sm[sl ^ s1] = v.a[1];
     }
 }
 
 template <typename R, bool RAW = false>
-__device__ __forceinline__ void tile_scatter(const C2<R>* sm, SC2<R>* gs, uint32_t gt, uint32_t st,
-                                             const uint2* koff, int nk, int T, int t) {
+__device__ __forceinline__ void tile_scatter(const C2<R>* sm, SC2<R>* gs, uint32_t gt, uint32_t st, uint32_t s1,
+                                             const uint2* koff, int nk) {
     using V = typename VecSel<R, RAW>::t;
     constexpr int APV = 16 / sizeof(C2<R>);
     for (int k = 0; k < nk; ++k) {
         V v;
         const uint32_t sl = st ^ koff[k].y;
-#pragma unroll
-        for (int e = 0; e < APV; ++e) v.a[e] = sm[sl ^ e];
-        v.st(gs + (gt | koff[k].x));
+        v.a[0] = sm[sl];
+        if constexpr (APV == 2) v.a[1] = sm[sl ^ s1];
+        v.st(gs + (gt ^ koff[k].x));
     }
 }
 
@@ -164,15 +156,15 @@ __device__ __forceinline__ void tile_prefetch(const SC2<R>* gs, uint32_t gt, con
                                               int t) {
     if (t & 7) return;
     for (int k = 0; k < nk; ++k)
-        asm volatile("prefetch.global.L2 [%0];" ::"l"(gs + (gt | koff[k].x)));
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(gs + (gt ^ koff[k].x)));
 }
 
 // FULL: tile groups span whole warps (2^(m-K) >= 32 threads; every production
 // tile), see sweep_kernel.
 template <typename R, int K, int MODE, bool FULL, bool PH2 = true>
 __global__ void __launch_bounds__(256, 2) pass_kernel(const __grid_constant__ PArgs<St<R>> A) {
-    if (geometry_bad(blockDim.x != (unsigned)(A.S << A.tbits) || A.tbits != A.m - K ||
-                         A.stage_end <= A.stage_begin,
+    if (geometry_bad(blockDim.x != (unsigned)(A.S << A.tbits) || A.tbits != A.m - K || A.nstages < 1 ||
+                         A.m > kMaxTileBits || A.nout > kMaxOuterBits,
                      A.err, kErrPassGeometry))
         return;
     extern __shared__ __align__(16) unsigned char smem[];
@@ -182,30 +174,21 @@ __global__ void __launch_bounds__(256, 2) pass_kernel(const __grid_constant__ PA
     C2<R>* lam_all = reinterpret_cast<C2<R>*>(smem + A.sm_lam);
     R* acc_all = reinterpret_cast<R*>(smem + A.sm_acc);
     R* red_all = reinterpret_cast<R*>(smem + A.sm_red);
+    const int nthr = blockDim.x, nst = A.nstages;
 
-    const unsigned char* smt = nullptr;
-    const unsigned char* sms = nullptr;
-    if (A.plan_smem) {
-        unsigned char* t = smem + A.sm_plan;
-        unsigned char* u = t + ((A.tab_bytes + 15) & ~15);
-        copy_region(t, A.plan + A.tab_off, A.tab_bytes);
-        copy_region(u, A.plan + A.sched_off, A.sched_bytes);
-        smt = t;
-        sms = u;
-    }
-    grid_dep_wait();
-    grid_dep_launch();
-    const DOp* P_ops = rebase(A.ops, A.plan, A.sched_off, sms);
-    const DStage* P_stages = rebase(A.stages, A.plan, A.sched_off, sms);
-    const int32_t* P_pass_entries = rebase(A.pass_entries, A.plan, A.sched_off, sms);
-    const int32_t* P_pass_accs = rebase(A.pass_accs, A.plan, A.sched_off, sms);
-    const DEntry* P_entries = rebase(A.entries, A.plan, A.tab_off, smt);
-    const DConst* P_consts = rebase(A.consts, A.plan, A.tab_off, smt);
-    const R* P_cmat = reinterpret_cast<const R*>(
-        rebase(reinterpret_cast<const unsigned char*>(A.cmat), A.plan, A.tab_off, smt));
-    const R* P_cang = reinterpret_cast<const R*>(
-        rebase(reinterpret_cast<const unsigned char*>(A.cang), A.plan, A.tab_off, smt));
-    if (A.plan_smem) __syncthreads();
+    // the pass's program (no kernel writes the plan, so this may precede the wait)
+    FStage* stages = reinterpret_cast<FStage*>(smem + A.sm_plan);
+    FFinal* fin = reinterpret_cast<FFinal*>(stages + nst);
+    uint2* ops = reinterpret_cast<uint2*>(fin + 1);
+    FFlip* flips = reinterpret_cast<FFlip*>(ops + A.nops);
+    async_region(reinterpret_cast<unsigned char*>(stages), reinterpret_cast<const unsigned char*>(A.stages),
+                 nst * (int)sizeof(FStage));
+    if (A.fin)
+        async_region(reinterpret_cast<unsigned char*>(fin), reinterpret_cast<const unsigned char*>(A.fin),
+                     sizeof(FFinal));
+    for (int i = threadIdx.x; i < A.nops; i += nthr) async_elem<uint2>(ops + i, reinterpret_cast<const uint2*>(A.ops) + i);
+    for (int i = threadIdx.x; i < nst * A.nout; i += nthr)
+        async_elem<uint2>(reinterpret_cast<uint2*>(flips) + i, reinterpret_cast<const uint2*>(A.flips) + i);
 
     const int n = A.n, G = A.G, tdim = 1 << A.m;
     const long long total_tiles = (long long)A.B * A.ntiles;
@@ -221,118 +204,125 @@ __global__ void __launch_bounds__(256, 2) pass_kernel(const __grid_constant__ PA
     q.mask = blockDim.x >= 32 ? 0xffffffffu : ((1u << blockDim.x) - 1u);
     const int lane = q.t & 31;
     const int warp_in_group = q.t >> 5;
-    const int nthr = blockDim.x;
 
     // Tile copy geometry: vectors v = t + k*T of APV amplitudes.
     constexpr int APV = 16 / sizeof(C2<R>);
     const int nvec = tdim / APV;
     const int nk = (nvec + q.T - 1) / q.T;
-    uint2* koff = reinterpret_cast<uint2*>(smem + A.sm_koff);
+    uint2* koff_g = reinterpret_cast<uint2*>(smem + A.sm_koff);
+    uint2* koff_s = koff_g + nk;
     for (int k = threadIdx.x; k < nk; k += nthr) {
         const uint32_t u = (uint32_t)k * q.T * APV;
-        koff[k] = make_uint2(tile_global(u, 0, A.tile_q, G), swz(u, G));
+        koff_g[k] = make_uint2(xor_cols(A.ga, u), xor_cols(A.gs, u));
+        koff_s[k] = make_uint2(xor_cols(A.sa, u), xor_cols(A.ss, u));
     }
     const uint32_t u_t = (uint32_t)q.t * APV;
-    const uint32_t st_t = swz(u_t, G) ^ (uint32_t)q.h;
+    const uint32_t g_addr = xor_cols(A.ga, u_t), g_slot = xor_cols(A.gs, u_t) ^ (uint32_t)q.h;
+    const uint32_t s_addr = xor_cols(A.sa, u_t), s_slot = xor_cols(A.ss, u_t) ^ (uint32_t)q.h;
+    const uint32_t g_one = (uint32_t)A.gs[0], s_one = (uint32_t)A.ss[0];
 
-    for (int i = threadIdx.x; i < A.sh_count; i += nthr) {
-        const DEntry e = P_entries[vqc_ld(&P_pass_entries[A.sh_begin + i])];
-        eval_entry<R>(e, P_consts, static_cast<const St<R>*>(nullptr), A.w, P_cang, P_cmat,
-                      sh_tab + EntryWords<R>::value * i);
+    grid_dep_wait();
+    grid_dep_launch();
+    {   // the pass's shared entries
+        constexpr int V = EntryWords<R>::value * (int)sizeof(R) / 16;   // 16-byte vectors per entry
+        const unsigned char* gtab = static_cast<const unsigned char*>(A.sh_g);
+        for (int i = threadIdx.x; i < A.sh_count * V; i += nthr) {
+            const int k = i / V, v = i - k * V;
+            async_copy<16>(reinterpret_cast<unsigned char*>(sh_tab) + 16 * i,
+                           gtab + 16 * ((size_t)vqc_ld(&A.pass_entries[A.sh_begin + k]) * V + v));
+        }
     }
+    async_wait();
     __syncthreads();
 
     C2<R>* psi = psi_all + (size_t)q.g * tdim;
     C2<R>* lam = lam_all + (size_t)q.g * tdim;
     R* ps_tab = ps_all + (size_t)q.g * A.ps_count * EntryWords<R>::value;
     R* acc = acc_all + (size_t)q.g * A.acc_count * q.wg * 8;
+    uint2* tfl_all = reinterpret_cast<uint2*>(smem + A.sm_tfl);
+    const uint2* tfl = tfl_all + q.g * (nst + 1);
 
     for (long long unit = blockIdx.x; unit < A.nunits; unit += gridDim.x) {
         const long long tid_raw = unit * A.S + q.g;
         const bool valid = tid_raw < total_tiles;
         const long long tile_id = valid ? tid_raw : total_tiles - 1;
         const int b = (int)(tile_id / A.ntiles);
-        const int tau = (int)(tile_id % A.ntiles);
-        uint32_t tile_base = 0;
-        for (int j = 0; j < A.nout; ++j)
-            if ((tau >> j) & 1) tile_base |= 1u << A.out_q[j];
+        const uint32_t tau = (uint32_t)(tile_id % A.ntiles);
 
-        if (MODE == 1 && std::is_same<R, float>::value) {
-            // the complex64 backward evaluates its per-sample entries itself: with
-            // the table copy instead its register allocation spilled more and it
-            // measured 0.7% slower (the other kernels read the table)
-            for (int i = threadIdx.x; i < A.S * A.ps_count; i += nthr) {
-                const int gg = i / A.ps_count, k = i % A.ps_count;
-                const long long tt = min(unit * A.S + gg, total_tiles - 1);
-                const int bb = (int)(tt / A.ntiles);
-                const DEntry e = P_entries[vqc_ld(&P_pass_entries[A.ps_begin + k])];
-                eval_entry<R>(e, P_consts, A.x + (size_t)bb * A.Px, A.w, P_cang, P_cmat,
-                              ps_all + ((size_t)gg * A.ps_count + k) * EntryWords<R>::value);
+        // the tile's flip of each stage, and its logical parities
+        for (int i = threadIdx.x; i < A.S * (nst + 1); i += nthr) {
+            const int gg = i / (nst + 1), s = i - gg * (nst + 1);
+            const uint32_t tt = (uint32_t)(min(unit * A.S + gg, total_tiles - 1) % A.ntiles);
+            uint2 f = make_uint2(0, 0);
+            if (s < nst) {
+                for (int o = 0; o < A.nout; ++o)
+                    if ((tt >> o) & 1) {
+                        f.x ^= (uint32_t)flips[s * A.nout + o].slot;
+                        f.y ^= flips[s * A.nout + o].mask;
+                    }
+            } else if (A.fin) {
+                f.x = xor_cols(fin->omask, tt);
             }
-        } else if (A.ps_count) {   // the pass's per-sample entries, copied from the sample's precomputed table
-            constexpr int V = EntryWords<R>::value * (int)sizeof(R) / 16;   // 16-byte vectors per entry
+            tfl_all[i] = f;
+        }
+        if (A.ps_count) {   // the pass's per-sample entries
+            constexpr int V = EntryWords<R>::value * (int)sizeof(R) / 16;
             const int4* gtab = static_cast<const int4*>(A.ps_g);
             int4* stab = reinterpret_cast<int4*>(ps_all);
             const int per = A.ps_count * V;
             for (int i = threadIdx.x; i < A.S * per; i += nthr) {
                 const int gg = i / per, r = i - gg * per, k = r / V, v = r - k * V;
                 const int bb = (int)(min(unit * A.S + gg, total_tiles - 1) / A.ntiles);
-                const int slot = P_entries[vqc_ld(&P_pass_entries[A.ps_begin + k])].slot;
-                stab[((size_t)gg * A.ps_count + k) * V + v] = gtab[((size_t)bb * A.n_ps + slot) * V + v];
+                stab[i] = gtab[((size_t)bb * A.n_ps + vqc_ld(&A.pass_entries[A.ps_begin + k])) * V + v];
             }
         }
         const size_t sbase = (size_t)b << n;
-        const uint32_t gt = tile_global(u_t, tile_base, A.tile_q, G);
+        const uint32_t ga = g_addr ^ xor_cols(A.go, tau);
         if (A.src_psi) {
-            if (DDK && A.src_raw) tile_gather<R, DDK>(psi, A.src_psi + sbase, gt, st_t, koff, nk, q.T, q.t);
+            if (DDK && A.src_raw) tile_gather<R, DDK>(psi, A.src_psi + sbase, ga, g_slot, g_one, koff_g, nk);
             else   // 16 loads in flight where one state is gathered, 8 beside lam's registers
-                tile_gather<R, false, MODE == 0 ? 16 : 8>(psi, A.src_psi + sbase, gt, st_t, koff, nk, q.T, q.t);
+                tile_gather<R, false, MODE == 0 ? 16 : 8>(psi, A.src_psi + sbase, ga, g_slot, g_one, koff_g, nk);
         }
         if (MODE == 1 && A.src_lam) {
-            if (DDK && A.lam_raw) tile_gather<R, DDK>(lam, A.src_lam + sbase, gt, st_t, koff, nk, q.T, q.t);
-            else tile_gather<R>(lam, A.src_lam + sbase, gt, st_t, koff, nk, q.T, q.t);
+            if (DDK && A.lam_raw) tile_gather<R, DDK>(lam, A.src_lam + sbase, ga, g_slot, g_one, koff_g, nk);
+            else tile_gather<R>(lam, A.src_lam + sbase, ga, g_slot, g_one, koff_g, nk);
         }
         if (unit + gridDim.x < A.nunits) {   // the CTA's next tile into L2 during this one's stages
             const long long nt = min((unit + gridDim.x) * A.S + q.g, total_tiles - 1);
-            const int nb = (int)(nt / A.ntiles), ntau = (int)(nt % A.ntiles);
-            uint32_t nbase = 0;
-            for (int j = 0; j < A.nout; ++j)
-                if ((ntau >> j) & 1) nbase |= 1u << A.out_q[j];
-            const uint32_t ngt = tile_global(u_t, nbase, A.tile_q, G);
-            const size_t nsb = (size_t)nb << n;
-            if (A.src_psi) tile_prefetch<R>(A.src_psi + nsb, ngt, koff, nk, q.t);
-            if (MODE == 1 && A.src_lam) tile_prefetch<R>(A.src_lam + nsb, ngt, koff, nk, q.t);
+            const uint32_t nga = g_addr ^ xor_cols(A.go, (uint32_t)(nt % A.ntiles));
+            const size_t nsb = (size_t)(nt / A.ntiles) << n;
+            if (A.src_psi) tile_prefetch<R>(A.src_psi + nsb, nga, koff_g, nk, q.t);
+            if (MODE == 1 && A.src_lam) tile_prefetch<R>(A.src_lam + nsb, nga, koff_g, nk, q.t);
         }
         __syncthreads();
 
         C2<R> a[1 << K];
         int32_t sg[K];
         StageView v{0, 0};
-        if (MODE == 0) {
-            for (int s = A.stage_begin; s < A.stage_end; ++s) {
-                const DStage* sp = P_stages + s;
-                v = stage_view<K>(sp, q.t, q.h, sg);
-                v.pb |= tile_base;
-                if (s == A.stage_begin && !A.src_psi) {
+        if constexpr (MODE == 0) {
+            for (int s = 0; s < nst; ++s) {
+                const FStage* sp = stages + s;
+                const uint2 fl = tfl[s];
+                v = frame_view<K>(sp, q.t, fl.x, fl.y, q.h, sg);
+                if (s == 0 && !A.src_psi) {
 #pragma unroll
                     for (int r = 0; r < (1 << K); ++r) a[r] = cm<R>(0, 0);
-                    if (v.pb == 0) a[0] = cm<R>(1, 0);
+                    if ((q.t | tau) == 0) a[0] = cm<R>(1, 0);
                 } else {
                     block_load<R, K>(a, psi, v.swb, sg);
                 }
-                run_ops<R, K, 0, true, FULL, PH2>(P_ops, vqc_ld(&sp->op_begin), vqc_ld(&sp->op_end), v.pb, a, a,
-                                 sh_tab, ps_tab, nullptr, q, lane, warp_in_group);
-                if (s + 1 < A.stage_end || A.dst_psi) {   // store map: absorbed CX gates
-                    if (vqc_ld(&sp->nperm)) group_sync<R>(q);   // all loads of the stage first
-                    int32_t s2[K];
-                    const uint32_t b2 = map_base<K, true>(sp, q.t, q.h, s2);
-                    block_store<R, K>(a, psi, b2, s2);
+                run_ops<R, K, 0, false, FULL, PH2>(reinterpret_cast<const DOp*>(ops), sp->op_begin - A.op_begin,
+                                                   sp->op_end - A.op_begin, v.pb, a, a, sh_tab, ps_tab, nullptr, q,
+                                                   lane, warp_in_group);
+                if (s + 1 < nst || A.dst_psi) {
+                    block_store<R, K>(a, psi, v.swb, sg);
                     group_sync<R>(q);
                 }
             }
             if (A.E_part) {
                 R* red = red_all + (size_t)q.g * q.wg * n;
-                expz_partials<R, K>(P_stages + (A.stage_end - 1), v.pb, a, n, red, q, warp_in_group);
+                const uint32_t pbf = tfl[nst].x ^ xor_bits(fin->tmask, A.tbits, q.t);
+                expz_frame<R, K, FULL>(fin->lmask, pbf, a, n, red, q, lane, warp_in_group);
                 __syncthreads();
                 if (valid)
                     for (int j = q.t; j < n; j += q.T) {
@@ -343,61 +333,58 @@ __global__ void __launch_bounds__(256, 2) pass_kernel(const __grid_constant__ PA
             }
             __syncthreads();
             if (A.dst_psi && valid) {
-                if (DDK && A.dst_raw) tile_scatter<R, DDK>(psi, A.dst_psi + sbase, gt, st_t, koff, nk, q.T, q.t);
-                else tile_scatter<R>(psi, A.dst_psi + sbase, gt, st_t, koff, nk, q.T, q.t);
+                const uint32_t da = s_addr ^ xor_cols(A.so, tau), ds = s_slot ^ xor_cols(A.sosl, tau);
+                if (DDK && A.dst_raw) tile_scatter<R, DDK>(psi, A.dst_psi + sbase, da, ds, s_one, koff_s, nk);
+                else tile_scatter<R>(psi, A.dst_psi + sbase, da, ds, s_one, koff_s, nk);
             }
             __syncthreads();
-            continue;
-        }
-
-        // backward: stages of the pass in reverse
-        for (int s = A.stage_end - 1; s >= A.stage_begin; --s) {
-            const DStage* sp = P_stages + s;
-            C2<R> l[1 << K];
-            v = stage_view<K>(sp, q.t, q.h, sg);
-            v.pb |= tile_base;
-            {   // the forward left this stage's output in its store map
-                int32_t s2[K];
-                const uint32_t b2 = map_base<K, true>(sp, q.t, q.h, s2);
-                block_load<R, K>(a, psi, b2, s2);
-                if (s == A.stage_end - 1 && !A.src_lam)
-                    lambda_init<R, K>(sp, v.pb, A.gE + (size_t)b * n, n, a, l);
-                else
-                    block_load<R, K>(l, lam, b2, s2);
+        } else {
+            // backward: stages of the pass in reverse
+            for (int s = nst - 1; s >= 0; --s) {
+                const FStage* sp = stages + s;
+                const uint2 fl = tfl[s];
+                C2<R> l[1 << K];
+                v = frame_view<K>(sp, q.t, fl.x, fl.y, q.h, sg);
+                block_load<R, K>(a, psi, v.swb, sg);
+                if (s == nst - 1 && !A.src_lam) {
+                    const uint32_t pbf = tfl[nst].x ^ xor_bits(fin->tmask, A.tbits, q.t);
+                    lambda_frame<R, K>(fin->lmask, pbf, A.gE + (size_t)b * n, n, a, l);
+                } else {
+                    block_load<R, K>(l, lam, v.swb, sg);
+                }
+                run_ops<R, K, 1, false, FULL, PH2>(reinterpret_cast<const DOp*>(ops), sp->op_begin - A.op_begin,
+                                                   sp->op_end - A.op_begin, v.pb, a, l, sh_tab, ps_tab, acc, q, lane,
+                                                   warp_in_group);
+                if (s > 0 || A.dst_psi) {
+                    block_store<R, K>(a, psi, v.swb, sg);
+                    block_store<R, K>(l, lam, v.swb, sg);
+                }
+                group_sync<R>(q);
             }
-            run_ops<R, K, 1, true, FULL, PH2>(P_ops, vqc_ld(&sp->op_begin), vqc_ld(&sp->op_end), v.pb, a, l, sh_tab,
-                             ps_tab, acc, q, lane, warp_in_group);
-            if (s > A.stage_begin || A.dst_psi) {   // back to the stage's load map
-                if (vqc_ld(&sp->nperm)) group_sync<R>(q);   // all loads of the stage first
-                int32_t s2[K];
-                const uint32_t b2 = map_base<K, false>(sp, q.t, q.h, s2);
-                block_store<R, K>(a, psi, b2, s2);
-                block_store<R, K>(l, lam, b2, s2);
+            __syncthreads();
+            if (valid && A.dst_psi) {
+                const uint32_t da = s_addr ^ xor_cols(A.so, tau);
+                if (DDK && A.dst_raw) {
+                    tile_scatter<R, DDK>(psi, A.dst_psi + sbase, da, s_slot, s_one, koff_s, nk);
+                    tile_scatter<R, DDK>(lam, A.dst_lam + sbase, da, s_slot, s_one, koff_s, nk);
+                } else {
+                    tile_scatter<R>(psi, A.dst_psi + sbase, da, s_slot, s_one, koff_s, nk);
+                    tile_scatter<R>(lam, A.dst_lam + sbase, da, s_slot, s_one, koff_s, nk);
+                }
             }
-            group_sync<R>(q);
-        }
-        __syncthreads();
-        if (valid && A.dst_psi) {
-            if (DDK && A.dst_raw) {
-                tile_scatter<R, DDK>(psi, A.dst_psi + sbase, gt, st_t, koff, nk, q.T, q.t);
-                tile_scatter<R, DDK>(lam, A.dst_lam + sbase, gt, st_t, koff, nk, q.T, q.t);
-            } else {
-                tile_scatter<R>(psi, A.dst_psi + sbase, gt, st_t, koff, nk, q.T, q.t);
-                tile_scatter<R>(lam, A.dst_lam + sbase, gt, st_t, koff, nk, q.T, q.t);
+            // the tile's rho sums (warps in order), in parallel over accumulators and
+            // components; the per-sample turn into terms is reduce_terms' work
+            for (int i = threadIdx.x; i < A.S * A.acc_count * 3; i += nthr) {
+                const int gg = i / (A.acc_count * 3), r = i % (A.acc_count * 3), k = r / 3, c = r % 3;
+                const long long tt = unit * A.S + gg;
+                if (tt >= total_tiles) continue;
+                const R* ap = acc_all + ((size_t)gg * A.acc_count + k) * q.wg * 8 + c;
+                R sum = 0;
+                for (int wi = 0; wi < q.wg; ++wi) sum += ap[wi * 8];
+                A.rho[((size_t)tt * A.n_accs + vqc_ld(&A.pass_accs[A.acc_begin + k])) * 4 + c] = as_out<St<R>>(sum);
             }
+            __syncthreads();
         }
-        // the tile's rho sums (warps in order), in parallel over accumulators and
-        // components; the per-sample turn into terms is reduce_terms' work
-        for (int i = threadIdx.x; i < A.S * A.acc_count * 3; i += nthr) {
-            const int gg = i / (A.acc_count * 3), r = i % (A.acc_count * 3), k = r / 3, c = r % 3;
-            const long long tt = unit * A.S + gg;
-            if (tt >= total_tiles) continue;
-            const R* ap = acc_all + ((size_t)gg * A.acc_count + k) * q.wg * 8 + c;
-            R sum = 0;
-            for (int wi = 0; wi < q.wg; ++wi) sum += ap[wi * 8];
-            A.rho[((size_t)tt * A.n_accs + vqc_ld(&P_pass_accs[A.acc_begin + k])) * 4 + c] = as_out<St<R>>(sum);
-        }
-        __syncthreads();
     }
 }
 
@@ -415,22 +402,28 @@ __global__ void reduce_expz(const R* E_part, int B, int ntiles, int n, R* E) {
     }
 }
 
-// Per-sample table entries of every sample (the x-dependent runs), evaluated
-// once per call for all passes: out [B][n_ps][entry words], in the kernels'
-// real type R (slot order = ps_list order).
+// Table entries, evaluated once per call for all passes, in the kernels' real
+// type R: the shared ones to out_sh [n_sh][entry words], every sample's
+// x-dependent ones to out_ps [B][n_ps][entry words] (slot order = list order).
 template <typename R>
-__global__ void __launch_bounds__(256) ps_tables(const DEntry* entries, const int32_t* ps_list,
-                                                 const DConst* consts, const R* cang, const R* cmat,
-                                                 const St<R>* x, int Px, const St<R>* w, int B, int n_ps,
-                                                 R* out) {
+__global__ void __launch_bounds__(256) run_tables(const DEntry* entries, const int32_t* ps_list,
+                                                  const int32_t* sh_list, const DConst* consts, const R* cang,
+                                                  const R* cmat, const St<R>* x, int Px, const St<R>* w, int B,
+                                                  int n_ps, int n_sh, R* out_ps, R* out_sh) {
     grid_dep_wait();
     grid_dep_launch();
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < (long long)B * n_ps;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < (long long)B * n_ps + n_sh;
          i += (long long)gridDim.x * blockDim.x) {
-        const long long b = i / n_ps;
-        const DEntry e = entries[vqc_ld(&ps_list[i % n_ps])];
+        if (i < n_sh) {
+            const DEntry e = entries[vqc_ld(&sh_list[i])];
+            eval_entry<R>(e, consts, static_cast<const St<R>*>(nullptr), w, cang, cmat,
+                          out_sh + (size_t)e.slot * EntryWords<R>::value);
+            continue;
+        }
+        const long long j = i - n_sh, b = j / n_ps;
+        const DEntry e = entries[vqc_ld(&ps_list[j % n_ps])];
         eval_entry<R>(e, consts, x + b * Px, w, cang, cmat,
-                      out + ((size_t)b * n_ps + e.slot) * EntryWords<R>::value);
+                      out_ps + ((size_t)b * n_ps + e.slot) * EntryWords<R>::value);
     }
 }
 
@@ -463,34 +456,23 @@ __global__ void __launch_bounds__(256) reduce_terms(const St<R>* rho, int B, int
     }
 }
 
-// dx[b, p] = sum_tau sum_{terms j of x column p} terms[b * ntiles + tau, j]
+// dx[b, p] = sum over the terms of x column p, in order: the element i of dx.
 template <typename R>
-__global__ void reduce_dx(const R* terms, int B, int ntiles, int nt, const int32_t* ptr,
-                          const int32_t* occ, int Px, R* dx) {
-    grid_dep_wait();
-    grid_dep_launch();
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < (long long)B * Px;
-         i += (long long)gridDim.x * blockDim.x) {
-        const long long b = i / Px;
-        const int p = (int)(i % Px);
-        R s = 0;
-        for (int t = 0; t < ntiles; ++t) {
-            const R* row = terms + (b * ntiles + t) * nt;
-            for (int k = vqc_ld(&ptr[p]); k < vqc_ld(&ptr[p + 1]); ++k) s += row[vqc_ld(&occ[k])];
-        }
-        dx[i] = s;
-    }
+__device__ __forceinline__ void dx_element(const R* terms, long long i, int nt, const int32_t* ptr,
+                                           const int32_t* occ, int Px, R* dx) {
+    const R* row = terms + (i / Px) * nt;
+    const int p = (int)(i % Px);
+    R s = 0;
+    for (int k = vqc_ld(&ptr[p]); k < vqc_ld(&ptr[p + 1]); ++k) s += row[vqc_ld(&occ[k])];
+    dx[i] = s;
 }
 
-// dw[p] = sum over every tile row of the terms of w index p: one block per p,
-// fixed strided partial sums then a fixed-shape tree.
+// dw[p] = sum over every row of the terms of w index p: one block per p, fixed
+// strided partial sums then a fixed-shape tree.
 template <typename R>
-__global__ void __launch_bounds__(256) reduce_dw(const R* terms, long long rows, int nt,
-                                                 const int32_t* ptr, const int32_t* occ, R* dw) {
+__device__ __forceinline__ void dw_column(const R* terms, long long rows, int nt, const int32_t* ptr,
+                                          const int32_t* occ, int p, R* dw) {
     __shared__ R part[256];
-    const int p = blockIdx.x;
-    grid_dep_wait();
-    grid_dep_launch();
     const int k0 = vqc_ld(&ptr[p]), k1 = vqc_ld(&ptr[p + 1]);
     R s = 0;
     for (long long r = threadIdx.x; r < rows; r += 256) {
@@ -504,6 +486,39 @@ __global__ void __launch_bounds__(256) reduce_dw(const R* terms, long long rows,
         __syncthreads();
     }
     if (threadIdx.x == 0) dw[p] = part[0];
+}
+
+template <typename R>
+__global__ void reduce_dx(const R* terms, int B, int nt, const int32_t* ptr, const int32_t* occ, int Px, R* dx) {
+    grid_dep_wait();
+    grid_dep_launch();
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < (long long)B * Px;
+         i += (long long)gridDim.x * blockDim.x)
+        dx_element<R>(terms, i, nt, ptr, occ, Px, dx);
+}
+
+template <typename R>
+__global__ void __launch_bounds__(256) reduce_dw(const R* terms, long long rows, int nt,
+                                                 const int32_t* ptr, const int32_t* occ, R* dw) {
+    grid_dep_wait();
+    grid_dep_launch();
+    dw_column<R>(terms, rows, nt, ptr, occ, blockIdx.x, dw);
+}
+
+// Both in one launch (complex64): the first Pw blocks take dw, the others dx.
+template <typename R>
+__global__ void __launch_bounds__(256) reduce_grads(const R* terms, int B, int nt, const int32_t* xptr,
+                                                    const int32_t* xocc, int Px, R* dx, const int32_t* wptr,
+                                                    const int32_t* wocc, int Pw, R* dw) {
+    grid_dep_wait();
+    grid_dep_launch();
+    if ((int)blockIdx.x < Pw) {
+        dw_column<R>(terms, B, nt, wptr, wocc, blockIdx.x, dw);
+        return;
+    }
+    for (long long i = (blockIdx.x - Pw) * (long long)blockDim.x + threadIdx.x; i < (long long)B * Px;
+         i += (long long)(gridDim.x - Pw) * blockDim.x)
+        dx_element<R>(terms, i, nt, xptr, xocc, Px, dx);
 }
 
 // probs[i] = |psi[i]|^2 over count amplitudes (the probabilities output).
