@@ -692,10 +692,9 @@ vqc_status run_cluster_backward(const HostPlan& p, int B, const void* x, const v
 struct PassGeo {
     const FrameSchedule* s = nullptr;
     int K = 0, T = 0, S = 0, block = 0, grid = 0, wg = 1, ntiles = 1;
-    long long nunits = 0;
+    int nunits = 0;
     size_t smem = 0;
-    int sm_sh = 0, sm_ps = 0, sm_psi = 0, sm_lam = 0, sm_acc = 0, sm_red = 0, sm_plan = 0,
-        sm_tfl = 0, sm_koff = 0;
+    int sm_sh = 0, sm_ps = 0, sm_lam = 0, sm_acc = 0, sm_red = 0, sm_plan = 0, sm_tfl = 0, sm_koff = 0, sm_toff = 0, sm_tbase = 0;
     const void* fn = nullptr;
 };
 
@@ -729,7 +728,7 @@ vqc_status plan_hbm_uncached(const HostPlan& p, int mode, int B, PassGeo& L) {
                         (size_t)nst_max * L.s->nout * sizeof(FFlip);
     const size_t fixed = align16((size_t)sh_max * ew * rs) + align16(prog) + align16(2 * nk * 8) + 8 * 16;
     const size_t per_tile = (size_t)ps_max * ew * rs + tdim * cs * (mode == 1 ? 2 : 1) + (size_t)(nst_max + 1) * 8 +
-                            (mode == 1 ? (size_t)acc_max * L.wg * 8 * rs : (size_t)L.wg * p.n * rs);
+                            (size_t)L.T * (16 + 4 * nst_max) + (mode == 1 ? (size_t)acc_max * L.wg * 8 * rs : (size_t)L.wg * p.n * rs);
     int S = std::max(1, 128 / L.T);
     if ((size_t)di.smem_optin <= fixed + per_tile)
         S = (size_t)di.smem_optin >= fixed + per_tile ? 1 : 0;
@@ -746,27 +745,31 @@ vqc_status plan_hbm_uncached(const HostPlan& p, int mode, int B, PassGeo& L) {
         off = align16(off + bytes);
         return (int)o;
     };
+    take((size_t)S * tdim * cs);   // psi tiles at offset 0
+    L.sm_lam = take(mode == 1 ? (size_t)S * tdim * cs : 0);
     L.sm_sh = take((size_t)sh_max * ew * rs);
     L.sm_ps = take((size_t)S * ps_max * ew * rs);
-    L.sm_psi = take((size_t)S * tdim * cs);
-    L.sm_lam = take(mode == 1 ? (size_t)S * tdim * cs : 0);
     L.sm_acc = take(mode == 1 ? (size_t)S * acc_max * L.wg * 8 * rs : 0);
     L.sm_red = take(mode == 0 ? (size_t)S * L.wg * p.n * rs : 0);
     L.sm_koff = take(2 * nk * 8);   // tile-copy offsets: one uint2 per vector round, read and written
+    L.sm_toff = take((size_t)L.block * 16);   // and each thread's own part
+    L.sm_tbase = take((size_t)nst_max * L.block * 4);
     L.sm_plan = take(prog);
     L.sm_tfl = take((size_t)S * (nst_max + 1) * 8);
     L.smem = off;
     L.fn = p.dfloat ? pass_ptr_dd(mode, L.K, L.T >= 32)
-           : (!dbl && mode == 0 && !p.has_ph2) ? pass_ptr_f32_fwd_nph(L.K, L.T >= 32)   // no phase cases
-                                               : pass_ptr(dbl, mode, L.K, L.T >= 32);
+           : (!dbl && !p.has_ph2) ? pass_ptr_f32_nph(mode, L.K, L.T >= 32)   // no phase cases
+                                  : pass_ptr(dbl, mode, L.K, L.T >= 32);
     if (!L.fn) return fail(VQC_ERR_UNSUPPORTED, "pass kernel not instantiated for this K");
     st = allow_max_smem(L.fn, dev, di.smem_optin);
     if (st != VQC_OK) return st;
     int per_sm = 0;
     VQC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, L.fn, L.block, L.smem));
     if (per_sm < 1) return fail(VQC_ERR_UNSUPPORTED, "pass kernel cannot be resident");
-    L.nunits = ((long long)B * L.ntiles + S - 1) / S;
-    L.grid = (int)std::max<long long>(1, std::min<long long>(L.nunits, (long long)per_sm * di.sms));
+    const long long nunits = ((long long)B * L.ntiles + S - 1) / S;
+    if ((long long)B * L.ntiles > 0x3fffffffLL) return fail(VQC_ERR_UNSUPPORTED, "too many tiles");
+    L.nunits = (int)nunits;
+    L.grid = std::max(1, std::min(L.nunits, per_sm * di.sms));
     return VQC_OK;
 }
 
@@ -872,7 +875,6 @@ void fill_pass_args(const HostPlan& p, const PassGeo& L, const FPass& ps, const 
     a.G = p.G_swz;
     a.S = L.S;
     a.nout = s.nout;
-    a.ntiles = L.ntiles;
     a.nstages = ps.stage_end - ps.stage_begin;
     a.nops = ps.op_end - ps.op_begin;
     a.op_begin = ps.op_begin;
@@ -898,9 +900,10 @@ void fill_pass_args(const HostPlan& p, const PassGeo& L, const FPass& ps, const 
         a.so[i] = back ? ps.oin[i] : ps.oout[i];
         a.sosl[i] = back ? 0 : ps.oslot[i];
     }
-    a.sm_sh = L.sm_sh; a.sm_ps = L.sm_ps; a.sm_psi = L.sm_psi; a.sm_lam = L.sm_lam;
+    a.sm_sh = L.sm_sh; a.sm_ps = L.sm_ps; a.sm_lam = L.sm_lam;
     a.sm_acc = L.sm_acc; a.sm_red = L.sm_red; a.sm_koff = L.sm_koff;
-    a.sm_plan = L.sm_plan; a.sm_tfl = L.sm_tfl;
+    a.sm_plan = L.sm_plan; a.sm_tfl = L.sm_tfl; a.sm_toff = L.sm_toff;
+    a.sm_tbase = L.sm_tbase;
 }
 
 // The forward passes: psi0 (nullptr: |0...0>) -> out in logical order (nullptr:

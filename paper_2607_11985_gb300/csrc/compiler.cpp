@@ -721,10 +721,10 @@ vqc_status compile_host(const vqc_gate* gates, int32_t G, int32_t n, int32_t nx,
     for (int mode = 0; mode < 2; ++mode) {
         const Schedule* h = find_hbm_schedule(p, mode);
         if (!h) continue;
-        int fm = std::min(frame_tile_qubits(mode, dtype), n - 1);
+        std::vector<int> tiles = frame_tile_qubits(mode, dtype, n);
         const int env_m = std::getenv("VQC_HBM_TILE_QUBITS") ? std::atoi(std::getenv("VQC_HBM_TILE_QUBITS")) : 0;
-        if (env_m > p.G_swz && env_m < n) fm = h->m;
-        p.frames.push_back(build_frame_schedule(p, mode, VQC_PATH_HBM, fm, h->K));
+        if (env_m > p.G_swz && env_m < n) tiles = {h->m};
+        p.frames.push_back(build_frame_schedule(p, mode, VQC_PATH_HBM, tiles, h->K));
     }
     return VQC_OK;
 }

@@ -91,10 +91,16 @@ inline int hbm_k(int mode, int dtype) {
     return mode == 0 ? 4 : 3;
 }
 
-// Tile qubits of the frame schedules of the HBM passes.
-inline int frame_tile_qubits(int mode, int dtype) {
-    if (dtype == VQC_C64) return mode == 0 ? 13 : 12;
-    return mode == 0 ? 12 : 11;
+// Tile bits offered to the frame schedules of the HBM passes.  complex64: 32 KiB of
+// forward tile (18-qubit / batch-48 forward 468 us, 500 with 13 bits, 502 with 11),
+// or one bit less where that costs no pass and no stage (16-qubit / batch-512 step
+// 6.39 ms against 6.66): a pass is bound by the latency of its stages, and smaller
+// tiles mean more CTAs per SM, each waiting for fewer warps.  complex128: 64 KiB
+// (16-qubit double-float step 9.72 ms, 10.3 with 11 / 10 bits).
+inline std::vector<int> frame_tile_qubits(int mode, int dtype, int n) {
+    auto fit = [n](int m) { return m < n - 1 ? m : n - 1; };
+    if (dtype == VQC_C64) return {fit(12), fit(11)};
+    return {fit(mode == 0 ? 12 : 11)};
 }
 
 // Maximum K per (mode, dtype) for register-resident blocks.

@@ -28,19 +28,68 @@ __device__ __forceinline__ uint32_t xor_bits(const void* v, int nb, int t) {
     return b;
 }
 
-// Slot base (and, when the stage needs them, outside parities) of thread t; fl is
-// the tile's flip of the stage.
-template <int K>
-__device__ __forceinline__ StageView frame_view(const FStage* sp, int t, uint32_t fl_slot, uint32_t fl_mask,
-                                                int h, int32_t (&sg)[K]) {
+// A thread's block in a stage: the byte offset of its base in the group's tiles and
+// (when the stage needs them) its outside parities; sb the local bits' byte offsets.
+// base: the offset in the tile that does not depend on the tile (frame_base); fl:
+// the tile's flip of the stage, as a byte offset, and its parities.
+struct FrameView {
+    uint32_t off, pb;
+};
+template <typename R>
+__device__ __forceinline__ uint32_t frame_base(const FStage* sp, int t, uint32_t g0) {
+    return (g0 ^ xor_bits(sp->tau, sp->nthreadbits, t)) * (uint32_t)sizeof(C2<R>);
+}
+template <typename R, int K>
+__device__ __forceinline__ FrameView frame_view(const FStage* sp, int t, uint32_t base, uint2 fl,
+                                                uint32_t (&sb)[K]) {
 #pragma unroll
-    for (int j = 0; j < K; ++j) sg[j] = sp->sigma[j];
-    const int nb = sp->nthreadbits;
-    StageView v;
-    v.swb = (uint32_t)h ^ fl_slot ^ xor_bits(sp->tau, nb, t);
+    for (int j = 0; j < K; ++j) sb[j] = (uint32_t)sp->sigma[j] * (uint32_t)sizeof(C2<R>);
+    FrameView v;
+    v.off = base ^ fl.x;
     v.pb = 0;
-    if (sp->nsel) v.pb = fl_mask ^ xor_bits(sp->tmask, nb, t);
+    if (sp->nsel) v.pb = fl.y ^ xor_bits(sp->tmask, sp->nthreadbits, t);
     return v;
+}
+
+// The block's amplitudes between registers and shared memory, in Gray-code order:
+// one XOR per access on a running byte offset (two of them, for the two halves of
+// the block).  tiles: start of the CTA's tiles.
+template <typename R, int K>
+__device__ __forceinline__ void frame_load(C2<R> (&a)[1 << K], const unsigned char* tiles, uint32_t off,
+                                           const uint32_t (&sb)[K]) {
+    constexpr int H = 1 << (K - 1);
+    uint32_t o0 = off, o1 = off ^ sb[K - 1];
+#pragma unroll
+    for (int i = 0; i < H; ++i) {
+        const int r = i ^ (i >> 1);
+        a[r] = *reinterpret_cast<const C2<R>*>(tiles + o0);
+        a[r | H] = *reinterpret_cast<const C2<R>*>(tiles + o1);
+        if (i + 1 < H) {
+            const int b = (i & 1) == 0 ? 0 : (i & 2) == 0 ? 1 : (i & 4) == 0 ? 2 : 3;   // the bit that changes
+            o0 ^= sb[b];
+            o1 ^= sb[b];
+        }
+    }
+}
+// (An empty asm hides off's value from the compiler, so that it does not keep the
+// load's offsets live in registers across the stage's ops.)
+template <typename R, int K>
+__device__ __forceinline__ void frame_store(const C2<R> (&a)[1 << K], unsigned char* tiles, uint32_t off,
+                                            const uint32_t (&sb)[K]) {
+    constexpr int H = 1 << (K - 1);
+    asm volatile("" : "+r"(off));
+    uint32_t o0 = off, o1 = off ^ sb[K - 1];
+#pragma unroll
+    for (int i = 0; i < H; ++i) {
+        const int r = i ^ (i >> 1);
+        *reinterpret_cast<C2<R>*>(tiles + o0) = a[r];
+        *reinterpret_cast<C2<R>*>(tiles + o1) = a[r | H];
+        if (i + 1 < H) {
+            const int b = (i & 1) == 0 ? 0 : (i & 2) == 0 ? 1 : (i & 4) == 0 ? 2 : 3;
+            o0 ^= sb[b];
+            o1 ^= sb[b];
+        }
+    }
 }
 
 // In place: v[c] becomes the sum over r of (-1)^parity(c & r) v[r].
@@ -107,6 +156,128 @@ __device__ __forceinline__ void lambda_frame(const uint8_t* lmask, uint32_t pbf,
     walsh<R, K>(g);
 #pragma unroll
     for (int r = 0; r < (1 << K); ++r) l[r] = cm<R>(g[r] * a[r].x, g[r] * a[r].y);
+}
+
+// ---------------------------------------------------------------- pure stages
+// A stage of 2x2 updates only, at most one per local position: straight-line code
+// over the positions, each under one uniform branch, instead of a descriptor load
+// and a jump per op.
+template <typename R>
+__device__ __forceinline__ const R* op_table(uint2 raw, const R* sh_tab, const R* ps_tab) {
+    return (((raw.x >> 24) & OPF_PER_SAMPLE) ? ps_tab : sh_tab) + EntryWords<R>::value * (raw.y & 0xffff);
+}
+
+template <typename R, int K>
+__device__ __forceinline__ void pure_forward(const uint2* ops, unsigned pm, C2<R> (&a)[1 << K], const R* sh_tab,
+                                             const R* ps_tab) {
+    const R* tp[K];
+    {
+        int o = 0;
+#pragma unroll
+        for (int j = 0; j < K; ++j) {
+            tp[j] = op_table<R>(ops[o], sh_tab, ps_tab);
+            o += (pm >> j) & 1;
+        }
+    }
+#define VQC_PURE(T_) \
+    if constexpr (T_ < K) if ((pm >> T_) & 1) m1_entry<R, K, T_, false>(a, tp[T_]);
+    VQC_PURE(0) VQC_PURE(1) VQC_PURE(2) VQC_PURE(3) VQC_PURE(4)
+#undef VQC_PURE
+}
+
+// Sum the three components of K <= 4 ops over a warp by one reduce-scatter
+// butterfly (13 shuffles for 4 ops).  Returns 4 op + component for the lanes
+// that end up with a sum (in v[0][0]), -1 for the others.
+template <typename R, int K>
+__device__ __forceinline__ int reduce_runs(R (&v)[K][3], int lane) {
+    static_assert(K >= 1 && K <= 4, "K");
+    const unsigned full = 0xffffffffu;
+    const int u0 = (lane >> 4) & 1, u1 = (lane >> 3) & 1, u2 = (lane >> 2) & 1, u3 = (lane >> 1) & 1;
+#pragma unroll
+    for (int i = 0; i < (K > 1 ? 2 : 1); ++i)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            if (i + 2 < K) {
+                const R send = u0 ? v[i][c] : v[i + 2 < K ? i + 2 : 0][c];
+                const R keep = u0 ? v[i + 2 < K ? i + 2 : 0][c] : v[i][c];
+                v[i][c] = keep + shx<R>(send, 16, full);
+            } else {
+                v[i][c] += shx<R>(v[i][c], 16, full);
+            }
+        }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        if (K > 1) {
+            const R send = u1 ? v[0][c] : v[K > 1 ? 1 : 0][c];
+            const R keep = u1 ? v[K > 1 ? 1 : 0][c] : v[0][c];
+            v[0][c] = keep + shx<R>(send, 8, full);
+        } else {
+            v[0][c] += shx<R>(v[0][c], 8, full);
+        }
+    }
+    const R p = shx<R>(u2 ? v[0][0] : v[0][2], 4, full), r = shx<R>(v[0][1], 4, full);
+    R x = (u2 ? v[0][2] : v[0][0]) + p, y = v[0][1] + r;
+    const R send = u2 ? x : (u3 ? x : y), keep = u2 ? x : (u3 ? y : x);
+    x = keep + shx<R>(send, 2, full);
+    x += shx<R>(x, 1, full);
+    v[0][0] = x;
+    const int op = 2 * u0 + u1;
+    return (lane & 1) || (u2 && u3) || op >= K ? -1 : 4 * op + (u2 ? 2 : u3);
+}
+
+// The adjoint of a pure stage.  Its runs act on different local bits, so every
+// run's (tx, ty, tz) can be taken at the stage's output, and one butterfly sums all
+// of them over the warp before the updates, whose registers it would otherwise
+// hold (16-qubit step 6.90 -> 6.74 ms).  Packed forms of the sums (two components
+// per FFMA2, the tz of all runs from one product per amplitude) execute fewer
+// instructions but measured 2-3% slower.
+template <int K>
+__device__ __forceinline__ void pure_backward(const uint2* ops, unsigned pm, float2 (&a)[1 << K],
+                                              float2 (&l)[1 << K], const float* sh_tab, const float* ps_tab,
+                                              float* acc, int wg, int lane, int warp_in_group) {
+    uint2 raw[K];
+    unsigned am = 0;   // positions that accumulate
+    {
+        int o = 0;
+#pragma unroll
+        for (int j = 0; j < K; ++j) {
+            raw[j] = ops[o];
+            const unsigned on = (pm >> j) & 1;
+            o += on;
+            am |= (on && ((raw[j].x >> 24) & OPF_HAS_ACC)) ? 1u << j : 0u;
+        }
+    }
+    if (am) {
+        float v[K][3];
+#pragma unroll
+        for (int j = 0; j < K; ++j) v[j][0] = v[j][1] = v[j][2] = 0;
+#define VQC_PURE(T_)                                     \
+        if constexpr (T_ < K)                            \
+            if ((am >> T_) & 1) {                        \
+                float t[4] = {0, 0, 0, 0};               \
+                m1_t3<float, K, T_>(a, l, t);            \
+                v[T_][0] = t[0];                         \
+                v[T_][1] = t[1];                         \
+                v[T_][2] = t[2];                         \
+            }
+        VQC_PURE(0) VQC_PURE(1) VQC_PURE(2) VQC_PURE(3)
+#undef VQC_PURE
+        const int idx = reduce_runs<float, K>(v, lane);
+        const int j = idx >> 2;
+        if (idx >= 0 && ((am >> j) & 1)) {
+            const unsigned aux = ops[__popc(pm & ((1u << j) - 1u))].y >> 16;
+            acc[((size_t)aux * wg + warp_in_group) * 8 + (idx & 3)] = v[0][0];
+        }
+    }
+#define VQC_PURE(T_)                                                                 \
+    if constexpr (T_ < K)                                                            \
+        if ((pm >> T_) & 1) {                                                        \
+            const float* tp = op_table<float>(raw[T_], sh_tab, ps_tab);              \
+            m1_entry<float, K, T_, true>(a, tp);                                     \
+            m1_entry<float, K, T_, true>(l, tp);                                     \
+        }
+    VQC_PURE(0) VQC_PURE(1) VQC_PURE(2) VQC_PURE(3)
+#undef VQC_PURE
 }
 
 }  // namespace vqc

@@ -105,7 +105,7 @@ struct FrameSchedule {
 struct HostPlan;
 
 // frames.cpp
-FrameSchedule build_frame_schedule(const HostPlan& p, int mode, int path, int m, int K);
+FrameSchedule build_frame_schedule(const HostPlan& p, int mode, int path, std::vector<int> tiles, int K);
 std::vector<uint8_t> export_frames(const HostPlan& p);
 
 }  // namespace vqc

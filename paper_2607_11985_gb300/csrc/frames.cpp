@@ -261,23 +261,19 @@ struct Rng {   // small deterministic generator (xorshift32) for the swizzle sea
     }
 };
 
-}  // namespace
-
-FrameSchedule build_frame_schedule(const HostPlan& p, int mode, int path, int m, int K) {
-    const int n = p.n, G = std::min(p.G_swz, m);
-    const bool tiled = path == VQC_PATH_HBM;
-    FrameSchedule S;
-    S.mode = mode;
-    S.K = K;
-    S.m = m;
-    S.path = path;
-    S.nout = n - m;
-    const int nout = n - m;
-
-    // the op list in the storage frame
-    std::vector<uint32_t> dir(n), sel(n);
-    for (int q = 0; q < n; ++q) dir[q] = sel[q] = 1u << q;
+// The op list in the storage frame, and the frame at its end.
+struct FrameOps {
+    std::vector<uint32_t> dir, sel;
     std::vector<FOp> f;
+};
+
+FrameOps lower(const HostPlan& p) {
+    const int n = p.n;
+    FrameOps L;
+    std::vector<uint32_t>&dir = L.dir, &sel = L.sel;
+    dir.resize(n);
+    sel.resize(n);
+    for (int q = 0; q < n; ++q) dir[q] = sel[q] = 1u << q;
     for (size_t i = 0; i < p.ops.size(); ++i) {
         const HOp& o = p.ops[i];
         if (o.type == OP_CX) {
@@ -291,8 +287,17 @@ FrameSchedule build_frame_schedule(const HostPlan& p, int mode, int path, int m,
         g.r = sel[o.q0];
         if (g.run) g.d = dir[o.q0];
         else g.r2 = sel[o.q1];
-        f.push_back(g);
+        L.f.push_back(g);
     }
+    return L;
+}
+
+// The passes over tiles of m bits (the resident path: one pass, m = n) and their
+// stages of K directions.
+std::vector<PassPlan> plan_passes(const HostPlan& p, const FrameOps& L, int mode, bool tiled, int m, int K) {
+    const int n = p.n, G = std::min(p.G_swz, m);
+    const std::vector<FOp>& f = L.f;
+    const std::vector<uint32_t>& dir = L.dir;
 
     // ---- passes: each takes, in time order, every op that commutes with the ops
     // it leaves behind while the tile has room for its direction.  At most m - G
@@ -392,8 +397,6 @@ FrameSchedule build_frame_schedule(const HostPlan& p, int mode, int path, int m,
             if (end) break;
         }
     }
-    const int np = (int)passes.size();
-
     // ---- stages of each pass; a stage whose diagonal ops leave no room for its
     // pads gives its later diagonal ops to a stage of their own
     for (PassPlan& ps : passes) {
@@ -418,6 +421,38 @@ FrameSchedule build_frame_schedule(const HostPlan& p, int mode, int path, int m,
         }
         ps.stages = std::move(out);
     }
+    return passes;
+}
+
+}  // namespace
+
+FrameSchedule build_frame_schedule(const HostPlan& p, int mode, int path, std::vector<int> tiles, int K) {
+    const int n = p.n;
+    const bool tiled = path == VQC_PATH_HBM;
+    const FrameOps L = lower(p);
+    const std::vector<FOp>& f = L.f;
+    const std::vector<uint32_t>&dir = L.dir, &sel = L.sel;
+
+    // of the tile sizes offered, the first unless a later one takes no more passes and stages
+    int m = 0;
+    size_t nst = 0;
+    std::vector<PassPlan> passes;
+    for (int t : tiles) {
+        std::vector<PassPlan> q = plan_passes(p, L, mode, tiled, t, K);
+        size_t c = 0;
+        for (const PassPlan& ps : q) c += ps.stages.size();
+        if (m && (q.size() > passes.size() || c > nst)) continue;
+        m = t;
+        nst = c;
+        passes = std::move(q);
+    }
+    const int G = std::min(p.G_swz, m), np = (int)passes.size(), nout = n - m;
+    FrameSchedule S;
+    S.mode = mode;
+    S.K = K;
+    S.m = m;
+    S.path = path;
+    S.nout = nout;
 
     // ---- addresses, slots and records, in the order the passes run (the backward
     // from the last).  A pass reads the state at the addresses M s; the forward

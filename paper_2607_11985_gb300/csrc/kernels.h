@@ -18,7 +18,7 @@ const void* sweep_ptr_f32_fused(int K, bool full);   // backward that also write
 const void* sweep_ptr_f32_fwd_nph(int K, bool full);
 const void* sweep_ptr_f32_bwd_nph(int K, bool full);
 const void* sweep_ptr_f32_fused_nph(int K, bool full);
-const void* pass_ptr_f32_fwd_nph(int K, bool full);
+const void* pass_ptr_f32_nph(int mode, int K, bool full);
 const void* sweep_ptr_f64_fused(int K, bool full);
 // double-float arithmetic on complex128 storage (VQC_C128_DF plans)
 const void* sweep_ptr_dd_fwd(int K, bool full);

@@ -24,13 +24,13 @@ struct PArgs {
     const FFinal* fin;            // last pass only (forward: <Z>; backward: lam = O psi)
     const int32_t* pass_entries;  // table slots of the pass's entries
     const int32_t* pass_accs;
-    int n, m, tbits, G, S, nout, ntiles, nstages, nops, op_begin;
+    int n, m, tbits, G, S, nout, nstages, nops, op_begin;
     int ps_begin, ps_count, sh_begin, sh_count, acc_begin, acc_count, n_accs;
     const void* ps_g;       // per-sample table entries [B][n_ps][entry words], kernel real type
     const void* sh_g;       // shared table entries [n_sh][entry words] (both from run_tables)
     int n_ps;
     int B;
-    long long nunits;
+    int nunits;
     uint32_t ga[kMaxTileBits], sa[kMaxTileBits];   // tile bit -> address, read and written order
     int32_t gs[kMaxTileBits], ss[kMaxTileBits];    // tile bit -> slot, read and written order
     uint32_t go[kMaxOuterBits], so[kMaxOuterBits]; // tile index bit -> address
@@ -42,9 +42,11 @@ struct PArgs {
     C2<R>* dst_lam;
     R* E_part;              // forward, last pass: [B * ntiles, n]
     R* rho;                 // backward: per-tile rho sums [B * ntiles][n_accs][4] (3 used)
-    int sm_sh, sm_ps, sm_psi, sm_lam, sm_acc, sm_red;
+    int sm_sh, sm_ps, sm_lam, sm_acc, sm_red;
     int sm_plan;            // copies of the pass's stages, ops, flips and fin
     int sm_tfl;             // per tile: each stage's flip (uint2), then the logical parities
+    int sm_tbase;           // each thread's block base in every stage: [nstages][threads]
+    int sm_toff;            // tile-copy offsets of each thread: uint4
     int sm_koff;            // tile-copy offsets per vector round, read order then written order: uint2
     unsigned* err;          // the plan's error word (launch self-check)
     // double-float kernels only: src_psi / src_lam / dst_psi and dst_lam hold
@@ -170,8 +172,8 @@ __global__ void __launch_bounds__(256, 2) pass_kernel(const __grid_constant__ PA
     extern __shared__ __align__(16) unsigned char smem[];
     R* sh_tab = reinterpret_cast<R*>(smem + A.sm_sh);
     R* ps_all = reinterpret_cast<R*>(smem + A.sm_ps);
-    C2<R>* psi_all = reinterpret_cast<C2<R>*>(smem + A.sm_psi);
-    C2<R>* lam_all = reinterpret_cast<C2<R>*>(smem + A.sm_lam);
+    unsigned char* psi_t = smem;                // the CTA's S tiles first, so that a slot's byte
+    unsigned char* lam_t = smem + A.sm_lam;     // offset is its address up to a constant
     R* acc_all = reinterpret_cast<R*>(smem + A.sm_acc);
     R* red_all = reinterpret_cast<R*>(smem + A.sm_red);
     const int nthr = blockDim.x, nst = A.nstages;
@@ -191,8 +193,13 @@ __global__ void __launch_bounds__(256, 2) pass_kernel(const __grid_constant__ PA
         async_elem<uint2>(reinterpret_cast<uint2*>(flips) + i, reinterpret_cast<const uint2*>(A.flips) + i);
 
     const int n = A.n, G = A.G, tdim = 1 << A.m;
-    const long long total_tiles = (long long)A.B * A.ntiles;
+    const int total_tiles = A.B << A.nout;   // (at most states in memory over 64 amplitudes)
+    const uint32_t tmask = (1u << A.nout) - 1u;
     constexpr bool DDK = !std::is_same<St<R>, R>::value;   // double-float kernel
+    // straight-line stages: complex64 only (16-qubit workload 7.61 -> 7.24 ms); the
+    // double-float and FP64 updates are long enough to hide the dispatch, and the
+    // extra code costs them registers (double-float 9.87 -> 10.05 ms)
+    constexpr bool PURE = FULL && std::is_same<R, float>::value;
     Geo q;
     q.T = 1 << A.tbits;
     q.lanes = q.T < 32 ? q.T : 32;
@@ -216,9 +223,13 @@ __global__ void __launch_bounds__(256, 2) pass_kernel(const __grid_constant__ PA
         koff_g[k] = make_uint2(xor_cols(A.ga, u), xor_cols(A.gs, u));
         koff_s[k] = make_uint2(xor_cols(A.sa, u), xor_cols(A.ss, u));
     }
-    const uint32_t u_t = (uint32_t)q.t * APV;
-    const uint32_t g_addr = xor_cols(A.ga, u_t), g_slot = xor_cols(A.gs, u_t) ^ (uint32_t)q.h;
-    const uint32_t s_addr = xor_cols(A.sa, u_t), s_slot = xor_cols(A.ss, u_t) ^ (uint32_t)q.h;
+    // each thread's own part, kept in shared memory: four registers across the stages
+    uint4* toff = reinterpret_cast<uint4*>(smem + A.sm_toff) + threadIdx.x;
+    {
+        const uint32_t u = (uint32_t)q.t * APV;
+        *toff = make_uint4(xor_cols(A.ga, u), xor_cols(A.gs, u) ^ (uint32_t)q.h, xor_cols(A.sa, u),
+                           xor_cols(A.ss, u) ^ (uint32_t)q.h);
+    }
     const uint32_t g_one = (uint32_t)A.gs[0], s_one = (uint32_t)A.ss[0];
 
     grid_dep_wait();
@@ -235,29 +246,33 @@ __global__ void __launch_bounds__(256, 2) pass_kernel(const __grid_constant__ PA
     async_wait();
     __syncthreads();
 
-    C2<R>* psi = psi_all + (size_t)q.g * tdim;
-    C2<R>* lam = lam_all + (size_t)q.g * tdim;
+    C2<R>* psi = reinterpret_cast<C2<R>*>(psi_t) + (size_t)q.g * tdim;
+    C2<R>* lam = reinterpret_cast<C2<R>*>(lam_t) + (size_t)q.g * tdim;
+    const uint32_t g0 = (uint32_t)(q.g * tdim) ^ (uint32_t)q.h;
     R* ps_tab = ps_all + (size_t)q.g * A.ps_count * EntryWords<R>::value;
     R* acc = acc_all + (size_t)q.g * A.acc_count * q.wg * 8;
     uint2* tfl_all = reinterpret_cast<uint2*>(smem + A.sm_tfl);
     const uint2* tfl = tfl_all + q.g * (nst + 1);
+    // each thread's block base in every stage (read by itself only)
+    uint32_t* tbase = reinterpret_cast<uint32_t*>(smem + A.sm_tbase) + threadIdx.x;
+    for (int s = 0; s < nst; ++s) tbase[s * nthr] = frame_base<R>(stages + s, q.t, g0);
 
-    for (long long unit = blockIdx.x; unit < A.nunits; unit += gridDim.x) {
-        const long long tid_raw = unit * A.S + q.g;
+    for (int unit = blockIdx.x; unit < A.nunits; unit += gridDim.x) {
+        const int tid_raw = unit * A.S + q.g;
         const bool valid = tid_raw < total_tiles;
-        const long long tile_id = valid ? tid_raw : total_tiles - 1;
-        const int b = (int)(tile_id / A.ntiles);
-        const uint32_t tau = (uint32_t)(tile_id % A.ntiles);
+        const int tile_id = valid ? tid_raw : total_tiles - 1;
+        const int b = tile_id >> A.nout;
+        const uint32_t tau = (uint32_t)tile_id & tmask;
 
         // the tile's flip of each stage, and its logical parities
         for (int i = threadIdx.x; i < A.S * (nst + 1); i += nthr) {
             const int gg = i / (nst + 1), s = i - gg * (nst + 1);
-            const uint32_t tt = (uint32_t)(min(unit * A.S + gg, total_tiles - 1) % A.ntiles);
+            const uint32_t tt = (uint32_t)min(unit * A.S + gg, total_tiles - 1) & tmask;
             uint2 f = make_uint2(0, 0);
             if (s < nst) {
                 for (int o = 0; o < A.nout; ++o)
                     if ((tt >> o) & 1) {
-                        f.x ^= (uint32_t)flips[s * A.nout + o].slot;
+                        f.x ^= (uint32_t)flips[s * A.nout + o].slot * (uint32_t)sizeof(C2<R>);
                         f.y ^= flips[s * A.nout + o].mask;
                     }
             } else if (A.fin) {
@@ -272,12 +287,13 @@ __global__ void __launch_bounds__(256, 2) pass_kernel(const __grid_constant__ PA
             const int per = A.ps_count * V;
             for (int i = threadIdx.x; i < A.S * per; i += nthr) {
                 const int gg = i / per, r = i - gg * per, k = r / V, v = r - k * V;
-                const int bb = (int)(min(unit * A.S + gg, total_tiles - 1) / A.ntiles);
+                const int bb = min(unit * A.S + gg, total_tiles - 1) >> A.nout;
                 stab[i] = gtab[((size_t)bb * A.n_ps + vqc_ld(&A.pass_entries[A.ps_begin + k])) * V + v];
             }
         }
         const size_t sbase = (size_t)b << n;
-        const uint32_t ga = g_addr ^ xor_cols(A.go, tau);
+        const uint2 gto = *reinterpret_cast<const uint2*>(toff);
+        const uint32_t ga = gto.x ^ xor_cols(A.go, tau), g_slot = gto.y;
         if (A.src_psi) {
             if (DDK && A.src_raw) tile_gather<R, DDK>(psi, A.src_psi + sbase, ga, g_slot, g_one, koff_g, nk);
             else   // 16 loads in flight where one state is gathered, 8 beside lam's registers
@@ -287,35 +303,38 @@ __global__ void __launch_bounds__(256, 2) pass_kernel(const __grid_constant__ PA
             if (DDK && A.lam_raw) tile_gather<R, DDK>(lam, A.src_lam + sbase, ga, g_slot, g_one, koff_g, nk);
             else tile_gather<R>(lam, A.src_lam + sbase, ga, g_slot, g_one, koff_g, nk);
         }
-        if (unit + gridDim.x < A.nunits) {   // the CTA's next tile into L2 during this one's stages
-            const long long nt = min((unit + gridDim.x) * A.S + q.g, total_tiles - 1);
-            const uint32_t nga = g_addr ^ xor_cols(A.go, (uint32_t)(nt % A.ntiles));
-            const size_t nsb = (size_t)(nt / A.ntiles) << n;
+        if (unit + (int)gridDim.x < A.nunits) {   // the CTA's next tile into L2 during this one's stages
+            const int nt = min((int)(unit + gridDim.x) * A.S + q.g, total_tiles - 1);
+            const uint32_t nga = gto.x ^ xor_cols(A.go, (uint32_t)nt & tmask);
+            const size_t nsb = (size_t)(nt >> A.nout) << n;
             if (A.src_psi) tile_prefetch<R>(A.src_psi + nsb, nga, koff_g, nk, q.t);
             if (MODE == 1 && A.src_lam) tile_prefetch<R>(A.src_lam + nsb, nga, koff_g, nk, q.t);
         }
         __syncthreads();
 
         C2<R> a[1 << K];
-        int32_t sg[K];
-        StageView v{0, 0};
+        uint32_t sb[K];
+        FrameView v{0, 0};
         if constexpr (MODE == 0) {
             for (int s = 0; s < nst; ++s) {
                 const FStage* sp = stages + s;
                 const uint2 fl = tfl[s];
-                v = frame_view<K>(sp, q.t, fl.x, fl.y, q.h, sg);
+                v = frame_view<R, K>(sp, q.t, tbase[s * nthr], fl, sb);
                 if (s == 0 && !A.src_psi) {
 #pragma unroll
                     for (int r = 0; r < (1 << K); ++r) a[r] = cm<R>(0, 0);
                     if ((q.t | tau) == 0) a[0] = cm<R>(1, 0);
                 } else {
-                    block_load<R, K>(a, psi, v.swb, sg);
+                    frame_load<R, K>(a, psi_t, v.off, sb);
                 }
-                run_ops<R, K, 0, false, FULL, PH2>(reinterpret_cast<const DOp*>(ops), sp->op_begin - A.op_begin,
-                                                   sp->op_end - A.op_begin, v.pb, a, a, sh_tab, ps_tab, nullptr, q,
-                                                   lane, warp_in_group);
+                if (PURE && sp->pure)
+                    pure_forward<R, K>(ops + (sp->op_begin - A.op_begin), sp->pmask, a, sh_tab, ps_tab);
+                else
+                    run_ops<R, K, 0, false, FULL, PH2>(reinterpret_cast<const DOp*>(ops), sp->op_begin - A.op_begin,
+                                                       sp->op_end - A.op_begin, v.pb, a, a, sh_tab, ps_tab, nullptr,
+                                                       q, lane, warp_in_group);
                 if (s + 1 < nst || A.dst_psi) {
-                    block_store<R, K>(a, psi, v.swb, sg);
+                    frame_store<R, K>(a, psi_t, v.off, sb);
                     group_sync<R>(q);
                 }
             }
@@ -328,12 +347,13 @@ __global__ void __launch_bounds__(256, 2) pass_kernel(const __grid_constant__ PA
                     for (int j = q.t; j < n; j += q.T) {
                         R e = 0;
                         for (int k = 0; k < q.wg; ++k) e += red[k * n + j];
-                        A.E_part[tile_id * n + j] = as_out<St<R>>(e);
+                        A.E_part[(size_t)tile_id * n + j] = as_out<St<R>>(e);
                     }
             }
             __syncthreads();
             if (A.dst_psi && valid) {
-                const uint32_t da = s_addr ^ xor_cols(A.so, tau), ds = s_slot ^ xor_cols(A.sosl, tau);
+                const uint2 sto = *(reinterpret_cast<const uint2*>(toff) + 1);
+                const uint32_t da = sto.x ^ xor_cols(A.so, tau), ds = sto.y ^ xor_cols(A.sosl, tau);
                 if (DDK && A.dst_raw) tile_scatter<R, DDK>(psi, A.dst_psi + sbase, da, ds, s_one, koff_s, nk);
                 else tile_scatter<R>(psi, A.dst_psi + sbase, da, ds, s_one, koff_s, nk);
             }
@@ -344,26 +364,35 @@ __global__ void __launch_bounds__(256, 2) pass_kernel(const __grid_constant__ PA
                 const FStage* sp = stages + s;
                 const uint2 fl = tfl[s];
                 C2<R> l[1 << K];
-                v = frame_view<K>(sp, q.t, fl.x, fl.y, q.h, sg);
-                block_load<R, K>(a, psi, v.swb, sg);
+                v = frame_view<R, K>(sp, q.t, tbase[s * nthr], fl, sb);
+                frame_load<R, K>(a, psi_t, v.off, sb);
                 if (s == nst - 1 && !A.src_lam) {
                     const uint32_t pbf = tfl[nst].x ^ xor_bits(fin->tmask, A.tbits, q.t);
                     lambda_frame<R, K>(fin->lmask, pbf, A.gE + (size_t)b * n, n, a, l);
                 } else {
-                    block_load<R, K>(l, lam, v.swb, sg);
+                    frame_load<R, K>(l, lam_t, v.off, sb);
                 }
-                run_ops<R, K, 1, false, FULL, PH2>(reinterpret_cast<const DOp*>(ops), sp->op_begin - A.op_begin,
-                                                   sp->op_end - A.op_begin, v.pb, a, l, sh_tab, ps_tab, acc, q, lane,
-                                                   warp_in_group);
+                bool pure = false;
+                if constexpr (PURE) {
+                    pure = sp->pure;
+                    if (pure)
+                        pure_backward<K>(ops + (sp->op_begin - A.op_begin), sp->pmask, a, l, sh_tab, ps_tab, acc,
+                                         q.wg, lane, warp_in_group);
+                }
+                if (!pure)
+                    run_ops<R, K, 1, false, FULL, PH2>(reinterpret_cast<const DOp*>(ops), sp->op_begin - A.op_begin,
+                                                       sp->op_end - A.op_begin, v.pb, a, l, sh_tab, ps_tab, acc, q,
+                                                       lane, warp_in_group);
                 if (s > 0 || A.dst_psi) {
-                    block_store<R, K>(a, psi, v.swb, sg);
-                    block_store<R, K>(l, lam, v.swb, sg);
+                    frame_store<R, K>(a, psi_t, v.off, sb);
+                    frame_store<R, K>(l, lam_t, v.off, sb);
                 }
                 group_sync<R>(q);
             }
             __syncthreads();
             if (valid && A.dst_psi) {
-                const uint32_t da = s_addr ^ xor_cols(A.so, tau);
+                const uint2 sto = *(reinterpret_cast<const uint2*>(toff) + 1);
+                const uint32_t da = sto.x ^ xor_cols(A.so, tau), s_slot = sto.y;
                 if (DDK && A.dst_raw) {
                     tile_scatter<R, DDK>(psi, A.dst_psi + sbase, da, s_slot, s_one, koff_s, nk);
                     tile_scatter<R, DDK>(lam, A.dst_lam + sbase, da, s_slot, s_one, koff_s, nk);
@@ -376,7 +405,7 @@ __global__ void __launch_bounds__(256, 2) pass_kernel(const __grid_constant__ PA
             // components; the per-sample turn into terms is reduce_terms' work
             for (int i = threadIdx.x; i < A.S * A.acc_count * 3; i += nthr) {
                 const int gg = i / (A.acc_count * 3), r = i % (A.acc_count * 3), k = r / 3, c = r % 3;
-                const long long tt = unit * A.S + gg;
+                const int tt = unit * A.S + gg;
                 if (tt >= total_tiles) continue;
                 const R* ap = acc_all + ((size_t)gg * A.acc_count + k) * q.wg * 8 + c;
                 R sum = 0;
