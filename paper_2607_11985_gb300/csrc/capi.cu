@@ -119,11 +119,12 @@ size_t align256(size_t v) { return (v + 255) & ~size_t(255); }
 
 // Launch geometry of one call.
 struct Launch {
-    const Schedule* s = nullptr;
-    int K = 0, T = 0, S = 0, block = 0, grid = 0, nunits = 0, wg = 1, bpt = 1;
+    const Schedule* s = nullptr;        // cluster path
+    const FrameSchedule* f = nullptr;   // resident path
+    int K = 0, T = 0, S = 0, block = 0, grid = 0, nunits = 0, wg = 1;
     size_t smem = 0;
     int sm_sh = 0, sm_ps = 0, sm_psi = 0, sm_lam = 0, sm_acc = 0, sm_terms = 0, sm_dw = 0,
-        sm_red = 0, sm_plan = 0, sm_w = 0, sm_xg = 0;
+        sm_red = 0, sm_plan = 0, sm_w = 0, sm_xg = 0, sm_io = 0;
     int cl = 0, sm_ecl = 0;   // cluster path: log2 CTAs per sample, <Z> gather area
     bool plan_smem = false;
     const void* fn = nullptr;
@@ -170,15 +171,15 @@ int cta_threads() {
 // extra warps hide latency.
 int choose_k(const HostPlan& p, int mode, int B, int sms) {
     int forced = env_int(mode == 0 ? "VQC_FORCE_K_FWD" : "VQC_FORCE_K_BWD", 0);
-    if (forced > 0 && find_schedule(p, mode, forced)) return forced;
+    if (forced > 0 && find_frame(p, mode, VQC_PATH_RESIDENT, forced)) return forced;
     int kmax = 0;
-    for (const auto& s : p.scheds)
+    for (const auto& s : p.frames)
         if (s.mode == mode && s.path == VQC_PATH_RESIDENT) kmax = std::max(kmax, s.K);
     if (kmax == 0) return 0;
     const int kmin = std::min(kmax, 3);
     const double want = (double)sms * 4 * 32;
     int K = kmax;
-    while (K > kmin && (double)B * std::ldexp(1.0, p.n - K) < want && find_schedule(p, mode, K - 1))
+    while (K > kmin && (double)B * std::ldexp(1.0, p.n - K) < want && find_frame(p, mode, VQC_PATH_RESIDENT, K - 1))
         --K;
     return K;
 }
@@ -192,22 +193,20 @@ vqc_status plan_launch_uncached(const HostPlan& p, int launch_mode, int B, Launc
     vqc_status st = device_info(dev, di);
     if (st != VQC_OK) return st;
     L.K = choose_k(p, mode, B, di.sms);
-    L.s = L.K ? find_schedule(p, mode, L.K) : nullptr;
-    if (!L.s)
+    L.f = L.K ? find_frame(p, mode, VQC_PATH_RESIDENT, L.K) : nullptr;
+    if (!L.f)
         return fail(VQC_ERR_UNSUPPORTED, "no resident schedule for this circuit (n = " +
                                              std::to_string(p.n) + ")");
     const bool dbl = p.dtype == VQC_C128;
     const size_t rs = dbl ? 8 : 4, cs = 2 * rs;
-    // A sample needs 2^(n-K) register blocks; a group of at most 256 threads
-    // holds them, bpt blocks per thread.
-    L.T = std::min(1 << (p.n - L.K), sweep_max_threads(dbl, mode, L.K));
-    L.bpt = (1 << (p.n - L.K)) / L.T;
+    L.T = 1 << (p.n - L.K);   // one register block per thread (n - K <= 9)
     L.wg = L.T > 32 ? L.T / 32 : 1;
     // Shared memory: a fixed part per CTA and a part per resident sample.
     const size_t dim = (size_t)1 << p.n;
     const size_t ew = dbl ? 8 : 32;   // reals per table entry
+    const size_t io = (size_t)8 << L.K;   // slot offsets of the state copies
     const size_t fixed = align16((size_t)p.n_sh * ew * rs) + align16(mode == 1 ? (size_t)p.num_w * rs : 0) +
-                         align16((size_t)p.num_w * rs) + 10 * 16;
+                         align16((size_t)p.num_w * rs) + io + 10 * 16;
     const size_t per_sample = (size_t)p.n_ps * ew * rs + dim * cs * (mode == 1 ? 2 : 1) +
                               (size_t)(p.num_x + p.n) * rs +
                               (mode == 1 ? p.accs.size() * L.wg * 8 * rs + p.term_src.size() * rs : 0) +
@@ -229,7 +228,7 @@ vqc_status plan_launch_uncached(const HostPlan& p, int launch_mode, int B, Launc
     if (L.T < 32 && S * L.T > 32) S -= S % (32 / L.T);
     L.S = S;
     L.block = L.S * L.T;
-    if (L.block > sweep_max_threads(dbl, mode, L.K))
+    if (L.block > kSweepMaxThreads)
         return fail(VQC_ERR_UNSUPPORTED, "thread group too large for this kernel");
     size_t off = 0;
     auto take = [&](size_t bytes) {
@@ -237,10 +236,11 @@ vqc_status plan_launch_uncached(const HostPlan& p, int launch_mode, int B, Launc
         off = align16(off + bytes);
         return (int)o;
     };
+    take((size_t)L.S * dim * cs);   // psi at offset 0
+    L.sm_lam = take(mode == 1 ? (size_t)L.S * dim * cs : 0);
     L.sm_sh = take((size_t)p.n_sh * ew * rs);
     L.sm_ps = take((size_t)L.S * p.n_ps * ew * rs);
-    L.sm_psi = take((size_t)L.S * dim * cs);
-    L.sm_lam = take(mode == 1 ? (size_t)L.S * dim * cs : 0);
+    L.sm_io = take(io);
     L.sm_acc = take(mode == 1 ? (size_t)L.S * p.accs.size() * L.wg * 8 * rs : 0);
     L.sm_terms = take(mode == 1 ? (size_t)L.S * p.term_src.size() * rs : 0);
     L.sm_dw = take(mode == 1 ? (size_t)p.num_w * rs : 0);
@@ -249,7 +249,7 @@ vqc_status plan_launch_uncached(const HostPlan& p, int launch_mode, int B, Launc
     L.sm_xg = take((size_t)L.S * (p.num_x + p.n) * rs);
     // the plan's table data and this schedule go to shared memory when they fit
     const size_t plan_bytes = align16(p.dev_tab_end - p.dev_tab_begin) +
-                              (L.s->dev_region_end - L.s->dev_region_begin);
+                              (L.f->dev_region_end - L.f->dev_region_begin);
     L.plan_smem = off + plan_bytes <= (size_t)di.smem_optin && env_int("VQC_PLAN_IN_SMEM", 1) != 0;
     L.sm_plan = L.plan_smem ? take(plan_bytes) : 0;
     L.smem = off;
@@ -301,9 +301,24 @@ vqc_status plan_launch(const HostPlan& p, int mode, int B, Launch& L) {
 template <typename R>
 void fill_plan_args(const HostPlan& p, const Launch& L, KArgs<R>& a) {
     const char* base = static_cast<const char*>(p.dbuf);
-    a.ops = reinterpret_cast<const DOp*>(base + L.s->dev_ops);
-    a.stages = reinterpret_cast<const DStage*>(base + L.s->dev_stages);
-    a.nstages = (int)L.s->stages.size();
+    if (L.f) {
+        a.ops = reinterpret_cast<const DOp*>(base + L.f->dev_ops);
+        a.fstages = reinterpret_cast<const FStage*>(base + L.f->dev_stages);
+        a.fin = reinterpret_cast<const FFinal*>(base + L.f->dev_fin);
+        a.nstages = (int)L.f->stages.size();
+        for (int i = 0; i < p.n; ++i) {
+            a.sin[i] = L.f->passes[0].sin[i];
+            a.sout[i] = L.f->passes[0].sout[i];
+        }
+        a.sched_off = (int)L.f->dev_region_begin;
+        a.sched_bytes = (int)(L.f->dev_region_end - L.f->dev_region_begin);
+    } else {
+        a.ops = reinterpret_cast<const DOp*>(base + L.s->dev_ops);
+        a.stages = reinterpret_cast<const DStage*>(base + L.s->dev_stages);
+        a.nstages = (int)L.s->stages.size();
+        a.sched_off = (int)L.s->dev_region_begin;
+        a.sched_bytes = (int)(L.s->dev_region_end - L.s->dev_region_begin);
+    }
     a.entries = reinterpret_cast<const DEntry*>(base + p.dev_entries);
     a.ps_list = reinterpret_cast<const int32_t*>(base + p.dev_ps_list);
     a.sh_list = reinterpret_cast<const int32_t*>(base + p.dev_sh_list);
@@ -322,7 +337,6 @@ void fill_plan_args(const HostPlan& p, const Launch& L, KArgs<R>& a) {
     a.G = p.G_swz;
     a.S = L.S;
     a.tpg = L.T;
-    a.bpt = L.bpt;
     a.n_ps = p.n_ps;
     a.n_sh = p.n_sh;
     a.n_accs = (int)p.accs.size();
@@ -332,12 +346,10 @@ void fill_plan_args(const HostPlan& p, const Launch& L, KArgs<R>& a) {
     a.Pw = p.num_w;
     a.sm_sh = L.sm_sh; a.sm_ps = L.sm_ps; a.sm_psi = L.sm_psi; a.sm_lam = L.sm_lam;
     a.sm_acc = L.sm_acc; a.sm_terms = L.sm_terms; a.sm_dw = L.sm_dw; a.sm_red = L.sm_red;
-    a.sm_w = L.sm_w; a.sm_xg = L.sm_xg;
+    a.sm_w = L.sm_w; a.sm_xg = L.sm_xg; a.sm_io = L.sm_io;
     a.plan = static_cast<const unsigned char*>(p.dbuf);
     a.tab_off = (int)p.dev_tab_begin;
     a.tab_bytes = (int)(p.dev_tab_end - p.dev_tab_begin);
-    a.sched_off = (int)L.s->dev_region_begin;
-    a.sched_bytes = (int)(L.s->dev_region_end - L.s->dev_region_begin);
     a.sm_plan = L.sm_plan;
     a.plan_smem = L.plan_smem ? 1 : 0;
     a.cl = L.cl;
@@ -400,10 +412,12 @@ vqc_status upload(HostPlan& p) {
         s.dev_region_end = blob.size();
     }
     for (auto& s : p.frames) {
+        s.dev_region_begin = blob.size();
         s.dev_ops = put(s.ops.data(), s.ops.size() * sizeof(DOp));
         s.dev_stages = put(s.stages.data(), s.stages.size() * sizeof(FStage));
-        s.dev_flips = put(s.flips.data(), s.flips.size() * sizeof(FFlip));
         s.dev_fin = put(&s.fin, sizeof(FFinal));
+        s.dev_region_end = blob.size();
+        s.dev_flips = put(s.flips.data(), s.flips.size() * sizeof(FFlip));
         // the passes copy their entries from the tables by slot
         std::vector<int32_t> slots;
         for (int32_t e : s.pass_entries) slots.push_back(p.entries[e].slot);
@@ -513,7 +527,6 @@ vqc_status plan_cluster(const HostPlan& p, int mode, int B, Launch& L) {
     L.T = 1 << (p.n - L.K);           // threads of a sample group, over the whole cluster
     L.block = L.T >> L.cl;            // 2^cta_bits: 256 or 512
     L.S = 1;
-    L.bpt = 1;
     L.wg = L.block / 32;
     size_t off = 0;
     auto take = [&](size_t bytes) {
@@ -1587,32 +1600,33 @@ vqc_status vqc_plan_info(const vqc_plan* plan, int32_t batch, vqc_plan_stats* ou
         const bool clu = use_cluster(p, mode);
         const bool hbm = !clu && (ndev > 0 ? use_hbm(p, mode, B)
                                            : (K == 0 && find_frame(p, mode, VQC_PATH_HBM) != nullptr));
-        if (hbm) {
-            const FrameSchedule* s = find_frame(p, mode, VQC_PATH_HBM);
-            const int P = (int)s->passes.size();
+        if (clu) {
+            const Schedule* s = find_cluster_schedule(p, mode);
             *path = s->path;
             *kk = s->K;
             *ns = (int)s->stages.size();
             *tq = s->m;
-            *np = P;
-            *tps = (1 << (s->m - s->K)) << (p.n - s->m);
-            // state traffic: forward reads and writes the state once per pass;
-            // the backward reads psi (and lam after the first pass) and writes
-            // both (except after the last pass)
-            *hb = mode == 0 ? 2.0 * P * sbytes : (4.0 * P - 3.0) * sbytes;
+            *np = 1;
+            *tps = 1 << (p.n - s->K);
             continue;
         }
-        const Schedule* s = clu ? find_cluster_schedule(p, mode) : (K ? find_schedule(p, mode, K) : nullptr);
+        const FrameSchedule* s = hbm ? find_frame(p, mode, VQC_PATH_HBM)
+                                     : K ? find_frame(p, mode, VQC_PATH_RESIDENT, K) : nullptr;
         if (!s) {
             *path = -1;
             continue;
         }
+        const int P = (int)s->passes.size();
         *path = s->path;
         *kk = s->K;
         *ns = (int)s->stages.size();
         *tq = s->m;
-        *np = 1;
-        *tps = 1 << (p.n - s->K);
+        *np = P;
+        *tps = (1 << (s->m - s->K)) << s->nout;
+        // state traffic of the HBM passes: forward reads and writes the state once
+        // per pass; the backward reads psi (and lam after the first pass) and writes
+        // both (except after the last pass)
+        if (hbm) *hb = mode == 0 ? 2.0 * P * sbytes : (4.0 * P - 3.0) * sbytes;
     }
     g_err = saved;
     return VQC_OK;

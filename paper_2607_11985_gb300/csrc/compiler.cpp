@@ -570,6 +570,32 @@ void build_hbm_schedule(const HostPlan& p, Schedule& s) {
     } while (!remaining.empty());
 }
 
+// Tile qubits and block size of the HBM passes, false when the circuit has none (the
+// pass kernels exist for one K per mode and type).
+bool hbm_shape(const HostPlan& p, int mode, int& m, int& K) {
+    const int n = p.n, k = hbm_k(mode, p.dtype);
+    m = std::min(hbm_tile_qubits(mode, p.dtype, p.G_swz), n - 1);
+    K = std::min(k, m - 1);
+    if (n < p.G_swz + 2 || K < 1 || m <= p.G_swz) return false;
+    if (p.env_tile) {
+        m = std::min(std::max(p.env_tile, k + 1), k + 8);
+        K = std::min(k, m - 1);
+    }
+    return K == k;
+}
+
+// Whether every launch of the resident path fits a CTA's shared memory, with some
+// room to spare (the launch code's own layout decides): all sizes a launch may choose.
+bool resident_fits(const HostPlan& p) {
+    if (p.n > resident_max_qubits(1, p.dtype)) return false;
+    const size_t rs = p.dtype == VQC_C128 ? 8 : 4, ew = p.dtype == VQC_C128 ? 8 : 32;
+    const size_t wg = std::max(1, std::min(512, 1 << std::max(0, p.n - 3)) / 32);
+    const size_t need = (size_t)(p.n_sh + p.n_ps) * ew * rs + 2 * (size_t)p.num_w * rs +
+                        ((size_t)4 << p.n) * rs + (size_t)(p.num_x + p.n) * rs + p.accs.size() * wg * 8 * rs +
+                        p.term_src.size() * rs + wg * p.n * rs;
+    return need <= 216 * 1024;
+}
+
 template <class T>
 void put_vec(std::vector<uint8_t>& out, const std::vector<T>& v) {
     int32_t count = (int32_t)v.size();
@@ -640,21 +666,9 @@ vqc_status compile_host(const vqc_gate* gates, int32_t G, int32_t n, int32_t nx,
     p.recompute_flops = f * dim;
     p.fwd_flops = (f + 3 + n) * dim;
     p.bwd_flops = (fb + n + 2) * dim;
-    // Stage schedules for every usable (mode, K) on the resident path.
-    for (int mode = 0; mode < 2; ++mode) {
-        for (int K = 1; K <= std::min(max_k(mode, dtype), n); ++K) {
-            // at most 512 register blocks per sample: one block per thread, which
-            // the folded CX gates need (a thread holding two blocks would store
-            // one before loading the other)
-            if (n - K > 9) continue;
-            if (n > resident_max_qubits(mode, dtype)) continue;
-            Schedule s;
-            s.mode = mode;
-            s.K = K;
-            s.path = VQC_PATH_RESIDENT;
-            build_schedule(p, s);
-            p.scheds.push_back(std::move(s));
-        }
+    if (const char* t = std::getenv("VQC_HBM_TILE_QUBITS")) {
+        const int env_m = std::atoi(t);
+        if (env_m > p.G_swz && env_m < n) p.env_tile = env_m;
     }
     // Cluster schedules: states up to 16 qubits over 2..8 CTAs of a thread-block
     // cluster, one register block per thread (2^(n-K) threads) and at most 128
@@ -696,35 +710,31 @@ vqc_status compile_host(const vqc_gate* gates, int32_t G, int32_t n, int32_t nx,
             p.scheds.push_back(std::move(s));
         }
     }
-    // HBM-tiled pass schedules (tile of m qubits, K fixed per mode and type).
+    // Frame schedules on the resident path, one block per thread (at most 512 threads
+    // per sample): the block sizes that a launch chooses from (choose_k: 3 and up where
+    // the circuit has them), and the smaller ones when the environment asks for a size
+    // at compile time; then the HBM passes.
+    const FrameBuilder frames(p);
+    const bool all_k = std::getenv("VQC_FORCE_K_FWD") || std::getenv("VQC_FORCE_K_BWD");
     for (int mode = 0; mode < 2; ++mode) {
-        int m = std::min(hbm_tile_qubits(mode, dtype, p.G_swz), n - 1);
-        int K = std::min(hbm_k(mode, dtype), m - 1);
-        if (n < p.G_swz + 2 || K < 1 || m <= p.G_swz) continue;
-        const int env_m = std::getenv("VQC_HBM_TILE_QUBITS") ? std::atoi(std::getenv("VQC_HBM_TILE_QUBITS")) : 0;
-        if (env_m > p.G_swz && env_m < n) {
-            m = std::min(std::max(env_m, hbm_k(mode, dtype) + 1), hbm_k(mode, dtype) + 8);
-            K = std::min(hbm_k(mode, dtype), m - 1);
-        }
-        if (K != hbm_k(mode, dtype)) continue;   // pass kernels exist for this K only
+        const int kmax = std::min(max_k(mode, dtype), n);
+        for (int K = all_k ? 1 : std::min(kmax, 3); K <= kmax; ++K)
+            if (n - K <= 9 && n <= resident_max_qubits(mode, dtype))
+                p.frames.push_back(frames.build(mode, VQC_PATH_RESIDENT, {n}, K));
+    }
+    // (Circuits whose sweeps fit one CTA in both modes never take the passes, unless
+    // the environment asks for them at compile time.)
+    const bool want_hbm = std::getenv("VQC_FORCE_PATH") || p.env_tile || !resident_fits(p);
+    for (int mode = 0; mode < 2; ++mode) {
+        int m, K;
+        if (!hbm_shape(p, mode, m, K)) continue;
         // the backward passes recompute the final state with the forward passes
         // when the caller gives none: no backward schedule without a forward one
-        if (mode == 1 && !find_hbm_schedule(p, 0)) continue;
-        Schedule s;
-        s.mode = mode;
-        s.K = K;
-        s.m = m;
-        s.path = VQC_PATH_HBM;
-        build_hbm_schedule(p, s);
-        p.scheds.push_back(std::move(s));
-    }
-    for (int mode = 0; mode < 2; ++mode) {
-        const Schedule* h = find_hbm_schedule(p, mode);
-        if (!h) continue;
+        if (mode == 1 && !find_frame(p, 0, VQC_PATH_HBM)) continue;
+        if (!want_hbm) break;
         std::vector<int> tiles = frame_tile_qubits(mode, dtype, n);
-        const int env_m = std::getenv("VQC_HBM_TILE_QUBITS") ? std::atoi(std::getenv("VQC_HBM_TILE_QUBITS")) : 0;
-        if (env_m > p.G_swz && env_m < n) tiles = {h->m};
-        p.frames.push_back(build_frame_schedule(p, mode, VQC_PATH_HBM, tiles, h->K));
+        if (p.env_tile) tiles = {m};
+        p.frames.push_back(frames.build(mode, VQC_PATH_HBM, tiles, K));
     }
     return VQC_OK;
 }
@@ -735,22 +745,43 @@ const FrameSchedule* find_frame(const HostPlan& p, int mode, int path, int K) {
     return nullptr;
 }
 
-const Schedule* find_schedule(const HostPlan& p, int mode, int K) {
-    for (const auto& s : p.scheds)
-        if (s.mode == mode && s.K == K && s.path == VQC_PATH_RESIDENT) return &s;
-    return nullptr;
-}
-
 const Schedule* find_cluster_schedule(const HostPlan& p, int mode) {
     for (const auto& s : p.scheds)
         if (s.mode == mode && s.path == VQC_PATH_CLUSTER) return &s;
     return nullptr;
 }
 
-const Schedule* find_hbm_schedule(const HostPlan& p, int mode) {
-    for (const auto& s : p.scheds)
-        if (s.mode == mode && s.path == VQC_PATH_HBM) return &s;
-    return nullptr;
+// The schedules of the plan's export: axis-aligned tiles and blocks, CX gates folded
+// into the store maps.  The kernels run the frame schedules (and, of these, the
+// cluster ones); the others are built here only, when an export asks for them.
+static std::vector<Schedule> export_schedules(const HostPlan& p) {
+    std::vector<Schedule> out;
+    const int n = p.n, dtype = p.dtype;
+    // every (mode, K) on the resident path: at most 512 register blocks per sample
+    for (int mode = 0; mode < 2; ++mode)
+        for (int K = 1; K <= std::min(max_k(mode, dtype), n); ++K) {
+            if (n - K > 9 || n > resident_max_qubits(mode, dtype)) continue;
+            Schedule s;
+            s.mode = mode;
+            s.K = K;
+            s.path = VQC_PATH_RESIDENT;
+            build_schedule(p, s);
+            out.push_back(std::move(s));
+        }
+    out.insert(out.end(), p.scheds.begin(), p.scheds.end());
+    for (int mode = 0; mode < 2; ++mode) {
+        int m, K;
+        if (!hbm_shape(p, mode, m, K) || (mode == 1 && !hbm_shape(p, 0, m, K))) continue;
+        hbm_shape(p, mode, m, K);
+        Schedule s;
+        s.mode = mode;
+        s.K = K;
+        s.m = m;
+        s.path = VQC_PATH_HBM;
+        build_hbm_schedule(p, s);
+        out.push_back(std::move(s));
+    }
+    return out;
 }
 
 std::vector<uint8_t> export_plan(const HostPlan& p) {
@@ -779,8 +810,9 @@ std::vector<uint8_t> export_plan(const HostPlan& p) {
     put_vec(out, p.xocc);
     put_vec(out, p.wocc_ptr);
     put_vec(out, p.wocc);
-    put_i32(out, (int32_t)p.scheds.size());
-    for (const auto& s : p.scheds) {
+    const std::vector<Schedule> scheds = export_schedules(p);
+    put_i32(out, (int32_t)scheds.size());
+    for (const auto& s : scheds) {
         for (int v : {s.mode, s.K, s.m, s.path, s.thread_bits, s.group_lanes_log2, s.cta_bits})
             put_i32(out, v);
         put_vec(out, s.ops);

@@ -61,8 +61,9 @@ struct HostPlan {
     std::vector<int32_t> xocc_ptr, xocc, wocc_ptr, wocc;   // terms of each x column / w index
     int n_ps = 0, n_sh = 0;                // per-sample / shared table sizes
     int n_runs = 0;
-    std::vector<Schedule> scheds;
-    std::vector<FrameSchedule> frames;     // what the HBM-tiled kernels run
+    int env_tile = 0;                      // VQC_HBM_TILE_QUBITS at compile time, 0: none
+    std::vector<Schedule> scheds;          // of the cluster path
+    std::vector<FrameSchedule> frames;     // of the resident and HBM-tiled kernels
     double fwd_flops = 0, bwd_flops = 0, recompute_flops = 0;
 
     // device copy
@@ -112,8 +113,6 @@ inline int max_k(int mode, int dtype) {
 // compiler.cpp
 vqc_status compile_host(const vqc_gate* gates, int32_t G, int32_t n, int32_t nx, int32_t nw,
                         int dtype, HostPlan& out, std::string& err);
-const Schedule* find_schedule(const HostPlan& p, int mode, int K);
-const Schedule* find_hbm_schedule(const HostPlan& p, int mode);
 const Schedule* find_cluster_schedule(const HostPlan& p, int mode);
 const FrameSchedule* find_frame(const HostPlan& p, int mode, int path, int K = 0);
 std::vector<uint8_t> export_plan(const HostPlan& p);

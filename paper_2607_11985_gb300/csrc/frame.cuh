@@ -28,6 +28,15 @@ __device__ __forceinline__ uint32_t xor_bits(const void* v, int nb, int t) {
     return b;
 }
 
+// XOR of cols[i] over the set bits of v.
+template <typename T, int N>
+__device__ __forceinline__ uint32_t xor_cols(const T (&cols)[N], uint32_t v) {
+    uint32_t r = 0;
+    for (int i = 0; v; ++i, v >>= 1)
+        if (v & 1u) r ^= (uint32_t)cols[i];
+    return r;
+}
+
 // A thread's block in a stage: the byte offset of its base in the group's tiles and
 // (when the stage needs them) its outside parities; sb the local bits' byte offsets.
 // base: the offset in the tile that does not depend on the tile (frame_base); fl:
@@ -106,37 +115,44 @@ __device__ __forceinline__ void walsh(R (&v)[1 << K]) {
             }
 }
 
-// Per-warp sums of E_j = sum (-1)^{bit j} |a|^2 over the group's blocks, to
-// red[warp_in_group * n + j].  One Walsh transform of the block's |a|^2 holds the
-// signed sum of every local mask; qubit j takes its own, signed by its outside
-// parity (bit j of pbf).  Full-warp groups sum 16 qubits at a time by a
-// reduce-scatter butterfly.
-template <typename R, int K, bool FULL>
+// Per-warp sums of E_j = sum (-1)^{bit j} |a|^2 over the group's blocks: put(j, sum)
+// in one lane per qubit.  One Walsh transform of the block's |a|^2 holds the signed
+// sum of every local mask; qubit j takes its own, signed by its outside parity (bit
+// j of pbf).  Full-warp groups sum 16 (or 8) qubits at a time by a reduce-scatter
+// butterfly.
+template <typename R, int K, int NV, typename Put>
+__device__ __forceinline__ void expz_group(const uint8_t* lmask, uint32_t pbf, const R (&W)[1 << K], int n, int j0,
+                                           int lane, Put put) {
+    R ez[NV];
+#pragma unroll
+    for (int j = 0; j < NV; ++j) {
+        ez[j] = 0;
+        if (j0 + j < n) {
+            const R s = W[lmask[j0 + j]];
+            ez[j] = ((pbf >> (j0 + j)) & 1u) ? -s : s;
+        }
+    }
+    const int j = j0 + warp_reduce_scatter<R, NV>(ez, lane);
+    if ((lane & (32 / NV - 1)) == 0 && j < n) put(j, ez[0]);
+}
+template <typename R, int K, bool FULL, typename Put>
 __device__ __forceinline__ void expz_frame(const uint8_t* lmask, uint32_t pbf, const C2<R> (&a)[1 << K], int n,
-                                           R* red, const Geo& q, int lane, int warp_in_group) {
+                                           const Geo& q, int lane, Put put) {
     R W[1 << K];
 #pragma unroll
     for (int r = 0; r < (1 << K); ++r) W[r] = fma(a[r].x, a[r].x, a[r].y * a[r].y);
     walsh<R, K>(W);
     if constexpr (FULL) {
-        for (int j0 = 0; j0 < n; j0 += 16) {
-            R ez[16];
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                ez[j] = 0;
-                if (j0 + j < n) {
-                    const R s = W[lmask[j0 + j]];
-                    ez[j] = ((pbf >> (j0 + j)) & 1u) ? -s : s;
-                }
-            }
-            const int j = j0 + warp_reduce_scatter<R, 16>(ez, lane);
-            if ((lane & 1) == 0 && j < n) red[warp_in_group * n + j] = ez[0];
+        if (n <= 8) {
+            expz_group<R, K, 8>(lmask, pbf, W, n, 0, lane, put);
+        } else {
+            for (int j0 = 0; j0 < n; j0 += 16) expz_group<R, K, 16>(lmask, pbf, W, n, j0, lane, put);
         }
     } else {
         for (int j = 0; j < n; ++j) {
             const R s = W[lmask[j]];
             const R val = reduce1<R>(((pbf >> j) & 1u) ? -s : s, q.lanes, q.mask);
-            if ((q.t & (q.lanes - 1)) == 0) red[warp_in_group * n + j] = val;
+            if ((q.t & (q.lanes - 1)) == 0) put(j, val);
         }
     }
 }

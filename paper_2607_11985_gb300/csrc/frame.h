@@ -29,6 +29,7 @@
 #pragma once
 
 #include <cstdint>
+#include <memory>
 #include <string>
 #include <vector>
 
@@ -100,12 +101,24 @@ struct FrameSchedule {
     std::vector<int32_t> pass_entries, pass_accs;
     FFinal fin{};
     size_t dev_ops = 0, dev_stages = 0, dev_flips = 0, dev_fin = 0, dev_pass_entries = 0, dev_pass_accs = 0;
+    size_t dev_region_begin = 0, dev_region_end = 0;   // ops, stages, fin in the plan's device blob
 };
 
 struct HostPlan;
 
-// frames.cpp
-FrameSchedule build_frame_schedule(const HostPlan& p, int mode, int path, std::vector<int> tiles, int K);
+// frames.cpp: builds a plan's frame schedules.
+struct FrameOps;
+class FrameBuilder {
+  public:
+    explicit FrameBuilder(const HostPlan& p);
+    ~FrameBuilder();
+    // tiles: the tile sizes to choose from (the resident path: the qubit count)
+    FrameSchedule build(int mode, int path, const std::vector<int>& tiles, int K) const;
+
+  private:
+    const HostPlan& p;
+    std::unique_ptr<FrameOps> ops;
+};
 std::vector<uint8_t> export_frames(const HostPlan& p);
 
 }  // namespace vqc

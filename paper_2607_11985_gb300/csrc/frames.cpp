@@ -7,7 +7,43 @@
 namespace vqc {
 namespace {
 
-bool odd(uint32_t v) { return (__builtin_popcount(v) & 1) != 0; }
+// A short list of vectors of the index space (or selectors), held in place: a plan
+// builds thousands of them.
+struct Vecs {
+    uint32_t v[32];
+    int n = 0;
+    Vecs() = default;
+    explicit Vecs(size_t count) : n((int)count) { std::memset(v, 0, sizeof(v)); }
+    Vecs(const Vecs& o) : n(o.n) { std::memcpy(v, o.v, sizeof(uint32_t) * n); }
+    Vecs& operator=(const Vecs& o) {
+        n = o.n;
+        std::memmove(v, o.v, sizeof(uint32_t) * n);
+        return *this;
+    }
+    size_t size() const { return (size_t)n; }
+    bool empty() const { return n == 0; }
+    void clear() { n = 0; }
+    void push_back(uint32_t x) { v[n++] = x; }
+    uint32_t& operator[](size_t i) { return v[i]; }
+    uint32_t operator[](size_t i) const { return v[i]; }
+    uint32_t* begin() { return v; }
+    uint32_t* end() { return v + n; }
+    const uint32_t* begin() const { return v; }
+    const uint32_t* end() const { return v + n; }
+    void append(const Vecs& o) {
+        for (uint32_t x : o) push_back(x);
+    }
+    void erase(int i) {
+        for (--n; i < n; ++i) v[i] = v[i + 1];
+    }
+    Vecs first(int count) const {
+        Vecs r;
+        for (int i = 0; i < count; ++i) r.push_back(v[i]);
+        return r;
+    }
+};
+
+inline bool odd(uint32_t v) { return __builtin_parity(v) != 0; }
 
 // An op in the storage frame: a run (direction d, selector r), or a diagonal op
 // on the parities r and r2.
@@ -17,16 +53,9 @@ struct FOp {
     int hop = -1;
 };
 
-bool commute(const FOp& a, const FOp& b) {
-    if (a.run && b.run) return !odd(a.r & b.d) && !odd(b.r & a.d);
-    if (a.run) return !odd(b.r & a.d) && !odd(b.r2 & a.d);
-    if (b.run) return !odd(a.r & b.d) && !odd(a.r2 & b.d);
-    return true;
-}
-
 // The subspace spanned by the vectors added so far.
 struct Span {
-    uint32_t piv[32] = {0};   // by highest set bit
+    uint32_t piv[24] = {0};   // by highest set bit (at most 24 qubits)
     int dim = 0;
     uint32_t reduce(uint32_t v) const {
         while (v) {
@@ -43,18 +72,45 @@ struct Span {
         ++dim;
         return true;
     }
-    std::vector<uint32_t> basis() const {
-        std::vector<uint32_t> b;
+    Vecs basis() const {
+        Vecs b;
         for (uint32_t v : piv)
             if (v) b.push_back(v);
         return b;
     }
 };
 
+// The ops that a scan in time order leaves behind.  An op commutes with all of them
+// when its selectors are even on their directions and its direction on their
+// selectors: both are tests against a basis.  Once the directions fill the space
+// nothing later can pass.
+struct Waiting {
+    Span d, s;
+    uint32_t dv[24], sv[24];   // the bases, dense
+    int nd = 0, ns = 0;
+    bool passes(const FOp& o) const {
+        if (o.run) {
+            for (int i = 0; i < nd; ++i)
+                if (odd(o.r & dv[i])) return false;
+            for (int i = 0; i < ns; ++i)
+                if (odd(o.d & sv[i])) return false;
+        } else {
+            for (int i = 0; i < nd; ++i)
+                if (odd(o.r & dv[i]) || odd(o.r2 & dv[i])) return false;
+        }
+        return true;
+    }
+    void add(const FOp& o) {
+        if (o.run && d.add(o.d)) dv[nd++] = o.d;
+        if (s.add(o.r)) sv[ns++] = o.r;
+        if (!o.run && s.add(o.r2)) sv[ns++] = o.r2;
+    }
+};
+
 // Coordinates in a basis: coord(v) has bit i set when basis vector i is in v.
 struct Coords {
     uint32_t piv[32] = {0}, comb[32] = {0};
-    explicit Coords(const std::vector<uint32_t>& b) {
+    explicit Coords(const Vecs& b) {
         for (size_t i = 0; i < b.size(); ++i) {
             uint32_t v = b[i], c = 1u << i;
             while (v) {
@@ -81,7 +137,7 @@ struct Coords {
 };
 
 // The vectors of span(vs) on which every functional of `sel` is even (a basis).
-std::vector<uint32_t> annihilated(std::vector<uint32_t> vs, const std::vector<uint32_t>& sel) {
+Vecs annihilated(Vecs vs, const Vecs& sel) {
     for (uint32_t s : sel) {
         int k = -1;
         for (size_t i = 0; i < vs.size(); ++i)
@@ -89,21 +145,21 @@ std::vector<uint32_t> annihilated(std::vector<uint32_t> vs, const std::vector<ui
                 if (k < 0) k = (int)i;
                 else vs[i] ^= vs[k];
             }
-        if (k >= 0) vs.erase(vs.begin() + k);
+        if (k >= 0) vs.erase(k);
     }
     return vs;
 }
 
-uint32_t image(const std::vector<uint32_t>& cols, uint32_t v) {   // XOR of cols[i] over v's bits
+uint32_t image(const Vecs& cols, uint32_t v) {   // XOR of cols[i] over v's bits
     uint32_t r = 0;
     for (size_t i = 0; i < cols.size(); ++i)
         if ((v >> i) & 1) r ^= cols[i];
     return r;
 }
 
-std::vector<uint32_t> inverse(std::vector<uint32_t> cols) {   // of an invertible matrix, as columns
+Vecs inverse(Vecs cols) {   // of an invertible matrix, as columns
     const size_t n = cols.size();
-    std::vector<uint32_t> inv(n);
+    Vecs inv(n);
     for (size_t i = 0; i < n; ++i) inv[i] = 1u << i;
     for (size_t b = 0; b < n; ++b) {
         size_t k = b;
@@ -119,58 +175,55 @@ std::vector<uint32_t> inverse(std::vector<uint32_t> cols) {   // of an invertibl
     return inv;
 }
 
-// Ops looked ahead of the first one that has to wait.  Beyond a few layers of
-// the widest circuit nothing can run early any more.
-constexpr size_t kLookahead = 160;
 // Table entries and accumulators of one pass: bounds its shared memory.
 constexpr int kMaxPassEntries = 96;
 
 struct StagePlan {
     std::vector<int> ops;              // indices into the FOp list, time order
-    std::vector<uint32_t> D, R;        // directions and selectors of its runs, by local position
-    std::vector<uint32_t> sels;        // distinct selectors of its diagonal ops
+    Vecs D, R;        // directions and selectors of its runs, by local position
+    Vecs sels;        // distinct selectors of its diagonal ops
 };
 
 // Cut a pass's ops into stages of at most K directions.
-std::vector<StagePlan> cut(const std::vector<FOp>& f, const std::vector<int>& ops, int K) {
+std::vector<StagePlan> cut(const std::vector<FOp>& f, const std::vector<int>& ops, int n, int K) {
     std::vector<StagePlan> out;
     std::vector<int> rem = ops;
     do {   // an empty op list still gets one (empty) stage
         StagePlan s;
         std::vector<int> defer;
+        Waiting w;
+        Span sp;   // of D
         size_t i = 0;
-        for (; i < rem.size() && defer.size() <= kLookahead; ++i) {
+        for (; i < rem.size() && w.d.dim < n; ++i) {
             const FOp& o = f[rem[i]];
-            bool ok = true;
-            for (int x : defer)
-                if (!commute(o, f[x])) { ok = false; break; }
+            bool ok = w.passes(o);
             if (ok && o.run) {
                 size_t j = 0;
                 while (j < s.D.size() && !(s.D[j] == o.d && s.R[j] == o.r)) ++j;
                 if (j == s.D.size()) {   // a new direction: dual to the others and to the parities
                     ok = (int)s.D.size() < K;
-                    Span sp;
-                    for (uint32_t d : s.D) sp.add(d);
                     ok = ok && sp.reduce(o.d) != 0;
                     for (size_t k = 0; ok && k < s.D.size(); ++k)
                         ok = !odd(s.R[k] & o.d) && !odd(o.r & s.D[k]);
                     for (size_t k = 0; ok && k < s.sels.size(); ++k)
                         ok = !odd(s.sels[k] & o.d) || s.sels[k] == o.r;
                     if (ok) {
+                        sp.add(o.d);
                         s.D.push_back(o.d);
                         s.R.push_back(o.r);
                     }
                 }
             } else if (ok) {
-                std::vector<uint32_t> add;
+                Vecs add;
                 for (uint32_t r : {o.r, o.r2}) {   // a parity that a run changes is that run's own
                     for (size_t k = 0; k < s.D.size(); ++k) ok = ok && (!odd(r & s.D[k]) || r == s.R[k]);
                     if (std::find(s.sels.begin(), s.sels.end(), r) == s.sels.end()) add.push_back(r);
                 }
                 ok = ok && s.sels.size() + add.size() <= (size_t)kMaxSelectors;
-                if (ok) s.sels.insert(s.sels.end(), add.begin(), add.end());
+                if (ok) s.sels.append(add);
             }
             (ok ? s.ops : defer).push_back(rem[i]);
+            if (!ok) w.add(o);
         }
         defer.insert(defer.end(), rem.begin() + i, rem.end());
         out.push_back(std::move(s));
@@ -182,12 +235,12 @@ std::vector<StagePlan> cut(const std::vector<FOp>& f, const std::vector<int>& op
 // Complete a stage's D to K vectors of the tile: every pad is even on the runs'
 // selectors, meets at most one diagonal selector, and no selector meets two of D.
 // False when the diagonal ops leave no such pads.
-bool pad(StagePlan& s, const std::vector<uint32_t>& V, int K) {
-    std::vector<uint32_t> A = annihilated(V, s.R);
-    std::vector<uint32_t> free = annihilated(A, s.sels);
+bool pad(StagePlan& s, const Vecs& V, int K) {
+    Vecs A = annihilated(V, s.R);
+    Vecs free = annihilated(A, s.sels);
     // A's vectors dual to the diagonal selectors that D does not meet yet, then the free ones
-    std::vector<uint32_t> cand = free;
-    std::vector<uint32_t> rest = A;
+    Vecs cand = free;
+    Vecs rest = A;
     for (size_t i = 0; i < s.sels.size(); ++i) {
         int k = -1;
         for (size_t j = 0; j < rest.size(); ++j)
@@ -197,7 +250,7 @@ bool pad(StagePlan& s, const std::vector<uint32_t>& V, int K) {
             }
         if (k < 0) continue;
         uint32_t v = rest[k];
-        rest.erase(rest.begin() + k);
+        rest.erase(k);
         for (size_t l = i + 1; l < s.sels.size(); ++l)   // even on the later selectors if the rest allows it
             if (odd(v & s.sels[l]))
                 for (uint32_t t : rest) {
@@ -229,7 +282,7 @@ bool pad(StagePlan& s, const std::vector<uint32_t>& V, int K) {
 
 struct PassPlan {
     std::vector<int> ops;
-    std::vector<uint32_t> V;           // basis of the tile's subspace
+    Vecs V;           // basis of the tile's subspace
     std::vector<StagePlan> stages;
 };
 
@@ -245,7 +298,7 @@ uint32_t settle(const StagePlan& s, uint32_t v) {
     return v;
 }
 
-int rank_of(const std::vector<uint32_t>& v) {
+int rank_of(const Vecs& v) {
     Span s;
     for (uint32_t x : v) s.add(x);
     return s.dim;
@@ -261,19 +314,24 @@ struct Rng {   // small deterministic generator (xorshift32) for the swizzle sea
     }
 };
 
+}  // namespace
+
 // The op list in the storage frame, and the frame at its end.
 struct FrameOps {
-    std::vector<uint32_t> dir, sel;
+    Vecs dir, sel;
     std::vector<FOp> f;
 };
+
+namespace {
 
 FrameOps lower(const HostPlan& p) {
     const int n = p.n;
     FrameOps L;
-    std::vector<uint32_t>&dir = L.dir, &sel = L.sel;
-    dir.resize(n);
-    sel.resize(n);
-    for (int q = 0; q < n; ++q) dir[q] = sel[q] = 1u << q;
+    Vecs &dir = L.dir, &sel = L.sel;
+    for (int q = 0; q < n; ++q) {
+        dir.push_back(1u << q);
+        sel.push_back(1u << q);
+    }
     for (size_t i = 0; i < p.ops.size(); ++i) {
         const HOp& o = p.ops[i];
         if (o.type == OP_CX) {
@@ -297,7 +355,7 @@ FrameOps lower(const HostPlan& p) {
 std::vector<PassPlan> plan_passes(const HostPlan& p, const FrameOps& L, int mode, bool tiled, int m, int K) {
     const int n = p.n, G = std::min(p.G_swz, m);
     const std::vector<FOp>& f = L.f;
-    const std::vector<uint32_t>& dir = L.dir;
+    const Vecs& dir = L.dir;
 
     // ---- passes: each takes, in time order, every op that commutes with the ops
     // it leaves behind while the tile has room for its direction.  At most m - G
@@ -313,7 +371,7 @@ std::vector<PassPlan> plan_passes(const HostPlan& p, const FrameOps& L, int mode
         for (int q = 0; q < n; ++q) ps.V.push_back(1u << q);
         passes.push_back(std::move(ps));
     } else {
-        std::vector<uint32_t> prev, last_dirs(dir.begin(), dir.begin() + G);
+        Vecs prev, last_dirs = dir.first(G);
         // the forward's first tile holds the lines of the given state; the
         // backward's first is its last to run and writes nothing
         for (int i = 0; i < G; ++i) prev.push_back(1u << i);
@@ -333,18 +391,17 @@ std::vector<PassPlan> plan_passes(const HostPlan& p, const FrameOps& L, int mode
                     return true;
                 }
             };
-            auto attempt = [&](const std::vector<uint32_t>& pre, Try& t) {
+            auto attempt = [&](const Vecs& pre, Try& t) {
                 for (uint32_t d : prev) t.mod.add(d);
                 for (uint32_t d : pre)
                     if (!t.add(d, m, room)) return false;
                 int entries = 0;
                 std::vector<char> have(p.entries.size(), 0);
+                Waiting w;
                 size_t i = 0;
-                for (; i < rem.size() && t.left.size() <= kLookahead; ++i) {
+                for (; i < rem.size() && w.d.dim < n; ++i) {
                     const FOp& o = f[rem[i]];
-                    bool ok = true;
-                    for (int x : t.left)
-                        if (!commute(o, f[x])) { ok = false; break; }
+                    bool ok = w.passes(o);
                     const int e = p.ops[o.hop].entry;
                     const bool newe = e >= 0 && !have[e];
                     if (ok && newe) ok = entries < kMaxPassEntries;
@@ -354,34 +411,32 @@ std::vector<PassPlan> plan_passes(const HostPlan& p, const FrameOps& L, int mode
                         ++entries;
                     }
                     (ok ? t.taken : t.left).push_back(rem[i]);
+                    if (!ok) w.add(o);
                 }
                 t.left.insert(t.left.end(), rem.begin() + i, rem.end());
                 return true;
             };
-            Try fin, t;
-            const bool can_end = attempt(last_dirs, fin);
-            const bool end = can_end && fin.left.empty();
-            if (!end) {
-                attempt({}, t);
-                if (t.left.empty()) {
-                    if (can_end) {
-                        t = fin;
-                    } else {   // move towards the last tile
-                        for (uint32_t d : last_dirs) t.add(d, m, room);
-                    }
+            Try t;
+            bool end = false;
+            attempt(Vecs(), t);
+            if (t.left.empty()) {
+                Try fin;
+                if (attempt(last_dirs, fin)) {   // the last tile, or all of it but what it has no room for
+                    end = fin.left.empty();
+                    t = fin;
+                } else {   // move towards the last tile
+                    for (uint32_t d : last_dirs) t.add(d, m, room);
                 }
-            } else {
-                t = fin;
             }
             // fill up: G directions shared with the previous tile (its last-tile
             // directions first), then unit vectors
             {
-                std::vector<uint32_t> shared;
+                Vecs shared;
                 Span pv;
                 for (uint32_t d : prev) pv.add(d);
                 for (uint32_t d : last_dirs)
                     if (!pv.reduce(d)) shared.push_back(d);
-                shared.insert(shared.end(), prev.begin(), prev.end());
+                shared.append(prev);
                 for (uint32_t d : shared)
                     if (t.v.dim - t.fresh < G) t.add(d, m, room);
                 for (int q = 0; q < n; ++q) t.add(1u << q, m, room);
@@ -400,7 +455,7 @@ std::vector<PassPlan> plan_passes(const HostPlan& p, const FrameOps& L, int mode
     // ---- stages of each pass; a stage whose diagonal ops leave no room for its
     // pads gives its later diagonal ops to a stage of their own
     for (PassPlan& ps : passes) {
-        std::vector<StagePlan> st = cut(f, ps.ops, K), out;
+        std::vector<StagePlan> st = cut(f, ps.ops, n, K), out;
         for (StagePlan& s : st) {
             std::vector<StagePlan> work{s};
             while (!work.empty()) {
@@ -414,7 +469,7 @@ std::vector<PassPlan> plan_passes(const HostPlan& p, const FrameOps& L, int mode
                 // split in time order: the first half's ops, then the second's
                 std::vector<int> a(w0.ops.begin(), w0.ops.begin() + (w0.ops.size() + 1) / 2),
                     b(w0.ops.begin() + (w0.ops.size() + 1) / 2, w0.ops.end());
-                std::vector<StagePlan> sb = cut(f, b, K), sa = cut(f, a, K);
+                std::vector<StagePlan> sb = cut(f, b, n, K), sa = cut(f, a, n, K);
                 for (size_t i = sb.size(); i-- > 0;) work.push_back(sb[i]);
                 for (size_t i = sa.size(); i-- > 0;) work.push_back(sa[i]);
             }
@@ -426,18 +481,23 @@ std::vector<PassPlan> plan_passes(const HostPlan& p, const FrameOps& L, int mode
 
 }  // namespace
 
-FrameSchedule build_frame_schedule(const HostPlan& p, int mode, int path, std::vector<int> tiles, int K) {
+FrameBuilder::FrameBuilder(const HostPlan& plan) : p(plan), ops(new FrameOps(lower(plan))) {}
+FrameBuilder::~FrameBuilder() = default;
+
+FrameSchedule FrameBuilder::build(int mode, int path, const std::vector<int>& tiles, int K) const {
     const int n = p.n;
     const bool tiled = path == VQC_PATH_HBM;
-    const FrameOps L = lower(p);
+    const FrameOps& L = *ops;
     const std::vector<FOp>& f = L.f;
-    const std::vector<uint32_t>&dir = L.dir, &sel = L.sel;
+    const Vecs &dir = L.dir, &sel = L.sel;
 
     // of the tile sizes offered, the first unless a later one takes no more passes and stages
     int m = 0;
     size_t nst = 0;
     std::vector<PassPlan> passes;
-    for (int t : tiles) {
+    for (size_t i = 0; i < tiles.size(); ++i) {
+        const int t = tiles[i];
+        if (i && t == tiles[i - 1]) continue;
         std::vector<PassPlan> q = plan_passes(p, L, mode, tiled, t, K);
         size_t c = 0;
         for (const PassPlan& ps : q) c += ps.stages.size();
@@ -458,7 +518,7 @@ FrameSchedule build_frame_schedule(const HostPlan& p, int mode, int path, std::v
     // from the last).  A pass reads the state at the addresses M s; the forward
     // starts at M = 1 (a state in logical order before the first gate) and writes
     // logical order at its end, the backward starts there.
-    std::vector<uint32_t> M(n), Minv(n);   // columns: address of e_i; index vector of address bit i
+    Vecs M(n), Minv(n);   // columns: address of e_i; index vector of address bit i
     for (int i = 0; i < n; ++i) {
         M[i] = Minv[i] = 1u << i;
         if (mode == 1) {
@@ -476,25 +536,25 @@ FrameSchedule build_frame_schedule(const HostPlan& p, int mode, int path, std::v
         const bool last = pi == np - 1, end = step == np - 1;
         FPass fp{};
         // the tile's addresses as read: a reduced echelon basis with the G low units first
-        std::vector<uint32_t> gin, vin, opos, ovec;
-        auto echelon = [&](const std::vector<uint32_t>& addr, std::vector<uint32_t>& g) {
+        Vecs gin, vin, opos, ovec;
+        auto echelon = [&](const Vecs& addr, Vecs& g) {
             uint32_t lowm = (1u << G) - 1;
             g.clear();
             for (int i = 0; i < G; ++i) g.push_back(1u << i);
-            std::vector<uint32_t> r;
+            Vecs r;
             for (uint32_t a : addr) r.push_back(a & ~lowm);
             Span sp;
             for (uint32_t a : r) sp.add(a);
-            std::vector<uint32_t> b = sp.basis();   // ascending highest bit
+            Vecs b = sp.basis();   // ascending highest bit
             for (size_t i = 0; i < b.size(); ++i)   // fully reduce
                 for (size_t j = 0; j < i; ++j) {
                     const int h = 31 - __builtin_clz(b[j]);
                     if ((b[i] >> h) & 1) b[i] ^= b[j];
                 }
-            g.insert(g.end(), b.begin(), b.end());
+            g.append(b);
         };
         if (tiled) {
-            std::vector<uint32_t> addr;
+            Vecs addr;
             for (uint32_t v : ps.V) addr.push_back(image(M, v));
             echelon(addr, gin);
         } else {
@@ -512,12 +572,12 @@ FrameSchedule build_frame_schedule(const HostPlan& p, int mode, int path, std::v
 
         // directions that the written lines will hold: ones that the next tile has
         // too, at the forward's end the last logical ones
-        std::vector<uint32_t> line;
+        Vecs line;
         if (end) {
-            if (mode == 0) line.assign(dir.begin(), dir.begin() + G);
+            if (mode == 0) line = dir.first(G);
         } else {
             // V intersect V': vectors of V whose sum with V' vectors vanishes
-            const std::vector<uint32_t>&a = ps.V, &b = passes[pi + (mode == 0 ? 1 : -1)].V;
+            const Vecs &a = ps.V, &b = passes[pi + (mode == 0 ? 1 : -1)].V;
             uint32_t piv[32] = {0}, ca[32] = {0};
             auto ins = [&](uint32_t v, uint32_t c, bool fromb) {
                 while (v) {
@@ -537,20 +597,19 @@ FrameSchedule build_frame_schedule(const HostPlan& p, int mode, int path, std::v
             for (uint32_t v : b) ins(v, 0, true);
         }
 
-        // swizzle: slot bits 0..G-1 of tile bit i >= G also get column F[i]; a random
-        // choice whose lanes hit distinct banks in every stage and both copies
-        std::vector<uint32_t> F(m, 0);
+        // swizzle: slot bits 0..G-1 of tile bit i >= G also get column F[i], chosen so
+        // that lanes hit distinct banks in every stage and both copies
+        Vecs F(m);
         const int tb = m - K, gl = std::min(G, tb);   // lanes that must differ in the low gl slot bits
         auto slot_of = [&](uint32_t c) {
             uint32_t s = c;
-            for (int i = G; i < m; ++i)
-                if ((c >> i) & 1) s ^= F[i];
+            for (uint32_t hi = c >> G; hi; hi &= hi - 1) s ^= F[G + __builtin_ctz(hi)];
             return s;
         };
         auto bank = [&](uint32_t v) { return slot_of(coord(v)) & ((1u << G) - 1); };
         // the stages' thread spaces: V's vectors even on the runs' selectors, without the pads
         struct Threads {
-            std::vector<uint32_t> basis;
+            Vecs basis;
         };
         std::vector<Threads> th(ps.stages.size());
         for (size_t si = 0; si < ps.stages.size(); ++si) {
@@ -561,41 +620,75 @@ FrameSchedule build_frame_schedule(const HostPlan& p, int mode, int path, std::v
                 if (sp.add(v)) th[si].basis.push_back(settle(s, v));
         }
         const int vbits = p.dtype == VQC_C64 ? 1 : 0;   // bits inside a 16-byte vector of amplitudes
-        auto score = [&]() {
-            int bad = 0;
-            for (const Threads& t : th) {
-                std::vector<uint32_t> b;
-                for (uint32_t v : t.basis) b.push_back(bank(v) & ((1u << gl) - 1));
-                bad += gl - rank_of(b);
-            }
-            std::vector<uint32_t> b;
-            for (int i = vbits; i < std::min(m, G + vbits); ++i) b.push_back(bank(vin[i]));
-            bad += std::min((int)b.size(), G) - rank_of(b);
-            b.clear();
-            for (uint32_t v : line) b.push_back(bank(v));
-            if (!b.empty()) bad += 2 * std::max(0, G - vbits - rank_of(b));
-            return bad;
-        };
         {
-            std::vector<uint32_t> best = F;
-            int best_bad = 1 << 20;
-            for (int trial = 0; trial < 256 && best_bad > 0; ++trial) {
-                for (int i = G; i < m; ++i)   // the first trial: the plain fold of the high bits
-                    F[i] = trial == 0 ? 1u << (i % G) : (rng.next() >> 8) & ((1u << G) - 1);
-                const int bad = score();
-                if (bad < best_bad) {
-                    best_bad = bad;
-                    best = F;
-                }
+            // sets of tile coordinates whose banks should be independent, and how many
+            struct Want {
+                int rank, weight;
+                uint32_t mask;
+                Vecs c, b;   // tile coordinates, their banks under F
+            };
+            std::vector<Want> want;
+            want.reserve(th.size() + 2);
+            for (const Threads& t : th) {
+                want.push_back(Want{gl, 1, (1u << gl) - 1, {}, {}});
+                for (uint32_t v : t.basis) want.back().c.push_back(coord(v));
             }
-            F = best;
+            want.push_back(Want{0, 1, (1u << G) - 1, {}, {}});
+            for (int i = vbits; i < std::min(m, G + vbits); ++i) want.back().c.push_back(1u << i);
+            want.back().rank = (int)want.back().c.size();
+            if (!line.empty()) {
+                want.push_back(Want{G - vbits, 2, (1u << G) - 1, {}, {}});
+                for (uint32_t v : line) want.back().c.push_back(coord(v));
+            }
+            auto score = [&](int limit) {
+                int bad = 0;
+                for (const Want& w : want) {
+                    uint32_t piv[4] = {0, 0, 0, 0};
+                    int rank = 0;
+                    for (size_t i = 0; i < w.b.size() && rank < w.rank; ++i) {
+                        uint32_t v = w.b[i] & w.mask;
+                        while (v) {
+                            const int h = 31 - __builtin_clz(v);
+                            if (!piv[h]) {
+                                piv[h] = v;
+                                ++rank;
+                                break;
+                            }
+                            v ^= piv[h];
+                        }
+                    }
+                    bad += w.weight * (w.rank - rank);
+                    if (bad > limit) break;
+                }
+                return bad;
+            };
+            auto turn = [&](int i, uint32_t delta) {   // F[i] ^= delta
+                F[i] ^= delta;
+                for (Want& w : want)
+                    for (size_t k = 0; k < w.c.size(); ++k)
+                        if ((w.c[k] >> i) & 1) w.b[k] ^= delta;
+            };
+            // from the plain fold of the high bits, one random column at a time
+            for (int i = G; i < m; ++i) F[i] = 1u << (i % G);
+            for (Want& w : want)
+                for (uint32_t c : w.c) w.b.push_back(slot_of(c) & ((1u << G) - 1));
+            int best = score(1 << 20);
+            for (int trial = 0; trial < 64 && best > 0 && m > G; ++trial) {
+                const int i = G + (int)((rng.next() >> 4) % (uint32_t)(m - G));
+                const uint32_t delta = (rng.next() >> 8) & ((1u << G) - 1);
+                if (!delta) continue;
+                turn(i, delta);
+                const int bad = score(best);
+                if (bad <= best) best = bad;
+                else turn(i, delta);
+            }
         }
 
         // written order: the line's directions lowest, chosen so that the lanes that
         // read the tile back differ in their banks
-        std::vector<uint32_t> gout, vout;
+        Vecs gout, vout;
         if (end && mode == 0 && tiled) {
-            std::vector<uint32_t> addr;
+            Vecs addr;
             for (uint32_t v : ps.V) {
                 uint32_t a = 0;
                 for (int j = 0; j < n; ++j) a |= (uint32_t)odd(sel[j] & v) << j;
@@ -603,19 +696,21 @@ FrameSchedule build_frame_schedule(const HostPlan& p, int mode, int path, std::v
             }
             echelon(addr, gout);
             for (uint32_t g : gout) vout.push_back(image(dir, g));
-        } else if (!tiled && mode == 0) {
+        } else if (!tiled) {   // given and final order of whole states
             gout = gin;
             vout = dir;
+            if (mode == 1)
+                for (int i = 0; i < n; ++i) vout[i] = 1u << i;
         } else if (end) {   // the backward's end: nothing is written
             gout = gin;
             vout = vin;
         } else {
             gout = gin;
-            std::vector<uint32_t> l = line, pickd;
+            Vecs l = line, pickd;
             Span bs;
             if (vbits) {   // the vector's own bit: the one whose bank the others can spare
                 for (size_t i = 0; i < l.size(); ++i) {
-                    std::vector<uint32_t> b;
+                    Vecs b;
                     for (size_t j = 0; j < l.size(); ++j)
                         if (j != i) b.push_back(bank(l[j]));
                     if (rank_of(b) == (int)l.size() - 1 || i + 1 == l.size()) {
@@ -628,7 +723,7 @@ FrameSchedule build_frame_schedule(const HostPlan& p, int mode, int path, std::v
             Span sp;
             for (uint32_t v : vout) sp.add(v);
             for (size_t i = vbits; i < vout.size(); ++i) bs.add(bank(vout[i]));
-            std::vector<uint32_t> others;
+            Vecs others;
             for (uint32_t v : vin)
                 if (sp.add(v)) others.push_back(v);
             for (size_t i = 0; i < others.size(); ++i)
@@ -636,7 +731,7 @@ FrameSchedule build_frame_schedule(const HostPlan& p, int mode, int path, std::v
                     std::swap(others[0], others[i]);
                     break;
                 }
-            vout.insert(vout.end(), others.begin(), others.end());
+            vout.append(others);
         }
         if (end && mode == 0 && tiled && vbits) {   // the same for the final order's fifth bit
             Span bs;
@@ -702,16 +797,16 @@ FrameSchedule build_frame_schedule(const HostPlan& p, int mode, int path, std::v
             FStage st{};
             for (int k = 0; k < K; ++k) st.sigma[k] = (int32_t)slot_of(coord(s.D[k]));
             // thread vectors: the first gl with independent banks
-            std::vector<uint32_t> tv, others;
+            Vecs tv, others;
             Span bs;
             for (uint32_t v : th[si].basis) {
                 if ((int)tv.size() < gl && bs.add(bank(v) & ((1u << gl) - 1))) tv.push_back(v);
                 else others.push_back(v);
             }
-            tv.insert(tv.end(), others.begin(), others.end());
+            tv.append(others);
             st.nthreadbits = (uint8_t)tv.size();
             // parities outside the registers
-            std::vector<uint32_t> outside;
+            Vecs outside;
             auto ref = [&](uint32_t r) -> uint8_t {
                 for (int k = 0; k < K; ++k)
                     if (odd(r & s.D[k])) return (uint8_t)k;
@@ -805,7 +900,7 @@ FrameSchedule build_frame_schedule(const HostPlan& p, int mode, int path, std::v
 
         // the frame after the pass: M' vout[i] = gin[i], M' = M on the outer vectors
         if (!end) {
-            std::vector<uint32_t> Mi(n, 0);
+            Vecs Mi(n);
             for (int o = 0; o < nout; ++o) Mi[31 - __builtin_clz(opos[o])] = ovec[o];
             for (int i = 0; i < m; ++i) {
                 const int h = 31 - __builtin_clz(gin[i]);

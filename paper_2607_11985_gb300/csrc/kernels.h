@@ -42,12 +42,7 @@ const void* abs2_ptr(bool dbl);   // |psi|^2, elementwise
 const void* cluster_ptr(bool dbl);   // cluster-path forward (K = 5 / 4 for complex64 / 128)
 const void* cluster_bwd_ptr(bool dbl, bool dfloat);   // cluster-path backward (K = 4 / 3)
 
-// Largest block (threads) each instantiation is compiled for.
-inline int sweep_max_threads(bool is_double, int mode, int K) {
-    (void)is_double;
-    (void)mode;
-    (void)K;
-    return 512;   // sweep kernels: __launch_bounds__(512) (<= 128 registers)
-}
+// Largest block of the sweep kernels (__launch_bounds__(512): <= 128 registers).
+constexpr int kSweepMaxThreads = 512;
 
 }  // namespace vqc

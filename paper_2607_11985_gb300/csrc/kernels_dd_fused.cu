@@ -2,7 +2,7 @@
 // forward itself and writes E; vqc_forward_backward) with double-float
 // arithmetic (complex128 storage), full-warp and sub-warp sample groups.
 #include "kernels.h"
-#include "sweep.cuh"
+#include "resident.cuh"
 
 namespace vqc {
 

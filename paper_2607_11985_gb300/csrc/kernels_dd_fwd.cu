@@ -1,7 +1,7 @@
 // kernels_dd_fwd.cu -- instantiations of the sweep kernel with double-float
 // arithmetic (complex128 storage), mode 0: full-warp and sub-warp sample groups.
 #include "kernels.h"
-#include "sweep.cuh"
+#include "resident.cuh"
 
 namespace vqc {
 

@@ -2,7 +2,7 @@
 // with FUSED: the backward that sweeps forward itself and writes E
 // (vqc_forward_backward), for full-warp and sub-warp sample groups.
 #include "kernels.h"
-#include "sweep.cuh"
+#include "resident.cuh"
 
 namespace vqc {
 

@@ -2,7 +2,7 @@
 // (fused) sweep kernel for plans without diagonal two-qubit phase ops (CRZ,
 // RZZ): the switch has no phase cases, which frees registers (see apply_op).
 #include "kernels.h"
-#include "sweep.cuh"
+#include "resident.cuh"
 
 namespace vqc {
 

@@ -1,7 +1,7 @@
 // kernels_f32_fwd.cu -- instantiations of the sweep kernel for float, mode 0, sample
 // groups of at least one warp (full-warp reductions).
 #include "kernels.h"
-#include "sweep.cuh"
+#include "resident.cuh"
 
 namespace vqc {
 

@@ -1,7 +1,7 @@
 // kernels_f32_fwd_small.cu -- instantiations of the sweep kernel for float, mode 0, sample
 // groups of fewer than 32 threads (small circuits or large blocks).
 #include "kernels.h"
-#include "sweep.cuh"
+#include "resident.cuh"
 
 namespace vqc {
 

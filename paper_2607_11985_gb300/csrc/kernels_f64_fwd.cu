@@ -1,7 +1,7 @@
 // kernels_f64_fwd.cu -- instantiations of the sweep kernel for double, mode 0, sample
 // groups of at least one warp (full-warp reductions).
 #include "kernels.h"
-#include "sweep.cuh"
+#include "resident.cuh"
 
 namespace vqc {
 

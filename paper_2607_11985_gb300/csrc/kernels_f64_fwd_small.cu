@@ -1,7 +1,7 @@
 // kernels_f64_fwd_small.cu -- instantiations of the sweep kernel for double, mode 0, sample
 // groups of fewer than 32 threads (small circuits or large blocks).
 #include "kernels.h"
-#include "sweep.cuh"
+#include "resident.cuh"
 
 namespace vqc {
 

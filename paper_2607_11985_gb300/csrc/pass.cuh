@@ -55,15 +55,6 @@ struct PArgs {
     int src_raw, lam_raw, dst_raw;
 };
 
-// XOR of cols[i] over the set bits of v.
-template <typename T, int N>
-__device__ __forceinline__ uint32_t xor_cols(const T (&cols)[N], uint32_t v) {
-    uint32_t r = 0;
-    for (int i = 0; v; ++i, v >>= 1)
-        if (v & 1u) r ^= (uint32_t)cols[i];
-    return r;
-}
-
 // 16-byte vectors of amplitudes, moved without taking register addresses.
 template <typename R> struct Vec16;
 template <> struct Vec16<float> {
@@ -341,7 +332,8 @@ __global__ void __launch_bounds__(256, 2) pass_kernel(const __grid_constant__ PA
             if (A.E_part) {
                 R* red = red_all + (size_t)q.g * q.wg * n;
                 const uint32_t pbf = tfl[nst].x ^ xor_bits(fin->tmask, A.tbits, q.t);
-                expz_frame<R, K, FULL>(fin->lmask, pbf, a, n, red, q, lane, warp_in_group);
+                expz_frame<R, K, FULL>(fin->lmask, pbf, a, n, q, lane,
+                                       [&](int j, R e) { red[warp_in_group * n + j] = e; });
                 __syncthreads();
                 if (valid)
                     for (int j = q.t; j < n; j += q.T) {

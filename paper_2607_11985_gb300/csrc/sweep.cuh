@@ -27,6 +27,7 @@
 #include <type_traits>
 
 #include "dd.cuh"
+#include "frame.h"
 #include "plan.h"
 
 namespace vqc {
@@ -231,7 +232,7 @@ struct KArgs {
     const int32_t* wocc;
     unsigned* err;
     int n, K, tbits, G, S;     // S = samples per CTA
-    int tpg, bpt;              // threads per sample group, register blocks per thread (tpg * bpt = 2^tbits)
+    int tpg;                   // threads per sample group (2^tbits)
     int n_ps, n_sh, n_accs, n_terms, Px, Pw;
     // batch
     int B, nunits;
@@ -254,6 +255,12 @@ struct KArgs {
     // [sched_off, sched_off + sched_bytes) of the plan's device blob.
     const unsigned char* plan;
     int tab_off, tab_bytes, sched_off, sched_bytes, sm_plan, plan_smem;
+    // resident path (resident.cuh): the frame schedule, and the slots of the state's
+    // bits in the order of a given state (sin) and of the final one (sout)
+    const FStage* fstages;
+    const FFinal* fin;
+    int32_t sin[kMaxTileBits], sout[kMaxTileBits];
+    int sm_io;
     // cluster path only (cluster.cuh): log2 CTAs per sample, rank 0's <Z> gather area
     int cl, sm_ecl;
 };
@@ -1170,13 +1177,6 @@ __device__ void acc_terms(const DAcc& ac, const DEntry& e, const R* ap, int wg,
 }
 
 
-// ---------------------------------------------------------------- kernel
-// MODE 0: forward, MODE 1: backward.
-// FULL: every sample group spans whole warps (2^(n-K) >= 32 threads), so warp
-// reductions are fixed full-warp butterflies; the launch picks the variant.
-// FUSED (MODE 1 only): the backward that recomputes the states also writes E
-// (vqc_forward_backward); a separate instantiation keeps that code out of the
-// plain backward kernel.
 // Launch-geometry self-check (kernel side): the host derives the block size,
 // the sample groups and the register blocks from one plan; a launch whose
 // numbers disagree records `code` in the plan's error word (read back by
@@ -1187,343 +1187,6 @@ __device__ __forceinline__ bool geometry_bad(bool bad, unsigned* err, unsigned c
     return bad;
 }
 enum : unsigned { kErrSweepGeometry = 1u, kErrPassGeometry = 2u, kErrClusterGeometry = 4u };
-
-template <typename R, int K, int MODE, bool FULL, bool FUSED, bool PH2 = true>
-__global__ void __launch_bounds__(512) sweep_kernel(const __grid_constant__ KArgs<St<R>> A) {
-    if (geometry_bad(blockDim.x != (unsigned)(A.S * A.tpg) || A.bpt * A.tpg != (1 << A.tbits) ||
-                         A.tbits != A.n - K || A.nstages < 1,
-                     A.err, kErrSweepGeometry))
-        return;
-    extern __shared__ __align__(16) unsigned char smem[];
-    R* sh_tab = reinterpret_cast<R*>(smem + A.sm_sh);
-    R* ps_all = reinterpret_cast<R*>(smem + A.sm_ps);
-    C2<R>* psi_all = reinterpret_cast<C2<R>*>(smem + A.sm_psi);
-    C2<R>* lam_all = reinterpret_cast<C2<R>*>(smem + A.sm_lam);
-    R* acc_all = reinterpret_cast<R*>(smem + A.sm_acc);
-    R* terms_all = reinterpret_cast<R*>(smem + A.sm_terms);
-    R* dw_cta = reinterpret_cast<R*>(smem + A.sm_dw);
-    R* red_all = reinterpret_cast<R*>(smem + A.sm_red);
-
-    const int n = A.n, G = A.G;
-    const int dim = 1 << n;
-    Geo q;
-    q.T = A.tpg;
-    q.lanes = q.T < 32 ? q.T : 32;
-    q.wg = q.T > 32 ? q.T / 32 : 1;
-    q.g = threadIdx.x / q.T;
-    q.t = threadIdx.x % q.T;
-    q.h = 0;
-    if (A.tbits < G) q.h = ((q.g & ((1 << (G - A.tbits)) - 1)) << A.tbits) & (dim - 1);
-    q.mask = blockDim.x >= 32 ? 0xffffffffu : ((1u << blockDim.x) - 1u);
-    const int lane = q.t & 31;
-    const int warp_in_group = q.t >> 5;
-    const int nthr = blockDim.x;
-
-    R* w_sm = reinterpret_cast<R*>(smem + A.sm_w);
-    R* xg_all = reinterpret_cast<R*>(smem + A.sm_xg);
-    const int xgw = A.Px + n;   // row width of the x / gE staging area
-    C2<R>* psi = psi_all + (size_t)q.g * dim;
-    C2<R>* lam = lam_all + (size_t)q.g * dim;
-
-    // initial (forward) or final (backward) state source; null: |0...0>
-    const SC2<R>* src = MODE == 1 ? A.psi_final : A.psi0;
-    if (MODE == 1 && !src) src = A.psi0;
-    const bool from_global = src != nullptr;
-
-    // One unit's inputs to shared memory, asynchronously: x (and, backward,
-    // gE) rows of its samples and each sample's initial / final state
-    // (coalesced reads, swizzled slots).
-    // (Double-float kernels copy the stored doubles as they are and split them
-    // in place afterwards, unit_to_dd: both types are 8 bytes.)
-    St<R>* xg_st = reinterpret_cast<St<R>*>(xg_all);
-    SC2<R>* psi_st = reinterpret_cast<SC2<R>*>(psi);
-    auto stage_unit = [&](int unit) {
-        for (int i = threadIdx.x; i < A.S * xgw; i += nthr) {
-            const int gg = i / xgw, c = i % xgw;
-            const int bb = min(unit * A.S + gg, A.B - 1);
-            if (c < A.Px) async_elem<St<R>>(xg_st + i, A.x + (size_t)bb * A.Px + c);
-            else if (MODE == 1) async_elem<St<R>>(xg_st + i, A.gE + (size_t)bb * n + (c - A.Px));
-        }
-        if (from_global) {
-            const int b = min(unit * A.S + q.g, A.B - 1);
-            const SC2<R>* gs = src + (size_t)b * dim;
-            for (int u = q.t; u < dim; u += q.T) async_elem<SC2<R>>(psi_st + (swz(u, G) ^ q.h), gs + u);
-        }
-    };
-    // after async_wait(): stored doubles -> dd in place, each by the thread that
-    // issued its copy (its own copies are visible to it); a barrier follows
-    auto unit_to_dd = [&]() {
-        if constexpr (!std::is_same<St<R>, R>::value) {
-            for (int i = threadIdx.x; i < A.S * xgw; i += nthr) {
-                const int c = i % xgw;
-                if (c < A.Px || MODE == 1) xg_all[i] = R(xg_st[i]);
-            }
-            if (from_global)
-                for (int u = q.t; u < dim; u += q.T) {
-                    const int sl = swz(u, G) ^ q.h;
-                    psi[sl] = c2_in<R>(psi_st[sl]);
-                }
-        }
-    };
-
-    // Prologue: the plan regions, w and the first unit's inputs all in flight
-    // at once, one wait.
-    const unsigned char* smt = nullptr;
-    const unsigned char* sms = nullptr;
-    if (A.plan_smem) {
-        unsigned char* t = smem + A.sm_plan;
-        unsigned char* u = t + ((A.tab_bytes + 15) & ~15);
-        async_region(t, A.plan + A.tab_off, A.tab_bytes);
-        async_region(u, A.plan + A.sched_off, A.sched_bytes);
-        smt = t;
-        sms = u;
-    }
-    grid_dep_wait();
-    grid_dep_launch();
-    for (int i = threadIdx.x; i < A.Pw; i += nthr)
-        async_elem<St<R>>(reinterpret_cast<St<R>*>(w_sm) + i, A.w + i);
-    if ((int)blockIdx.x < A.nunits) stage_unit(blockIdx.x);
-    if (MODE == 1)
-        for (int i = threadIdx.x; i < A.Pw; i += nthr) dw_cta[i] = 0;
-    PlanPtrs P;
-    P.ops = rebase(A.ops, A.plan, A.sched_off, sms);
-    P.stages = rebase(A.stages, A.plan, A.sched_off, sms);
-    P.entries = rebase(A.entries, A.plan, A.tab_off, smt);
-    P.ps_list = rebase(A.ps_list, A.plan, A.tab_off, smt);
-    P.sh_list = rebase(A.sh_list, A.plan, A.tab_off, smt);
-    P.consts = rebase(A.consts, A.plan, A.tab_off, smt);
-    P.cmat = rebase(reinterpret_cast<const unsigned char*>(A.cmat), A.plan, A.tab_off, smt);
-    P.cang = rebase(reinterpret_cast<const unsigned char*>(A.cang), A.plan, A.tab_off, smt);
-    P.accs = rebase(A.accs, A.plan, A.tab_off, smt);
-    P.xocc_ptr = rebase(A.xocc_ptr, A.plan, A.tab_off, smt);
-    P.xocc = rebase(A.xocc, A.plan, A.tab_off, smt);
-    P.wocc_ptr = rebase(A.wocc_ptr, A.plan, A.tab_off, smt);
-    P.wocc = rebase(A.wocc, A.plan, A.tab_off, smt);
-    const R* Pcmat = reinterpret_cast<const R*>(P.cmat);
-    const R* Pcang = reinterpret_cast<const R*>(P.cang);
-    async_wait();
-    if constexpr (!std::is_same<St<R>, R>::value) {
-        for (int i = threadIdx.x; i < A.Pw; i += nthr) w_sm[i] = R(reinterpret_cast<const St<R>*>(w_sm)[i]);
-        if ((int)blockIdx.x < A.nunits) unit_to_dd();
-    }
-    __syncthreads();
-
-    // shared table (w and constants) once per CTA, on the CTA's last threads
-    // so that it runs beside the first unit's per-sample table
-    for (int i = nthr - 1 - threadIdx.x; i < A.n_sh; i += nthr) {
-        const int id = vqc_ld(&P.sh_list[i]);
-        const DEntry e = P.entries[id];
-        eval_entry<R>(e, P.consts, static_cast<const R*>(nullptr), w_sm, Pcang, Pcmat,
-                      sh_tab + EntryWords<R>::value * e.slot);
-    }
-
-    R* ps_tab = ps_all + (size_t)q.g * A.n_ps * EntryWords<R>::value;
-    R* acc = acc_all + (size_t)q.g * A.n_accs * q.wg * 8;
-    R* terms = terms_all + (size_t)q.g * A.n_terms;
-
-    for (int unit = blockIdx.x; unit < A.nunits; unit += gridDim.x) {
-        const int b_raw = unit * A.S + q.g;
-        const bool valid = b_raw < A.B;
-        const int b = valid ? b_raw : A.B - 1;
-        if (unit != (int)blockIdx.x) {
-            stage_unit(unit);
-            async_wait();
-            if constexpr (!std::is_same<St<R>, R>::value) unit_to_dd();
-            __syncthreads();
-        }
-        const R* xrow = xg_all + (size_t)q.g * xgw;
-
-        // per-sample table (x-dependent runs): threads of the CTA over (sample, entry)
-        for (int i = threadIdx.x; i < A.S * A.n_ps; i += nthr) {
-            const int gg = i / A.n_ps, k = i % A.n_ps;
-            const int id = vqc_ld(&P.ps_list[k]);
-            const DEntry e = P.entries[id];
-            eval_entry<R>(e, P.consts, xg_all + (size_t)gg * xgw, w_sm, Pcang, Pcmat,
-                          ps_all + ((size_t)gg * A.n_ps + e.slot) * EntryWords<R>::value);
-        }
-        __syncthreads();
-
-        C2<R> a[1 << K];
-        int32_t sg[K];
-        StageView v{0, 0};
-        const bool recompute = MODE == 1 && A.psi_final == nullptr;
-        const int ns = A.nstages;
-
-        // -------- forward sweep (forward mode, or backward recompute; the
-        // recompute also writes E when the caller asks for it)
-        R* red = red_all + (size_t)q.g * q.wg * n;
-        const bool want_E = MODE == 0 || (FUSED && recompute && A.E != nullptr);
-        if (MODE == 0 || recompute) {
-            for (int s = 0; s < ns; ++s) {
-                const DStage* sp = P.stages + s;
-                const bool last = s + 1 == ns;
-                const bool store = !last || (MODE == 0 && A.state_out) || (MODE == 1 && A.bpt > 1);
-                R eacc = 0;   // full-warp groups: this lane's share of the warp's <Z> sums
-                int eidx = 0;
-                for (int bj = 0; bj < A.bpt; ++bj) {
-                    v = stage_view<K>(sp, q.t + bj * q.T, q.h, sg);
-                    if (s == 0 && !from_global) {
-#pragma unroll
-                        for (int r = 0; r < (1 << K); ++r) a[r] = cm<R>(0, 0);
-                        if (v.pb == 0) a[0] = cm<R>(1, 0);
-                    } else {
-                        block_load<R, K>(a, psi, v.swb, sg);
-                    }
-                    run_ops<R, K, 0, false, FULL, PH2>(P.ops, vqc_ld(&sp->op_begin), vqc_ld(&sp->op_end), v.pb, a, a,
-                                     sh_tab, ps_tab, nullptr, q, lane, warp_in_group);
-                    if (want_E && last) {   // <Z_j> partials from the final blocks
-                        if constexpr (FULL) {   // butterfly over the warp (n <= 16 here)
-                            if (n <= 8) {
-                                R ez[8];
-#pragma unroll
-                                for (int j = 0; j < 8; ++j) ez[j] = 0;
-                                expz_accum<R, K, 8>(sp, v.pb, a, ez);
-                                eidx = warp_reduce_scatter<R, 8>(ez, lane);
-                                eacc += ez[0];
-                            } else {
-                                R ez[16];
-#pragma unroll
-                                for (int j = 0; j < 16; ++j) ez[j] = 0;
-                                expz_accum<R, K, 16>(sp, v.pb, a, ez);
-                                eidx = warp_reduce_scatter<R, 16>(ez, lane);
-                                eacc += ez[0];
-                            }
-                        } else {
-                            expz_partials<R, K>(sp, v.pb, a, n, red, q, warp_in_group, bj > 0);
-                        }
-                    }
-                    if (store) {   // through the store map (absorbed CX gates)
-                        // a permuting store writes slots other threads load in this
-                        // stage: every load of the group must be done first
-                        if (vqc_ld(&sp->nperm)) group_sync<R>(q);
-                        int32_t s2[K];
-                        const uint32_t b2 = map_base<K, true>(sp, q.t + bj * q.T, q.h, s2);
-                        block_store<R, K>(a, psi, b2, s2);
-                    }
-                }
-                if (want_E && last && FULL) {
-                    // a single-warp group writes E itself
-                    const int low = n <= 8 ? 3 : 1;   // lane bits below the scatter bits
-                    if ((lane & low) == 0 && eidx < n) {
-                        if (q.wg == 1) {
-                            if (valid) A.E[(size_t)b * n + eidx] = as_out<St<R>>(eacc);
-                        } else {
-                            red[warp_in_group * n + eidx] = eacc;
-                        }
-                    }
-                }
-                if (store) group_sync<R>(q);
-            }
-        }
-
-        if (MODE == 0) {
-            const bool direct = FULL && q.wg == 1;   // E already written
-            if (!direct || A.state_out) {
-                __syncthreads();
-                if (valid) {
-                    if (!direct) {
-                        for (int j = q.t; j < n; j += q.T) {
-                            R e = 0;
-                            for (int k = 0; k < q.wg; ++k) e += red[k * n + j];
-                            A.E[(size_t)b * n + j] = as_out<St<R>>(e);
-                        }
-                    }
-                    if (A.state_out) {
-                        SC2<R>* go = A.state_out + (size_t)b * dim;
-                        for (int u = q.t; u < dim; u += q.T) go[u] = c2_out<R>(psi[swz(u, G) ^ q.h]);
-                    }
-                }
-            }
-            if (unit + (int)gridDim.x < A.nunits) __syncthreads();
-            continue;
-        }
-
-        if (MODE == 1 && want_E && !(FULL && q.wg == 1)) {   // E of the recomputed states
-            __syncthreads();
-            if (valid)
-                for (int j = q.t; j < n; j += q.T) {
-                    R e = 0;
-                    for (int k = 0; k < q.wg; ++k) e += red[k * n + j];
-                    A.E[(size_t)b * n + j] = as_out<St<R>>(e);
-                }
-        }
-
-        // -------- backward: reverse sweep with psi and lam
-        for (int s = ns - 1; s >= 0; --s) {
-            const DStage* sp = P.stages + s;
-            for (int bj = 0; bj < A.bpt; ++bj) {
-                C2<R> l[1 << K];
-                v = stage_view<K>(sp, q.t + bj * q.T, q.h, sg);
-                if (s == ns - 1) {
-                    if (!recompute || A.bpt > 1) block_load<R, K>(a, psi, v.swb, sg);
-                    lambda_init<R, K>(sp, v.pb, xrow + A.Px, n, a, l);
-                } else {   // the forward left this stage's output in its store map
-                    int32_t s2[K];
-                    const uint32_t b2 = map_base<K, true>(sp, q.t + bj * q.T, q.h, s2);
-                    block_load<R, K>(a, psi, b2, s2);
-                    block_load<R, K>(l, lam, b2, s2);
-                }
-                run_ops<R, K, 1, false, FULL, PH2>(P.ops, vqc_ld(&sp->op_begin), vqc_ld(&sp->op_end), v.pb, a, l,
-                                 sh_tab, ps_tab, acc, q, lane, warp_in_group, bj > 0);
-                if (s > 0) {   // back to the stage's input layout (load map)
-                    if (vqc_ld(&sp->nperm)) group_sync<R>(q);   // see the forward's store
-                    int32_t s2[K];
-                    const uint32_t b2 = map_base<K, false>(sp, q.t + bj * q.T, q.h, s2);
-                    block_store<R, K>(a, psi, b2, s2);
-                    block_store<R, K>(l, lam, b2, s2);
-                }
-            }
-            group_sync<R>(q);
-        }
-        __syncthreads();
-
-        // -------- gradient terms from the accumulated rho / scalars
-        for (int i = threadIdx.x; i < A.S * A.n_accs; i += nthr) {
-            const int gg = i / A.n_accs, k = i % A.n_accs;
-            const DAcc ac = P.accs[k];
-            acc_terms<R>(ac, P.entries[ac.entry], acc_all + ((size_t)gg * A.n_accs + k) * q.wg * 8,
-                         q.wg, P.consts, xg_all + (size_t)gg * xgw, w_sm, Pcang, Pcmat,
-                         terms_all + (size_t)gg * A.n_terms);
-        }
-        __syncthreads();
-        // dx rows of this CTA's samples; dw partial of this CTA (fixed order)
-        if (A.dx) {
-            for (int i = threadIdx.x; i < A.S * A.Px; i += nthr) {
-                const int gg = i / A.Px, p = i % A.Px;
-                const int bb = unit * A.S + gg;
-                if (bb >= A.B) continue;
-                const R* tm = terms_all + (size_t)gg * A.n_terms;
-                const int k0 = vqc_ld(&P.xocc_ptr[p]), k1 = vqc_ld(&P.xocc_ptr[p + 1]);
-                R sum = 0;
-                for (int k = k0; k < k1; ++k) sum += tm[vqc_ld(&P.xocc[k])];
-                A.dx[(size_t)bb * A.Px + p] = as_out<St<R>>(sum);
-            }
-        }
-        const int nvalid = min(A.S, A.B - unit * A.S);
-        for (int p = threadIdx.x; p < A.Pw; p += nthr) {
-            // samples in order, each sample's occurrences in order
-            const int k0 = vqc_ld(&P.wocc_ptr[p]), k1 = vqc_ld(&P.wocc_ptr[p + 1]);
-            R sum = dw_cta[p];
-            if (k1 - k0 == 1) {   // the common case: independent loads
-                const int j = vqc_ld(&P.wocc[k0]);
-                for (int gg = 0; gg < nvalid; ++gg) sum += terms_all[(size_t)gg * A.n_terms + j];
-            } else {
-                for (int gg = 0; gg < nvalid; ++gg) {
-                    const R* tm = terms_all + (size_t)gg * A.n_terms;
-                    for (int k = k0; k < k1; ++k) sum += tm[vqc_ld(&P.wocc[k])];
-                }
-            }
-            dw_cta[p] = sum;
-        }
-        __syncthreads();
-    }
-
-    if (MODE == 1 && A.Pw > 0 && A.dw) {
-        // per-CTA partial of dw; reduce_cols sums the partials in CTA order
-        for (int p = threadIdx.x; p < A.Pw; p += nthr)
-            A.dw_part[(size_t)blockIdx.x * A.Pw + p] = as_out<St<R>>(dw_cta[p]);
-    }
-}
 
 // out[c] = sum over rows r of part[r * cols + c]: one block per column,
 // fixed strided partial sums, then a fixed-shape tree (deterministic).

@@ -275,9 +275,9 @@ def check(spec, x, w, gE, psi0, dtype):
     for s in fr:
         em = Emulator(pl, s, xs[0], w)
         p0 = None if psi0 is None else psi0[0]
-        if s["mode"] == 0:
+        if s["mode"] == 0 or s["path"] == 0:   # the resident backward recomputes with its own stages
             assert np.allclose(em.forward(p0), st[0], atol=1e-12)
-        else:
+        if s["mode"] == 1:
             dx, dw = em.backward(st[0], gE[0])
             assert np.allclose(dx, dx_ref[0] if spec.num_x else dx, atol=1e-10)
             assert np.allclose(dw, dw_ref, atol=1e-10)
