@@ -582,30 +582,44 @@ vqc_status plan_cluster(const HostPlan& p, int mode, int B, Launch& L) {
     return VQC_OK;
 }
 
-// The cluster forward by default for 2-CTA clusters (complex64 15 qubits,
-// complex128 14): measured 16-24% / ~5% faster than the HBM-tiled passes there.
-// Larger clusters measured slower (0.7x at 16 qubits: one sample per cluster
-// leaves too few warps per SM to hide the per-stage cluster barriers), so they
-// run only when VQC_FORCE_PATH=cluster asks; VQC_FORCE_PATH=hbm turns it off.
-// The cluster backward (psi and lam over the cluster) follows the same rule:
-// by default for 2-CTA clusters (complex64 14 qubits, complex128 13), where it
-// measured 1-7% faster than the backward passes, and 0.78-0.90x with 4-8 CTAs
-// (0.80x on the 16-qubit / batch-512 workload); it also needs its shared-memory
-// layout (two slices, the per-warp rho partials, the tables) to fit one CTA.
-bool use_cluster(const HostPlan& p, int mode) {
+// Whether a 2-CTA cluster schedule exists and (backward) its shared-memory layout --
+// two slices, the per-warp rho partials, the tables -- fits one CTA.
+bool cluster_fits(const HostPlan& p, int mode) {
     const Schedule* s = find_cluster_schedule(p, mode);
     if (!s) return false;
-    const char* f = std::getenv("VQC_FORCE_PATH");
-    const bool forced = f && std::string(f) == "cluster";
-    if (f && std::string(f) == "hbm") return false;
-    const bool two_cta = p.n - s->K - s->cta_bits == 1;
-    if (mode == 0) return forced || two_cta;
-    if (!forced && !two_cta) return false;
+    if (mode == 0) return true;
     Launch L;
     const std::string saved = g_err;
     const bool ok = plan_cluster(p, 1, 1, L) == VQC_OK;
     g_err = saved;
     return ok;
+}
+
+// By default 2-CTA clusters (complex64 15 qubits forward, 14 backward; complex128 one
+// less) take batches of at most one wave, a cluster per sample, which need no state
+// in HBM; beyond that the HBM passes run, which then measured faster on every
+// circuit: complex64 14 qubits, batch 100, backward 257 / 358 / 469 us by clusters
+// (layered / RZZ rings / random) and 159 / 269 / 327 us by passes; 15 qubits forward
+// 191 / 232 / 312 and 118 / 172 / 200 us; complex128 1.0 to 1.3 times.  (Within a wave
+// the passes are 1.0 to 2.2 times faster too; that choice is kept for its workspace,
+// which holds no states.)  The double-float backward stays on clusters: 762 / 1319 /
+// 1555 us at batch 152 against 770 / 2203 / 1558 by passes.  Larger clusters run only
+// when VQC_FORCE_PATH=cluster asks; VQC_FORCE_PATH=hbm turns them off.
+bool use_cluster(const HostPlan& p, int mode, int B) {
+    const Schedule* s = find_cluster_schedule(p, mode);
+    if (!s) return false;
+    const char* f = std::getenv("VQC_FORCE_PATH");
+    if (f && std::string(f) == "cluster") return cluster_fits(p, mode);
+    if (f && std::string(f) == "hbm") return false;
+    if (p.n - s->K - s->cta_bits != 1) return false;
+    if (!(p.dfloat && mode == 1) && find_frame(p, mode, VQC_PATH_HBM)) {
+        int dev = 0, sms = 152;   // without a device: GB300's SM count
+        DevInfo di;
+        if (cudaGetDevice(&dev) == cudaSuccess && device_info(dev, di) == VQC_OK) sms = di.sms;
+        else (void)cudaGetLastError();
+        if (B > sms / 2) return false;
+    }
+    return cluster_fits(p, mode);
 }
 
 template <typename R>
@@ -1188,8 +1202,19 @@ vqc_status backward_with_scratch(const vqc_plan* plan, int32_t batch, const void
     // the same path choice as vqc_backward: the cluster backward when the
     // environment asks for it, resident when the batch fits a resident launch,
     // else the HBM-tiled passes (each with its own workspace layout)
-    const bool clu = use_cluster(p, 1);
-    const bool hbm = !clu && use_hbm(p, 1, batch);
+    bool clu = use_cluster(p, 1, batch);
+    bool hbm = !clu && use_hbm(p, 1, batch);
+    if (hbm && !std::getenv("VQC_FORCE_PATH")) {   // states that do not fit the scratch may fit a cluster
+        const Schedule* s = find_cluster_schedule(p, 1);
+        PassGeo L;
+        st = plan_hbm(p, 1, batch, L);
+        if (st != VQC_OK) return st;
+        if (s && p.n - s->K - s->cta_bits == 1 && hbm_layout(p, 1, batch, L.ntiles).total > scratch_bytes &&
+            cluster_fits(p, 1)) {
+            clu = true;
+            hbm = false;
+        }
+    }
     size_t need = 0;
     if (clu) {
         Launch L;
@@ -1305,7 +1330,7 @@ size_t vqc_workspace_bytes(const vqc_plan* plan, int32_t batch, int32_t mode) {
         const HostPlan& p = plan->hp;
         Launch L;
         const std::string saved = g_err;
-        if (batch > 0 && !use_cluster(p, 0) && !use_hbm(p, 0, batch) && !use_hbm(p, 1, batch)) {
+        if (batch > 0 && !use_cluster(p, 0, batch) && !use_hbm(p, 0, batch) && !use_hbm(p, 1, batch)) {
             if (resident_two_calls(p, batch)) {
                 const size_t cs = p.dtype == VQC_C128 ? 16 : 8;
                 need = std::max(need, two_call_state_offset(p, batch) + align256(((size_t)batch << p.n) * cs));
@@ -1313,11 +1338,11 @@ size_t vqc_workspace_bytes(const vqc_plan* plan, int32_t batch, int32_t mode) {
                 need = std::max(need, bwd_workspace(p, L));
             }
         }
-        if (batch > 0 && !use_cluster(p, 1) && use_hbm(p, 1, batch)) {
+        if (batch > 0 && !use_cluster(p, 1, batch) && use_hbm(p, 1, batch)) {
             // the final states in the backward's psi region, the forward's workspace behind them
             need = std::max(need, hbm_state_bytes(p, batch) + vqc_workspace_bytes(plan, batch, 0));
         }
-        if (batch > 0 && use_cluster(p, 1)) {   // [either call's workspace | final states]
+        if (batch > 0 && use_cluster(p, 1, batch)) {   // [either call's workspace | final states]
             const size_t cs = p.dtype == VQC_C128 ? 16 : 8;
             need = align256(need) + align256(((size_t)batch << p.n) * cs);
         }
@@ -1332,7 +1357,7 @@ size_t vqc_workspace_bytes(const vqc_plan* plan, int32_t batch, int32_t mode) {
     }
     if ((mode != 0 && mode != 1) || batch <= 0) return 0;
     const HostPlan& p = plan->hp;
-    if (use_cluster(p, mode)) {
+    if (use_cluster(p, mode, batch)) {
         if (mode == 0) return 0;
         Launch L;
         if (plan_cluster(p, 1, batch, L) != VQC_OK) return 0;
@@ -1405,7 +1430,7 @@ vqc_status vqc_forward(const vqc_plan* plan, int32_t batch, const void* x, const
         st = check_out_ptrs(p, {expz_out}, {state_out});
         if (st != VQC_OK) return st;
         cudaStream_t s = static_cast<cudaStream_t>(stream);
-        if (use_cluster(p, 0)) {
+        if (use_cluster(p, 0, batch)) {
             if (p.dtype == VQC_C64)
                 return run_cluster_forward<float>(p, batch, x, w, psi0, expz_out, state_out, s);
             return run_cluster_forward<double>(p, batch, x, w, psi0, expz_out, state_out, s);
@@ -1446,7 +1471,7 @@ vqc_status vqc_backward(const vqc_plan* plan, int32_t batch, const void* x, cons
         if (!grad_expz) return fail(VQC_ERR_INVALID_ARG, "grad_expz is NULL");
         st = check_out_ptrs(p, {grad_expz, grad_x, grad_w}, {});
         if (st != VQC_OK) return st;
-        if (use_cluster(p, 1)) {
+        if (use_cluster(p, 1, batch)) {
             if (p.dtype == VQC_C64)
                 return run_cluster_backward<float>(p, batch, x, w, psi0, psi_final, grad_expz, grad_x,
                                                    grad_w, workspace, workspace_bytes, s);
@@ -1489,7 +1514,7 @@ vqc_status vqc_forward_backward(const vqc_plan* plan, int32_t batch, const void*
         if (!expz_out) return fail(VQC_ERR_INVALID_ARG, "expz_out is NULL");
         st = check_out_ptrs(p, {expz_out, grad_expz, grad_x, grad_w}, {});
         if (st != VQC_OK) return st;
-        if (!use_cluster(p, 0) && !use_hbm(p, 0, batch) && !use_hbm(p, 1, batch) &&
+        if (!use_cluster(p, 0, batch) && !use_hbm(p, 0, batch) && !use_hbm(p, 1, batch) &&
             resident_two_calls(p, batch)) {
             // the forward (larger register blocks) saves the final states after the
             // backward's workspace; the backward starts from them
@@ -1503,7 +1528,7 @@ vqc_status vqc_forward_backward(const vqc_plan* plan, int32_t batch, const void*
             return vqc_backward(plan, batch, x, w, psi0, psi_final, grad_expz, grad_x, grad_w, workspace,
                                 workspace_bytes, stream);
         }
-        if (!use_cluster(p, 0) && !use_hbm(p, 0, batch) && !use_hbm(p, 1, batch)) {
+        if (!use_cluster(p, 0, batch) && !use_hbm(p, 0, batch) && !use_hbm(p, 1, batch)) {
             // one launch: the backward kernel sweeps forward itself (the state stays in
             // shared memory), writes E, then sweeps back
             if (p.dtype == VQC_C64)
@@ -1512,7 +1537,7 @@ vqc_status vqc_forward_backward(const vqc_plan* plan, int32_t batch, const void*
             return run<double>(p, 2, batch, x, w, psi0, nullptr, grad_expz, expz_out, nullptr, grad_x,
                                grad_w, workspace, workspace_bytes, s);
         }
-        if (use_cluster(p, 1)) {
+        if (use_cluster(p, 1, batch)) {
             // the forward leaves the final states after the larger of the two calls'
             // workspaces; the cluster backward starts from them
             const size_t need = vqc_workspace_bytes(plan, batch, 3);
@@ -1597,7 +1622,7 @@ vqc_status vqc_plan_info(const vqc_plan* plan, int32_t batch, vqc_plan_stats* ou
         int* tq = mode == 0 ? &out->fwd_tile_qubits : &out->bwd_tile_qubits;
         double* hb = mode == 0 ? &out->fwd_hbm_bytes_per_eval : &out->bwd_hbm_bytes_per_eval;
         const int K = choose_k(p, mode, B, sms);
-        const bool clu = use_cluster(p, mode);
+        const bool clu = use_cluster(p, mode, B);
         const bool hbm = !clu && (ndev > 0 ? use_hbm(p, mode, B)
                                            : (K == 0 && find_frame(p, mode, VQC_PATH_HBM) != nullptr));
         if (clu) {
