@@ -124,7 +124,7 @@ struct Launch {
     int K = 0, T = 0, S = 0, block = 0, grid = 0, nunits = 0, wg = 1;
     size_t smem = 0;
     int sm_sh = 0, sm_ps = 0, sm_psi = 0, sm_lam = 0, sm_acc = 0, sm_terms = 0, sm_dw = 0,
-        sm_red = 0, sm_plan = 0, sm_w = 0, sm_xg = 0, sm_io = 0;
+        sm_red = 0, sm_plan = 0, sm_w = 0, sm_xg = 0, sm_io = 0, sm_dg = 0;
     int cl = 0, sm_ecl = 0;   // cluster path: log2 CTAs per sample, <Z> gather area
     bool plan_smem = false;
     const void* fn = nullptr;
@@ -203,11 +203,12 @@ vqc_status plan_launch_uncached(const HostPlan& p, int launch_mode, int B, Launc
     L.wg = L.T > 32 ? L.T / 32 : 1;
     // Shared memory: a fixed part per CTA and a part per resident sample.
     const size_t dim = (size_t)1 << p.n;
-    const size_t ew = dbl ? 8 : 32;   // reals per table entry
+    const size_t ew = entry_reals(dbl);
     const size_t io = (size_t)8 << L.K;   // slot offsets of the state copies
     const size_t fixed = align16((size_t)p.n_sh * ew * rs) + align16(mode == 1 ? (size_t)p.num_w * rs : 0) +
                          align16((size_t)p.num_w * rs) + io + 10 * 16;
-    const size_t per_sample = (size_t)p.n_ps * ew * rs + dim * cs * (mode == 1 ? 2 : 1) +
+    const size_t dgb = dbl && L.T >= 32 ? (L.f->stages.size() << (L.K + 1)) * cs : 0;   // stage diagonals
+    const size_t per_sample = dgb + (size_t)p.n_ps * ew * rs + dim * cs * (mode == 1 ? 2 : 1) +
                               (size_t)(p.num_x + p.n) * rs +
                               (mode == 1 ? p.accs.size() * L.wg * 8 * rs + p.term_src.size() * rs : 0) +
                               (size_t)L.wg * p.n * rs;
@@ -241,6 +242,7 @@ vqc_status plan_launch_uncached(const HostPlan& p, int launch_mode, int B, Launc
     L.sm_sh = take((size_t)p.n_sh * ew * rs);
     L.sm_ps = take((size_t)L.S * p.n_ps * ew * rs);
     L.sm_io = take(io);
+    L.sm_dg = take(L.S * dgb);
     L.sm_acc = take(mode == 1 ? (size_t)L.S * p.accs.size() * L.wg * 8 * rs : 0);
     L.sm_terms = take(mode == 1 ? (size_t)L.S * p.term_src.size() * rs : 0);
     L.sm_dw = take(mode == 1 ? (size_t)p.num_w * rs : 0);
@@ -346,7 +348,7 @@ void fill_plan_args(const HostPlan& p, const Launch& L, KArgs<R>& a) {
     a.Pw = p.num_w;
     a.sm_sh = L.sm_sh; a.sm_ps = L.sm_ps; a.sm_psi = L.sm_psi; a.sm_lam = L.sm_lam;
     a.sm_acc = L.sm_acc; a.sm_terms = L.sm_terms; a.sm_dw = L.sm_dw; a.sm_red = L.sm_red;
-    a.sm_w = L.sm_w; a.sm_xg = L.sm_xg; a.sm_io = L.sm_io;
+    a.sm_w = L.sm_w; a.sm_xg = L.sm_xg; a.sm_io = L.sm_io; a.sm_dg = L.sm_dg;
     a.plan = static_cast<const unsigned char*>(p.dbuf);
     a.tab_off = (int)p.dev_tab_begin;
     a.tab_bytes = (int)(p.dev_tab_end - p.dev_tab_begin);
@@ -521,7 +523,7 @@ vqc_status plan_cluster(const HostPlan& p, int mode, int B, Launch& L) {
     vqc_status st = device_info(dev, di);
     if (st != VQC_OK) return st;
     const bool dbl = p.dtype == VQC_C128;
-    const size_t rs = dbl ? 8 : 4, cs = 2 * rs, ew = dbl ? 8 : 32;
+    const size_t rs = dbl ? 8 : 4, cs = 2 * rs, ew = entry_reals(dbl);
     L.K = L.s->K;
     L.cl = p.n - L.K - L.s->cta_bits;
     L.T = 1 << (p.n - L.K);           // threads of a sample group, over the whole cluster
@@ -721,7 +723,7 @@ struct PassGeo {
     int K = 0, T = 0, S = 0, block = 0, grid = 0, wg = 1, ntiles = 1;
     int nunits = 0;
     size_t smem = 0;
-    int sm_sh = 0, sm_ps = 0, sm_lam = 0, sm_acc = 0, sm_red = 0, sm_plan = 0, sm_tfl = 0, sm_koff = 0, sm_toff = 0, sm_tbase = 0;
+    int sm_sh = 0, sm_ps = 0, sm_lam = 0, sm_acc = 0, sm_red = 0, sm_plan = 0, sm_tfl = 0, sm_koff = 0, sm_toff = 0, sm_tbase = 0, sm_dg = 0;
     const void* fn = nullptr;
 };
 
@@ -749,12 +751,13 @@ vqc_status plan_hbm_uncached(const HostPlan& p, int mode, int B, PassGeo& L) {
         ops_max = std::max(ops_max, ps.op_end - ps.op_begin);
     }
     const size_t tdim = (size_t)1 << m;
-    const size_t ew = dbl ? 8 : 32;   // reals per table entry
+    const size_t ew = entry_reals(dbl);
     const size_t apv = 16 / cs, nk = (tdim / apv + L.T - 1) / L.T;
     const size_t prog = (size_t)nst_max * sizeof(FStage) + sizeof(FFinal) + (size_t)ops_max * sizeof(DOp) +
                         (size_t)nst_max * L.s->nout * sizeof(FFlip);
     const size_t fixed = align16((size_t)sh_max * ew * rs) + align16(prog) + align16(2 * nk * 8) + 8 * 16;
-    const size_t per_tile = (size_t)ps_max * ew * rs + tdim * cs * (mode == 1 ? 2 : 1) + (size_t)(nst_max + 1) * 8 +
+    const size_t dgb = dbl && L.T >= 32 ? ((size_t)nst_max << (L.K + 1)) * cs : 0;   // stage diagonals
+    const size_t per_tile = dgb + (size_t)ps_max * ew * rs + tdim * cs * (mode == 1 ? 2 : 1) + (size_t)(nst_max + 1) * 8 +
                             (size_t)L.T * (16 + 4 * nst_max) + (mode == 1 ? (size_t)acc_max * L.wg * 8 * rs : (size_t)L.wg * p.n * rs);
     int S = std::max(1, 128 / L.T);
     if ((size_t)di.smem_optin <= fixed + per_tile)
@@ -780,6 +783,7 @@ vqc_status plan_hbm_uncached(const HostPlan& p, int mode, int B, PassGeo& L) {
     L.sm_red = take(mode == 0 ? (size_t)S * L.wg * p.n * rs : 0);
     L.sm_koff = take(2 * nk * 8);   // tile-copy offsets: one uint2 per vector round, read and written
     L.sm_toff = take((size_t)L.block * 16);   // and each thread's own part
+    L.sm_dg = take(S * dgb);
     L.sm_tbase = take((size_t)nst_max * L.block * 4);
     L.sm_plan = take(prog);
     L.sm_tfl = take((size_t)S * (nst_max + 1) * 8);
@@ -843,7 +847,7 @@ size_t hbm_state_bytes(const HostPlan& p, int B) {
 HbmWs hbm_layout(const HostPlan& p, int mode, int B, int ntiles) {
     const size_t rs = p.dtype == VQC_C128 ? 8 : 4;
     const size_t sbytes = hbm_state_bytes(p, B);
-    const size_t entry = (p.dtype == VQC_C128 ? 8 : 32) * rs;
+    const size_t entry = entry_reals(p.dtype == VQC_C128) * rs;
     HbmWs w;
     w.state = 256;
     if (mode == 0) {
@@ -931,6 +935,7 @@ void fill_pass_args(const HostPlan& p, const PassGeo& L, const FPass& ps, const 
     a.sm_acc = L.sm_acc; a.sm_red = L.sm_red; a.sm_koff = L.sm_koff;
     a.sm_plan = L.sm_plan; a.sm_tfl = L.sm_tfl; a.sm_toff = L.sm_toff;
     a.sm_tbase = L.sm_tbase;
+    a.sm_dg = L.sm_dg;
 }
 
 // The forward passes: psi0 (nullptr: |0...0>) -> out in logical order (nullptr:

@@ -109,4 +109,46 @@ __device__ __forceinline__ dd dot4(dd a0, dd b0, dd a1, dd b1, dd a2, dd b2, dd 
     return dd(h, __fsub_rn(err, __fsub_rn(h, s)));
 }
 
+// a0 b0 + a1 b1, the same way (19 operations; a product and a fused multiply-add
+// take 29).
+__device__ __forceinline__ dd dot2(dd a0, dd b0, dd a1, dd b1) {
+    const float p0 = __fmul_rn(a0.hi, b0.hi), p1 = __fmul_rn(a1.hi, b1.hi);
+    float err = __fmaf_rn(a0.hi, b0.hi, -p0);
+    err = __fmaf_rn(a0.hi, b0.lo, err);
+    err = __fmaf_rn(a0.lo, b0.hi, err);
+    const float e = __fmaf_rn(a1.hi, b1.hi, -p1);
+    const float s = __fadd_rn(p0, p1);
+    const float v = __fsub_rn(s, p0);
+    const float r = __fadd_rn(__fsub_rn(p0, __fsub_rn(s, v)), __fsub_rn(p1, v));
+    err = __fadd_rn(err, r);
+    err = __fmaf_rn(a1.hi, b1.lo, err);
+    err = __fmaf_rn(a1.lo, b1.hi, err);
+    err = __fadd_rn(err, e);
+    const float h = __fadd_rn(s, err);
+    return dd(h, __fsub_rn(err, __fsub_rn(h, s)));
+}
+
+// A running compensated dot product: 12 operations a term, one normalization at the
+// end.  The error of err is a few float roundings of float-sized errors, some 2^-46
+// of the terms' magnitudes over the 32 terms of a register block.
+struct ddsum {
+    float s = 0.f, err = 0.f;
+    __device__ __forceinline__ void add(dd a, dd b) {
+        const float p = __fmul_rn(a.hi, b.hi);
+        const float e = __fmaf_rn(a.hi, b.hi, -p);
+        const float t = __fadd_rn(s, p);
+        const float v = __fsub_rn(t, s);
+        const float r = __fadd_rn(__fsub_rn(s, __fsub_rn(t, v)), __fsub_rn(p, v));
+        s = t;
+        err = __fadd_rn(err, r);
+        err = __fmaf_rn(a.hi, b.lo, err);
+        err = __fmaf_rn(a.lo, b.hi, err);
+        err = __fadd_rn(err, e);
+    }
+    __device__ __forceinline__ dd value() const {
+        const float h = __fadd_rn(s, err);
+        return dd(h, __fsub_rn(err, __fsub_rn(h, s)));
+    }
+};
+
 }  // namespace vqc

@@ -296,4 +296,123 @@ __device__ __forceinline__ void pure_backward(const uint2* ops, unsigned pm, flo
 #undef VQC_PURE
 }
 
+// ---------------------------------------------------------------- factored stages
+// complex128 stages of runs: with every run as diag(p) rotation diag(q), a stage is one
+// diagonal over the block's 2^K amplitudes (the product of its runs' q), K real
+// rotations, one more diagonal (their p).  A rotation takes half the arithmetic of a
+// 2x2 update -- for double-float 4 two-term dot products a pair instead of 4 four-term
+// ones -- and complex128 is bound by its arithmetic (FP64, or the FP32 pipe in
+// double-float).  The diagonals are tabulated in shared memory, [stage][q, p][2^K].
+template <typename R, int K>
+__device__ __forceinline__ void build_diagonals(const FStage* stages, int nst, const uint2* ops, int op_base,
+                                                const R* sh_tab, const R* ps_tab, bool per_sample, int t, int T,
+                                                C2<R>* dg) {
+    for (int i = t; i < (nst << (K + 1)); i += T) {
+        const FStage* sp = stages + (i >> (K + 1));
+        const int which = (i >> K) & 1, r = i & ((1 << K) - 1);
+        if (!(sp->pure & (which ? kStageP : kStageQ)) || ((sp->pure & kStagePs) != 0) != per_sample) continue;
+        const uint2* op = ops + (sp->op_begin - op_base);
+        C2<R> f = cm<R>(1, 0);
+        for (int j = 0; j < K; ++j)
+            if ((sp->pmask >> j) & 1) {
+                const R* e = op_table<R>(*op++, sh_tab, ps_tab) + 8 + (which ? 2 : 6) + 2 * ((r >> j) & 1);
+                f = cmul<R>(f, cm<R>(e[0], e[1]));
+            }
+        dg[i] = f;
+    }
+}
+
+template <typename R, int K, bool ADJ>
+__device__ __forceinline__ void apply_diagonal(C2<R> (&a)[1 << K], const C2<R>* f) {
+#pragma unroll
+    for (int r = 0; r < (1 << K); ++r) a[r] = cmul<R>(a[r], ADJ ? cconj<R>(f[r]) : f[r]);
+}
+
+// [[C, -S], [S, C]] on local bit T (ADJ: its transpose).
+template <typename R, int K, int T, bool ADJ>
+__device__ __forceinline__ void rotate(C2<R> (&a)[1 << K], const R* e) {
+    const R C = e[0], S = ADJ ? -e[1] : e[1], M = -S;
+#pragma unroll
+    for (int p = 0; p < (1 << (K - 1)); ++p) {
+        const int i0 = pair_lo<T>(p), i1 = i0 | (1 << T);
+        const C2<R> u = a[i0], v = a[i1];
+        if constexpr (std::is_same<R, dd>::value) {
+            a[i0] = cm<R>(dot2(C, u.x, M, v.x), dot2(C, u.y, M, v.y));
+            a[i1] = cm<R>(dot2(S, u.x, C, v.x), dot2(S, u.y, C, v.y));
+        } else {
+            a[i0] = cm<R>(fma(C, u.x, M * v.x), fma(C, u.y, M * v.y));
+            a[i1] = cm<R>(fma(S, u.x, C * v.x), fma(S, u.y, C * v.y));
+        }
+    }
+}
+
+template <typename R, int K>
+__device__ __forceinline__ void factored_forward(const FStage* sp, const uint2* ops, C2<R> (&a)[1 << K],
+                                                 const R* sh_tab, const R* ps_tab, const C2<R>* dg) {
+    if (sp->pure & kStageQ) apply_diagonal<R, K, false>(a, dg);
+    const unsigned pm = sp->pmask;
+#define VQC_PURE(T_) \
+    if constexpr (T_ < K) if ((pm >> T_) & 1) rotate<R, K, T_, false>(a, op_table<R>(*ops++, sh_tab, ps_tab) + 8);
+    VQC_PURE(0) VQC_PURE(1) VQC_PURE(2) VQC_PURE(3) VQC_PURE(4)
+#undef VQC_PURE
+    if (sp->pure & kStageP) apply_diagonal<R, K, false>(a, dg + (1 << K));
+}
+
+// The adjoint, the runs' rho first as in pure_backward.
+template <typename R, int K>
+__device__ __forceinline__ void factored_backward(const FStage* sp, const uint2* ops, C2<R> (&a)[1 << K],
+                                                  C2<R> (&l)[1 << K], const R* sh_tab, const R* ps_tab,
+                                                  const C2<R>* dg, R* acc, int wg, int lane, int warp_in_group) {
+    const unsigned pm = sp->pmask;
+    unsigned am = 0;
+    {
+        const uint2* o = ops;
+#pragma unroll
+        for (int j = 0; j < K; ++j)
+            if ((pm >> j) & 1) {
+                if (((o->x) >> 24) & OPF_HAS_ACC) am |= 1u << j;
+                ++o;
+            }
+    }
+    if (am) {
+        R v[K][3];
+#pragma unroll
+        for (int j = 0; j < K; ++j) v[j][0] = v[j][1] = v[j][2] = 0;
+#define VQC_PURE(T_)                                     \
+        if constexpr (T_ < K)                            \
+            if ((am >> T_) & 1) {                        \
+                R t[4] = {0, 0, 0, 0};                   \
+                m1_t3<R, K, T_>(a, l, t);                \
+                v[T_][0] = t[0];                         \
+                v[T_][1] = t[1];                         \
+                v[T_][2] = t[2];                         \
+            }
+        VQC_PURE(0) VQC_PURE(1) VQC_PURE(2) VQC_PURE(3)
+#undef VQC_PURE
+        const int idx = reduce_runs<R, K>(v, lane);
+        const int j = idx >> 2;
+        if (idx >= 0 && ((am >> j) & 1)) {
+            const unsigned aux = ops[__popc(pm & ((1u << j) - 1u))].y >> 16;
+            acc[((size_t)aux * wg + warp_in_group) * 8 + (idx & 3)] = v[0][0];
+        }
+    }
+    if (sp->pure & kStageP) {
+        apply_diagonal<R, K, true>(a, dg + (1 << K));
+        apply_diagonal<R, K, true>(l, dg + (1 << K));
+    }
+#define VQC_PURE(T_)                                                             \
+    if constexpr (T_ < K)                                                        \
+        if ((pm >> T_) & 1) {                                                    \
+            const R* e = op_table<R>(*ops++, sh_tab, ps_tab) + 8;                \
+            rotate<R, K, T_, true>(a, e);                                        \
+            rotate<R, K, T_, true>(l, e);                                        \
+        }
+    VQC_PURE(0) VQC_PURE(1) VQC_PURE(2) VQC_PURE(3)
+#undef VQC_PURE
+    if (sp->pure & kStageQ) {
+        apply_diagonal<R, K, true>(a, dg);
+        apply_diagonal<R, K, true>(l, dg);
+    }
+}
+
 }  // namespace vqc

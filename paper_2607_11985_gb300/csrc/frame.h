@@ -52,8 +52,14 @@ struct FStage {
     int32_t sigma[kMaxK];
     int32_t op_begin, op_end;
     uint8_t nthreadbits, nsel;   // nsel: parities in pb (0: pb is not needed)
-    uint8_t pure;                // 1: the ops are 2x2 updates only, one per local position at most,
-    uint8_t pmask;               //    in the order of their positions; pmask: positions that have one
+    uint8_t pure;                // kStagePure: the ops are 2x2 updates only, at most one per local position,
+                                 // in the order of their positions; then also kStageQ, kStageP, kStagePs
+    uint8_t pmask;               // positions that have one
+};
+enum : uint8_t {
+    kStagePure = 1,
+    kStageQ = 2, kStageP = 4,    // some run needs its diagonal before / after the rotation (run_form)
+    kStagePs = 8                 // some run depends on the sample
 };
 static_assert(sizeof(FStage) == 160, "FStage layout");
 

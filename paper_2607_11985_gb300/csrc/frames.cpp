@@ -866,7 +866,15 @@ FrameSchedule FrameBuilder::build(int mode, int path, const std::vector<int>& ti
             if (pure) std::sort(recs.begin(), recs.end(), [](const DOp& a, const DOp& b) { return a.a < b.a; });
             S.ops.insert(S.ops.end(), recs.begin(), recs.end());
             st.op_end = (int32_t)S.ops.size();
-            st.pure = pure ? 1 : 0;
+            st.pure = pure ? kStagePure : 0;
+            for (const DOp& d : recs)
+                if (pure && (d.flags & OPF_PER_SAMPLE)) st.pure |= kStagePs;
+            if (pure)
+                for (int x : s.ops) {
+                    const DEntry& e = p.entries[p.ops[f[x].hop].entry];
+                    const int form = run_form(&p.consts[e.cfirst], e.ccount);
+                    st.pure |= (uint8_t)((form & 1 ? kStageQ : 0) | (form & 2 ? kStageP : 0));
+                }
             st.pmask = pure ? pm : 0;
             st.nsel = (uint8_t)outside.size();
             auto word = [&](uint32_t v) {

@@ -45,6 +45,7 @@ struct PArgs {
     int sm_sh, sm_ps, sm_lam, sm_acc, sm_red;
     int sm_plan;            // copies of the pass's stages, ops, flips and fin
     int sm_tfl;             // per tile: each stage's flip (uint2), then the logical parities
+    int sm_dg;              // complex128: the stages' diagonals (build_diagonals), per tile of the CTA
     int sm_tbase;           // each thread's block base in every stage: [nstages][threads]
     int sm_toff;            // tile-copy offsets of each thread: uint4
     int sm_koff;            // tile-copy offsets per vector round, read order then written order: uint2
@@ -187,10 +188,10 @@ __global__ void __launch_bounds__(256, 2) pass_kernel(const __grid_constant__ PA
     const int total_tiles = A.B << A.nout;   // (at most states in memory over 64 amplitudes)
     const uint32_t tmask = (1u << A.nout) - 1u;
     constexpr bool DDK = !std::is_same<St<R>, R>::value;   // double-float kernel
-    // straight-line stages: complex64 only (16-qubit workload 7.61 -> 7.24 ms); the
-    // double-float and FP64 updates are long enough to hide the dispatch, and the
-    // extra code costs them registers (double-float 9.87 -> 10.05 ms)
+    // stages of runs: complex64 as straight-line code (16-qubit workload 7.61 -> 7.24
+    // ms against the op switch), complex128 factored
     constexpr bool PURE = FULL && std::is_same<R, float>::value;
+    constexpr bool FACT = FULL && !std::is_same<R, float>::value;   // factored stages
     Geo q;
     q.T = 1 << A.tbits;
     q.lanes = q.T < 32 ? q.T : 32;
@@ -242,6 +243,8 @@ __global__ void __launch_bounds__(256, 2) pass_kernel(const __grid_constant__ PA
     const uint32_t g0 = (uint32_t)(q.g * tdim) ^ (uint32_t)q.h;
     R* ps_tab = ps_all + (size_t)q.g * A.ps_count * EntryWords<R>::value;
     R* acc = acc_all + (size_t)q.g * A.acc_count * q.wg * 8;
+    C2<R>* dg = reinterpret_cast<C2<R>*>(smem + A.sm_dg) + (((size_t)q.g * nst) << (K + 1));
+    if constexpr (FACT) build_diagonals<R, K>(stages, nst, ops, A.op_begin, sh_tab, ps_tab, false, q.t, q.T, dg);
     uint2* tfl_all = reinterpret_cast<uint2*>(smem + A.sm_tfl);
     const uint2* tfl = tfl_all + q.g * (nst + 1);
     // each thread's block base in every stage (read by itself only)
@@ -302,6 +305,11 @@ __global__ void __launch_bounds__(256, 2) pass_kernel(const __grid_constant__ PA
             if (MODE == 1 && A.src_lam) tile_prefetch<R>(A.src_lam + nsb, nga, koff_g, nk, q.t);
         }
         __syncthreads();
+        if constexpr (FACT)
+            if (A.ps_count) {
+                build_diagonals<R, K>(stages, nst, ops, A.op_begin, sh_tab, ps_tab, true, q.t, q.T, dg);
+                __syncthreads();
+            }
 
         C2<R> a[1 << K];
         uint32_t sb[K];
@@ -318,8 +326,11 @@ __global__ void __launch_bounds__(256, 2) pass_kernel(const __grid_constant__ PA
                 } else {
                     frame_load<R, K>(a, psi_t, v.off, sb);
                 }
-                if (PURE && sp->pure)
+                if (PURE && (sp->pure & kStagePure))
                     pure_forward<R, K>(ops + (sp->op_begin - A.op_begin), sp->pmask, a, sh_tab, ps_tab);
+                else if (FACT && (sp->pure & kStagePure))
+                    factored_forward<R, K>(sp, ops + (sp->op_begin - A.op_begin), a, sh_tab, ps_tab,
+                                           dg + ((size_t)s << (K + 1)));
                 else
                     run_ops<R, K, 0, false, FULL, PH2>(reinterpret_cast<const DOp*>(ops), sp->op_begin - A.op_begin,
                                                        sp->op_end - A.op_begin, v.pb, a, a, sh_tab, ps_tab, nullptr,
@@ -364,12 +375,16 @@ __global__ void __launch_bounds__(256, 2) pass_kernel(const __grid_constant__ PA
                 } else {
                     frame_load<R, K>(l, lam_t, v.off, sb);
                 }
-                bool pure = false;
+                const bool pure = (PURE || FACT) && (sp->pure & kStagePure);
                 if constexpr (PURE) {
-                    pure = sp->pure;
                     if (pure)
                         pure_backward<K>(ops + (sp->op_begin - A.op_begin), sp->pmask, a, l, sh_tab, ps_tab, acc,
                                          q.wg, lane, warp_in_group);
+                }
+                if constexpr (FACT) {
+                    if (pure)
+                        factored_backward<R, K>(sp, ops + (sp->op_begin - A.op_begin), a, l, sh_tab, ps_tab,
+                                                dg + ((size_t)s << (K + 1)), acc, q.wg, lane, warp_in_group);
                 }
                 if (!pure)
                     run_ops<R, K, 1, false, FULL, PH2>(reinterpret_cast<const DOp*>(ops), sp->op_begin - A.op_begin,

@@ -124,6 +124,34 @@ struct DEntry {
 };
 static_assert(sizeof(DEntry) == 12, "DEntry layout");
 
+// Reals of one table entry.  complex64: see EntryWords (sweep.cuh).  complex128: the
+// 2x2 matrix (or the phases) in the first 8, then the run's factors (Factored).
+constexpr int kEntryReals32 = 32, kEntryReals64 = 20;
+constexpr int entry_reals(bool dbl) { return dbl ? kEntryReals64 : kEntryReals32; }
+
+#ifdef __CUDACC__
+#define VQC_HD __host__ __device__
+#else
+#define VQC_HD
+#endif
+
+// A run as diag(p0, p1) [[C, -S], [S, C]] diag(q0, q1), the phases of modulus 1: which
+// of the two diagonals it needs (bit 0: q, bit 1: p).  Rotations about Z (and scalar
+// phases) before and after nothing but rotations about Y need only theirs.
+VQC_HD inline int run_form(const DConst* c, int count) {
+    int first = count, last = -1;
+    bool general = false;
+    for (int k = 0; k < count; ++k) {
+        if (c[k].kind == CK_RZ || c[k].kind == CK_GPHASE) continue;
+        if (first == count) first = k;
+        last = k;
+        general = general || c[k].kind != CK_RY;
+    }
+    if (last < 0) return 2;   // diagonal
+    for (int k = first; k < last; ++k) general = general || c[k].kind != CK_RY;
+    return general ? 3 : (first > 0 ? 1 : 0) | (last + 1 < count ? 2 : 0);
+}
+
 // One pass of the HBM-tiled path: its stages act on tiles of m qubits; the
 // other n - m qubits index the tiles of a sample.
 struct DPass {

@@ -29,6 +29,7 @@ __global__ void __launch_bounds__(512) sweep_kernel(const __grid_constant__ KArg
     R* red_all = reinterpret_cast<R*>(smem + A.sm_red);
 
     constexpr bool PURE = FULL && std::is_same<R, float>::value;   // straight-line stages (see pass_kernel)
+    constexpr bool FACT = FULL && !std::is_same<R, float>::value;  // factored stages
     const int n = A.n, G = A.G;
     const int dim = 1 << n;
     Geo q;
@@ -180,6 +181,14 @@ __global__ void __launch_bounds__(512) sweep_kernel(const __grid_constant__ KArg
                           ps_all + ((size_t)gg * A.n_ps + e.slot) * EntryWords<R>::value);
         }
         __syncthreads();
+        C2<R>* dg = reinterpret_cast<C2<R>*>(smem + A.sm_dg) + (((size_t)q.g * A.nstages) << (K + 1));
+        if constexpr (FACT) {
+            const uint2* ops = reinterpret_cast<const uint2*>(P.ops);
+            if (unit == (int)blockIdx.x)
+                build_diagonals<R, K>(stages, A.nstages, ops, 0, sh_tab, ps_tab, false, q.t, q.T, dg);
+            build_diagonals<R, K>(stages, A.nstages, ops, 0, sh_tab, ps_tab, true, q.t, q.T, dg);
+            __syncthreads();
+        }
 
         C2<R> a[1 << K];
         uint32_t sb[K];
@@ -201,9 +210,12 @@ __global__ void __launch_bounds__(512) sweep_kernel(const __grid_constant__ KArg
                 } else {
                     frame_load<R, K>(a, psi_t, v.off, sb);
                 }
-                if (PURE && sp->pure)
+                if (PURE && (sp->pure & kStagePure))
                     pure_forward<R, K>(reinterpret_cast<const uint2*>(P.ops) + sp->op_begin, sp->pmask, a, sh_tab,
                                        ps_tab);
+                else if (FACT && (sp->pure & kStagePure))
+                    factored_forward<R, K>(sp, reinterpret_cast<const uint2*>(P.ops) + sp->op_begin, a, sh_tab,
+                                           ps_tab, dg + ((size_t)s << (K + 1)));
                 else
                     run_ops<R, K, 0, false, FULL, PH2>(P.ops, sp->op_begin, sp->op_end, v.pb, a, a, sh_tab, ps_tab,
                                                        nullptr, q, lane, warp_in_group);
@@ -269,12 +281,17 @@ __global__ void __launch_bounds__(512) sweep_kernel(const __grid_constant__ KArg
                     lambda_frame<R, K>(fin->lmask, xor_bits(fin->tmask, A.tbits, q.t), xrow + A.Px, n, a, l);
                 else
                     frame_load<R, K>(l, lam_t, v.off, sb);
-                bool pure = false;
+                const bool pure = (PURE || FACT) && (sp->pure & kStagePure);
                 if constexpr (PURE) {
-                    pure = sp->pure;
                     if (pure)
                         pure_backward<K>(reinterpret_cast<const uint2*>(P.ops) + sp->op_begin, sp->pmask, a, l,
                                          sh_tab, ps_tab, acc, q.wg, lane, warp_in_group);
+                }
+                if constexpr (FACT) {
+                    if (pure)
+                        factored_backward<R, K>(sp, reinterpret_cast<const uint2*>(P.ops) + sp->op_begin, a, l,
+                                                sh_tab, ps_tab, dg + ((size_t)s << (K + 1)), acc, q.wg, lane,
+                                                warp_in_group);
                 }
                 if (!pure)
                     run_ops<R, K, 1, false, FULL, PH2>(P.ops, sp->op_begin, sp->op_end, v.pb, a, l, sh_tab, ps_tab,

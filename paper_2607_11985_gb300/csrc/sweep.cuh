@@ -73,7 +73,10 @@ __device__ __forceinline__ C2<R> cm(R x, R y) { C2<R> r; r.x = x; r.y = y; retur
 
 template <typename R>
 __device__ __forceinline__ C2<R> cmul(C2<R> a, C2<R> b) {
-    return cm<R>(fma(a.x, b.x, -a.y * b.y), fma(a.x, b.y, a.y * b.x));
+    if constexpr (std::is_same<R, dd>::value)
+        return cm<R>(dot2(a.x, b.x, -a.y, b.y), dot2(a.x, b.y, a.y, b.x));
+    else
+        return cm<R>(fma(a.x, b.x, -a.y * b.y), fma(a.x, b.y, a.y * b.x));
 }
 // m0 * u + m1 * v
 template <typename R>
@@ -260,7 +263,7 @@ struct KArgs {
     const FStage* fstages;
     const FFinal* fin;
     int32_t sin[kMaxTileBits], sout[kMaxTileBits];
-    int sm_io;
+    int sm_io, sm_dg;
     // cluster path only (cluster.cuh): log2 CTAs per sample, rank 0's <Z> gather area
     int cl, sm_ecl;
 };
@@ -286,9 +289,63 @@ struct PlanPtrs {
 // operand form of the packed-FP32 update (see m1_apply_f2w): U at [0, 16) and
 // U^dag at [16, 32), each as the pairs (m, i m) = (Re m, Im m), (-Im m, Re m) of
 // its four entries m.
-// complex128 stores U once (8 reals).  Phase entries use the first 8 reals.
-template <typename R> struct EntryWords { static constexpr int value = sizeof(R) == 4 ? 32 : 8; };
+// complex128 stores U (8 reals) and its factors (Factored).  Phase entries use the
+// first 8 reals.
+template <typename R> struct EntryWords { static constexpr int value = entry_reals(sizeof(R) == 8); };
 
+// A complex128 run's factors at offset 8 of its entry: C, S, then p0, p1, q0, q1 with
+// U = diag(p0, p1) [[C, -S], [S, C]] diag(q0, q1).  Stages of runs apply the real
+// rotations one by one and the diagonals of all of them at once (frame.cuh).  Each
+// phase comes from the larger of two entries, so a vanishing one costs no accuracy.
+// double-float entries are factored in double.
+template <typename R>
+__device__ __forceinline__ void store_factors(const M2<R>& m, int form, R* o) {
+    if constexpr (sizeof(R) == 8) {
+        auto d2 = [](C2<R> v) { const SC2<R> w = c2_out<R>(v); return make_double2(w.x, w.y); };
+        auto scale = [](double2 v, double f) { return make_double2(v.x * f, v.y * f); };
+        auto mulc = [](double2 x, double2 y) {   // x conj(y)
+            return make_double2(fma(x.x, y.x, x.y * y.y), fma(x.y, y.x, -x.x * y.y));
+        };
+        const double2 a = d2(m.a), b = d2(m.b), c = d2(m.c), d = d2(m.d), one = make_double2(1, 0);
+        double2 p0 = one, p1 = one, q0 = one, q1 = one;
+        double C = a.x, S = c.x;
+        if (form != 0) {
+            const double na = sqrt(fma(a.x, a.x, a.y * a.y)), nc = sqrt(fma(c.x, c.x, c.y * c.y));
+            const bool big = na >= nc;
+            C = na;
+            S = nc;
+            if (form == 3) {   // q0 = 1
+                p0 = na > 0 || !(nc > 0) ? scale(a, 1 / na) : one;
+                p1 = nc > 0 || !(na > 0) ? scale(c, 1 / nc) : one;
+                q1 = big ? scale(mulc(d, p1), 1 / na) : scale(mulc(b, p0), -1 / nc);
+            } else if (form == 2) {
+                if (big) {
+                    p0 = scale(a, 1 / na);
+                    p1 = scale(d, 1 / na);
+                    S = mulc(c, p1).x;
+                } else {
+                    p1 = scale(c, 1 / nc);
+                    p0 = scale(b, -1 / nc);
+                    C = mulc(a, p0).x;
+                }
+            } else {
+                if (big) {
+                    q0 = scale(a, 1 / na);
+                    q1 = scale(d, 1 / na);
+                    S = mulc(c, q0).x;
+                } else {
+                    q0 = scale(c, 1 / nc);
+                    q1 = scale(b, -1 / nc);
+                    C = mulc(a, q0).x;
+                }
+            }
+        }
+        o[0] = R(C); o[1] = R(S);
+        o[2] = R(p0.x); o[3] = R(p0.y); o[4] = R(p1.x); o[5] = R(p1.y);
+        o[6] = R(q0.x); o[7] = R(q0.y); o[8] = R(q1.x); o[9] = R(q1.y);
+        o[10] = R(0); o[11] = R(0);
+    }
+}
 
 template <typename R>
 __device__ __forceinline__ void store_matrix(const M2<R>& m, R* out) {
@@ -363,6 +420,7 @@ __device__ __forceinline__ void eval_entry(const DEntry& e, const DConst* consts
         m = mmul<R>(constituent<R>(c, xb, w, cang, cmat), m);
     }
     store_matrix<R>(m, out);
+    store_factors<R>(m, run_form(consts + e.cfirst, e.ccount), out + 8);
 }
 
 template <typename R>
@@ -401,6 +459,21 @@ __device__ __forceinline__ void m1_apply(C2<R> (&a)[1 << K], const M2<R>& m) {
 template <typename R, int K, int T>
 __device__ __forceinline__ void m1_t3(const C2<R> (&ps)[1 << K], const C2<R> (&la)[1 << K],
                                       R (&v)[4]) {
+    if constexpr (std::is_same<R, dd>::value) {   // each component one long compensated dot product
+        ddsum sx, sy, sz;
+#pragma unroll
+        for (int p = 0; p < (1 << (K - 1)); ++p) {
+            const int i0 = pair_lo<T>(p), i1 = i0 | (1 << T);
+            const dd2 u = ps[i0], w = ps[i1], q0 = la[i0], q1 = la[i1];
+            sx.add(u.y, q1.x); sx.add(-u.x, q1.y); sx.add(w.y, q0.x); sx.add(-w.x, q0.y);
+            sy.add(u.x, q1.x); sy.add(u.y, q1.y); sy.add(-w.x, q0.x); sy.add(-w.y, q0.y);
+            sz.add(u.y, q0.x); sz.add(-u.x, q0.y); sz.add(-w.y, q1.x); sz.add(w.x, q1.y);
+        }
+        v[0] += sx.value();
+        v[1] += sy.value();
+        v[2] += sz.value();
+        return;
+    }
     R xa = 0, ya = 0, za = 0;
 #pragma unroll
     for (int p = 0; p < (1 << (K - 1)); ++p) {

@@ -164,7 +164,8 @@ class Emulator:
         ops = self.s["ops"][st["op_begin"]:st["op_end"]]
         runs = [pe.op_type(o)[0] == pe.OP_M1 for o in ops]
         pos = [int(o["a"]) for o in ops]
-        if st["pure"]:
+        if st["pure"] & 1:
+            assert bool(st["pure"] & 8) == any(int(o["flags"]) & pe.OPF_PER_SAMPLE for o in ops)
             assert all(runs) and pos == sorted(set(pos)) and st["pmask"] == sum(1 << q for q in pos)
 
     def logical(self, tau):
