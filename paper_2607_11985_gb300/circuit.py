@@ -22,6 +22,17 @@ def _ptr(t):
     return None if t is None else t.data_ptr()
 
 
+def _here():
+    """(current device index, its current stream's address)."""
+    dev = torch.cuda.current_device()
+    return dev, _raw_stream(dev)
+
+
+# the current stream's address without building a Stream object (about 3 us a call)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or \
+    (lambda dev: torch.cuda.current_stream(dev).cuda_stream)
+
+
 class Circuit:
     """A compiled static circuit (see ``workloads.CircuitSpec`` for the format)."""
 
@@ -74,21 +85,27 @@ class Circuit:
     def _check(self, t, dtype, shape, name):
         if t is None:
             return None
-        if not t.is_cuda or t.dtype != dtype or tuple(t.shape) != tuple(shape):
+        if t.dtype is not dtype or t.shape != shape or not t.is_cuda:
             raise ValueError("%s must be a CUDA %s tensor of shape %s (got %s %s %s)"
                              % (name, dtype, tuple(shape), t.device, t.dtype, tuple(t.shape)))
-        return t.contiguous()
+        return t if t.is_contiguous() else t.contiguous()
 
     def workspace(self, batch: int, mode: int, stream=None):
-        nbytes = B.vqc_workspace_bytes(self.plan, batch, mode)
+        if stream is None:
+            dev, sp = _here()
+        else:
+            dev, sp = torch.cuda.current_device(), stream.cuda_stream
+        return self._workspace(batch, mode, dev, sp)
+
+    def _workspace(self, batch, mode, dev, sp):
+        nbytes = B.lib().vqc_workspace_bytes(self.plan, batch, mode)
         if nbytes == 0:
             return None, 0
-        stream = stream or torch.cuda.current_stream()
-        key = (mode, stream.cuda_stream, torch.cuda.current_device())
+        key = (mode, sp, dev)
         buf = self._ws.get(key)
         if buf is None or buf.numel() < nbytes:
             buf = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
-            B.vqc_workspace_init(buf.data_ptr(), nbytes, stream.cuda_stream)
+            B.vqc_workspace_init(buf.data_ptr(), nbytes, sp)
             self._ws[key] = buf
         return buf, buf.numel()
 
@@ -103,10 +120,10 @@ class Circuit:
         st = state_out
         if want_state and st is None:
             st = torch.empty(batch, 1 << self.n, dtype=self.cplx, device="cuda")
-        stream = torch.cuda.current_stream()
-        ws, wsb = self.workspace(batch, 0, stream)
+        dev, sp = _here()
+        ws, wsb = self._workspace(batch, 0, dev, sp)
         B.vqc_forward(self.plan, batch, _ptr(x), _ptr(w), _ptr(psi0), _ptr(E), _ptr(st),
-                      _ptr(ws), wsb, stream.cuda_stream)
+                      _ptr(ws), wsb, sp)
         return (E, st) if want_state else E
 
     def probabilities(self, x, w, psi0=None, out=None):
@@ -116,10 +133,10 @@ class Circuit:
         w = self._check(w, self.real, (self.num_w,), "w") if self.num_w else None
         psi0 = self._check(psi0, self.cplx, (batch, 1 << self.n), "psi0")
         P = out if out is not None else torch.empty(batch, 1 << self.n, dtype=self.real, device="cuda")
-        stream = torch.cuda.current_stream()
-        ws, wsb = self.workspace(batch, 2, stream)
+        dev, sp = _here()
+        ws, wsb = self._workspace(batch, 2, dev, sp)
         B.vqc_probabilities(self.plan, batch, _ptr(x), _ptr(w), _ptr(psi0), _ptr(P), _ptr(ws), wsb,
-                            stream.cuda_stream)
+                            sp)
         return P
 
     def backward(self, x, w, grad_expz, psi0=None, psi_final=None, need_x=True, need_w=True,
@@ -137,10 +154,10 @@ class Circuit:
         dw = grad_w
         if dw is None and need_w and self.num_w:
             dw = torch.empty(self.num_w, dtype=self.real, device="cuda")
-        stream = torch.cuda.current_stream()
-        ws, wsb = self.workspace(batch, 1, stream)
+        dev, sp = _here()
+        ws, wsb = self._workspace(batch, 1, dev, sp)
         B.vqc_backward(self.plan, batch, _ptr(x), _ptr(w), _ptr(psi0), _ptr(psi_final),
-                       _ptr(gE), _ptr(dx), _ptr(dw), _ptr(ws), wsb, stream.cuda_stream)
+                       _ptr(gE), _ptr(dx), _ptr(dw), _ptr(ws), wsb, sp)
         return dx, dw
 
     def forward_backward(self, x, w, grad_expz, psi0=None, out=None):
@@ -158,10 +175,10 @@ class Circuit:
             dw = torch.empty(self.num_w, dtype=self.real, device="cuda") if self.num_w else None
         else:
             E, dx, dw = out
-        stream = torch.cuda.current_stream()
-        ws, wsb = self.workspace(batch, 3, stream)
+        dev, sp = _here()
+        ws, wsb = self._workspace(batch, 3, dev, sp)
         B.vqc_forward_backward(self.plan, batch, _ptr(x), _ptr(w), _ptr(psi0), _ptr(gE), _ptr(E),
-                               _ptr(dx), _ptr(dw), _ptr(ws), wsb, stream.cuda_stream)
+                               _ptr(dx), _ptr(dw), _ptr(ws), wsb, sp)
         return E, dx, dw
 
     def evaluate_host(self, x, w, grad_expz=None, out=None, stream=None):
@@ -263,8 +280,7 @@ class VQCFunction(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, x, w, circuit, psi0=None):
-        E, st = circuit.forward(x.detach() if x is not None else None,
-                                w.detach() if w is not None else None, psi0=psi0, want_state=True)
+        E, st = circuit.forward(x, w, psi0=psi0, want_state=True)
         ctx.circuit = circuit
         ctx.save_for_backward(x, w, psi0, st)
         return E

@@ -135,15 +135,49 @@ int env_int(const char* name, int dflt) {
     return v && *v ? std::atoi(v) : dflt;
 }
 
+int cta_threads() {
+    const int t = env_int("VQC_CTA_THREADS", 128);
+    return t >= 32 && t <= 512 ? t : 128;
+}
+
+// The environment switches, read once per call from outside (a call asks for some of
+// them dozens of times, and each getenv walks the environment).
+struct Env {
+    int k_fwd = 0, k_bwd = 0, cta = 128;
+    bool plan_smem = true, force = false, hbm = false, cluster = false;
+};
+thread_local Env t_env;
+thread_local int t_env_depth = 0;
+struct EnvScope {
+    EnvScope() {
+        if (t_env_depth++) return;
+        Env e;
+        e.k_fwd = env_int("VQC_FORCE_K_FWD", 0);
+        e.k_bwd = env_int("VQC_FORCE_K_BWD", 0);
+        e.cta = cta_threads();
+        e.plan_smem = env_int("VQC_PLAN_IN_SMEM", 1) != 0;
+        if (const char* f = std::getenv("VQC_FORCE_PATH")) {
+            e.force = true;
+            e.hbm = !std::strcmp(f, "hbm");
+            e.cluster = !std::strcmp(f, "cluster");
+        }
+        t_env = e;
+    }
+    ~EnvScope() { --t_env_depth; }
+};
+
 // Launch with programmatic stream serialisation: the kernel may be scheduled
 // while the previous kernel in the stream finishes, and waits for it (every
 // kernel calls grid_dep_wait() before touching caller memory), which hides most
 // of the launch gap between the back-to-back kernels of one call and between
 // consecutive calls.  VQC_PDL=0 turns it off (plain stream order).
+bool use_pdl() {
+    static const bool pdl = env_int("VQC_PDL", 1) != 0;
+    return pdl;
+}
 cudaError_t launch(const void* fn, dim3 grid, dim3 block, void** args, size_t smem,
                    cudaStream_t stream) {
-    static const bool pdl = env_int("VQC_PDL", 1) != 0;
-    if (!pdl) return cudaLaunchKernel(fn, grid, block, args, smem, stream);
+    if (!use_pdl()) return cudaLaunchKernel(fn, grid, block, args, smem, stream);
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -157,11 +191,6 @@ cudaError_t launch(const void* fn, dim3 grid, dim3 block, void** args, size_t sm
     return cudaLaunchKernelExC(&cfg, fn, args);
 }
 
-int cta_threads() {
-    const int t = env_int("VQC_CTA_THREADS", 128);
-    return t >= 32 && t <= 512 ? t : 128;
-}
-
 // Pick the register-block size: the largest K that still gives the batch
 // enough threads to cover every SM's schedulers (SMs x 4 warps), but not below
 // 3 (a block of 8 amplitudes) where the circuit allows it.  A forced-K sweep on
@@ -170,7 +199,7 @@ int cta_threads() {
 // blocks add stages (shared-memory round trips and barriers) faster than the
 // extra warps hide latency.
 int choose_k(const HostPlan& p, int mode, int B, int sms) {
-    int forced = env_int(mode == 0 ? "VQC_FORCE_K_FWD" : "VQC_FORCE_K_BWD", 0);
+    const int forced = mode == 0 ? t_env.k_fwd : t_env.k_bwd;
     if (forced > 0 && find_frame(p, mode, VQC_PATH_RESIDENT, forced)) return forced;
     int kmax = 0;
     for (const auto& s : p.frames)
@@ -213,7 +242,7 @@ vqc_status plan_launch_uncached(const HostPlan& p, int launch_mode, int B, Launc
                               (mode == 1 ? p.accs.size() * L.wg * 8 * rs + p.term_src.size() * rs : 0) +
                               (size_t)L.wg * p.n * rs;
     // samples per CTA: groups up to VQC_CTA_THREADS (default 128) threads
-    int S = std::max(1, cta_threads() / L.T);
+    int S = std::max(1, t_env.cta / L.T);
     if ((size_t)di.smem_optin > fixed) {
         size_t fit = ((size_t)di.smem_optin - fixed) / per_sample;
         S = (int)std::min<size_t>((size_t)S, fit);
@@ -252,7 +281,7 @@ vqc_status plan_launch_uncached(const HostPlan& p, int launch_mode, int B, Launc
     // the plan's table data and this schedule go to shared memory when they fit
     const size_t plan_bytes = align16(p.dev_tab_end - p.dev_tab_begin) +
                               (L.f->dev_region_end - L.f->dev_region_begin);
-    L.plan_smem = off + plan_bytes <= (size_t)di.smem_optin && env_int("VQC_PLAN_IN_SMEM", 1) != 0;
+    L.plan_smem = off + plan_bytes <= (size_t)di.smem_optin && t_env.plan_smem;
     L.sm_plan = L.plan_smem ? take(plan_bytes) : 0;
     L.smem = off;
     if (L.smem > (size_t)di.smem_optin)
@@ -277,8 +306,7 @@ GeoKey geo_key(const HostPlan& p, int mode, int B, int hbm) {
     int dev = -1;
     cudaGetDevice(&dev);
     // environment switches that change the geometry are part of the key
-    const int env = env_int("VQC_FORCE_K_FWD", 0) * 1000 + env_int("VQC_FORCE_K_BWD", 0) * 10 +
-                    (env_int("VQC_PLAN_IN_SMEM", 1) != 0 ? 1 : 0) + cta_threads() * 1000000;
+    const int env = t_env.k_fwd * 1000 + t_env.k_bwd * 10 + (t_env.plan_smem ? 1 : 0) + t_env.cta * 1000000;
     return GeoKey{&p, mode, B, dev, hbm * 100000 + env};
 }
 
@@ -555,7 +583,7 @@ vqc_status plan_cluster(const HostPlan& p, int mode, int B, Launch& L) {
     }
     const size_t plan_bytes = align16(p.dev_tab_end - p.dev_tab_begin) +
                               (L.s->dev_region_end - L.s->dev_region_begin);
-    L.plan_smem = off + plan_bytes <= (size_t)di.smem_optin && env_int("VQC_PLAN_IN_SMEM", 1) != 0;
+    L.plan_smem = off + plan_bytes <= (size_t)di.smem_optin && t_env.plan_smem;
     L.sm_plan = L.plan_smem ? take(plan_bytes) : 0;
     L.smem = off;
     if (L.smem > (size_t)di.smem_optin)
@@ -610,9 +638,8 @@ bool cluster_fits(const HostPlan& p, int mode) {
 bool use_cluster(const HostPlan& p, int mode, int B) {
     const Schedule* s = find_cluster_schedule(p, mode);
     if (!s) return false;
-    const char* f = std::getenv("VQC_FORCE_PATH");
-    if (f && std::string(f) == "cluster") return cluster_fits(p, mode);
-    if (f && std::string(f) == "hbm") return false;
+    if (t_env.cluster) return cluster_fits(p, mode);
+    if (t_env.hbm) return false;
     if (p.n - s->K - s->cta_bits != 1) return false;
     if (!(p.dfloat && mode == 1) && find_frame(p, mode, VQC_PATH_HBM)) {
         int dev = 0, sms = 152;   // without a device: GB300's SM count
@@ -654,7 +681,7 @@ vqc_status run_cluster_forward(const HostPlan& p, int B, const void* x, const vo
     cfg.dynamicSmemBytes = L.smem;
     cfg.stream = stream;
     cfg.attrs = attr;
-    cfg.numAttrs = env_int("VQC_PDL", 1) != 0 ? 2 : 1;
+    cfg.numAttrs = use_pdl() ? 2 : 1;
     VQC_CUDA(cudaLaunchKernelExC(&cfg, L.fn, args));
     return VQC_OK;
 }
@@ -705,7 +732,7 @@ vqc_status run_cluster_backward(const HostPlan& p, int B, const void* x, const v
     cfg.dynamicSmemBytes = L.smem;
     cfg.stream = stream;
     cfg.attrs = attr;
-    cfg.numAttrs = env_int("VQC_PDL", 1) != 0 ? 2 : 1;
+    cfg.numAttrs = use_pdl() ? 2 : 1;
     VQC_CUDA(cudaLaunchKernelExC(&cfg, L.fn, args));
     if (dw && p.num_w > 0) {
         const R* part = a.dw_part;
@@ -1096,8 +1123,7 @@ vqc_status run_hbm_backward(const HostPlan& p, int B, const void* x, const void*
 // The resident path when it can take the batch (and VQC_FORCE_PATH does not
 // ask for the HBM path), else the HBM path.
 bool use_hbm(const HostPlan& p, int mode, int B) {
-    const char* f = std::getenv("VQC_FORCE_PATH");
-    if (f && std::string(f) == "hbm" && find_frame(p, mode, VQC_PATH_HBM)) return true;
+    if (t_env.hbm && find_frame(p, mode, VQC_PATH_HBM)) return true;
     Launch L;
     std::string saved = g_err;
     if (plan_launch(p, mode, B, L) == VQC_OK) return false;
@@ -1190,6 +1216,7 @@ vqc_status backward_with_scratch(const vqc_plan* plan, int32_t batch, const void
                                  const void* w, const void* psi0, const void* psi_final,
                                  const void* grad_expz, void* grad_x, void* grad_w, void* scratch,
                                  size_t scratch_bytes, void* stream, bool clear_control) {
+    const EnvScope env;
     vqc_status st = check_common(plan, batch);
     if (st != VQC_OK) return st;
     const HostPlan& p = plan->hp;
@@ -1209,7 +1236,7 @@ vqc_status backward_with_scratch(const vqc_plan* plan, int32_t batch, const void
     // else the HBM-tiled passes (each with its own workspace layout)
     bool clu = use_cluster(p, 1, batch);
     bool hbm = !clu && use_hbm(p, 1, batch);
-    if (hbm && !std::getenv("VQC_FORCE_PATH")) {   // states that do not fit the scratch may fit a cluster
+    if (hbm && !t_env.force) {   // states that do not fit the scratch may fit a cluster
         const Schedule* s = find_cluster_schedule(p, 1);
         PassGeo L;
         st = plan_hbm(p, 1, batch, L);
@@ -1330,6 +1357,7 @@ void vqc_free(vqc_plan* plan) {
 
 size_t vqc_workspace_bytes(const vqc_plan* plan, int32_t batch, int32_t mode) {
     if (!plan) return (size_t)-1;
+    const EnvScope env;
     if (mode == 3) {   // vqc_forward_backward: its one-launch form, or either call's workspace
         size_t need = std::max(vqc_workspace_bytes(plan, batch, 0), vqc_workspace_bytes(plan, batch, 1));
         const HostPlan& p = plan->hp;
@@ -1383,6 +1411,7 @@ vqc_status vqc_probabilities(const vqc_plan* plan, int32_t batch, const void* x,
                              const void* psi0, void* probs_out, void* workspace,
                              size_t workspace_bytes, void* stream) {
     try {
+        const EnvScope env;
         vqc_status st = check_common(plan, batch);
         if (st != VQC_OK) return st;
         if (batch == 0) return VQC_OK;
@@ -1425,6 +1454,7 @@ vqc_status vqc_forward(const vqc_plan* plan, int32_t batch, const void* x, const
                        const void* psi0, void* expz_out, void* state_out, void* workspace,
                        size_t workspace_bytes, void* stream) {
     try {
+        const EnvScope env;
         vqc_status st = check_common(plan, batch);
         if (st != VQC_OK) return st;
         if (batch == 0) return VQC_OK;
@@ -1462,6 +1492,7 @@ vqc_status vqc_backward(const vqc_plan* plan, int32_t batch, const void* x, cons
                         void* grad_x, void* grad_w, void* workspace, size_t workspace_bytes,
                         void* stream) {
     try {
+        const EnvScope env;
         vqc_status st = check_common(plan, batch);
         if (st != VQC_OK) return st;
         const HostPlan& p = plan->hp;
@@ -1504,6 +1535,7 @@ vqc_status vqc_forward_backward(const vqc_plan* plan, int32_t batch, const void*
                                 const void* psi0, const void* grad_expz, void* expz_out, void* grad_x,
                                 void* grad_w, void* workspace, size_t workspace_bytes, void* stream) {
     try {
+        const EnvScope env;
         vqc_status st = check_common(plan, batch);
         if (st != VQC_OK) return st;
         const HostPlan& p = plan->hp;
@@ -1589,6 +1621,7 @@ vqc_status vqc_forward_backward(const vqc_plan* plan, int32_t batch, const void*
 }
 
 vqc_status vqc_plan_info(const vqc_plan* plan, int32_t batch, vqc_plan_stats* out) {
+    const EnvScope env;
     if (!plan || !out) return fail(VQC_ERR_INVALID_ARG, "NULL argument");
     const HostPlan& p = plan->hp;
     std::memset(out, 0, sizeof(*out));
