@@ -232,11 +232,11 @@ vqc_status plan_launch_uncached(const HostPlan& p, int launch_mode, int B, Launc
     L.wg = L.T > 32 ? L.T / 32 : 1;
     // Shared memory: a fixed part per CTA and a part per resident sample.
     const size_t dim = (size_t)1 << p.n;
-    const size_t ew = entry_reals(dbl);
+    const size_t ew = entry_reals(dbl, p.dfloat);
     const size_t io = (size_t)8 << L.K;   // slot offsets of the state copies
     const size_t fixed = align16((size_t)p.n_sh * ew * rs) + align16(mode == 1 ? (size_t)p.num_w * rs : 0) +
                          align16((size_t)p.num_w * rs) + io + 10 * 16;
-    const size_t dgb = dbl && L.T >= 32 ? (L.f->stages.size() << (L.K + 1)) * cs : 0;   // stage diagonals
+    const size_t dgb = p.dfloat && L.T >= 32 ? (L.f->stages.size() << (L.K + 1)) * cs : 0;   // stage diagonals
     const size_t per_sample = dgb + (size_t)p.n_ps * ew * rs + dim * cs * (mode == 1 ? 2 : 1) +
                               (size_t)(p.num_x + p.n) * rs +
                               (mode == 1 ? p.accs.size() * L.wg * 8 * rs + p.term_src.size() * rs : 0) +
@@ -551,7 +551,7 @@ vqc_status plan_cluster(const HostPlan& p, int mode, int B, Launch& L) {
     vqc_status st = device_info(dev, di);
     if (st != VQC_OK) return st;
     const bool dbl = p.dtype == VQC_C128;
-    const size_t rs = dbl ? 8 : 4, cs = 2 * rs, ew = entry_reals(dbl);
+    const size_t rs = dbl ? 8 : 4, cs = 2 * rs, ew = entry_reals(dbl, p.dfloat);
     L.K = L.s->K;
     L.cl = p.n - L.K - L.s->cta_bits;
     L.T = 1 << (p.n - L.K);           // threads of a sample group, over the whole cluster
@@ -778,12 +778,12 @@ vqc_status plan_hbm_uncached(const HostPlan& p, int mode, int B, PassGeo& L) {
         ops_max = std::max(ops_max, ps.op_end - ps.op_begin);
     }
     const size_t tdim = (size_t)1 << m;
-    const size_t ew = entry_reals(dbl);
+    const size_t ew = entry_reals(dbl, p.dfloat);
     const size_t apv = 16 / cs, nk = (tdim / apv + L.T - 1) / L.T;
     const size_t prog = (size_t)nst_max * sizeof(FStage) + sizeof(FFinal) + (size_t)ops_max * sizeof(DOp) +
                         (size_t)nst_max * L.s->nout * sizeof(FFlip);
     const size_t fixed = align16((size_t)sh_max * ew * rs) + align16(prog) + align16(2 * nk * 8) + 8 * 16;
-    const size_t dgb = dbl && L.T >= 32 ? ((size_t)nst_max << (L.K + 1)) * cs : 0;   // stage diagonals
+    const size_t dgb = p.dfloat && L.T >= 32 ? ((size_t)nst_max << (L.K + 1)) * cs : 0;   // stage diagonals
     const size_t per_tile = dgb + (size_t)ps_max * ew * rs + tdim * cs * (mode == 1 ? 2 : 1) + (size_t)(nst_max + 1) * 8 +
                             (size_t)L.T * (16 + 4 * nst_max) + (mode == 1 ? (size_t)acc_max * L.wg * 8 * rs : (size_t)L.wg * p.n * rs);
     int S = std::max(1, 128 / L.T);
@@ -874,7 +874,7 @@ size_t hbm_state_bytes(const HostPlan& p, int B) {
 HbmWs hbm_layout(const HostPlan& p, int mode, int B, int ntiles) {
     const size_t rs = p.dtype == VQC_C128 ? 8 : 4;
     const size_t sbytes = hbm_state_bytes(p, B);
-    const size_t entry = entry_reals(p.dtype == VQC_C128) * rs;
+    const size_t entry = entry_reals(p.dtype == VQC_C128, p.dfloat) * rs;
     HbmWs w;
     w.state = 256;
     if (mode == 0) {

@@ -588,7 +588,7 @@ bool hbm_shape(const HostPlan& p, int mode, int& m, int& K) {
 // room to spare (the launch code's own layout decides): all sizes a launch may choose.
 bool resident_fits(const HostPlan& p) {
     if (p.n > resident_max_qubits(1, p.dtype)) return false;
-    const size_t rs = p.dtype == VQC_C128 ? 8 : 4, ew = entry_reals(p.dtype == VQC_C128);
+    const size_t rs = p.dtype == VQC_C128 ? 8 : 4, ew = entry_reals(p.dtype == VQC_C128, p.dtype == VQC_C128);
     const size_t wg = std::max(1, std::min(512, 1 << std::max(0, p.n - 3)) / 32);
     const size_t need = (size_t)(p.n_sh + p.n_ps) * ew * rs + 2 * (size_t)p.num_w * rs +
                         ((size_t)4 << p.n) * rs + (size_t)(p.num_x + p.n) * rs + p.accs.size() * wg * 8 * rs +

@@ -297,12 +297,12 @@ __device__ __forceinline__ void pure_backward(const uint2* ops, unsigned pm, flo
 }
 
 // ---------------------------------------------------------------- factored stages
-// complex128 stages of runs: with every run as diag(p) rotation diag(q), a stage is one
-// diagonal over the block's 2^K amplitudes (the product of its runs' q), K real
-// rotations, one more diagonal (their p).  A rotation takes half the arithmetic of a
-// 2x2 update -- for double-float 4 two-term dot products a pair instead of 4 four-term
-// ones -- and complex128 is bound by its arithmetic (FP64, or the FP32 pipe in
-// double-float).  The diagonals are tabulated in shared memory, [stage][q, p][2^K].
+// double-float stages of runs: with every run as diag(p) rotation diag(q), a stage is
+// one diagonal over the block's 2^K amplitudes (the product of its runs' q), K real
+// rotations, one more diagonal (their p).  A rotation is 4 two-term dot products a
+// pair (76 operations) where a 2x2 update is 4 four-term ones (172), and double-float
+// is bound by the FP32 pipe: 16 qubits x 77 step 9.64 -> 7.82 ms (with the running rho
+// sums of ddsum).  The diagonals are tabulated in shared memory, [stage][q, p][2^K].
 template <typename R, int K>
 __device__ __forceinline__ void build_diagonals(const FStage* stages, int nst, const uint2* ops, int op_base,
                                                 const R* sh_tab, const R* ps_tab, bool per_sample, int t, int T,
@@ -312,13 +312,14 @@ __device__ __forceinline__ void build_diagonals(const FStage* stages, int nst, c
         const int which = (i >> K) & 1, r = i & ((1 << K) - 1);
         if (!(sp->pure & (which ? kStageP : kStageQ)) || ((sp->pure & kStagePs) != 0) != per_sample) continue;
         const uint2* op = ops + (sp->op_begin - op_base);
-        C2<R> f = cm<R>(1, 0);
+        double2 f = make_double2(1, 0);
         for (int j = 0; j < K; ++j)
             if ((sp->pmask >> j) & 1) {
-                const R* e = op_table<R>(*op++, sh_tab, ps_tab) + 8 + (which ? 2 : 6) + 2 * ((r >> j) & 1);
-                f = cmul<R>(f, cm<R>(e[0], e[1]));
+                const R* e = op_table<R>(*op++, sh_tab, ps_tab) + 10;
+                const double2 ph = reinterpret_cast<const double2*>(e)[(which ? 0 : 2) + ((r >> j) & 1)];
+                f = make_double2(fma(f.x, ph.x, -f.y * ph.y), fma(f.x, ph.y, f.y * ph.x));
             }
-        dg[i] = f;
+        dg[i] = cm<R>(R(f.x), R(f.y));
     }
 }
 

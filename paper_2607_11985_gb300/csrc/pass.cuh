@@ -45,7 +45,7 @@ struct PArgs {
     int sm_sh, sm_ps, sm_lam, sm_acc, sm_red;
     int sm_plan;            // copies of the pass's stages, ops, flips and fin
     int sm_tfl;             // per tile: each stage's flip (uint2), then the logical parities
-    int sm_dg;              // complex128: the stages' diagonals (build_diagonals), per tile of the CTA
+    int sm_dg;              // double-float: the stages' diagonals (build_diagonals), per tile of the CTA
     int sm_tbase;           // each thread's block base in every stage: [nstages][threads]
     int sm_toff;            // tile-copy offsets of each thread: uint4
     int sm_koff;            // tile-copy offsets per vector round, read order then written order: uint2
@@ -189,9 +189,9 @@ __global__ void __launch_bounds__(256, 2) pass_kernel(const __grid_constant__ PA
     const uint32_t tmask = (1u << A.nout) - 1u;
     constexpr bool DDK = !std::is_same<St<R>, R>::value;   // double-float kernel
     // stages of runs: complex64 as straight-line code (16-qubit workload 7.61 -> 7.24
-    // ms against the op switch), complex128 factored
+    // ms against the op switch), double-float factored
     constexpr bool PURE = FULL && std::is_same<R, float>::value;
-    constexpr bool FACT = FULL && !std::is_same<R, float>::value;   // factored stages
+    constexpr bool FACT = FULL && std::is_same<R, dd>::value;   // factored stages
     Geo q;
     q.T = 1 << A.tbits;
     q.lanes = q.T < 32 ? q.T : 32;

@@ -125,9 +125,8 @@ struct DEntry {
 static_assert(sizeof(DEntry) == 12, "DEntry layout");
 
 // Reals of one table entry.  complex64: see EntryWords (sweep.cuh).  complex128: the
-// 2x2 matrix (or the phases) in the first 8, then the run's factors (Factored).
-constexpr int kEntryReals32 = 32, kEntryReals64 = 20;
-constexpr int entry_reals(bool dbl) { return dbl ? kEntryReals64 : kEntryReals32; }
+// 2x2 matrix or the phases; double-float: then the run's factors (store_factors).
+constexpr int entry_reals(bool dbl, bool dfloat) { return dfloat ? 20 : dbl ? 8 : 32; }
 
 #ifdef __CUDACC__
 #define VQC_HD __host__ __device__

@@ -29,7 +29,7 @@ __global__ void __launch_bounds__(512) sweep_kernel(const __grid_constant__ KArg
     R* red_all = reinterpret_cast<R*>(smem + A.sm_red);
 
     constexpr bool PURE = FULL && std::is_same<R, float>::value;   // straight-line stages (see pass_kernel)
-    constexpr bool FACT = FULL && !std::is_same<R, float>::value;  // factored stages
+    constexpr bool FACT = FULL && std::is_same<R, dd>::value;  // factored stages
     const int n = A.n, G = A.G;
     const int dim = 1 << n;
     Geo q;

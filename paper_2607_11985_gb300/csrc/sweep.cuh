@@ -289,18 +289,23 @@ struct PlanPtrs {
 // operand form of the packed-FP32 update (see m1_apply_f2w): U at [0, 16) and
 // U^dag at [16, 32), each as the pairs (m, i m) = (Re m, Im m), (-Im m, Re m) of
 // its four entries m.
-// complex128 stores U (8 reals) and its factors (Factored).  Phase entries use the
-// first 8 reals.
-template <typename R> struct EntryWords { static constexpr int value = entry_reals(sizeof(R) == 8); };
+// complex128 stores U (8 reals), double-float also its factors (store_factors).  Phase
+// entries use the first 8 reals.
+template <typename R> struct EntryWords {
+    static constexpr int value = entry_reals(sizeof(R) == 8, std::is_same<R, dd>::value);
+};
 
-// A complex128 run's factors at offset 8 of its entry: C, S, then p0, p1, q0, q1 with
-// U = diag(p0, p1) [[C, -S], [S, C]] diag(q0, q1).  Stages of runs apply the real
-// rotations one by one and the diagonals of all of them at once (frame.cuh).  Each
-// phase comes from the larger of two entries, so a vanishing one costs no accuracy.
-// double-float entries are factored in double.
+// A double-float run's factors at offset 8 of its entry: C, S, then p0, p1, q0, q1 as
+// doubles, with U = diag(p0, p1) [[C, -S], [S, C]] diag(q0, q1).  Stages of runs apply
+// the real rotations one by one and the diagonals of all of them at once (frame.cuh).
+// Each phase comes from the larger of two entries, so a vanishing one costs no
+// accuracy; the phases stay doubles until the stage's products of them are split, so
+// that their roundings, the same for every amplitude, are not double-float's.
+// (Native complex128 keeps the 2x2 updates: factors rounded to double doubled its
+// gradients' error against 64 bits, 3.2e-15 -> 6.4e-15 at 16 qubits.)
 template <typename R>
 __device__ __forceinline__ void store_factors(const M2<R>& m, int form, R* o) {
-    if constexpr (sizeof(R) == 8) {
+    if constexpr (std::is_same<R, dd>::value) {
         auto d2 = [](C2<R> v) { const SC2<R> w = c2_out<R>(v); return make_double2(w.x, w.y); };
         auto scale = [](double2 v, double f) { return make_double2(v.x * f, v.y * f); };
         auto mulc = [](double2 x, double2 y) {   // x conj(y)
@@ -341,8 +346,8 @@ __device__ __forceinline__ void store_factors(const M2<R>& m, int form, R* o) {
             }
         }
         o[0] = R(C); o[1] = R(S);
-        o[2] = R(p0.x); o[3] = R(p0.y); o[4] = R(p1.x); o[5] = R(p1.y);
-        o[6] = R(q0.x); o[7] = R(q0.y); o[8] = R(q1.x); o[9] = R(q1.y);
+        double2* ph = reinterpret_cast<double2*>(o + 2);
+        ph[0] = p0; ph[1] = p1; ph[2] = q0; ph[3] = q1;
         o[10] = R(0); o[11] = R(0);
     }
 }
@@ -420,7 +425,7 @@ __device__ __forceinline__ void eval_entry(const DEntry& e, const DConst* consts
         m = mmul<R>(constituent<R>(c, xb, w, cang, cmat), m);
     }
     store_matrix<R>(m, out);
-    store_factors<R>(m, run_form(consts + e.cfirst, e.ccount), out + 8);
+    if constexpr (std::is_same<R, dd>::value) store_factors<R>(m, run_form(consts + e.cfirst, e.ccount), out + 8);
 }
 
 template <typename R>
