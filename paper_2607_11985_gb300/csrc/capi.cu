@@ -126,7 +126,7 @@ struct Launch {
     int sm_sh = 0, sm_ps = 0, sm_psi = 0, sm_lam = 0, sm_acc = 0, sm_terms = 0, sm_dw = 0,
         sm_red = 0, sm_plan = 0, sm_w = 0, sm_xg = 0, sm_io = 0, sm_dg = 0;
     int cl = 0, sm_ecl = 0;   // cluster path: log2 CTAs per sample, <Z> gather area
-    bool plan_smem = false;
+    bool plan_smem = false, tab_smem = true;   // resident: the plan's schedule / table data in shared memory
     const void* fn = nullptr;
 };
 
@@ -232,7 +232,7 @@ vqc_status plan_launch_uncached(const HostPlan& p, int launch_mode, int B, Launc
     L.wg = L.T > 32 ? L.T / 32 : 1;
     // Shared memory: a fixed part per CTA and a part per resident sample.
     const size_t dim = (size_t)1 << p.n;
-    const size_t ew = entry_reals(dbl, p.dfloat);
+    const size_t ew = entry_reals(dbl, p.dfloat) / (mode == 0 && !dbl ? 2 : 1);   // ForwardWords
     const size_t io = (size_t)8 << L.K;   // slot offsets of the state copies
     const size_t fixed = align16((size_t)p.n_sh * ew * rs) + align16(mode == 1 ? (size_t)p.num_w * rs : 0) +
                          align16((size_t)p.num_w * rs) + io + 10 * 16;
@@ -278,22 +278,46 @@ vqc_status plan_launch_uncached(const HostPlan& p, int launch_mode, int B, Launc
     L.sm_red = take((size_t)L.S * L.wg * p.n * rs);   // <Z> partials (forward, or recompute with E)
     L.sm_w = take((size_t)p.num_w * rs);
     L.sm_xg = take((size_t)L.S * (p.num_x + p.n) * rs);
-    // the plan's table data and this schedule go to shared memory when they fit
-    const size_t plan_bytes = align16(p.dev_tab_end - p.dev_tab_begin) +
-                              (L.f->dev_region_end - L.f->dev_region_begin);
-    L.plan_smem = off + plan_bytes <= (size_t)di.smem_optin && t_env.plan_smem;
-    L.sm_plan = L.plan_smem ? take(plan_bytes) : 0;
-    L.smem = off;
-    if (L.smem > (size_t)di.smem_optin)
-        return fail(VQC_ERR_UNSUPPORTED, "shared-memory layout exceeds the per-CTA limit");
     L.fn = kernel_ptr(p.dtype, p.dfloat, launch_mode, L.K, L.T >= 32, p.has_ph2);
     if (!L.fn) return fail(VQC_ERR_UNSUPPORTED, "kernel not instantiated for this K");
     st = allow_max_smem(L.fn, dev, di.smem_optin);
     if (st != VQC_OK) return st;
-    int per_sm = 0;
-    VQC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, L.fn, L.block, L.smem));
-    if (per_sm < 1) return fail(VQC_ERR_UNSUPPORTED, "kernel cannot be resident with this geometry");
     L.nunits = (B + L.S - 1) / L.S;
+    // The plan's table data and this schedule go to shared memory when they fit; the
+    // table data, which only the table evaluation reads, stays out when that lets more
+    // CTAs onto an SM and the batch has units for them (13-qubit random circuit x 256,
+    // 18 KB of table data: one wave of two CTAs an SM instead of two of one).
+    const size_t tab = align16(p.dev_tab_end - p.dev_tab_begin), sched = L.f->dev_region_end - L.f->dev_region_begin;
+    auto per_sm_with = [&](size_t extra, int& per_sm) -> vqc_status {
+        per_sm = 0;
+        if (off + extra > (size_t)di.smem_optin) return VQC_OK;
+        VQC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, L.fn, L.block, off + extra));
+        return VQC_OK;
+    };
+    int per_sm = 0, with_sched = 0;
+    if (t_env.plan_smem) {
+        st = per_sm_with(tab + sched, per_sm);
+        if (st != VQC_OK) return st;
+        L.plan_smem = L.tab_smem = per_sm > 0;
+        if (L.nunits > per_sm * di.sms) {
+            st = per_sm_with(sched, with_sched);
+            if (st != VQC_OK) return st;
+            if (with_sched > per_sm) {
+                per_sm = with_sched;
+                L.plan_smem = true;
+                L.tab_smem = false;
+            }
+        }
+    }
+    L.sm_plan = L.plan_smem ? take((L.tab_smem ? tab : 0) + sched) : 0;
+    L.smem = off;
+    if (L.smem > (size_t)di.smem_optin)
+        return fail(VQC_ERR_UNSUPPORTED, "shared-memory layout exceeds the per-CTA limit");
+    if (!L.plan_smem) {
+        st = per_sm_with(0, per_sm);
+        if (st != VQC_OK) return st;
+    }
+    if (per_sm < 1) return fail(VQC_ERR_UNSUPPORTED, "kernel cannot be resident with this geometry");
     L.grid = std::max(1, std::min(L.nunits, per_sm * di.sms));
     return VQC_OK;
 }
@@ -382,6 +406,7 @@ void fill_plan_args(const HostPlan& p, const Launch& L, KArgs<R>& a) {
     a.tab_bytes = (int)(p.dev_tab_end - p.dev_tab_begin);
     a.sm_plan = L.sm_plan;
     a.plan_smem = L.plan_smem ? 1 : 0;
+    a.tab_smem = L.tab_smem ? 1 : 0;
     a.cl = L.cl;
     a.sm_ecl = L.sm_ecl;
 }

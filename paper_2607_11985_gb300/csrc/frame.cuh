@@ -178,12 +178,12 @@ __device__ __forceinline__ void lambda_frame(const uint8_t* lmask, uint32_t pbf,
 // A stage of 2x2 updates only, at most one per local position: straight-line code
 // over the positions, each under one uniform branch, instead of a descriptor load
 // and a jump per op.
-template <typename R>
+template <typename R, int EW = EntryWords<R>::value>
 __device__ __forceinline__ const R* op_table(uint2 raw, const R* sh_tab, const R* ps_tab) {
-    return (((raw.x >> 24) & OPF_PER_SAMPLE) ? ps_tab : sh_tab) + EntryWords<R>::value * (raw.y & 0xffff);
+    return (((raw.x >> 24) & OPF_PER_SAMPLE) ? ps_tab : sh_tab) + EW * (raw.y & 0xffff);
 }
 
-template <typename R, int K>
+template <typename R, int K, int EW = EntryWords<R>::value>
 __device__ __forceinline__ void pure_forward(const uint2* ops, unsigned pm, C2<R> (&a)[1 << K], const R* sh_tab,
                                              const R* ps_tab) {
     const R* tp[K];
@@ -191,7 +191,7 @@ __device__ __forceinline__ void pure_forward(const uint2* ops, unsigned pm, C2<R
         int o = 0;
 #pragma unroll
         for (int j = 0; j < K; ++j) {
-            tp[j] = op_table<R>(ops[o], sh_tab, ps_tab);
+            tp[j] = op_table<R, EW>(ops[o], sh_tab, ps_tab);
             o += (pm >> j) & 1;
         }
     }

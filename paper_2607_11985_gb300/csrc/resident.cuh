@@ -30,6 +30,7 @@ __global__ void __launch_bounds__(512) sweep_kernel(const __grid_constant__ KArg
 
     constexpr bool PURE = FULL && std::is_same<R, float>::value;   // straight-line stages (see pass_kernel)
     constexpr bool FACT = FULL && std::is_same<R, dd>::value;  // factored stages
+    constexpr int EW = MODE == 0 ? ForwardWords<R>::value : EntryWords<R>::value;
     const int n = A.n, G = A.G;
     const int dim = 1 << n;
     Geo q;
@@ -109,10 +110,10 @@ __global__ void __launch_bounds__(512) sweep_kernel(const __grid_constant__ KArg
     const unsigned char* sms = nullptr;
     if (A.plan_smem) {
         unsigned char* t = smem + A.sm_plan;
-        unsigned char* u = t + ((A.tab_bytes + 15) & ~15);
-        async_region(t, A.plan + A.tab_off, A.tab_bytes);
+        unsigned char* u = t + (A.tab_smem ? (A.tab_bytes + 15) & ~15 : 0);
+        if (A.tab_smem) async_region(t, A.plan + A.tab_off, A.tab_bytes);
         async_region(u, A.plan + A.sched_off, A.sched_bytes);
-        smt = t;
+        smt = A.tab_smem ? t : nullptr;
         sms = u;
     }
     if (from_global) __syncthreads();   // ioff
@@ -152,11 +153,11 @@ __global__ void __launch_bounds__(512) sweep_kernel(const __grid_constant__ KArg
     for (int i = nthr - 1 - threadIdx.x; i < A.n_sh; i += nthr) {
         const int id = vqc_ld(&P.sh_list[i]);
         const DEntry e = P.entries[id];
-        eval_entry<R>(e, P.consts, static_cast<const R*>(nullptr), w_sm, Pcang, Pcmat,
-                      sh_tab + EntryWords<R>::value * e.slot);
+        eval_entry<R, EW>(e, P.consts, static_cast<const R*>(nullptr), w_sm, Pcang, Pcmat,
+                      sh_tab + EW * e.slot);
     }
 
-    R* ps_tab = ps_all + (size_t)q.g * A.n_ps * EntryWords<R>::value;
+    R* ps_tab = ps_all + (size_t)q.g * A.n_ps * EW;
     R* acc = acc_all + (size_t)q.g * A.n_accs * q.wg * 8;
     R* terms = terms_all + (size_t)q.g * A.n_terms;
 
@@ -177,8 +178,8 @@ __global__ void __launch_bounds__(512) sweep_kernel(const __grid_constant__ KArg
             const int gg = i / A.n_ps, k = i % A.n_ps;
             const int id = vqc_ld(&P.ps_list[k]);
             const DEntry e = P.entries[id];
-            eval_entry<R>(e, P.consts, xg_all + (size_t)gg * xgw, w_sm, Pcang, Pcmat,
-                          ps_all + ((size_t)gg * A.n_ps + e.slot) * EntryWords<R>::value);
+            eval_entry<R, EW>(e, P.consts, xg_all + (size_t)gg * xgw, w_sm, Pcang, Pcmat,
+                          ps_all + ((size_t)gg * A.n_ps + e.slot) * EW);
         }
         __syncthreads();
         C2<R>* dg = reinterpret_cast<C2<R>*>(smem + A.sm_dg) + (((size_t)q.g * A.nstages) << (K + 1));
@@ -211,13 +212,13 @@ __global__ void __launch_bounds__(512) sweep_kernel(const __grid_constant__ KArg
                     frame_load<R, K>(a, psi_t, v.off, sb);
                 }
                 if (PURE && (sp->pure & kStagePure))
-                    pure_forward<R, K>(reinterpret_cast<const uint2*>(P.ops) + sp->op_begin, sp->pmask, a, sh_tab,
+                    pure_forward<R, K, EW>(reinterpret_cast<const uint2*>(P.ops) + sp->op_begin, sp->pmask, a, sh_tab,
                                        ps_tab);
                 else if (FACT && (sp->pure & kStagePure))
                     factored_forward<R, K>(sp, reinterpret_cast<const uint2*>(P.ops) + sp->op_begin, a, sh_tab,
                                            ps_tab, dg + ((size_t)s << (K + 1)));
                 else
-                    run_ops<R, K, 0, false, FULL, PH2>(P.ops, sp->op_begin, sp->op_end, v.pb, a, a, sh_tab, ps_tab,
+                    run_ops<R, K, 0, false, FULL, PH2, EW>(P.ops, sp->op_begin, sp->op_end, v.pb, a, a, sh_tab, ps_tab,
                                                        nullptr, q, lane, warp_in_group);
                 if (s + 1 < ns || (MODE == 0 && A.state_out)) {
                     frame_store<R, K>(a, psi_t, v.off, sb);

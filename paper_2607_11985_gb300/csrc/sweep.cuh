@@ -257,7 +257,8 @@ struct KArgs {
     // table data [tab_off, tab_off + tab_bytes) and this schedule's
     // [sched_off, sched_off + sched_bytes) of the plan's device blob.
     const unsigned char* plan;
-    int tab_off, tab_bytes, sched_off, sched_bytes, sm_plan, plan_smem;
+    // (tab_smem 0: the table data is read where it lies, which leaves room for more CTAs)
+    int tab_off, tab_bytes, sched_off, sched_bytes, sm_plan, plan_smem, tab_smem;
     // resident path (resident.cuh): the frame schedule, and the slots of the state's
     // bits in the order of a given state (sin) and of the final one (sout)
     const FStage* fstages;
@@ -352,7 +353,13 @@ __device__ __forceinline__ void store_factors(const M2<R>& m, int form, R* o) {
     }
 }
 
-template <typename R>
+// Forward-only tables of the resident path: complex64 without U^dag (a 13-qubit random
+// circuit's tables 36 -> 18 KB per sample).
+template <typename R> struct ForwardWords {
+    static constexpr int value = sizeof(R) == 4 ? EntryWords<R>::value / 2 : EntryWords<R>::value;
+};
+
+template <typename R, int EW = EntryWords<R>::value>
 __device__ __forceinline__ void store_matrix(const M2<R>& m, R* out) {
     if constexpr (sizeof(R) == 4) {   // 16-byte stores (entries are 128-byte aligned)
         const C2<R> e[4] = {m.a, m.b, m.c, m.d};
@@ -361,7 +368,7 @@ __device__ __forceinline__ void store_matrix(const M2<R>& m, R* out) {
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             o4[k] = make_float4(e[k].x, e[k].y, -e[k].y, e[k].x);        // (m, i m)
-            o4[4 + k] = make_float4(d[k].x, d[k].y, -d[k].y, d[k].x);
+            if (EW == EntryWords<R>::value) o4[4 + k] = make_float4(d[k].x, d[k].y, -d[k].y, d[k].x);
         }
     } else {
         out[0] = m.a.x; out[1] = m.a.y; out[2] = m.b.x; out[3] = m.b.y;
@@ -402,7 +409,7 @@ __device__ __forceinline__ M2<R> constituent(const DConst& c, const XI* xb, cons
 }
 
 // Evaluate one table entry (8 reals) for sample row xb.
-template <typename R, typename XI, typename WI>
+template <typename R, int EW = EntryWords<R>::value, typename XI, typename WI>
 __device__ __forceinline__ void eval_entry(const DEntry& e, const DConst* consts, const XI* xb, const WI* w,
                            const R* cang, const R* cmat, R* out) {
     if (e.phase) {
@@ -424,7 +431,7 @@ __device__ __forceinline__ void eval_entry(const DEntry& e, const DConst* consts
         const DConst c = consts[e.cfirst + k];
         m = mmul<R>(constituent<R>(c, xb, w, cang, cmat), m);
     }
-    store_matrix<R>(m, out);
+    store_matrix<R, EW>(m, out);
     if constexpr (std::is_same<R, dd>::value) store_factors<R>(m, run_form(consts + e.cfirst, e.ccount), out + 8);
 }
 
@@ -942,14 +949,14 @@ __device__ __forceinline__ bool physbit(uint32_t pb, int ref) {
 // their register allocation then needs fewer spills (measured 8-11% faster on
 // the 12-qubit resident sweeps and the 16-qubit forward passes); the launch
 // code picks the instantiation from the plan.
-template <typename R, int K, int MODE, bool WITH_CX, bool FULL, bool WITH_PH2 = true>
+template <typename R, int K, int MODE, bool WITH_CX, bool FULL, bool WITH_PH2 = true, int EW = EntryWords<R>::value>
 __device__ __forceinline__ void apply_op(uint2 raw, uint32_t pb, C2<R> (&a)[1 << K],
                                          C2<R> (&l)[1 << K], const R* sh_tab, const R* ps_tab,
                                          R* acc, const Geo& q, int lane, int warp_in_group,
                                          bool acc_add) {
     const int code = raw.x & 0xff, ra = (raw.x >> 8) & 0xff, rb = (raw.x >> 16) & 0xff;
     const int flags = raw.x >> 24, slot = raw.y & 0xffff, aux = raw.y >> 16;
-    const R* tp = ((flags & OPF_PER_SAMPLE) ? ps_tab : sh_tab) + EntryWords<R>::value * slot;
+    const R* tp = ((flags & OPF_PER_SAMPLE) ? ps_tab : sh_tab) + EW * slot;
     R* accp = acc + ((size_t)aux * q.wg + warp_in_group) * 8;
     const int rlane = FULL ? lane : q.t;
     switch (code) {
@@ -1055,7 +1062,7 @@ __device__ __forceinline__ void apply_op(uint2 raw, uint32_t pb, C2<R> (&a)[1 <<
 // Run ops [ob, oe) of a stage (forward: in order; backward: reversed).  The
 // descriptor is read when the op starts: keeping a prefetched one live across
 // the dispatch switch costs more registers than the load latency it hides.
-template <typename R, int K, int MODE, bool WITH_CX, bool FULL, bool WITH_PH2 = true>
+template <typename R, int K, int MODE, bool WITH_CX, bool FULL, bool WITH_PH2 = true, int EW = EntryWords<R>::value>
 __device__ __forceinline__ void run_ops(const DOp* ops, int ob, int oe, uint32_t pb,
                                         C2<R> (&a)[1 << K], C2<R> (&l)[1 << K], const R* sh_tab,
                                         const R* ps_tab, R* acc, const Geo& q, int lane,
@@ -1063,11 +1070,11 @@ __device__ __forceinline__ void run_ops(const DOp* ops, int ob, int oe, uint32_t
     const uint2* op2 = reinterpret_cast<const uint2*>(ops);
     if (MODE == 0) {
         for (int o = ob; o < oe; ++o)
-            apply_op<R, K, MODE, WITH_CX, FULL, WITH_PH2>(vqc_ld(op2 + o), pb, a, l, sh_tab, ps_tab, acc, q, lane,
+            apply_op<R, K, MODE, WITH_CX, FULL, WITH_PH2, EW>(vqc_ld(op2 + o), pb, a, l, sh_tab, ps_tab, acc, q, lane,
                                           warp_in_group, acc_add);
     } else {
         for (int o = oe - 1; o >= ob; --o)
-            apply_op<R, K, MODE, WITH_CX, FULL, WITH_PH2>(vqc_ld(op2 + o), pb, a, l, sh_tab, ps_tab, acc, q, lane,
+            apply_op<R, K, MODE, WITH_CX, FULL, WITH_PH2, EW>(vqc_ld(op2 + o), pb, a, l, sh_tab, ps_tab, acc, q, lane,
                                           warp_in_group, acc_add);
     }
 }
