@@ -232,7 +232,7 @@ vqc_status plan_launch_uncached(const HostPlan& p, int launch_mode, int B, Launc
     L.wg = L.T > 32 ? L.T / 32 : 1;
     // Shared memory: a fixed part per CTA and a part per resident sample.
     const size_t dim = (size_t)1 << p.n;
-    const size_t ew = entry_reals(dbl, p.dfloat) / (mode == 0 && !dbl ? 2 : 1);   // ForwardWords
+    const size_t ew = entry_reals(dbl, p.dfloat && L.T >= 32) / (mode == 0 && !dbl ? 2 : 1);   // ResidentWords
     const size_t io = (size_t)8 << L.K;   // slot offsets of the state copies
     const size_t fixed = align16((size_t)p.n_sh * ew * rs) + align16(mode == 1 ? (size_t)p.num_w * rs : 0) +
                          align16((size_t)p.num_w * rs) + io + 10 * 16;

@@ -30,7 +30,7 @@ __global__ void __launch_bounds__(512) sweep_kernel(const __grid_constant__ KArg
 
     constexpr bool PURE = FULL && std::is_same<R, float>::value;   // straight-line stages (see pass_kernel)
     constexpr bool FACT = FULL && std::is_same<R, dd>::value;  // factored stages
-    constexpr int EW = MODE == 0 ? ForwardWords<R>::value : EntryWords<R>::value;
+    constexpr int EW = ResidentWords<R, MODE, FULL>::value;
     const int n = A.n, G = A.G;
     const int dim = 1 << n;
     Geo q;

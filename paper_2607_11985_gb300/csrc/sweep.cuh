@@ -304,6 +304,19 @@ template <typename R> struct EntryWords {
 // that their roundings, the same for every amplitude, are not double-float's.
 // (Native complex128 keeps the 2x2 updates: factors rounded to double doubled its
 // gradients' error against 64 bits, 3.2e-15 -> 6.4e-15 at 16 qubits.)
+constexpr double kTiny = 1e-36;   // squared moduli below this count as 0: their phase is never seen
+
+// 1 / sqrt(x) for x in [kTiny, 4]: a float start and two Newton steps, y (3 - x y^2) / 2
+// (relative error 2^-22 -> 2^-43 -> double); the FP64 pipe is slow and the library's
+// square root and divisions took longer than the rest of an entry.
+__device__ __forceinline__ double inv_sqrt(double x) {
+    if (!(x > kTiny)) return x != x ? x : 0.0;
+    double y = (double)rsqrtf((float)x);
+    const double h = 0.5 * x;
+    y = fma(y, fma(-h * y, y, 0.5), y);
+    return fma(y, fma(-h * y, y, 0.5), y);
+}
+
 template <typename R>
 __device__ __forceinline__ void store_factors(const M2<R>& m, int form, R* o) {
     if constexpr (std::is_same<R, dd>::value) {
@@ -316,32 +329,33 @@ __device__ __forceinline__ void store_factors(const M2<R>& m, int form, R* o) {
         double2 p0 = one, p1 = one, q0 = one, q1 = one;
         double C = a.x, S = c.x;
         if (form != 0) {
-            const double na = sqrt(fma(a.x, a.x, a.y * a.y)), nc = sqrt(fma(c.x, c.x, c.y * c.y));
-            const bool big = na >= nc;
-            C = na;
-            S = nc;
+            const double a2 = fma(a.x, a.x, a.y * a.y), c2 = fma(c.x, c.x, c.y * c.y);
+            const double ra = inv_sqrt(a2), rc = inv_sqrt(c2);   // 1 / |a|, 1 / |c|
+            const bool big = a2 >= c2;
+            C = a2 * ra;
+            S = c2 * rc;
             if (form == 3) {   // q0 = 1
-                p0 = na > 0 || !(nc > 0) ? scale(a, 1 / na) : one;
-                p1 = nc > 0 || !(na > 0) ? scale(c, 1 / nc) : one;
-                q1 = big ? scale(mulc(d, p1), 1 / na) : scale(mulc(b, p0), -1 / nc);
+                if (a2 > kTiny || !(c2 > kTiny)) p0 = scale(a, ra);
+                if (c2 > kTiny || !(a2 > kTiny)) p1 = scale(c, rc);
+                q1 = big ? scale(mulc(d, p1), ra) : scale(mulc(b, p0), -rc);
             } else if (form == 2) {
                 if (big) {
-                    p0 = scale(a, 1 / na);
-                    p1 = scale(d, 1 / na);
+                    p0 = scale(a, ra);
+                    p1 = scale(d, ra);
                     S = mulc(c, p1).x;
                 } else {
-                    p1 = scale(c, 1 / nc);
-                    p0 = scale(b, -1 / nc);
+                    p1 = scale(c, rc);
+                    p0 = scale(b, -rc);
                     C = mulc(a, p0).x;
                 }
             } else {
                 if (big) {
-                    q0 = scale(a, 1 / na);
-                    q1 = scale(d, 1 / na);
+                    q0 = scale(a, ra);
+                    q1 = scale(d, ra);
                     S = mulc(c, q0).x;
                 } else {
-                    q0 = scale(c, 1 / nc);
-                    q1 = scale(b, -1 / nc);
+                    q0 = scale(c, rc);
+                    q1 = scale(b, -rc);
                     C = mulc(a, q0).x;
                 }
             }
@@ -353,10 +367,13 @@ __device__ __forceinline__ void store_factors(const M2<R>& m, int form, R* o) {
     }
 }
 
-// Forward-only tables of the resident path: complex64 without U^dag (a 13-qubit random
-// circuit's tables 36 -> 18 KB per sample).
-template <typename R> struct ForwardWords {
-    static constexpr int value = sizeof(R) == 4 ? EntryWords<R>::value / 2 : EntryWords<R>::value;
+// Tables of the resident path: complex64 forward ones without U^dag (a 13-qubit random
+// circuit's tables 36 -> 18 KB per sample), double-float ones of groups below a warp,
+// which run no factored stages, without the factors.
+template <typename R, int MODE, bool FULL> struct ResidentWords {
+    static constexpr bool dbf = std::is_same<R, dd>::value;
+    static constexpr int value = dbf && !FULL ? entry_reals(true, false)
+                                              : EntryWords<R>::value / (!dbf && sizeof(R) == 4 && MODE == 0 ? 2 : 1);
 };
 
 template <typename R, int EW = EntryWords<R>::value>
@@ -432,7 +449,8 @@ __device__ __forceinline__ void eval_entry(const DEntry& e, const DConst* consts
         m = mmul<R>(constituent<R>(c, xb, w, cang, cmat), m);
     }
     store_matrix<R, EW>(m, out);
-    if constexpr (std::is_same<R, dd>::value) store_factors<R>(m, run_form(consts + e.cfirst, e.ccount), out + 8);
+    if constexpr (std::is_same<R, dd>::value && EW == EntryWords<R>::value)
+        store_factors<R>(m, run_form(consts + e.cfirst, e.ccount), out + 8);
 }
 
 template <typename R>
