@@ -124,7 +124,7 @@ struct Launch {
     int K = 0, T = 0, S = 0, block = 0, grid = 0, nunits = 0, wg = 1;
     size_t smem = 0;
     int sm_sh = 0, sm_ps = 0, sm_psi = 0, sm_lam = 0, sm_acc = 0, sm_terms = 0, sm_dw = 0,
-        sm_red = 0, sm_plan = 0, sm_w = 0, sm_xg = 0, sm_io = 0, sm_dg = 0;
+        sm_red = 0, sm_plan = 0, sm_w = 0, sm_xg = 0, sm_io = 0, sm_dg = 0, ndg = 0;
     int cl = 0, sm_ecl = 0;   // cluster path: log2 CTAs per sample, <Z> gather area
     bool plan_smem = false, tab_smem = true;   // resident: the plan's schedule / table data in shared memory
     const void* fn = nullptr;
@@ -236,7 +236,9 @@ vqc_status plan_launch_uncached(const HostPlan& p, int launch_mode, int B, Launc
     const size_t io = (size_t)8 << L.K;   // slot offsets of the state copies
     const size_t fixed = align16((size_t)p.n_sh * ew * rs) + align16(mode == 1 ? (size_t)p.num_w * rs : 0) +
                          align16((size_t)p.num_w * rs) + io + 10 * 16;
-    const size_t dgb = p.dfloat && L.T >= 32 ? (L.f->stages.size() << (L.K + 1)) * cs : 0;   // stage diagonals
+    // diagonal tables: two-local phases, and double-float's own (complex128 schedules count both)
+    L.ndg = L.T >= 32 && dbl && (p.dfloat || p.has_ph2) ? L.f->passes[0].ndg : 0;
+    const size_t dgb = ((size_t)L.ndg << L.K) * cs;
     const size_t per_sample = dgb + (size_t)p.n_ps * ew * rs + dim * cs * (mode == 1 ? 2 : 1) +
                               (size_t)(p.num_x + p.n) * rs +
                               (mode == 1 ? p.accs.size() * L.wg * 8 * rs + p.term_src.size() * rs : 0) +
@@ -358,6 +360,8 @@ void fill_plan_args(const HostPlan& p, const Launch& L, KArgs<R>& a) {
     if (L.f) {
         a.ops = reinterpret_cast<const DOp*>(base + L.f->dev_ops);
         a.fstages = reinterpret_cast<const FStage*>(base + L.f->dev_stages);
+        a.segs = reinterpret_cast<const FSeg*>(base + L.f->dev_segs);
+        a.nsegs = (int)L.f->segs.size();
         a.fin = reinterpret_cast<const FFinal*>(base + L.f->dev_fin);
         a.nstages = (int)L.f->stages.size();
         for (int i = 0; i < p.n; ++i) {
@@ -400,7 +404,7 @@ void fill_plan_args(const HostPlan& p, const Launch& L, KArgs<R>& a) {
     a.Pw = p.num_w;
     a.sm_sh = L.sm_sh; a.sm_ps = L.sm_ps; a.sm_psi = L.sm_psi; a.sm_lam = L.sm_lam;
     a.sm_acc = L.sm_acc; a.sm_terms = L.sm_terms; a.sm_dw = L.sm_dw; a.sm_red = L.sm_red;
-    a.sm_w = L.sm_w; a.sm_xg = L.sm_xg; a.sm_io = L.sm_io; a.sm_dg = L.sm_dg;
+    a.sm_w = L.sm_w; a.sm_xg = L.sm_xg; a.sm_io = L.sm_io; a.sm_dg = L.sm_dg; a.ndg = L.ndg;
     a.plan = static_cast<const unsigned char*>(p.dbuf);
     a.tab_off = (int)p.dev_tab_begin;
     a.tab_bytes = (int)(p.dev_tab_end - p.dev_tab_begin);
@@ -470,6 +474,7 @@ vqc_status upload(HostPlan& p) {
         s.dev_region_begin = blob.size();
         s.dev_ops = put(s.ops.data(), s.ops.size() * sizeof(DOp));
         s.dev_stages = put(s.stages.data(), s.stages.size() * sizeof(FStage));
+        s.dev_segs = put(s.segs.data(), s.segs.size() * sizeof(FSeg));
         s.dev_fin = put(&s.fin, sizeof(FFinal));
         s.dev_region_end = blob.size();
         s.dev_flips = put(s.flips.data(), s.flips.size() * sizeof(FFlip));
@@ -776,6 +781,7 @@ struct PassGeo {
     int nunits = 0;
     size_t smem = 0;
     int sm_sh = 0, sm_ps = 0, sm_lam = 0, sm_acc = 0, sm_red = 0, sm_plan = 0, sm_tfl = 0, sm_koff = 0, sm_toff = 0, sm_tbase = 0, sm_dg = 0;
+    bool tables = false;   // the stages' diagonal tables are used
     const void* fn = nullptr;
 };
 
@@ -794,21 +800,24 @@ vqc_status plan_hbm_uncached(const HostPlan& p, int mode, int B, PassGeo& L) {
     L.T = 1 << (m - L.K);
     L.wg = L.T > 32 ? L.T / 32 : 1;
     L.ntiles = 1 << (p.n - m);
-    int ps_max = 0, sh_max = 0, acc_max = 0, nst_max = 0, ops_max = 0;
+    int ps_max = 0, sh_max = 0, acc_max = 0, nst_max = 0, ops_max = 0, ndg_max = 0, seg_max = 0;
     for (const FPass& ps : L.s->passes) {
         ps_max = std::max(ps_max, ps.ps_count);
         sh_max = std::max(sh_max, ps.sh_count);
         acc_max = std::max(acc_max, ps.acc_count);
         nst_max = std::max(nst_max, ps.stage_end - ps.stage_begin);
+        ndg_max = std::max(ndg_max, ps.ndg);
+        seg_max = std::max(seg_max, ps.seg_end - ps.seg_begin);
         ops_max = std::max(ops_max, ps.op_end - ps.op_begin);
     }
     const size_t tdim = (size_t)1 << m;
     const size_t ew = entry_reals(dbl, p.dfloat);
     const size_t apv = 16 / cs, nk = (tdim / apv + L.T - 1) / L.T;
     const size_t prog = (size_t)nst_max * sizeof(FStage) + sizeof(FFinal) + (size_t)ops_max * sizeof(DOp) +
-                        (size_t)nst_max * L.s->nout * sizeof(FFlip);
+                        (size_t)nst_max * L.s->nout * sizeof(FFlip) + (size_t)seg_max * sizeof(FSeg);
     const size_t fixed = align16((size_t)sh_max * ew * rs) + align16(prog) + align16(2 * nk * 8) + 8 * 16;
-    const size_t dgb = p.dfloat && L.T >= 32 ? ((size_t)nst_max << (L.K + 1)) * cs : 0;   // stage diagonals
+    L.tables = L.T >= 32 && dbl && (p.dfloat || p.has_ph2);   // as on the resident path
+    const size_t dgb = L.tables ? ((size_t)ndg_max << L.K) * cs : 0;
     const size_t per_tile = dgb + (size_t)ps_max * ew * rs + tdim * cs * (mode == 1 ? 2 : 1) + (size_t)(nst_max + 1) * 8 +
                             (size_t)L.T * (16 + 4 * nst_max) + (mode == 1 ? (size_t)acc_max * L.wg * 8 * rs : (size_t)L.wg * p.n * rs);
     int S = std::max(1, 128 / L.T);
@@ -960,6 +969,9 @@ void fill_pass_args(const HostPlan& p, const PassGeo& L, const FPass& ps, const 
     a.nout = s.nout;
     a.nstages = ps.stage_end - ps.stage_begin;
     a.nops = ps.op_end - ps.op_begin;
+    a.segs = reinterpret_cast<const FSeg*>(base + s.dev_segs) + ps.seg_begin;
+    a.nsegs = ps.seg_end - ps.seg_begin;
+    a.seg_begin = ps.seg_begin;
     a.op_begin = ps.op_begin;
     a.ps_begin = ps.ps_begin;
     a.ps_count = ps.ps_count;
@@ -988,6 +1000,7 @@ void fill_pass_args(const HostPlan& p, const PassGeo& L, const FPass& ps, const 
     a.sm_plan = L.sm_plan; a.sm_tfl = L.sm_tfl; a.sm_toff = L.sm_toff;
     a.sm_tbase = L.sm_tbase;
     a.sm_dg = L.sm_dg;
+    a.ndg = L.tables ? ps.ndg : 0;
 }
 
 // The forward passes: psi0 (nullptr: |0...0>) -> out in logical order (nullptr:

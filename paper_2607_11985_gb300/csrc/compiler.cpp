@@ -593,7 +593,8 @@ bool resident_fits(const HostPlan& p) {
     const size_t need = (size_t)(p.n_sh + p.n_ps) * ew * rs + 2 * (size_t)p.num_w * rs +
                         ((size_t)4 << p.n) * rs + (size_t)(p.num_x + p.n) * rs + p.accs.size() * wg * 8 * rs +
                         p.term_src.size() * rs + wg * p.n * rs +
-                        (p.dtype == VQC_C128 ? 5 * p.ops.size() * 16 * rs : 0);   // stage diagonals, generously
+                        // diagonal tables, at most two per op
+                        (p.dtype == VQC_C128 ? p.ops.size() * 2 * 32 * rs : 0);
     return need <= 216 * 1024;
 }
 

@@ -50,18 +50,38 @@ struct FStage {
     int32_t tau[kMaxThreadBits];
     uint32_t tmask[kMaxThreadBits];
     int32_t sigma[kMaxK];
+    int32_t seg_begin, seg_end;
     int32_t op_begin, op_end;
     uint8_t nthreadbits, nsel;   // nsel: parities in pb (0: pb is not needed)
-    uint8_t pure;                // kStagePure: the ops are 2x2 updates only, at most one per local position,
-                                 // in the order of their positions; then also kStageQ, kStageP, kStagePs
-    uint8_t pmask;               // positions that have one
+    uint8_t kind;                // kStagePure: one round of runs and no diagonal op (or no op at all);
+                                 // kStagePhases: it has CRZ or RZZ
+    uint8_t pmask;               // its positions
+    int32_t pad1[2];
 };
+static_assert(sizeof(FStage) == 176, "FStage layout");
+enum : uint8_t { kStagePure = 1, kStagePhases = 2 };
+
+// A stage's ops in rounds: diagonal ones [op_begin, run_begin), then runs [run_begin,
+// op_end) in the order of their local positions, at most one each.  The diagonal group
+// is ordered by where its qubits live: both outside the block, one local (by position),
+// both local (CZ, then phases).
+struct FSeg {
+    int32_t op_begin, run_begin, op_end;
+    uint8_t flags;
+    uint8_t pmask;               // positions that have a run
+    // diagonal tables of the pass (kNoDiagonal: none): the group's two-local phases and
+    // (complex128) the runs' q, the runs' p
+    uint16_t dg[2];
+    uint16_t pad;
+};
+static_assert(sizeof(FSeg) == 20, "FSeg layout");
 enum : uint8_t {
-    kStagePure = 1,
-    kStageQ = 2, kStageP = 4,    // some run needs its diagonal before / after the rotation (run_form)
-    kStagePs = 8                 // some run depends on the sample
+    kSegPs = 1,             // a table depends on the sample
+    kSegQ = 2, kSegP = 4,   // some run needs its diagonal before / after the rotation (run_form)
+    kSegA = 8,              // the group has gradient terms
+    kSegL = 16              // it has phases of two local positions
 };
-static_assert(sizeof(FStage) == 160, "FStage layout");
+constexpr uint16_t kNoDiagonal = 0xffff;
 
 // What tile bit o (of the n - m outer bits) adds to a stage: the slot offset of
 // the register block's base and its parities.
@@ -87,7 +107,7 @@ static_assert(sizeof(FFinal) == 176, "FFinal layout");
 // order, at other addresses than its tiles were read from.
 struct FPass {
     int32_t stage_begin, stage_end;
-    int32_t op_begin, op_end;
+    int32_t op_begin, op_end, seg_begin, seg_end;
     uint32_t gin[kMaxTileBits], gout[kMaxTileBits];
     int32_t sin[kMaxTileBits], sout[kMaxTileBits];
     uint32_t oin[kMaxOuterBits], oout[kMaxOuterBits];
@@ -95,6 +115,7 @@ struct FPass {
     int32_t ps_begin, ps_count;    // per-sample table entries of the pass (into pass_entries)
     int32_t sh_begin, sh_count;    // shared table entries of the pass
     int32_t acc_begin, acc_count;  // accumulators of the pass (into pass_accs)
+    int32_t ndg;                   // diagonal tables of its stages
 };
 
 struct FrameSchedule {
@@ -102,12 +123,13 @@ struct FrameSchedule {
     int nout = 0;
     std::vector<DOp> ops;
     std::vector<FStage> stages;
+    std::vector<FSeg> segs;
     std::vector<FFlip> flips;              // [stages][nout]
     std::vector<FPass> passes;             // one on the resident path
     std::vector<int32_t> pass_entries, pass_accs;
     FFinal fin{};
-    size_t dev_ops = 0, dev_stages = 0, dev_flips = 0, dev_fin = 0, dev_pass_entries = 0, dev_pass_accs = 0;
-    size_t dev_region_begin = 0, dev_region_end = 0;   // ops, stages, fin in the plan's device blob
+    size_t dev_ops = 0, dev_stages = 0, dev_segs = 0, dev_flips = 0, dev_fin = 0, dev_pass_entries = 0, dev_pass_accs = 0;
+    size_t dev_region_begin = 0, dev_region_end = 0;   // ops, stages, segs, fin in the plan's device blob
 };
 
 struct HostPlan;

@@ -792,6 +792,7 @@ FrameSchedule FrameBuilder::build(int mode, int path, const std::vector<int>& ti
         // stage records
         fp.stage_begin = (int32_t)S.stages.size();
         fp.op_begin = (int32_t)S.ops.size();
+        fp.seg_begin = (int32_t)S.segs.size();
         for (size_t si = 0; si < ps.stages.size(); ++si) {
             const StagePlan& s = ps.stages[si];
             FStage st{};
@@ -815,11 +816,7 @@ FrameSchedule FrameBuilder::build(int mode, int path, const std::vector<int>& ti
                 if (i == outside.size()) outside.push_back(r);
                 return (uint8_t)(kRefPhys + i);
             };
-            st.op_begin = (int32_t)S.ops.size();
-            std::vector<DOp> recs;
-            uint8_t pm = 0;
-            bool pure = true;
-            for (int x : s.ops) {
+            auto record = [&](int x) {
                 const FOp& o = f[x];
                 const HOp& h = p.ops[o.hop];
                 DOp d{};
@@ -835,47 +832,99 @@ FrameSchedule FrameBuilder::build(int mode, int path, const std::vector<int>& ti
                     while (s.D[k] != o.d || s.R[k] != o.r) ++k;
                     d.a = (uint8_t)k;
                     d.code = (uint8_t)(DC_M1 + k);
-                    pure = pure && !((pm >> k) & 1);
-                    pm |= (uint8_t)(1u << k);
-                } else {
-                    pure = false;
-                    uint8_t ra = ref(o.r), rb = ref(o.r2);
-                    const bool la = ra < kRefPhys, lb = rb < kRefPhys;
-                    if (h.type == OP_CZ) {
-                        if (la && lb) {
-                            if (ra > rb) std::swap(ra, rb);
-                            d.code = (uint8_t)(DC_CZ_LL + cz_pair_index(ra, rb));
-                        } else if (la || lb) {
-                            if (!la) std::swap(ra, rb);
-                            d.code = (uint8_t)(DC_CZ_PL + ra);
-                        } else {
-                            d.code = DC_CZ_PP;
-                        }
-                    } else if (la && lb) {
-                        d.code = (uint8_t)(DC_PH2_LL + cz_pair_index(std::min(ra, rb), std::max(ra, rb)));
+                    return d;
+                }
+                uint8_t ra = ref(o.r), rb = ref(o.r2);
+                const bool la = ra < kRefPhys, lb = rb < kRefPhys;
+                if (h.type == OP_CZ) {
+                    if (la && lb) {
+                        if (ra > rb) std::swap(ra, rb);
+                        d.code = (uint8_t)(DC_CZ_LL + cz_pair_index(ra, rb));
                     } else if (la || lb) {
-                        d.code = (uint8_t)(DC_PH2_PL + (la ? ra : rb));
+                        if (!la) std::swap(ra, rb);
+                        d.code = (uint8_t)(DC_CZ_PL + ra);
                     } else {
-                        d.code = DC_PH2_PP;
+                        d.code = DC_CZ_PP;
                     }
-                    d.a = ra;
-                    d.b = rb;
+                } else if (la && lb) {
+                    d.code = (uint8_t)(DC_PH2_LL + cz_pair_index(std::min(ra, rb), std::max(ra, rb)));
+                } else if (la || lb) {
+                    d.code = (uint8_t)(DC_PH2_PL + (la ? ra : rb));
+                } else {
+                    d.code = DC_PH2_PP;
                 }
-                recs.push_back(d);
+                d.a = ra;
+                d.b = rb;
+                return d;
+            };
+            // order of a diagonal group: PP, PL by position, LL CZ, LL phases
+            auto key = [](const DOp& d) {
+                if (d.code == DC_CZ_PP || d.code == DC_PH2_PP) return 0;
+                if (d.code >= DC_CZ_PL && d.code < DC_CZ_PP) return 1 + d.code - DC_CZ_PL;
+                if (d.code >= DC_PH2_PL && d.code < DC_PH2_PP) return 1 + d.code - DC_PH2_PL;
+                return d.code < DC_CZ_PL ? 10 : 11;
+            };
+            // each op's round: a run follows the diagonal ops it does not commute with in
+            // the same round or an earlier one, and the run before it on its position; a
+            // diagonal op follows such runs by a round
+            std::vector<int> round(s.ops.size(), 0);
+            int rounds = 1;
+            for (size_t i = 0; i < s.ops.size(); ++i) {
+                const FOp& o = f[s.ops[i]];
+                for (size_t k = 0; k < i; ++k) {
+                    const FOp& q = f[s.ops[k]];
+                    if (!o.run && !q.run) continue;
+                    const bool clash = o.run && q.run ? q.d == o.d
+                                     : o.run ? odd(q.r & o.d) || odd(q.r2 & o.d) : odd(o.r & q.d) || odd(o.r2 & q.d);
+                    if (clash) round[i] = std::max(round[i], round[k] + (q.run ? 1 : 0));
+                }
+                rounds = std::max(rounds, round[i] + 1);
             }
-            if (pure) std::sort(recs.begin(), recs.end(), [](const DOp& a, const DOp& b) { return a.a < b.a; });
-            S.ops.insert(S.ops.end(), recs.begin(), recs.end());
-            st.op_end = (int32_t)S.ops.size();
-            st.pure = pure ? kStagePure : 0;
-            for (const DOp& d : recs)
-                if (pure && (d.flags & OPF_PER_SAMPLE)) st.pure |= kStagePs;
-            if (pure)
-                for (int x : s.ops) {
-                    const DEntry& e = p.entries[p.ops[f[x].hop].entry];
-                    const int form = run_form(&p.consts[e.cfirst], e.ccount);
-                    st.pure |= (uint8_t)((form & 1 ? kStageQ : 0) | (form & 2 ? kStageP : 0));
+            st.op_begin = (int32_t)S.ops.size();
+            st.seg_begin = (int32_t)S.segs.size();
+            for (int rd = 0; rd < rounds && !s.ops.empty(); ++rd) {
+                FSeg sg{};
+                std::vector<DOp> diag, runs;
+                for (size_t i = 0; i < s.ops.size(); ++i) {
+                    if (round[i] != rd) continue;
+                    const int x = s.ops[i];
+                    const DOp d = record(x);
+                    if (f[x].run) {
+                        sg.pmask |= (uint8_t)(1u << d.a);
+                        if (d.flags & OPF_PER_SAMPLE) sg.flags |= kSegPs;
+                        const DEntry& e = p.entries[p.ops[f[x].hop].entry];
+                        const int form = run_form(&p.consts[e.cfirst], e.ccount);
+                        sg.flags |= (uint8_t)((form & 1 ? kSegQ : 0) | (form & 2 ? kSegP : 0));
+                        runs.push_back(d);
+                    } else {
+                        if (d.flags & OPF_HAS_ACC) sg.flags |= kSegA;
+                        if (key(d) == 11) sg.flags |= (uint8_t)(kSegL | (d.flags & OPF_PER_SAMPLE ? kSegPs : 0));
+                        diag.push_back(d);
+                    }
                 }
-            st.pmask = pure ? pm : 0;
+                std::stable_sort(diag.begin(), diag.end(), [&](const DOp& a, const DOp& b) { return key(a) < key(b); });
+                std::sort(runs.begin(), runs.end(), [](const DOp& a, const DOp& b) { return a.a < b.a; });
+                sg.op_begin = (int32_t)S.ops.size();
+                S.ops.insert(S.ops.end(), diag.begin(), diag.end());
+                sg.run_begin = (int32_t)S.ops.size();
+                S.ops.insert(S.ops.end(), runs.begin(), runs.end());
+                sg.op_end = (int32_t)S.ops.size();
+                // tables: two-local phases, and (double-float) the runs' own diagonals
+                const bool factors = p.dtype == VQC_C128;
+                const bool has[2] = {(sg.flags & kSegL) || (factors && (sg.flags & kSegQ)),
+                                     factors && (sg.flags & kSegP)};
+                for (int k = 0; k < 2; ++k) sg.dg[k] = has[k] ? (uint16_t)fp.ndg++ : kNoDiagonal;
+                S.segs.push_back(sg);
+            }
+            st.seg_end = (int32_t)S.segs.size();
+            if (st.seg_begin == st.seg_end ||
+                (st.seg_begin + 1 == st.seg_end && S.segs.back().op_begin == S.segs.back().run_begin)) {
+                st.kind = kStagePure;
+                st.pmask = st.seg_begin < st.seg_end ? S.segs.back().pmask : 0;
+            }
+            for (int x : s.ops)
+                if (p.ops[f[x].hop].type == OP_PH2) st.kind |= kStagePhases;
+            st.op_end = (int32_t)S.ops.size();
             st.nsel = (uint8_t)outside.size();
             auto word = [&](uint32_t v) {
                 uint32_t w = 0;
@@ -904,6 +953,7 @@ FrameSchedule FrameBuilder::build(int mode, int path, const std::vector<int>& ti
         }
         fp.stage_end = (int32_t)S.stages.size();
         fp.op_end = (int32_t)S.ops.size();
+        fp.seg_end = (int32_t)S.segs.size();
         S.passes[pi] = fp;
 
         // the frame after the pass: M' vout[i] = gin[i], M' = M on the outer vectors
@@ -934,10 +984,11 @@ std::vector<uint8_t> export_frames(const HostPlan& p) {
     num((int32_t)p.frames.size());
     for (const FrameSchedule& s : p.frames) {
         for (int v : {s.mode, s.K, s.m, s.path, s.nout, (int)s.ops.size(), (int)s.stages.size(),
-                      (int)s.passes.size(), (int)s.pass_entries.size(), (int)s.pass_accs.size()})
+                      (int)s.passes.size(), (int)s.pass_entries.size(), (int)s.pass_accs.size(), (int)s.segs.size()})
             num(v);
         put(s.ops.data(), s.ops.size() * sizeof(DOp));
         put(s.stages.data(), s.stages.size() * sizeof(FStage));
+        put(s.segs.data(), s.segs.size() * sizeof(FSeg));
         put(s.flips.data(), s.flips.size() * sizeof(FFlip));
         put(s.passes.data(), s.passes.size() * sizeof(FPass));
         put(s.pass_entries.data(), s.pass_entries.size() * 4);

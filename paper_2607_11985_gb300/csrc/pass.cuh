@@ -20,11 +20,12 @@ template <typename R>
 struct PArgs {
     const DOp* ops;               // the pass's ops and stages
     const FStage* stages;
+    const FSeg* segs;
     const FFlip* flips;           // [stages][nout]
     const FFinal* fin;            // last pass only (forward: <Z>; backward: lam = O psi)
     const int32_t* pass_entries;  // table slots of the pass's entries
     const int32_t* pass_accs;
-    int n, m, tbits, G, S, nout, nstages, nops, op_begin;
+    int n, m, tbits, G, S, nout, nstages, nops, op_begin, nsegs, seg_begin;
     int ps_begin, ps_count, sh_begin, sh_count, acc_begin, acc_count, n_accs;
     const void* ps_g;       // per-sample table entries [B][n_ps][entry words], kernel real type
     const void* sh_g;       // shared table entries [n_sh][entry words] (both from run_tables)
@@ -43,9 +44,9 @@ struct PArgs {
     R* E_part;              // forward, last pass: [B * ntiles, n]
     R* rho;                 // backward: per-tile rho sums [B * ntiles][n_accs][4] (3 used)
     int sm_sh, sm_ps, sm_lam, sm_acc, sm_red;
-    int sm_plan;            // copies of the pass's stages, ops, flips and fin
+    int sm_plan;            // copies of the pass's stages, ops, flips, rounds and fin
     int sm_tfl;             // per tile: each stage's flip (uint2), then the logical parities
-    int sm_dg;              // double-float: the stages' diagonals (build_diagonals), per tile of the CTA
+    int sm_dg, ndg;         // the stages' diagonal tables (build_diagonals), per tile of the CTA
     int sm_tbase;           // each thread's block base in every stage: [nstages][threads]
     int sm_toff;            // tile-copy offsets of each thread: uint4
     int sm_koff;            // tile-copy offsets per vector round, read order then written order: uint2
@@ -175,12 +176,15 @@ __global__ void __launch_bounds__(256, 2) pass_kernel(const __grid_constant__ PA
     FFinal* fin = reinterpret_cast<FFinal*>(stages + nst);
     uint2* ops = reinterpret_cast<uint2*>(fin + 1);
     FFlip* flips = reinterpret_cast<FFlip*>(ops + A.nops);
+    FSeg* segs = reinterpret_cast<FSeg*>(flips + nst * A.nout);
     async_region(reinterpret_cast<unsigned char*>(stages), reinterpret_cast<const unsigned char*>(A.stages),
                  nst * (int)sizeof(FStage));
     if (A.fin)
         async_region(reinterpret_cast<unsigned char*>(fin), reinterpret_cast<const unsigned char*>(A.fin),
                      sizeof(FFinal));
     for (int i = threadIdx.x; i < A.nops; i += nthr) async_elem<uint2>(ops + i, reinterpret_cast<const uint2*>(A.ops) + i);
+    for (int i = threadIdx.x; i < A.nsegs * (int)(sizeof(FSeg) / 4); i += nthr)
+        async_elem<int>(reinterpret_cast<int*>(segs) + i, reinterpret_cast<const int*>(A.segs) + i);
     for (int i = threadIdx.x; i < nst * A.nout; i += nthr)
         async_elem<uint2>(reinterpret_cast<uint2*>(flips) + i, reinterpret_cast<const uint2*>(A.flips) + i);
 
@@ -188,10 +192,7 @@ __global__ void __launch_bounds__(256, 2) pass_kernel(const __grid_constant__ PA
     const int total_tiles = A.B << A.nout;   // (at most states in memory over 64 amplitudes)
     const uint32_t tmask = (1u << A.nout) - 1u;
     constexpr bool DDK = !std::is_same<St<R>, R>::value;   // double-float kernel
-    // stages of runs: complex64 as straight-line code (16-qubit workload 7.61 -> 7.24
-    // ms against the op switch), double-float factored
-    constexpr bool PURE = FULL && std::is_same<R, float>::value;
-    constexpr bool FACT = FULL && std::is_same<R, dd>::value;   // factored stages
+    constexpr bool DG = sizeof(R) == 8;   // the stages may have diagonal tables
     Geo q;
     q.T = 1 << A.tbits;
     q.lanes = q.T < 32 ? q.T : 32;
@@ -243,8 +244,9 @@ __global__ void __launch_bounds__(256, 2) pass_kernel(const __grid_constant__ PA
     const uint32_t g0 = (uint32_t)(q.g * tdim) ^ (uint32_t)q.h;
     R* ps_tab = ps_all + (size_t)q.g * A.ps_count * EntryWords<R>::value;
     R* acc = acc_all + (size_t)q.g * A.acc_count * q.wg * 8;
-    C2<R>* dg = reinterpret_cast<C2<R>*>(smem + A.sm_dg) + (((size_t)q.g * nst) << (K + 1));
-    if constexpr (FACT) build_diagonals<R, K>(stages, nst, ops, A.op_begin, sh_tab, ps_tab, false, q.t, q.T, dg);
+    C2<R>* dg = reinterpret_cast<C2<R>*>(smem + A.sm_dg) + (((size_t)q.g * A.ndg) << K);
+    if constexpr (FULL && DG) if (A.ndg)
+        build_diagonals<R, K>(segs, A.nsegs, ops, A.op_begin, sh_tab, ps_tab, false, q.t, q.T, dg);
     uint2* tfl_all = reinterpret_cast<uint2*>(smem + A.sm_tfl);
     const uint2* tfl = tfl_all + q.g * (nst + 1);
     // each thread's block base in every stage (read by itself only)
@@ -305,11 +307,10 @@ __global__ void __launch_bounds__(256, 2) pass_kernel(const __grid_constant__ PA
             if (MODE == 1 && A.src_lam) tile_prefetch<R>(A.src_lam + nsb, nga, koff_g, nk, q.t);
         }
         __syncthreads();
-        if constexpr (FACT)
-            if (A.ps_count) {
-                build_diagonals<R, K>(stages, nst, ops, A.op_begin, sh_tab, ps_tab, true, q.t, q.T, dg);
-                __syncthreads();
-            }
+        if constexpr (FULL && DG) if (A.ndg && A.ps_count) {
+            build_diagonals<R, K>(segs, A.nsegs, ops, A.op_begin, sh_tab, ps_tab, true, q.t, q.T, dg);
+            __syncthreads();
+        }
 
         C2<R> a[1 << K];
         uint32_t sb[K];
@@ -326,11 +327,9 @@ __global__ void __launch_bounds__(256, 2) pass_kernel(const __grid_constant__ PA
                 } else {
                     frame_load<R, K>(a, psi_t, v.off, sb);
                 }
-                if (PURE && (sp->pure & kStagePure))
-                    pure_forward<R, K>(ops + (sp->op_begin - A.op_begin), sp->pmask, a, sh_tab, ps_tab);
-                else if (FACT && (sp->pure & kStagePure))
-                    factored_forward<R, K>(sp, ops + (sp->op_begin - A.op_begin), a, sh_tab, ps_tab,
-                                           dg + ((size_t)s << (K + 1)));
+                if constexpr (FULL)
+                    stage_forward<R, K, PH2, EntryWords<R>::value>(sp, segs, A.seg_begin, ops, A.op_begin, v.pb, a,
+                                                                        sh_tab, ps_tab, dg, q, lane, warp_in_group);
                 else
                     run_ops<R, K, 0, false, FULL, PH2>(reinterpret_cast<const DOp*>(ops), sp->op_begin - A.op_begin,
                                                        sp->op_end - A.op_begin, v.pb, a, a, sh_tab, ps_tab, nullptr,
@@ -375,18 +374,10 @@ __global__ void __launch_bounds__(256, 2) pass_kernel(const __grid_constant__ PA
                 } else {
                     frame_load<R, K>(l, lam_t, v.off, sb);
                 }
-                const bool pure = (PURE || FACT) && (sp->pure & kStagePure);
-                if constexpr (PURE) {
-                    if (pure)
-                        pure_backward<K>(ops + (sp->op_begin - A.op_begin), sp->pmask, a, l, sh_tab, ps_tab, acc,
-                                         q.wg, lane, warp_in_group);
-                }
-                if constexpr (FACT) {
-                    if (pure)
-                        factored_backward<R, K>(sp, ops + (sp->op_begin - A.op_begin), a, l, sh_tab, ps_tab,
-                                                dg + ((size_t)s << (K + 1)), acc, q.wg, lane, warp_in_group);
-                }
-                if (!pure)
+                if constexpr (FULL)
+                    stage_backward<R, K, PH2>(sp, segs, A.seg_begin, ops, A.op_begin, v.pb, a, l, sh_tab, ps_tab, dg,
+                                              acc, q, lane, warp_in_group);
+                else
                     run_ops<R, K, 1, false, FULL, PH2>(reinterpret_cast<const DOp*>(ops), sp->op_begin - A.op_begin,
                                                        sp->op_end - A.op_begin, v.pb, a, l, sh_tab, ps_tab, acc, q,
                                                        lane, warp_in_group);

@@ -28,8 +28,7 @@ __global__ void __launch_bounds__(512) sweep_kernel(const __grid_constant__ KArg
     R* dw_cta = reinterpret_cast<R*>(smem + A.sm_dw);
     R* red_all = reinterpret_cast<R*>(smem + A.sm_red);
 
-    constexpr bool PURE = FULL && std::is_same<R, float>::value;   // straight-line stages (see pass_kernel)
-    constexpr bool FACT = FULL && std::is_same<R, dd>::value;  // factored stages
+    constexpr bool DG = sizeof(R) == 8;   // the stages may have diagonal tables
     constexpr int EW = ResidentWords<R, MODE, FULL>::value;
     const int n = A.n, G = A.G;
     const int dim = 1 << n;
@@ -127,6 +126,7 @@ __global__ void __launch_bounds__(512) sweep_kernel(const __grid_constant__ KArg
     PlanPtrs P;
     P.ops = rebase(A.ops, A.plan, A.sched_off, sms);
     const FStage* stages = rebase(A.fstages, A.plan, A.sched_off, sms);
+    const FSeg* segs = rebase(A.segs, A.plan, A.sched_off, sms);
     const FFinal* fin = rebase(A.fin, A.plan, A.sched_off, sms);
     P.entries = rebase(A.entries, A.plan, A.tab_off, smt);
     P.ps_list = rebase(A.ps_list, A.plan, A.tab_off, smt);
@@ -157,6 +157,7 @@ __global__ void __launch_bounds__(512) sweep_kernel(const __grid_constant__ KArg
                       sh_tab + EW * e.slot);
     }
 
+    const uint2* ops = reinterpret_cast<const uint2*>(P.ops);
     R* ps_tab = ps_all + (size_t)q.g * A.n_ps * EW;
     R* acc = acc_all + (size_t)q.g * A.n_accs * q.wg * 8;
     R* terms = terms_all + (size_t)q.g * A.n_terms;
@@ -182,12 +183,11 @@ __global__ void __launch_bounds__(512) sweep_kernel(const __grid_constant__ KArg
                           ps_all + ((size_t)gg * A.n_ps + e.slot) * EW);
         }
         __syncthreads();
-        C2<R>* dg = reinterpret_cast<C2<R>*>(smem + A.sm_dg) + (((size_t)q.g * A.nstages) << (K + 1));
-        if constexpr (FACT) {
-            const uint2* ops = reinterpret_cast<const uint2*>(P.ops);
+        C2<R>* dg = reinterpret_cast<C2<R>*>(smem + A.sm_dg) + (((size_t)q.g * A.ndg) << K);
+        if constexpr (FULL && DG) if (A.ndg) {
             if (unit == (int)blockIdx.x)
-                build_diagonals<R, K>(stages, A.nstages, ops, 0, sh_tab, ps_tab, false, q.t, q.T, dg);
-            build_diagonals<R, K>(stages, A.nstages, ops, 0, sh_tab, ps_tab, true, q.t, q.T, dg);
+                build_diagonals<R, K, EW>(segs, A.nsegs, ops, 0, sh_tab, ps_tab, false, q.t, q.T, dg);
+            build_diagonals<R, K, EW>(segs, A.nsegs, ops, 0, sh_tab, ps_tab, true, q.t, q.T, dg);
             __syncthreads();
         }
 
@@ -211,15 +211,11 @@ __global__ void __launch_bounds__(512) sweep_kernel(const __grid_constant__ KArg
                 } else {
                     frame_load<R, K>(a, psi_t, v.off, sb);
                 }
-                if (PURE && (sp->pure & kStagePure))
-                    pure_forward<R, K, EW>(reinterpret_cast<const uint2*>(P.ops) + sp->op_begin, sp->pmask, a, sh_tab,
-                                       ps_tab);
-                else if (FACT && (sp->pure & kStagePure))
-                    factored_forward<R, K>(sp, reinterpret_cast<const uint2*>(P.ops) + sp->op_begin, a, sh_tab,
-                                           ps_tab, dg + ((size_t)s << (K + 1)));
+                if constexpr (FULL)
+                    stage_forward<R, K, PH2, EW>(sp, segs, 0, ops, 0, v.pb, a, sh_tab, ps_tab, dg, q, lane, warp_in_group);
                 else
-                    run_ops<R, K, 0, false, FULL, PH2, EW>(P.ops, sp->op_begin, sp->op_end, v.pb, a, a, sh_tab, ps_tab,
-                                                       nullptr, q, lane, warp_in_group);
+                    run_ops<R, K, 0, false, FULL, PH2, EW>(P.ops, sp->op_begin, sp->op_end, v.pb, a, a, sh_tab,
+                                                           ps_tab, nullptr, q, lane, warp_in_group);
                 if (s + 1 < ns || (MODE == 0 && A.state_out)) {
                     frame_store<R, K>(a, psi_t, v.off, sb);
                     group_sync<R>(q);
@@ -282,21 +278,11 @@ __global__ void __launch_bounds__(512) sweep_kernel(const __grid_constant__ KArg
                     lambda_frame<R, K>(fin->lmask, xor_bits(fin->tmask, A.tbits, q.t), xrow + A.Px, n, a, l);
                 else
                     frame_load<R, K>(l, lam_t, v.off, sb);
-                const bool pure = (PURE || FACT) && (sp->pure & kStagePure);
-                if constexpr (PURE) {
-                    if (pure)
-                        pure_backward<K>(reinterpret_cast<const uint2*>(P.ops) + sp->op_begin, sp->pmask, a, l,
-                                         sh_tab, ps_tab, acc, q.wg, lane, warp_in_group);
-                }
-                if constexpr (FACT) {
-                    if (pure)
-                        factored_backward<R, K>(sp, reinterpret_cast<const uint2*>(P.ops) + sp->op_begin, a, l,
-                                                sh_tab, ps_tab, dg + ((size_t)s << (K + 1)), acc, q.wg, lane,
-                                                warp_in_group);
-                }
-                if (!pure)
-                    run_ops<R, K, 1, false, FULL, PH2>(P.ops, sp->op_begin, sp->op_end, v.pb, a, l, sh_tab, ps_tab,
-                                                       acc, q, lane, warp_in_group);
+                if constexpr (FULL)
+                    stage_backward<R, K, PH2>(sp, segs, 0, ops, 0, v.pb, a, l, sh_tab, ps_tab, dg, acc, q, lane, warp_in_group);
+                else
+                    run_ops<R, K, 1, false, FULL, PH2, EW>(P.ops, sp->op_begin, sp->op_end, v.pb, a, l, sh_tab,
+                                                           ps_tab, acc, q, lane, warp_in_group);
                 if (s > 0) {
                     frame_store<R, K>(a, psi_t, v.off, sb);
                     frame_store<R, K>(l, lam_t, v.off, sb);

@@ -262,9 +262,10 @@ struct KArgs {
     // resident path (resident.cuh): the frame schedule, and the slots of the state's
     // bits in the order of a given state (sin) and of the final one (sout)
     const FStage* fstages;
+    const FSeg* segs;
     const FFinal* fin;
     int32_t sin[kMaxTileBits], sout[kMaxTileBits];
-    int sm_io, sm_dg;
+    int sm_io, sm_dg, ndg, nsegs;
     // cluster path only (cluster.cuh): log2 CTAs per sample, rank 0's <Z> gather area
     int cl, sm_ecl;
 };

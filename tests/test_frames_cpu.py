@@ -18,13 +18,18 @@ from paper_2607_11985_gb300 import workloads as wl
 from tests import plan_emulator as pe
 
 DOP = pe.DOP
-FSTAGE = np.dtype([("tau", "<i4", 16), ("tmask", "<u4", 16), ("sigma", "<i4", 5), ("op_begin", "<i4"),
-                   ("op_end", "<i4"), ("nthreadbits", "u1"), ("nsel", "u1"), ("pure", "u1"), ("pmask", "u1")])
+FSTAGE = np.dtype([("tau", "<i4", 16), ("tmask", "<u4", 16), ("sigma", "<i4", 5), ("seg_begin", "<i4"),
+                   ("seg_end", "<i4"), ("op_begin", "<i4"), ("op_end", "<i4"), ("nthreadbits", "u1"),
+                   ("nsel", "u1"), ("kind", "u1"), ("pmask", "u1"), ("pad1", "<i4", 2)])
+FSEG = np.dtype([("op_begin", "<i4"), ("run_begin", "<i4"), ("op_end", "<i4"), ("flags", "u1"), ("pmask", "u1"),
+                 ("dg", "<u2", 2), ("pad", "<u2")])
+PS, Q, P_, ACC, LL = (1 << i for i in range(5))
+NO_DIAGONAL = 0xffff
 FFLIP = np.dtype([("slot", "<i4"), ("mask", "<u4")])
 FPASS = np.dtype([("stage_begin", "<i4"), ("stage_end", "<i4"), ("op_begin", "<i4"), ("op_end", "<i4"),
-                  ("gin", "<u4", 14), ("gout", "<u4", 14), ("sin", "<i4", 14), ("sout", "<i4", 14),
+                  ("seg_begin", "<i4"), ("seg_end", "<i4"), ("gin", "<u4", 14), ("gout", "<u4", 14), ("sin", "<i4", 14), ("sout", "<i4", 14),
                   ("oin", "<u4", 20), ("oout", "<u4", 20), ("oslot", "<i4", 20), ("ps_begin", "<i4"), ("ps_count", "<i4"),
-                  ("sh_begin", "<i4"), ("sh_count", "<i4"), ("acc_begin", "<i4"), ("acc_count", "<i4")])
+                  ("sh_begin", "<i4"), ("sh_count", "<i4"), ("acc_begin", "<i4"), ("acc_count", "<i4"), ("ndg", "<i4")])
 FFINAL = np.dtype([("tmask", "<u4", 16), ("omask", "<u4", 20), ("lmask", "u1", 32)])
 MAX_PASS_ENTRIES = 96
 
@@ -52,10 +57,10 @@ def frames(plan):
     off += 4
     out = []
     for _ in range(count):
-        mode, K, m, path, nout, nops, nst, nps, npe, npa = struct.unpack_from("<10i", blob, off)
-        off += 40
+        mode, K, m, path, nout, nops, nst, nps, npe, npa, nsg = struct.unpack_from("<11i", blob, off)
+        off += 44
         s = dict(mode=mode, K=K, m=m, path=path, nout=nout)
-        for name, dt, k in (("ops", DOP, nops), ("stages", FSTAGE, nst), ("flips", FFLIP, nst * nout),
+        for name, dt, k in (("ops", DOP, nops), ("stages", FSTAGE, nst), ("segs", FSEG, nsg), ("flips", FFLIP, nst * nout),
                             ("passes", FPASS, nps), ("pass_entries", np.dtype("<i4"), npe),
                             ("pass_accs", np.dtype("<i4"), npa), ("fin", FFINAL, 1)):
             s[name] = np.frombuffer(blob, dt, k, off)
@@ -160,13 +165,38 @@ class Emulator:
                 ph = ph.conj() if adj else ph
                 a *= ph[self.bit(oa, pb) + 2 * self.bit(ob, pb)]
 
-    def check_pure(self, st):
-        ops = self.s["ops"][st["op_begin"]:st["op_end"]]
-        runs = [pe.op_type(o)[0] == pe.OP_M1 for o in ops]
-        pos = [int(o["a"]) for o in ops]
-        if st["pure"] & 1:
-            assert bool(st["pure"] & 8) == any(int(o["flags"]) & pe.OPF_PER_SAMPLE for o in ops)
-            assert all(runs) and pos == sorted(set(pos)) and st["pmask"] == sum(1 << q for q in pos)
+    def check_rounds(self, st, ndg):
+        """A stage's rounds cover its ops; diagonal ops in the order the kernels walk
+        them, runs by position, flags and tables as they are read there."""
+        ops, at = self.s["ops"], st["op_begin"]
+        for sg in self.s["segs"][st["seg_begin"]:st["seg_end"]]:
+            assert sg["op_begin"] == at and sg["op_begin"] <= sg["run_begin"] <= sg["op_end"]
+            at = sg["op_end"]
+            diag, runs = ops[sg["op_begin"]:sg["run_begin"]], ops[sg["run_begin"]:sg["op_end"]]
+            pos = [int(o["a"]) for o in runs]
+            assert all(pe.op_type(o)[0] == pe.OP_M1 for o in runs)
+            assert pos == sorted(set(pos)) and sg["pmask"] == sum(1 << q for q in pos)
+            keys = []
+            for o in diag:
+                t, a, b = pe.op_type(o)
+                assert t in (pe.OP_CZ, pe.OP_PH2)
+                la, lb = a < 8, b < 8
+                keys.append((10 if t == pe.OP_CZ else 11) if la and lb else 1 + min(int(a), int(b)) if la or lb else 0)
+            assert keys == sorted(keys)
+            ps = any(int(o["flags"]) & pe.OPF_PER_SAMPLE for k, o in zip(keys, diag) if k == 11)
+            assert bool(sg["flags"] & PS) == (ps or any(int(o["flags"]) & pe.OPF_PER_SAMPLE for o in runs))
+            assert bool(sg["flags"] & ACC) == any(int(o["flags"]) & pe.OPF_HAS_ACC for o in diag)
+            assert bool(sg["flags"] & LL) == (11 in keys)
+            dbl = self.p.dtype == 1   # complex128 schedules count double-float's own tables
+            want = [11 in keys or (dbl and bool(sg["flags"] & Q)), dbl and bool(sg["flags"] & P_)]
+            for k in range(2):
+                assert (sg["dg"][k] != NO_DIAGONAL) == want[k] and (not want[k] or sg["dg"][k] < ndg)
+        assert at == st["op_end"]
+        sg = self.s["segs"][st["seg_begin"]:st["seg_end"]]
+        phases = any(pe.op_type(o)[0] == pe.OP_PH2 for o in ops[st["op_begin"]:st["op_end"]])
+        assert bool(st["kind"] & 2) == phases
+        assert bool(st["kind"] & 1) == (len(sg) == 0 or (len(sg) == 1 and sg[0]["op_begin"] == sg[0]["run_begin"]))
+        assert st["pmask"] == (sg[0]["pmask"] if st["kind"] & 1 and len(sg) else 0)
 
     def logical(self, tau):
         """Logical basis state of [thread, r] of the last stage's blocks of tile tau."""
@@ -196,7 +226,7 @@ class Emulator:
                 sm[si_] = mem[oi[tau] ^ ai]
                 for si in range(ps["stage_begin"], ps["stage_end"]):
                     st, idx, pb = self.stage(si, tau)
-                    self.check_pure(st)
+                    self.check_rounds(st, int(ps["ndg"]))
                     a = sm[idx]
                     for op in self.s["ops"][st["op_begin"]:st["op_end"]]:
                         self.op(op, pb, tabs, (a,), False, None)
