@@ -368,8 +368,9 @@ vqc_status vqc_stage_apply(int32_t method, int32_t batch, int32_t num_qubits, co
  * evaluation) for a batch of `batch` samples. */
 vqc_status vqc_plan_info(const vqc_plan* plan, int32_t batch, vqc_plan_stats* out);
 
-/* Serialise the host plan (fused ops, runs, constituents, term table and all
- * stage schedules) into buf.  *inout_bytes holds buf's capacity on entry and
+/* Serialise the host plan (fused ops, runs, constituents, term table and the
+ * axis-aligned stage schedules of every path, built for the export; the resident
+ * and HBM kernels run frame schedules of the same ops) into buf.  *inout_bytes holds buf's capacity on entry and
  * the bytes needed on return; buf may be NULL to query the size.  The bytes
  * are a deterministic function of the vqc_compile arguments. */
 vqc_status vqc_plan_export(const vqc_plan* plan, void* buf, size_t* inout_bytes);

@@ -221,7 +221,7 @@ __global__ void __launch_bounds__(512) cluster_fwd_kernel(const __grid_constant_
             } else {
                 cl_block_load<R, K>(a, psi_sa, slice, v.swb, sg);
             }
-            run_ops<R, K, 0, false, true>(P.ops, vqc_ld(&sp->op_begin), vqc_ld(&sp->op_end), v.pb, a, a,
+            run_ops<R, K, 0, true>(P.ops, vqc_ld(&sp->op_begin), vqc_ld(&sp->op_end), v.pb, a, a,
                                          sh_tab, ps_tab, nullptr, q, lane, warp);
             if (last) {   // <Z_j> partials: one butterfly per warp (n <= 16 here)
                 R ez[16];
@@ -416,7 +416,7 @@ __global__ void __launch_bounds__(512) cluster_bwd_kernel(const __grid_constant_
                 } else {
                     cl_block_load<R, K>(a, psi_sa, slice, v.swb, sg);
                 }
-                run_ops<R, K, 0, false, true>(P.ops, vqc_ld(&sp->op_begin), vqc_ld(&sp->op_end), v.pb, a, a,
+                run_ops<R, K, 0, true>(P.ops, vqc_ld(&sp->op_begin), vqc_ld(&sp->op_end), v.pb, a, a,
                                              sh_tab, ps_tab, nullptr, q, lane, warp);
                 if (s + 1 == ns) break;
                 if (vqc_ld(&sp->nperm)) {
@@ -453,7 +453,7 @@ __global__ void __launch_bounds__(512) cluster_bwd_kernel(const __grid_constant_
                     cl_block_load<R, K>(l, lam_sa, slice, b2, s2);
                 }
             }
-            run_ops<R, K, 1, false, true>(P.ops, vqc_ld(&sp->op_begin), vqc_ld(&sp->op_end), v.pb, a, l,
+            run_ops<R, K, 1, true>(P.ops, vqc_ld(&sp->op_begin), vqc_ld(&sp->op_end), v.pb, a, l,
                                          sh_tab, ps_tab, acc_w, qa, lane, warp_a);
             if (s > 0) {   // back to the stage's input layout (load map)
                 if (vqc_ld(&sp->nperm)) {

@@ -463,16 +463,10 @@ __device__ __forceinline__ void rotate(C2<R> (&a)[1 << K], const R* e) {
     for (int p = 0; p < (1 << (K - 1)); ++p) {
         const int i0 = pair_lo<T>(p), i1 = i0 | (1 << T);
         const C2<R> u = a[i0], v = a[i1];
-        if constexpr (std::is_same<R, dd>::value) {
-            a[i0] = cm<R>(dot2(C, u.x, M, v.x), dot2(C, u.y, M, v.y));
-            a[i1] = cm<R>(dot2(S, u.x, C, v.x), dot2(S, u.y, C, v.y));
-        } else {
-            a[i0] = cm<R>(fma(C, u.x, M * v.x), fma(C, u.y, M * v.y));
-            a[i1] = cm<R>(fma(S, u.x, C * v.x), fma(S, u.y, C * v.y));
-        }
+        a[i0] = cm<R>(dot2(C, u.x, M, v.x), dot2(C, u.y, M, v.y));
+        a[i1] = cm<R>(dot2(S, u.x, C, v.x), dot2(S, u.y, C, v.y));
     }
 }
-
 
 // The runs of a stage, forward.
 template <typename R, int K, int EW>
@@ -559,8 +553,7 @@ __device__ __forceinline__ void backward_runs(const uint2* ops, unsigned pm, C2<
                 rotate<R, K, T_, true>(a, tp[T_] + 8);                  \
                 rotate<R, K, T_, true>(l, tp[T_] + 8);                  \
             } else {                                                    \
-                m1_entry<R, K, T_, true>(a, tp[T_]);                    \
-                m1_entry<R, K, T_, true>(l, tp[T_]);                    \
+                m1_back<R, K, T_>(a, l, tp[T_]);                        \
             }                                                           \
         }
     VQC_RUN(0) VQC_RUN(1) VQC_RUN(2) VQC_RUN(3)
@@ -584,7 +577,7 @@ __device__ __forceinline__ void stage_forward(const FStage* st, const FSeg* segs
     constexpr bool PHASES = PH2 && std::is_same<R, double>::value;
     constexpr bool DG = sizeof(R) == 8;
     if (op_switch<R>(st->kind)) {
-        run_ops<R, K, 0, false, true, PH2, EW>(reinterpret_cast<const DOp*>(ops), st->op_begin - op_base,
+        run_ops<R, K, 0, true, PH2, EW>(reinterpret_cast<const DOp*>(ops), st->op_begin - op_base,
                                                st->op_end - op_base, pb, a, a, sh_tab, ps_tab, nullptr, q, lane,
                                                warp_in_group);
         return;
@@ -614,7 +607,7 @@ __device__ __forceinline__ void stage_backward(const FStage* st, const FSeg* seg
     constexpr bool DG = sizeof(R) == 8;
     const int wg = q.wg;
     if (op_switch<R>(st->kind)) {
-        run_ops<R, K, 1, false, true, PH2, EW>(reinterpret_cast<const DOp*>(ops), st->op_begin - op_base,
+        run_ops<R, K, 1, true, PH2, EW>(reinterpret_cast<const DOp*>(ops), st->op_begin - op_base,
                                                st->op_end - op_base, pb, a, l, sh_tab, ps_tab, acc, q, lane,
                                                warp_in_group);
         return;

@@ -331,7 +331,7 @@ __global__ void __launch_bounds__(256, 2) pass_kernel(const __grid_constant__ PA
                     stage_forward<R, K, PH2, EntryWords<R>::value>(sp, segs, A.seg_begin, ops, A.op_begin, v.pb, a,
                                                                         sh_tab, ps_tab, dg, q, lane, warp_in_group);
                 else
-                    run_ops<R, K, 0, false, FULL, PH2>(reinterpret_cast<const DOp*>(ops), sp->op_begin - A.op_begin,
+                    run_ops<R, K, 0, FULL, PH2>(reinterpret_cast<const DOp*>(ops), sp->op_begin - A.op_begin,
                                                        sp->op_end - A.op_begin, v.pb, a, a, sh_tab, ps_tab, nullptr,
                                                        q, lane, warp_in_group);
                 if (s + 1 < nst || A.dst_psi) {
@@ -378,7 +378,7 @@ __global__ void __launch_bounds__(256, 2) pass_kernel(const __grid_constant__ PA
                     stage_backward<R, K, PH2>(sp, segs, A.seg_begin, ops, A.op_begin, v.pb, a, l, sh_tab, ps_tab, dg,
                                               acc, q, lane, warp_in_group);
                 else
-                    run_ops<R, K, 1, false, FULL, PH2>(reinterpret_cast<const DOp*>(ops), sp->op_begin - A.op_begin,
+                    run_ops<R, K, 1, FULL, PH2>(reinterpret_cast<const DOp*>(ops), sp->op_begin - A.op_begin,
                                                        sp->op_end - A.op_begin, v.pb, a, l, sh_tab, ps_tab, acc, q,
                                                        lane, warp_in_group);
                 if (s > 0 || A.dst_psi) {

@@ -7,13 +7,14 @@
 //   * single-qubit gates that meet consecutively on a qubit are fused into a
 //     run; consecutive constant factors of a run are pre-multiplied on the host
 //     in fp64 (Alg. 1: "precompute and cache" constant matrices);
-//   * two-qubit gates become CX (conditional swap), CZ (sign) or a diagonal
-//     two-qubit phase (CRZ, RZZ); SWAP is lowered to three CX;
+//   * two-qubit gates become CX (a permutation of basis states that no kernel
+//     applies: a change of frame, or folded into a store map), CZ (sign) or a
+//     diagonal two-qubit phase (CRZ, RZZ); SWAP is lowered to three CX;
 //   * the op list is cut into stages.  In a stage every thread of a sample's
 //     thread group holds a register block of 2^K amplitudes spanned by the
-//     stage's K "active" qubits; every non-diagonal op of the stage acts on
-//     active qubits only, diagonal ops and CX controls may use any qubit.
-//     Between stages the state goes through shared memory.
+//     stage's K "active" qubits (frame schedules: K directions); every
+//     non-diagonal op of the stage acts on these only, diagonal ops may use any
+//     qubit.  Between stages the state goes through shared memory.
 //
 // Amplitude addressing in shared memory (per sample, tile-local index u):
 //   slot(u) = sw(u) ^ h_sample,   sw(u) = u ^ (fold_G(u >> G) & (2^G - 1))
@@ -73,15 +74,15 @@ struct DOp {
 static_assert(sizeof(DOp) == 8, "DOp layout");
 
 // ---- stages ----------------------------------------------------------------
-// A stage loads each block through its load map (sigma, tau), applies its ops
-// and stores the block through its store map (sigma_st, tau_st).  On the
-// resident path the compiler folds CX gates into the store map instead of
-// emitting them as ops: a CX is a permutation of basis states, linear over
-// GF(2) in the amplitude index, so storing amplitude k of the block at the slot
-// of pi(k) applies it at no arithmetic cost (pi = the stage's absorbed CX gates
-// in time order; every op of the stage that follows one of them in time acts on
-// other qubits, so it commutes with pi).  Without absorbed gates the two maps
-// are equal.
+// Stages of the cluster path and of exported schedules, on register blocks of K qubits
+// (the resident and HBM-tiled kernels run the frame schedules of frame.h).  A stage
+// loads each block through its load map (sigma, tau), applies its ops and stores the
+// block through its store map (sigma_st, tau_st).  CX gates are folded into the store
+// map: a CX is a permutation of basis states, linear over GF(2) in the amplitude
+// index, so storing amplitude k of the block at the slot of pi(k) applies it at no
+// arithmetic cost (pi = the stage's absorbed CX gates in time order; every op of the
+// stage that follows one of them in time acts on other qubits, so it commutes with
+// pi).  Without absorbed gates the two maps are equal.
 struct DStage {
     int32_t op_begin, op_end;
     int32_t sigma[kMaxK];             // load: swizzled slot offset of local bit j

@@ -214,7 +214,7 @@ __global__ void __launch_bounds__(512) sweep_kernel(const __grid_constant__ KArg
                 if constexpr (FULL)
                     stage_forward<R, K, PH2, EW>(sp, segs, 0, ops, 0, v.pb, a, sh_tab, ps_tab, dg, q, lane, warp_in_group);
                 else
-                    run_ops<R, K, 0, false, FULL, PH2, EW>(P.ops, sp->op_begin, sp->op_end, v.pb, a, a, sh_tab,
+                    run_ops<R, K, 0, FULL, PH2, EW>(P.ops, sp->op_begin, sp->op_end, v.pb, a, a, sh_tab,
                                                            ps_tab, nullptr, q, lane, warp_in_group);
                 if (s + 1 < ns || (MODE == 0 && A.state_out)) {
                     frame_store<R, K>(a, psi_t, v.off, sb);
@@ -281,7 +281,7 @@ __global__ void __launch_bounds__(512) sweep_kernel(const __grid_constant__ KArg
                 if constexpr (FULL)
                     stage_backward<R, K, PH2>(sp, segs, 0, ops, 0, v.pb, a, l, sh_tab, ps_tab, dg, acc, q, lane, warp_in_group);
                 else
-                    run_ops<R, K, 1, false, FULL, PH2, EW>(P.ops, sp->op_begin, sp->op_end, v.pb, a, l, sh_tab,
+                    run_ops<R, K, 1, FULL, PH2, EW>(P.ops, sp->op_begin, sp->op_end, v.pb, a, l, sh_tab,
                                                            ps_tab, acc, q, lane, warp_in_group);
                 if (s > 0) {
                     frame_store<R, K>(a, psi_t, v.off, sb);

@@ -13,8 +13,8 @@
 //
 // Execution model ("resident" path).  A sample's state lives in shared
 // memory.  A group of T = 2^(n-K) threads owns one sample; in each stage a
-// thread loads the 2^K amplitudes spanned by the stage's K active qubits into
-// registers (its block; the other n-K index bits come from the thread index),
+// thread loads the 2^K amplitudes spanned by the stage's K directions (frame.h)
+// into registers (its block; the other n-K index bits come from the thread index),
 // applies all of the stage's ops there, and stores the block back.  Blocks of
 // different threads are disjoint, so one group barrier per stage suffices.
 // Gate matrices are evaluated once per sample (sincos once per angle) into a
@@ -122,14 +122,6 @@ __device__ __forceinline__ M2<R> mident() {
 // or, when too large, in global memory.
 template <typename T>
 __device__ __forceinline__ T vqc_ld(const T* p) { return *p; }
-
-// Copy [src, src + bytes) (16-byte multiple) into shared memory; all loads are
-// independent, so a CTA pulls the whole plan in about one memory latency.
-__device__ __forceinline__ void copy_region(unsigned char* dst, const unsigned char* src, int bytes) {
-    const uint4* s = reinterpret_cast<const uint4*>(src);
-    uint4* d = reinterpret_cast<uint4*>(dst);
-    for (int i = threadIdx.x; i < bytes / 16; i += blockDim.x) d[i] = s[i];
-}
 
 // Asynchronous global -> shared copies (cp.async, 4/8/16 bytes, both addresses
 // aligned to the size).  They hold no registers while in flight, so a thread
@@ -530,8 +522,14 @@ __device__ __forceinline__ void m1_t3(const C2<R> (&ps)[1 << K], const C2<R> (&l
 // so a complex multiply-add is two FFMA2 and a pair update eight.  (The form
 // with the table's (Re m, Re m), (-Im m, Im m) pairs needs the swapped state
 // pair (u.im, u.re) instead and measured 2-8% slower.)
-template <int K, int T>
-__device__ __forceinline__ void m1_apply_f2w(float2 (&a)[1 << K], const float* wp) {
+//
+// Four pairs of a state at a time: the first product of all of them, then the second,
+// and so on, since each waits for the one before it.  (Pair by pair the compiler kept
+// most chains whole: 16-qubit step, B = 512, 6.41 ms against 6.24; BOTH
+// states of a backward stage together, eight pairs at a time, take another 1% off the
+// 12-qubit resident step, 1.69 -> 1.68 ms at B = 4096.)
+template <int K, int T, bool BOTH>
+__device__ __forceinline__ void m1_apply_f2w(float2 (&a)[1 << K], float2 (&l)[1 << K], const float* wp) {
     const float4 w0 = *reinterpret_cast<const float4*>(wp);
     const float4 w1 = *reinterpret_cast<const float4*>(wp + 4);
     const float4 w2 = *reinterpret_cast<const float4*>(wp + 8);
@@ -540,23 +538,40 @@ __device__ __forceinline__ void m1_apply_f2w(float2 (&a)[1 << K], const float* w
     const float2 br = make_float2(w1.x, w1.y), bi = make_float2(w1.z, w1.w);
     const float2 cr = make_float2(w2.x, w2.y), ci = make_float2(w2.z, w2.w);
     const float2 dr = make_float2(w3.x, w3.y), di = make_float2(w3.z, w3.w);
+    constexpr int N = 1 << (K - 1), H = N < 4 ? N : 4, GR = BOTH ? 2 * H : H;
 #pragma unroll
-    for (int p = 0; p < (1 << (K - 1)); ++p) {
-        const int i0 = pair_lo<T>(p), i1 = i0 | (1 << T);
-        const float2 u = a[i0], v = a[i1];
+    for (int p0 = 0; p0 < N; p0 += H) {
+        float2 u[GR], v[GR], nu[GR], nv[GR];
+#pragma unroll
+        for (int g = 0; g < GR; ++g) {
+            const int i0 = pair_lo<T>(p0 + g % H), i1 = i0 | (1 << T);
+            u[g] = g < H ? a[i0] : l[i0];
+            v[g] = g < H ? a[i1] : l[i1];
+        }
         // entries hold (m, i m): m u = u.re (m) + u.im (i m)
-        const float2 ux = make_float2(u.x, u.x), uy = make_float2(u.y, u.y);
-        const float2 vx = make_float2(v.x, v.x), vy = make_float2(v.y, v.y);
-        float2 nu = __fmul2_rn(ar, ux);
-        nu = __ffma2_rn(ai, uy, nu);
-        nu = __ffma2_rn(br, vx, nu);
-        nu = __ffma2_rn(bi, vy, nu);
-        float2 nv = __fmul2_rn(cr, ux);
-        nv = __ffma2_rn(ci, uy, nv);
-        nv = __ffma2_rn(dr, vx, nv);
-        nv = __ffma2_rn(di, vy, nv);
-        a[i0] = nu;
-        a[i1] = nv;
+#pragma unroll
+        for (int g = 0; g < GR; ++g) {
+            nu[g] = __fmul2_rn(ar, make_float2(u[g].x, u[g].x));
+            nv[g] = __fmul2_rn(cr, make_float2(u[g].x, u[g].x));
+        }
+#pragma unroll
+        for (int g = 0; g < GR; ++g) {
+            nu[g] = __ffma2_rn(ai, make_float2(u[g].y, u[g].y), nu[g]);
+            nv[g] = __ffma2_rn(ci, make_float2(u[g].y, u[g].y), nv[g]);
+        }
+#pragma unroll
+        for (int g = 0; g < GR; ++g) {
+            nu[g] = __ffma2_rn(br, make_float2(v[g].x, v[g].x), nu[g]);
+            nv[g] = __ffma2_rn(dr, make_float2(v[g].x, v[g].x), nv[g]);
+        }
+#pragma unroll
+        for (int g = 0; g < GR; ++g) {
+            const int i0 = pair_lo<T>(p0 + g % H), i1 = i0 | (1 << T);
+            nu[g] = __ffma2_rn(bi, make_float2(v[g].y, v[g].y), nu[g]);
+            nv[g] = __ffma2_rn(di, make_float2(v[g].y, v[g].y), nv[g]);
+            (g < H ? a : l)[i0] = nu[g];
+            (g < H ? a : l)[i1] = nv[g];
+        }
     }
 }
 
@@ -564,7 +579,7 @@ __device__ __forceinline__ void m1_apply_f2w(float2 (&a)[1 << K], const float* w
 template <typename R, int K, int T, bool ADJ>
 __device__ __forceinline__ void m1_entry(C2<R> (&a)[1 << K], const R* tp) {
     if constexpr (sizeof(R) == 4) {
-        m1_apply_f2w<K, T>(a, tp + (ADJ ? 16 : 0));
+        m1_apply_f2w<K, T, false>(a, a, tp + (ADJ ? 16 : 0));
     } else {
         M2<R> m = load_m2<R>(tp);
         if (ADJ) m = mdag<R>(m);
@@ -572,27 +587,14 @@ __device__ __forceinline__ void m1_entry(C2<R> (&a)[1 << K], const R* tp) {
     }
 }
 
-// X on local T when the predicate holds (control outside the block).
+// U^dag of the entry at tp on psi and lam.
 template <typename R, int K, int T>
-__device__ __forceinline__ void x_pred(C2<R> (&a)[1 << K], bool p) {
-#pragma unroll
-    for (int q = 0; q < (1 << (K - 1)); ++q) {
-        const int i0 = pair_lo<T>(q), i1 = i0 | (1 << T);
-        C2<R> u = a[i0], v = a[i1];
-        a[i0] = p ? v : u;
-        a[i1] = p ? u : v;
-    }
-}
-
-template <typename R, int K>
-__device__ __forceinline__ void x_pred_dispatch(int t, C2<R> (&a)[1 << K], bool p) {
-    switch (t) {
-    case 0: x_pred<R, K, 0>(a, p); break;
-    case 1: if constexpr (K > 1) x_pred<R, K, 1>(a, p); break;
-    case 2: if constexpr (K > 2) x_pred<R, K, 2>(a, p); break;
-    case 3: if constexpr (K > 3) x_pred<R, K, 3>(a, p); break;
-    case 4: if constexpr (K > 4) x_pred<R, K, 4>(a, p); break;
-    default: break;
+__device__ __forceinline__ void m1_back(C2<R> (&a)[1 << K], C2<R> (&l)[1 << K], const R* tp) {
+    if constexpr (sizeof(R) == 4) {
+        m1_apply_f2w<K, T, true>(a, l, tp + 16);
+    } else {
+        m1_entry<R, K, T, true>(a, tp);
+        m1_entry<R, K, T, true>(l, tp);
     }
 }
 
@@ -609,45 +611,6 @@ __device__ __forceinline__ void z1_pred(C2<R> (&a)[1 << K], bool p) {
 #pragma unroll
     for (int r = 0; r < (1 << K); ++r)
         if ((r >> A) & 1) a[r] = cm<R>(s * a[r].x, s * a[r].y);
-}
-
-template <typename R, int K>
-__device__ __forceinline__ void cz_dispatch(int ra, int rb, uint32_t pb, C2<R> (&a)[1 << K]) {
-    if (ra >= kRefPhys && rb >= kRefPhys) {
-        const bool p = ((pb >> (ra - kRefPhys)) & (pb >> (rb - kRefPhys)) & 1u) != 0;
-        const R s = p ? R(-1) : R(1);
-#pragma unroll
-        for (int r = 0; r < (1 << K); ++r) a[r] = cm<R>(s * a[r].x, s * a[r].y);
-        return;
-    }
-    if (ra >= kRefPhys || rb >= kRefPhys) {
-        const int l = ra >= kRefPhys ? rb : ra;
-        const int ph = ra >= kRefPhys ? ra : rb;
-        const bool p = ((pb >> (ph - kRefPhys)) & 1u) != 0;
-        switch (l) {
-        case 0: z1_pred<R, K, 0>(a, p); break;
-        case 1: if constexpr (K > 1) z1_pred<R, K, 1>(a, p); break;
-        case 2: if constexpr (K > 2) z1_pred<R, K, 2>(a, p); break;
-        case 3: if constexpr (K > 3) z1_pred<R, K, 3>(a, p); break;
-        case 4: if constexpr (K > 4) z1_pred<R, K, 4>(a, p); break;
-        default: break;
-        }
-        return;
-    }
-    const int lo = ra < rb ? ra : rb, hi = ra < rb ? rb : ra;
-#define VQC_ZCASE(A_, B_) \
-    case A_ * 8 + B_: if constexpr (A_ < K && B_ < K) z2_ll<R, K, A_, B_>(a); break;
-    switch (lo * 8 + hi) {
-        VQC_ZCASE(0, 1) VQC_ZCASE(0, 2) VQC_ZCASE(0, 3) VQC_ZCASE(0, 4)
-        VQC_ZCASE(1, 2) VQC_ZCASE(1, 3) VQC_ZCASE(1, 4)
-        VQC_ZCASE(2, 3) VQC_ZCASE(2, 4) VQC_ZCASE(3, 4)
-        default: break;
-    }
-#undef VQC_ZCASE
-}
-
-__device__ __forceinline__ int refbit(int ref, int r, uint32_t pb) {
-    return ref >= kRefPhys ? (int)((pb >> (ref - kRefPhys)) & 1u) : ((r >> ref) & 1);
 }
 
 // ---------------------------------------------------------------- reductions
@@ -956,19 +919,12 @@ __device__ __forceinline__ bool physbit(uint32_t pb, int ref) {
 // Apply op `raw` to the block(s).  MODE 0: forward on a.  MODE 1: backward --
 // accumulate the op's gradient slot, then un-apply on a (psi) and l (lam).
 // One switch over the dispatch code; every case has fixed local positions.
-// WITH_CX: the schedule may hold CX ops (HBM passes); resident schedules fold
-// every CX into stage store maps, and leaving those cases out of the switch
-// keeps the other cases' register allocation tight.  A pass schedule holds
-// only CX gates whose control lies outside the tile (the compiler folds every
-// CX with both qubits in the tile into a store map), so the switch has no case
-// for a local control: its code alone made the pass kernels spill (about 2.5x
-// the spill traffic under the 128-register cap).
 // WITH_PH2: the schedule may hold diagonal two-qubit phase ops (CRZ, RZZ).
 // Kernels for plans without them are instantiated with the cases left out:
 // their register allocation then needs fewer spills (measured 8-11% faster on
 // the 12-qubit resident sweeps and the 16-qubit forward passes); the launch
 // code picks the instantiation from the plan.
-template <typename R, int K, int MODE, bool WITH_CX, bool FULL, bool WITH_PH2 = true, int EW = EntryWords<R>::value>
+template <typename R, int K, int MODE, bool FULL, bool WITH_PH2 = true, int EW = EntryWords<R>::value>
 __device__ __forceinline__ void apply_op(uint2 raw, uint32_t pb, C2<R> (&a)[1 << K],
                                          C2<R> (&l)[1 << K], const R* sh_tab, const R* ps_tab,
                                          R* acc, const Geo& q, int lane, int warp_in_group,
@@ -1014,16 +970,6 @@ __device__ __forceinline__ void apply_op(uint2 raw, uint32_t pb, C2<R> (&a)[1 <<
         break;
         VQC_M1(0) VQC_M1(1) VQC_M1(2) VQC_M1(3) VQC_M1(4)
 #undef VQC_M1
-#define VQC_CXPL(T_)                                                                 \
-    case DC_CX_PL + T_:                                                              \
-        if constexpr (WITH_CX && T_ < K) {                                           \
-            const bool p_ = physbit(pb, ra);                                         \
-            x_pred<R, K, T_>(a, p_);                                                 \
-            if (MODE == 1) x_pred<R, K, T_>(l, p_);                                  \
-        }                                                                            \
-        break;
-        VQC_CXPL(0) VQC_CXPL(1) VQC_CXPL(2) VQC_CXPL(3) VQC_CXPL(4)
-#undef VQC_CXPL
 #define VQC_CZLL(A_, B_)                                                             \
     case DC_CZ_LL + cz_pair_index(A_, B_):                                           \
         if constexpr (A_ < K && B_ < K) {                                            \
@@ -1081,7 +1027,7 @@ __device__ __forceinline__ void apply_op(uint2 raw, uint32_t pb, C2<R> (&a)[1 <<
 // Run ops [ob, oe) of a stage (forward: in order; backward: reversed).  The
 // descriptor is read when the op starts: keeping a prefetched one live across
 // the dispatch switch costs more registers than the load latency it hides.
-template <typename R, int K, int MODE, bool WITH_CX, bool FULL, bool WITH_PH2 = true, int EW = EntryWords<R>::value>
+template <typename R, int K, int MODE, bool FULL, bool WITH_PH2 = true, int EW = EntryWords<R>::value>
 __device__ __forceinline__ void run_ops(const DOp* ops, int ob, int oe, uint32_t pb,
                                         C2<R> (&a)[1 << K], C2<R> (&l)[1 << K], const R* sh_tab,
                                         const R* ps_tab, R* acc, const Geo& q, int lane,
@@ -1089,11 +1035,11 @@ __device__ __forceinline__ void run_ops(const DOp* ops, int ob, int oe, uint32_t
     const uint2* op2 = reinterpret_cast<const uint2*>(ops);
     if (MODE == 0) {
         for (int o = ob; o < oe; ++o)
-            apply_op<R, K, MODE, WITH_CX, FULL, WITH_PH2, EW>(vqc_ld(op2 + o), pb, a, l, sh_tab, ps_tab, acc, q, lane,
+            apply_op<R, K, MODE, FULL, WITH_PH2, EW>(vqc_ld(op2 + o), pb, a, l, sh_tab, ps_tab, acc, q, lane,
                                           warp_in_group, acc_add);
     } else {
         for (int o = oe - 1; o >= ob; --o)
-            apply_op<R, K, MODE, WITH_CX, FULL, WITH_PH2, EW>(vqc_ld(op2 + o), pb, a, l, sh_tab, ps_tab, acc, q, lane,
+            apply_op<R, K, MODE, FULL, WITH_PH2, EW>(vqc_ld(op2 + o), pb, a, l, sh_tab, ps_tab, acc, q, lane,
                                           warp_in_group, acc_add);
     }
 }
@@ -1179,47 +1125,6 @@ __device__ __forceinline__ int warp_reduce_scatter(R (&v)[NV], int lane) {
 #pragma unroll
     for (; m >= 1; m >>= 1) v[0] += shx<R>(v[0], m, 0xffffffffu);
     return idx;
-}
-
-// Per-warp partial sums of E_j = sum (-1)^{bit j} |a|^2 over this group's
-// blocks, written to red[warp_in_group * n + j].
-template <typename R, int K>
-__device__ __forceinline__ void expz_partials(const DStage* sp, uint32_t pb,
-                                              const C2<R> (&a)[1 << K], int n, R* red,
-                                              const Geo& q, int warp_in_group, bool add = false) {
-    R ptot = 0;
-    R dloc[K];
-#pragma unroll
-    for (int j = 0; j < K; ++j) dloc[j] = 0;
-#pragma unroll
-    for (int r = 0; r < (1 << K); ++r) {
-        const R pr = fma(a[r].x, a[r].x, a[r].y * a[r].y);
-        ptot += pr;
-#pragma unroll
-        for (int j = 0; j < K; ++j) dloc[j] += ((r >> j) & 1) ? -pr : pr;
-    }
-    uint32_t actmask = 0;
-    int aq[K];
-#pragma unroll
-    for (int j = 0; j < K; ++j) {
-        aq[j] = vqc_ld(&sp->active[j]);
-        actmask |= 1u << aq[j];
-    }
-    for (int j = 0; j < n; ++j) {
-        R val;
-        if ((actmask >> j) & 1) {
-            val = 0;
-#pragma unroll
-            for (int k = 0; k < K; ++k) if (aq[k] == j) val = dloc[k];
-        } else {
-            val = ((pb >> j) & 1u) ? -ptot : ptot;
-        }
-        val = reduce1<R>(val, q.lanes, q.mask);
-        if ((q.t & (q.lanes - 1)) == 0) {
-            R* d = red + warp_in_group * n + j;
-            *d = add ? *d + val : val;
-        }
-    }
 }
 
 // Gradient terms of one accumulator slot (summed over the wg per-warp

@@ -280,11 +280,11 @@ __global__ void __launch_bounds__(256, 2) fp32_stage_kernel(const __grid_constan
             a[2 * i + 1] = make_float2(x.z, x.w);
         }
         for (int rep = 0; rep < A.repeats; ++rep) {
-            m1_apply_f2w<5, 0>(a, tab[0]);
-            m1_apply_f2w<5, 1>(a, tab[1]);
-            m1_apply_f2w<5, 2>(a, tab[2]);
-            m1_apply_f2w<5, 3>(a, tab[3]);
-            m1_apply_f2w<5, 4>(a, tab[4]);
+            m1_apply_f2w<5, 0, false>(a, a, tab[0]);
+            m1_apply_f2w<5, 1, false>(a, a, tab[1]);
+            m1_apply_f2w<5, 2, false>(a, a, tab[2]);
+            m1_apply_f2w<5, 3, false>(a, a, tab[3]);
+            m1_apply_f2w<5, 4, false>(a, a, tab[4]);
         }
         float4* dst = reinterpret_cast<float4*>(A.out + row * 32);
 #pragma unroll
