@@ -281,8 +281,10 @@ vqc_status vqc_probabilities(const vqc_plan* plan, int32_t batch, const void* x,
  * counterpart; it is a deployment convenience of this library.
  *   Arguments, outputs and results are those of vqc_backward.  The scratch is
  *   a fixed array of VQC_NOALLOC_SCRATCH_BYTES inside the library; a batch
- *   whose scratch need (vqc_workspace_bytes(plan, batch, 1)) exceeds it is
- *   rejected with VQC_ERR_WORKSPACE and a message giving both sizes.
+ *   whose scratch need (vqc_workspace_bytes(plan, batch, 1); for HBM passes the
+ *   states, the gradient terms, the per-sample matrices and one sum per gradient
+ *   slot and tile) exceeds it is rejected with VQC_ERR_WORKSPACE and a message
+ *   giving both sizes.
  *   No cudaMalloc, cudaFree or allocating library call is made.  Each call
  *   clears the array's control block on `stream` before its launch; all calls
  *   on a device share the array, so calls that overlap on the GPU race and must

@@ -71,7 +71,7 @@ struct HostPlan {
     void* dbuf = nullptr;
     size_t dbytes = 0;
     size_t dev_entries = 0, dev_ps_list = 0, dev_sh_list = 0, dev_consts = 0, dev_cmat = 0, dev_cang = 0;
-    size_t dev_xocc_ptr = 0, dev_xocc = 0, dev_wocc_ptr = 0, dev_wocc = 0, dev_accs = 0;
+    size_t dev_xocc_ptr = 0, dev_xocc = 0, dev_wocc_ptr = 0, dev_wocc = 0, dev_accs = 0, dev_iota = 0;
     unsigned* dev_error = nullptr;        // device error word (kernel self-checks)
     size_t dev_tab_begin = 0, dev_tab_end = 0;   // [entries .. wocc] in the blob
 };

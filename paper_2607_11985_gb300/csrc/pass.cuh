@@ -436,31 +436,34 @@ template <typename R>
 __global__ void __launch_bounds__(256) run_tables(const DEntry* entries, const int32_t* ps_list,
                                                   const int32_t* sh_list, const DConst* consts, const R* cang,
                                                   const R* cmat, const St<R>* x, int Px, const St<R>* w, int B,
-                                                  int n_ps, int n_sh, R* out_ps, R* out_sh) {
+                                                  int n_ps, int n_sh, const int32_t* ps_sel, const int32_t* sh_sel,
+                                                  R* out_ps, R* out_sh) {
     grid_dep_wait();
     grid_dep_launch();
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < (long long)B * n_ps + n_sh;
          i += (long long)gridDim.x * blockDim.x) {
         if (i < n_sh) {
-            const DEntry e = entries[vqc_ld(&sh_list[i])];
+            const DEntry e = entries[vqc_ld(&sh_list[sh_sel ? vqc_ld(&sh_sel[i]) : i])];
             eval_entry<R>(e, consts, static_cast<const St<R>*>(nullptr), w, cang, cmat,
-                          out_sh + (size_t)e.slot * EntryWords<R>::value);
+                          out_sh + (size_t)(sh_sel ? (int)i : e.slot) * EntryWords<R>::value);
             continue;
         }
         const long long j = i - n_sh, b = j / n_ps;
-        const DEntry e = entries[vqc_ld(&ps_list[j % n_ps])];
+        const int k = (int)(j % n_ps);
+        const DEntry e = entries[vqc_ld(&ps_list[ps_sel ? vqc_ld(&ps_sel[k]) : k])];
         eval_entry<R>(e, consts, x + b * Px, w, cang, cmat,
-                      out_ps + ((size_t)b * n_ps + e.slot) * EntryWords<R>::value);
+                      out_ps + ((size_t)b * n_ps + (ps_sel ? k : e.slot)) * EntryWords<R>::value);
     }
 }
 
 // Gradient terms of every accumulator of every sample: the sample's per-tile
 // rho sums added in tile order, then the constituent walk of acc_terms (one
 // partial), in the kernels' arithmetic R (the plan's constants are stored as R:
-// (hi, lo) float pairs for double-float plans).  terms: [B, n_terms].
+// (hi, lo) float pairs for double-float plans).  sel: the accumulators that rho holds
+// (nullptr: all of them).  terms: [B, n_terms].
 template <typename R>
 __global__ void __launch_bounds__(256) reduce_terms(const St<R>* rho, int B, int ntiles, int n_accs,
-                                                    const DAcc* accs, const DEntry* entries,
+                                                    const int32_t* sel, const DAcc* accs, const DEntry* entries,
                                                     const DConst* consts, const R* cang, const R* cmat,
                                                     const St<R>* x, int Px, const St<R>* w, int n_terms,
                                                     St<R>* terms) {
@@ -477,7 +480,7 @@ __global__ void __launch_bounds__(256) reduce_terms(const St<R>* rho, int B, int
             t[1] += as_r<R>(r[1]);
             t[2] += as_r<R>(r[2]);
         }
-        const DAcc ac = accs[k];
+        const DAcc ac = accs[sel ? vqc_ld(&sel[k]) : k];
         acc_terms<R>(ac, entries[ac.entry], t, 1, consts,
                      x ? x + b * Px : static_cast<const St<R>*>(nullptr), w, cang, cmat, terms + b * n_terms);
     }

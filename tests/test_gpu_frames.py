@@ -191,6 +191,55 @@ def test_noalloc_takes_clusters_beyond_its_scratch():
     assert maxerr(dw.cpu().numpy(), dw2) <= row.sum()
 
 
+@pytest.mark.parametrize("dtype,n", [("c64", 15), ("c128", 14), ("c128df", 14)])
+@pytest.mark.parametrize("saved", [True, False])
+def test_noalloc_takes_one_pass_at_a_time(monkeypatch, dtype, n, saved):
+    # the rho sums and table entries of the whole circuit exceed the built-in scratch,
+    # those of a pass do not: the same sums in the same order, bit by bit
+    monkeypatch.setenv("VQC_FORCE_PATH", "hbm")
+    spec = mixed(n, ("RX", "RY", "H", "CX"), layers=160 if dtype == "c64" else 115)
+    spec.add("RZZ", (0, n - 1), (("x", 1),))
+    c = C(spec, dtype)
+    w_, _ = draw(spec, 1, dtype, 7350)
+    assert B.vqc_workspace_bytes(c.plan, 1, 1) > 1 << 20
+    x, w, gE = dev(w_.x, dtype), dev(w_.w, dtype), dev(w_.gE, dtype)
+    st = c.forward(x, w, want_state=True)[1] if saved else None
+    dx_ref, dw_ref = c.backward(x, w, gE, psi_final=st)
+    dx, dw = torch.empty_like(x), torch.empty_like(w)
+    B.vqc_backward_noalloc(c.plan, 1, x.data_ptr(), w.data_ptr(), None, st.data_ptr() if saved else None,
+                           gE.data_ptr(), dx.data_ptr(), dw.data_ptr(), torch.cuda.current_stream().cuda_stream)
+    torch.cuda.synchronize()
+    assert torch.equal(dx, dx_ref) and torch.equal(dw, dw_ref)
+
+
+def test_noalloc_takes_fewer_ctas():
+    # dw partials of a full grid a little beyond the built-in scratch
+    num_w = 200
+    while True:
+        spec = wl.CircuitSpec(6, 6, num_w)
+        for q in range(6):
+            spec.add("RY", (q,), [("x", q)])
+        for j in range(num_w):
+            spec.add("RX", (j % 6,), [("w", j)])
+        c = C(spec, "c64")
+        need = B.vqc_workspace_bytes(c.plan, 4096, 1)
+        if need > 1 << 20:
+            break
+        num_w = num_w * 5 // 4
+    assert need < 2 << 20
+    w_, _ = draw(spec, 4096, "c64", 7370)
+    x, w, gE = dev(w_.x, "c64"), dev(w_.w, "c64"), dev(w_.gE, "c64")
+    dx_ref, dw_ref = c.backward(x, w, gE)
+    dx, dw = torch.empty_like(x), torch.empty_like(w)
+    B.vqc_backward_noalloc(c.plan, 4096, x.data_ptr(), w.data_ptr(), None, None, gE.data_ptr(), dx.data_ptr(),
+                           dw.data_ptr(), torch.cuda.current_stream().cuda_stream)
+    torch.cuda.synchronize()
+    assert torch.equal(dx, dx_ref)
+    # the same terms in another order: each of at most 4096 additions rounds by u
+    bound = 2 * 4096 * U["c64"] * np.abs(w_.gE).sum()
+    assert maxerr(dw.cpu().numpy(), dw_ref.cpu().numpy()) <= bound
+
+
 # runs of every factored form (rotation alone, a diagonal on either side or both, a
 # diagonal run), at angles where an entry of the matrix vanishes; groups below a warp
 # keep the 2x2 updates
