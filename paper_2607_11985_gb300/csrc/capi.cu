@@ -97,14 +97,16 @@ vqc_status allow_max_smem(const void* fn, int dev, int smem_optin) {
 }
 
 // mode 2: the backward with the forward sweep and E inside (vqc_forward_backward)
-const void* kernel_ptr(int dtype, bool dfloat, int mode, int K, bool full, bool ph2) {
+const void* kernel_ptr(int dtype, bool dfloat, int mode, int K, bool full, bool ph2,
+                       bool factored) {
     // complex64 sweeps of plans without CRZ / RZZ: the instantiations without
     // the phase cases (fewer spills)
     if (!dfloat && dtype == VQC_C64 && !ph2)
         return mode == 0 ? sweep_ptr_f32_fwd_nph(K, full)
              : mode == 1 ? sweep_ptr_f32_bwd_nph(K, full) : sweep_ptr_f32_fused_nph(K, full);
     if (dfloat)
-        return mode == 2 ? sweep_ptr_dd_fused(K, full) : mode == 0 ? sweep_ptr_dd_fwd(K, full) : sweep_ptr_dd_bwd(K, full);
+        return mode == 2 ? sweep_ptr_dd_fused(K, full, factored)
+             : mode == 0 ? sweep_ptr_dd_fwd(K, full, factored) : sweep_ptr_dd_bwd(K, full, factored);
     if (mode == 2) return dtype == VQC_C64 ? sweep_ptr_f32_fused(K, full) : sweep_ptr_f64_fused(K, full);
     if (full) {
         if (dtype == VQC_C64) return mode == 0 ? sweep_ptr_f32_fwd(K) : sweep_ptr_f32_bwd(K);
@@ -213,6 +215,18 @@ int choose_k(const HostPlan& p, int mode, int B, int sms) {
     return K;
 }
 
+// Double-float resident sweeps with factored stages: circuits without CRZ / RZZ (whose
+// stages take 2x2 updates; 9-qubit QAOA x 1600, 8 layers, forward 1036 us with the
+// factors beside them, 442 without), except small forwards of few stages, where the
+// factors and diagonals of a call, a chain of FP64 operations, take longer than they
+// save (RX RY RZ layers, CX ring, forward, factored / not: 8 qubits x 100, 1 layer 25 /
+// 22 us, 8 layers 72 / 77; 11 qubits x 1600, 1 layer 185 / 214; 12 x 100, 1 layer 47 / 54).
+bool factors_pay(const HostPlan& p, int mode, int B, const FrameSchedule& f, int sms) {
+    if (p.has_ph2) return false;
+    const bool small = p.n <= 11 && (double)B * std::ldexp(1.0, p.n) <= sms * 8192.0;
+    return mode == 1 || f.passes[0].ndg == 0 || !small || f.stages.size() >= 12;
+}
+
 vqc_status plan_launch_uncached(const HostPlan& p, int launch_mode, int B, Launch& L) {
     // mode 2 (fused) has the backward's schedule and layout, its own kernel
     const int mode = launch_mode == 2 ? 1 : launch_mode;
@@ -232,12 +246,13 @@ vqc_status plan_launch_uncached(const HostPlan& p, int launch_mode, int B, Launc
     L.wg = L.T > 32 ? L.T / 32 : 1;
     // Shared memory: a fixed part per CTA and a part per resident sample.
     const size_t dim = (size_t)1 << p.n;
-    const size_t ew = entry_reals(dbl, p.dfloat && L.T >= 32) / (mode == 0 && !dbl ? 2 : 1);   // ResidentWords
+    const bool factored = p.dfloat && L.T >= 32 && factors_pay(p, mode, B, *L.f, di.sms);
+    const size_t ew = entry_reals(dbl, factored) / (mode == 0 && !dbl ? 2 : 1);   // ResidentWords
     const size_t io = (size_t)8 << L.K;   // slot offsets of the state copies
     const size_t fixed = align16((size_t)p.n_sh * ew * rs) + align16(mode == 1 ? (size_t)p.num_w * rs : 0) +
                          align16((size_t)p.num_w * rs) + io + 10 * 16;
     // diagonal tables: two-local phases, and double-float's own (complex128 schedules count both)
-    L.ndg = L.T >= 32 && dbl && (p.dfloat || p.has_ph2) ? L.f->passes[0].ndg : 0;
+    L.ndg = L.T >= 32 && dbl && (p.dfloat ? factored : p.has_ph2) ? L.f->passes[0].ndg : 0;
     const size_t dgb = ((size_t)L.ndg << L.K) * cs;
     const size_t per_sample = dgb + (size_t)p.n_ps * ew * rs + dim * cs * (mode == 1 ? 2 : 1) +
                               (size_t)(p.num_x + p.n) * rs +
@@ -280,7 +295,7 @@ vqc_status plan_launch_uncached(const HostPlan& p, int launch_mode, int B, Launc
     L.sm_red = take((size_t)L.S * L.wg * p.n * rs);   // <Z> partials (forward, or recompute with E)
     L.sm_w = take((size_t)p.num_w * rs);
     L.sm_xg = take((size_t)L.S * (p.num_x + p.n) * rs);
-    L.fn = kernel_ptr(p.dtype, p.dfloat, launch_mode, L.K, L.T >= 32, p.has_ph2);
+    L.fn = kernel_ptr(p.dtype, p.dfloat, launch_mode, L.K, L.T >= 32, p.has_ph2, factored);
     if (!L.fn) return fail(VQC_ERR_UNSUPPORTED, "kernel not instantiated for this K");
     st = allow_max_smem(L.fn, dev, di.smem_optin);
     if (st != VQC_OK) return st;

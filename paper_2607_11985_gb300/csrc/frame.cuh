@@ -186,13 +186,14 @@ __device__ __forceinline__ void lambda_frame(const uint8_t* lmask, uint32_t pbf,
 // rings in double-float 1.60 -> 1.44).  Two kinds of stages take the op switch instead:
 // double-float ones with phases, whose collected factors round alike for a whole block
 // (error of <Z> of a 15-qubit random circuit 4.4e-14 -> 6.3e-14; 2.07 -> 1.49 ms on
-// 18-qubit RZZ rings, not kept), and complex64 ones with diagonal ops, where a
-// multiplication is cheap beside the walk over the group (13-qubit random circuit 216
+// 18-qubit RZZ rings, not kept; resident kernels of such circuits take 2x2 updates in
+// every stage), and complex64 ones with diagonal ops, where a
+// multiplication is cheap beside the walk over the group (scalar phases: 13-qubit random circuit 216
 // us, 247 in rounds; 15-qubit RZZ rings 797 us against 835).
-template <typename R>
+template <typename R, bool PH2>
 __device__ __forceinline__ bool op_switch(unsigned kind) {
     return std::is_same<R, float>::value ? !(kind & kStagePure)
-                                         : std::is_same<R, dd>::value && (kind & kStagePhases);
+                                         : std::is_same<R, dd>::value && PH2 && (kind & kStagePhases);
 }
 template <typename R, int EW = EntryWords<R>::value>
 __device__ __forceinline__ const R* op_table(uint2 raw, const R* sh_tab, const R* ps_tab) {
@@ -576,7 +577,7 @@ __device__ __forceinline__ void stage_forward(const FStage* st, const FSeg* segs
                                               int warp_in_group) {
     constexpr bool PHASES = PH2 && std::is_same<R, double>::value;
     constexpr bool DG = sizeof(R) == 8;
-    if (op_switch<R>(st->kind)) {
+    if (op_switch<R, PH2>(st->kind)) {
         run_ops<R, K, 0, true, PH2, EW>(reinterpret_cast<const DOp*>(ops), st->op_begin - op_base,
                                                st->op_end - op_base, pb, a, a, sh_tab, ps_tab, nullptr, q, lane,
                                                warp_in_group);
@@ -606,7 +607,7 @@ __device__ __forceinline__ void stage_backward(const FStage* st, const FSeg* seg
     constexpr bool PHASES = PH2 && std::is_same<R, double>::value;
     constexpr bool DG = sizeof(R) == 8;
     const int wg = q.wg;
-    if (op_switch<R>(st->kind)) {
+    if (op_switch<R, PH2>(st->kind)) {
         run_ops<R, K, 1, true, PH2, EW>(reinterpret_cast<const DOp*>(ops), st->op_begin - op_base,
                                                st->op_end - op_base, pb, a, l, sh_tab, ps_tab, acc, q, lane,
                                                warp_in_group);

@@ -21,9 +21,9 @@ const void* sweep_ptr_f32_fused_nph(int K, bool full);
 const void* pass_ptr_f32_nph(int mode, int K, bool full);
 const void* sweep_ptr_f64_fused(int K, bool full);
 // double-float arithmetic on complex128 storage (VQC_C128_DF plans)
-const void* sweep_ptr_dd_fwd(int K, bool full);
-const void* sweep_ptr_dd_bwd(int K, bool full);
-const void* sweep_ptr_dd_fused(int K, bool full);
+const void* sweep_ptr_dd_fwd(int K, bool full, bool factored);
+const void* sweep_ptr_dd_bwd(int K, bool full, bool factored);
+const void* sweep_ptr_dd_fused(int K, bool full, bool factored);
 const void* pass_ptr_dd(int mode, int K, bool full);
 const void* cluster_ptr_dd();
 const void* reduce_terms_ptr_dd();

@@ -12,6 +12,8 @@ namespace vqc {
 // FUSED (MODE 1 only): the backward that recomputes the states also writes E
 // (vqc_forward_backward); a separate instantiation keeps that code out of the
 // plain backward kernel.
+// PH2: the schedule may hold CRZ / RZZ.  Double-float: 2x2 updates throughout (else
+// factored stages, in groups of whole warps).
 template <typename R, int K, int MODE, bool FULL, bool FUSED, bool PH2 = true>
 __global__ void __launch_bounds__(512) sweep_kernel(const __grid_constant__ KArgs<St<R>> A) {
     if (geometry_bad(blockDim.x != (unsigned)(A.S * A.tpg) || A.tpg != (1 << A.tbits) ||
@@ -28,8 +30,10 @@ __global__ void __launch_bounds__(512) sweep_kernel(const __grid_constant__ KArg
     R* dw_cta = reinterpret_cast<R*>(smem + A.sm_dw);
     R* red_all = reinterpret_cast<R*>(smem + A.sm_red);
 
-    constexpr bool DG = sizeof(R) == 8;   // the stages may have diagonal tables
-    constexpr int EW = ResidentWords<R, MODE, FULL>::value;
+    constexpr bool DF = std::is_same<R, dd>::value;
+    constexpr bool ROUNDS = FULL && (!DF || Factored<R, FULL, PH2>::value);
+    constexpr bool DG = sizeof(R) == 8 && ROUNDS;   // the stages may have diagonal tables
+    constexpr int EW = ResidentWords<R, MODE, FULL, PH2>::value;
     const int n = A.n, G = A.G;
     const int dim = 1 << n;
     Geo q;
@@ -184,7 +188,7 @@ __global__ void __launch_bounds__(512) sweep_kernel(const __grid_constant__ KArg
         }
         __syncthreads();
         C2<R>* dg = reinterpret_cast<C2<R>*>(smem + A.sm_dg) + (((size_t)q.g * A.ndg) << K);
-        if constexpr (FULL && DG) if (A.ndg) {
+        if constexpr (DG) if (A.ndg) {
             if (unit == (int)blockIdx.x)
                 build_diagonals<R, K, EW>(segs, A.nsegs, ops, 0, sh_tab, ps_tab, false, q.t, q.T, dg);
             build_diagonals<R, K, EW>(segs, A.nsegs, ops, 0, sh_tab, ps_tab, true, q.t, q.T, dg);
@@ -211,7 +215,7 @@ __global__ void __launch_bounds__(512) sweep_kernel(const __grid_constant__ KArg
                 } else {
                     frame_load<R, K>(a, psi_t, v.off, sb);
                 }
-                if constexpr (FULL)
+                if constexpr (ROUNDS)
                     stage_forward<R, K, PH2, EW>(sp, segs, 0, ops, 0, v.pb, a, sh_tab, ps_tab, dg, q, lane, warp_in_group);
                 else
                     run_ops<R, K, 0, FULL, PH2, EW>(P.ops, sp->op_begin, sp->op_end, v.pb, a, a, sh_tab,
@@ -278,7 +282,7 @@ __global__ void __launch_bounds__(512) sweep_kernel(const __grid_constant__ KArg
                     lambda_frame<R, K>(fin->lmask, xor_bits(fin->tmask, A.tbits, q.t), xrow + A.Px, n, a, l);
                 else
                     frame_load<R, K>(l, lam_t, v.off, sb);
-                if constexpr (FULL)
+                if constexpr (ROUNDS)
                     stage_backward<R, K, PH2>(sp, segs, 0, ops, 0, v.pb, a, l, sh_tab, ps_tab, dg, acc, q, lane, warp_in_group);
                 else
                     run_ops<R, K, 1, FULL, PH2, EW>(P.ops, sp->op_begin, sp->op_end, v.pb, a, l, sh_tab,

@@ -361,11 +361,14 @@ __device__ __forceinline__ void store_factors(const M2<R>& m, int form, R* o) {
 }
 
 // Tables of the resident path: complex64 forward ones without U^dag (a 13-qubit random
-// circuit's tables 36 -> 18 KB per sample), double-float ones of groups below a warp,
-// which run no factored stages, without the factors.
-template <typename R, int MODE, bool FULL> struct ResidentWords {
+// circuit's tables 36 -> 18 KB per sample), double-float ones of the kernels without
+// factored stages (Factored) without the factors.
+template <typename R, bool FULL, bool PH2> struct Factored {
+    static constexpr bool value = std::is_same<R, dd>::value && FULL && !PH2;
+};
+template <typename R, int MODE, bool FULL, bool PH2> struct ResidentWords {
     static constexpr bool dbf = std::is_same<R, dd>::value;
-    static constexpr int value = dbf && !FULL ? entry_reals(true, false)
+    static constexpr int value = dbf && !Factored<R, FULL, PH2>::value ? entry_reals(true, false)
                                               : EntryWords<R>::value / (!dbf && sizeof(R) == 4 && MODE == 0 ? 2 : 1);
 };
 
