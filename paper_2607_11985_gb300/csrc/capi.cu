@@ -207,6 +207,9 @@ int choose_k(const HostPlan& p, int mode, int B, int sms) {
     for (const auto& s : p.frames)
         if (s.mode == mode && s.path == VQC_PATH_RESIDENT) kmax = std::max(kmax, s.K);
     if (kmax == 0) return 0;
+    // Double-float circuits with CRZ / RZZ: blocks of 8 where threads allow (ph2_any; 11-qubit
+    // QAOA x 1600, 8 layers, forward 1.57 ms, 2.40 with blocks of 16).
+    if (p.dfloat && p.has_ph2 && kmax > 3 && find_frame(p, mode, VQC_PATH_RESIDENT, 3)) kmax = 3;
     const int kmin = std::min(kmax, 3);
     const double want = (double)sms * 4 * 32;
     int K = kmax;

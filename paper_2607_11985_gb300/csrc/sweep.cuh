@@ -929,6 +929,35 @@ __device__ __forceinline__ void ph2_pp(int s, const R* tp, uint8_t flags, C2<R> 
     }
 }
 
+// The same for every place of a and b, their positions and the phase of an amplitude
+// taken at run time: double-float, whose products (about 40 instructions an amplitude)
+// hide that, and whose code for each place, 5 to 10 KB, does not fit the instruction
+// cache with the others' (QAOA circuits of 8 to 12 qubits, forward and backward, 1.18
+// times as fast in the mean).  Blocks of 16 amplitudes spill more with it (0.88 to 0.97
+// times at batch 1600) and keep the cases.
+template <typename R, int K, int MODE, bool FULL>
+__device__ __forceinline__ void ph2_any(int ra, int rb, uint32_t pb, const R* tp, uint8_t flags, C2<R> (&a)[1 << K],
+                                        C2<R> (&l)[1 << K], const Geo& q, R* accp, bool acc_add) {
+    const int pa = ra >= kRefPhys ? (int)((pb >> (ra - kRefPhys)) & 1u) : 0;
+    const int pc = rb >= kRefPhys ? (int)((pb >> (rb - kRefPhys)) & 1u) : 0;
+    const int ma = ra >= kRefPhys ? 0 : 1 << ra, mb = rb >= kRefPhys ? 0 : 1 << rb;
+    const C2<R>* ph = reinterpret_cast<const C2<R>*>(tp);
+    const bool acc = MODE == 1 && (flags & OPF_HAS_ACC);
+    R tv = 0;
+#pragma unroll
+    for (int r = 0; r < (1 << K); ++r) {
+        const int s = (pa | ((r & ma) ? 1 : 0)) + 2 * (pc | ((r & mb) ? 1 : 0));
+        C2<R> f = ph[s];
+        if (MODE == 1) {
+            f.y = -f.y;
+            if (acc) tv = fma(gen_at<R>(flags, s), im_conj_mul<R>(l[r], a[r]), tv);
+            l[r] = cmul<R>(l[r], f);
+        }
+        a[r] = cmul<R>(a[r], f);
+    }
+    if (acc) ph2_term_store<R, FULL>(tv, q, accp, acc_add);
+}
+
 // ---------------------------------------------------------------- op dispatch
 template <typename R> __device__ __forceinline__ M2<R> load_m2v(const R* p);
 template <> __device__ __forceinline__ M2<float> load_m2v<float>(const float* p) {
@@ -974,6 +1003,12 @@ __device__ __forceinline__ void apply_op(uint2 raw, uint32_t pb, C2<R> (&a)[1 <<
     const R* tp = ((flags & OPF_PER_SAMPLE) ? ps_tab : sh_tab) + EW * slot;
     R* accp = acc + ((size_t)aux * q.wg + warp_in_group) * 8;
     const int rlane = FULL ? lane : q.t;
+    constexpr bool ANY = std::is_same<R, dd>::value && K < 4;   // ph2_any
+    if constexpr (WITH_PH2 && ANY)
+        if (code >= DC_PH2_LL) {
+            ph2_any<R, K, MODE, FULL>(ra, rb, pb, tp, flags, a, l, q, accp, acc_add);
+            return;
+        }
     switch (code) {
 #define VQC_M1(T_)                                                                   \
     case DC_M1 + T_:                                                                 \
@@ -1042,7 +1077,7 @@ __device__ __forceinline__ void apply_op(uint2 raw, uint32_t pb, C2<R> (&a)[1 <<
     }
 #define VQC_PH2LL(LO_, HI_)                                                          \
     case DC_PH2_LL + cz_pair_index(LO_, HI_):                                        \
-        if constexpr (WITH_PH2 && LO_ < K && HI_ < K) ph2_ll<R, K, MODE, FULL, LO_, HI_>(ra > rb, tp, flags, a, l, q, accp, acc_add); \
+        if constexpr (WITH_PH2 && !ANY && LO_ < K && HI_ < K) ph2_ll<R, K, MODE, FULL, LO_, HI_>(ra > rb, tp, flags, a, l, q, accp, acc_add); \
         break;
         VQC_PH2LL(0, 1) VQC_PH2LL(0, 2) VQC_PH2LL(0, 3) VQC_PH2LL(0, 4)
         VQC_PH2LL(1, 2) VQC_PH2LL(1, 3) VQC_PH2LL(1, 4)
@@ -1050,12 +1085,12 @@ __device__ __forceinline__ void apply_op(uint2 raw, uint32_t pb, C2<R> (&a)[1 <<
 #undef VQC_PH2LL
 #define VQC_PH2PL(L_)                                                                \
     case DC_PH2_PL + L_:                                                             \
-        if constexpr (WITH_PH2 && L_ < K) ph2_pl<R, K, MODE, FULL, L_>(ra < kRefPhys, physbit(pb, ra < kRefPhys ? rb : ra), tp, flags, a, l, q, accp, acc_add); \
+        if constexpr (WITH_PH2 && !ANY && L_ < K) ph2_pl<R, K, MODE, FULL, L_>(ra < kRefPhys, physbit(pb, ra < kRefPhys ? rb : ra), tp, flags, a, l, q, accp, acc_add); \
         break;
         VQC_PH2PL(0) VQC_PH2PL(1) VQC_PH2PL(2) VQC_PH2PL(3) VQC_PH2PL(4)
 #undef VQC_PH2PL
     case DC_PH2_PP:
-        if constexpr (WITH_PH2)
+        if constexpr (WITH_PH2 && !ANY)
             ph2_pp<R, K, MODE, FULL>((int)physbit(pb, ra) + 2 * (int)physbit(pb, rb), tp, flags, a, l, q,
                                      accp, acc_add);
         break;
