@@ -242,14 +242,14 @@ def test_noalloc_takes_fewer_ctas():
 
 # runs of every factored form (rotation alone, a diagonal on either side or both, a
 # diagonal run), at angles where an entry of the matrix vanishes; groups below a warp
-# keep the 2x2 updates
-@pytest.mark.parametrize("n,path", [(3, None), (8, None), (11, None), (13, "hbm")])
+# and small forwards of few stages keep the 2x2 updates
+@pytest.mark.parametrize("n,path,layers", [(3, None, 2), (8, None, 2), (8, None, 6), (11, None, 2), (13, "hbm", 1)])
 @pytest.mark.parametrize("kinds", [("RY",), ("RY", "RZ"), ("RZ", "RY"), ("RX",), ("H",), ("RZ",), ("U3", "X")])
 @pytest.mark.parametrize("dtype", ["c128df", "c128"])
-def test_run_forms(monkeypatch, dtype, kinds, n, path):
+def test_run_forms(monkeypatch, dtype, kinds, n, path, layers):
     if path:
         monkeypatch.setenv("VQC_FORCE_PATH", path)
-    spec = mixed(n, kinds + ("CX",), layers=2 if n < 13 else 1)
+    spec = mixed(n, kinds + ("CX",), layers=layers)
     c = C(spec, dtype)
     for angles in ((0.0, np.pi, -np.pi, np.pi / 2), None):
         check(c, *draw(spec, 2, dtype, 7400 + n, angles=angles))
