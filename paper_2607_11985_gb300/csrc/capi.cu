@@ -833,26 +833,14 @@ vqc_status plan_hbm_uncached(const HostPlan& p, int mode, int B, PassGeo& L) {
     L.T = 1 << (m - L.K);
     L.wg = L.T > 32 ? L.T / 32 : 1;
     L.ntiles = 1 << (p.n - m);
-    int ps_max = 0, sh_max = 0, acc_max = 0, nst_max = 0, ops_max = 0, ndg_max = 0, seg_max = 0;
-    for (const FPass& ps : L.s->passes) {
-        ps_max = std::max(ps_max, ps.ps_count);
-        sh_max = std::max(sh_max, ps.sh_count);
-        acc_max = std::max(acc_max, ps.acc_count);
-        nst_max = std::max(nst_max, ps.stage_end - ps.stage_begin);
-        ndg_max = std::max(ndg_max, ps.ndg);
-        seg_max = std::max(seg_max, ps.seg_end - ps.seg_begin);
-        ops_max = std::max(ops_max, ps.op_end - ps.op_begin);
-    }
+    PassNeeds c;
+    for (const FPass& ps : L.s->passes) c.cover(ps);
     const size_t tdim = (size_t)1 << m;
     const size_t ew = entry_reals(dbl, p.dfloat);
     const size_t apv = 16 / cs, nk = (tdim / apv + L.T - 1) / L.T;
-    const size_t prog = (size_t)nst_max * sizeof(FStage) + sizeof(FFinal) + (size_t)ops_max * sizeof(DOp) +
-                        (size_t)nst_max * L.s->nout * sizeof(FFlip) + (size_t)seg_max * sizeof(FSeg);
-    const size_t fixed = align16((size_t)sh_max * ew * rs) + align16(prog) + align16(2 * nk * 8) + 8 * 16;
     L.tables = L.T >= 32 && dbl && (p.dfloat || p.has_ph2);   // as on the resident path
-    const size_t dgb = L.tables ? ((size_t)ndg_max << L.K) * cs : 0;
-    const size_t per_tile = dgb + (size_t)ps_max * ew * rs + tdim * cs * (mode == 1 ? 2 : 1) + (size_t)(nst_max + 1) * 8 +
-                            (size_t)L.T * (16 + 4 * nst_max) + (mode == 1 ? (size_t)acc_max * L.wg * 8 * rs : (size_t)L.wg * p.n * rs);
+    const PassBytes pb = pass_bytes(c, p.n, mode, p.dtype, p.dfloat, L.tables, m, L.K);
+    const size_t fixed = pb.fixed, per_tile = pb.tile;
     int S = std::max(1, 128 / L.T);
     if ((size_t)di.smem_optin <= fixed + per_tile)
         S = (size_t)di.smem_optin >= fixed + per_tile ? 1 : 0;
@@ -871,16 +859,16 @@ vqc_status plan_hbm_uncached(const HostPlan& p, int mode, int B, PassGeo& L) {
     };
     take((size_t)S * tdim * cs);   // psi tiles at offset 0
     L.sm_lam = take(mode == 1 ? (size_t)S * tdim * cs : 0);
-    L.sm_sh = take((size_t)sh_max * ew * rs);
-    L.sm_ps = take((size_t)S * ps_max * ew * rs);
-    L.sm_acc = take(mode == 1 ? (size_t)S * acc_max * L.wg * 8 * rs : 0);
+    L.sm_sh = take((size_t)c.sh * ew * rs);
+    L.sm_ps = take((size_t)S * c.ps * ew * rs);
+    L.sm_acc = take(mode == 1 ? (size_t)S * c.acc * L.wg * 8 * rs : 0);
     L.sm_red = take(mode == 0 ? (size_t)S * L.wg * p.n * rs : 0);
     L.sm_koff = take(2 * nk * 8);   // tile-copy offsets: one uint2 per vector round, read and written
     L.sm_toff = take((size_t)L.block * 16);   // and each thread's own part
-    L.sm_dg = take(S * dgb);
-    L.sm_tbase = take((size_t)nst_max * L.block * 4);
-    L.sm_plan = take(prog);
-    L.sm_tfl = take((size_t)S * (nst_max + 1) * 8);
+    L.sm_dg = take(S * pb.diagonals);
+    L.sm_tbase = take((size_t)c.stages * L.block * 4);
+    L.sm_plan = take(c.program(L.s->nout));
+    L.sm_tfl = take((size_t)S * (c.stages + 1) * 8);
     L.smem = off;
     L.fn = p.dfloat ? pass_ptr_dd(mode, L.K, L.T >= 32)
            : (!dbl && !p.has_ph2) ? pass_ptr_f32_nph(mode, L.K, L.T >= 32)   // no phase cases

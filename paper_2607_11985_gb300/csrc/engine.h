@@ -104,6 +104,49 @@ inline std::vector<int> frame_tile_qubits(int mode, int dtype, int n) {
     return {fit(mode == 0 ? 12 : 11)};
 }
 
+// Shared memory that a CTA can have on sm_103a (227 KB).
+constexpr size_t kCtaSharedMemory = 232448;
+
+// The largest of each count that sizes a launch of a pass: of one, or over all passes
+// of a schedule (whose launches share one layout).
+struct PassNeeds {
+    int ps = 0, sh = 0, acc = 0, stages = 0, ops = 0, segs = 0, ndg = 0;
+    void cover(const FPass& p) {
+        auto most = [](int& a, int b) { a = b > a ? b : a; };
+        most(ps, p.ps_count);
+        most(sh, p.sh_count);
+        most(acc, p.acc_count);
+        most(stages, p.stage_end - p.stage_begin);
+        most(ops, p.op_end - p.op_begin);
+        most(segs, p.seg_end - p.seg_begin);
+        most(ndg, p.ndg);
+    }
+    // the pass's program: copies of its stages, ops, flips, rounds and FFinal
+    size_t program(int nout) const {
+        return (size_t)stages * sizeof(FStage) + sizeof(FFinal) + (size_t)ops * sizeof(DOp) +
+               (size_t)stages * nout * sizeof(FFlip) + (size_t)segs * sizeof(FSeg);
+    }
+};
+
+// Shared memory of a pass launch (plan_hbm places the parts): bytes per CTA, and per
+// tile of the CTA.
+struct PassBytes {
+    size_t fixed, tile;
+    size_t diagonals;   // of the tile's: the stages' diagonal tables
+};
+inline PassBytes pass_bytes(const PassNeeds& c, int n, int mode, int dtype, bool dfloat, bool tables, int m, int K) {
+    const size_t rs = dtype == VQC_C128 ? 8 : 4, cs = 2 * rs, ew = entry_reals(dtype == VQC_C128, dfloat);
+    const size_t T = (size_t)1 << (m - K), wg = T > 32 ? T / 32 : 1, dim = (size_t)1 << m;
+    const size_t nk = (dim / (16 / cs) + T - 1) / T;
+    auto align16 = [](size_t v) { return (v + 15) & ~size_t(15); };
+    PassBytes b;
+    b.fixed = align16((size_t)c.sh * ew * rs) + align16(c.program(n - m)) + align16(2 * nk * 8) + 8 * 16;
+    b.diagonals = tables ? ((size_t)c.ndg << K) * cs : 0;
+    b.tile = b.diagonals + (size_t)c.ps * ew * rs + dim * cs * (mode == 1 ? 2 : 1) + (size_t)(c.stages + 1) * 8 +
+             T * (16 + 4 * (size_t)c.stages) + (mode == 1 ? (size_t)c.acc * wg * 8 * rs : wg * n * rs);
+    return b;
+}
+
 // Maximum K per (mode, dtype) for register-resident blocks.
 inline int max_k(int mode, int dtype) {
     if (dtype == VQC_C64) return mode == 0 ? 5 : 4;

@@ -175,8 +175,10 @@ Vecs inverse(Vecs cols) {   // of an invertible matrix, as columns
     return inv;
 }
 
-// Table entries and accumulators of one pass: bounds its shared memory.
+// Table entries and accumulators of one pass, and ops of one stage: what of a pass's
+// shared memory is not bounded by giving its later stages a pass of their own (split).
 constexpr int kMaxPassEntries = 96;
+constexpr size_t kMaxStageOps = 2048;
 
 struct StagePlan {
     std::vector<int> ops;              // indices into the FOp list, time order
@@ -196,7 +198,7 @@ std::vector<StagePlan> cut(const std::vector<FOp>& f, const std::vector<int>& op
         size_t i = 0;
         for (; i < rem.size() && w.d.dim < n; ++i) {
             const FOp& o = f[rem[i]];
-            bool ok = w.passes(o);
+            bool ok = w.passes(o) && s.ops.size() < kMaxStageOps;
             if (ok && o.run) {
                 size_t j = 0;
                 while (j < s.D.size() && !(s.D[j] == o.d && s.R[j] == o.r)) ++j;
@@ -479,6 +481,45 @@ std::vector<PassPlan> plan_passes(const HostPlan& p, const FrameOps& L, int mode
     return passes;
 }
 
+// Gives the later half of a pass's stages, on the same tile, to a pass of its own:
+// every pass that exceeds a CTA's shared memory by itself, or else the one that needs
+// most (the launches share the layout of the schedule's largest counts).  False when
+// no pass has two stages.
+bool split(std::vector<PassPlan>& passes, const FrameSchedule& S, const HostPlan& p) {
+    std::vector<size_t> bytes;
+    size_t most = 0;
+    for (size_t i = 0; i < passes.size(); ++i) {
+        PassNeeds c;
+        c.cover(S.passes[i]);
+        const bool dbl = p.dtype == VQC_C128;   // (double-float plans run the same schedules)
+        const PassBytes b = pass_bytes(c, p.n, S.mode, p.dtype, dbl, dbl, S.m, S.K);
+        bytes.push_back(passes[i].stages.size() > 1 ? b.fixed + b.tile : 0);
+        most = std::max(most, bytes.back());
+    }
+    if (most == 0) return false;
+    std::vector<PassPlan> out;
+    for (size_t i = 0; i < passes.size(); ++i) {
+        PassPlan& ps = passes[i];
+        if (bytes[i] < std::min(most, kCtaSharedMemory + 1)) {
+            out.push_back(std::move(ps));
+            continue;
+        }
+        const size_t half = (ps.stages.size() + 1) / 2;
+        for (size_t from : {(size_t)0, half}) {
+            PassPlan q;
+            q.V = ps.V;
+            q.stages.assign(ps.stages.begin() + from, from ? ps.stages.end() : ps.stages.begin() + half);
+            for (const StagePlan& s : q.stages) q.ops.insert(q.ops.end(), s.ops.begin(), s.ops.end());
+            out.push_back(std::move(q));
+        }
+    }
+    passes.swap(out);
+    return true;
+}
+
+FrameSchedule lay_out(const HostPlan& p, const FrameOps& L, int mode, int path, int m, int K,
+                      const std::vector<PassPlan>& passes);
+
 }  // namespace
 
 FrameBuilder::FrameBuilder(const HostPlan& plan) : p(plan), ops(new FrameOps(lower(plan))) {}
@@ -488,8 +529,6 @@ FrameSchedule FrameBuilder::build(int mode, int path, const std::vector<int>& ti
     const int n = p.n;
     const bool tiled = path == VQC_PATH_HBM;
     const FrameOps& L = *ops;
-    const std::vector<FOp>& f = L.f;
-    const Vecs &dir = L.dir, &sel = L.sel;
 
     // of the tile sizes offered, the first unless a later one takes no more passes and stages
     int m = 0;
@@ -506,6 +545,26 @@ FrameSchedule FrameBuilder::build(int mode, int path, const std::vector<int>& ti
         nst = c;
         passes = std::move(q);
     }
+    for (;;) {
+        FrameSchedule S = lay_out(p, L, mode, path, m, K, passes);
+        if (!tiled) return S;
+        PassNeeds c;
+        for (const FPass& ps : S.passes) c.cover(ps);
+        const bool dbl = p.dtype == VQC_C128;
+        const PassBytes b = pass_bytes(c, n, mode, p.dtype, dbl, dbl, m, K);
+        if (b.fixed + b.tile <= kCtaSharedMemory || !split(passes, S, p)) return S;
+    }
+}
+
+namespace {
+
+// The schedule's records from its passes and stages.
+FrameSchedule lay_out(const HostPlan& p, const FrameOps& L, int mode, int path, int m, int K,
+                      const std::vector<PassPlan>& passes) {
+    const int n = p.n;
+    const bool tiled = path == VQC_PATH_HBM;
+    const std::vector<FOp>& f = L.f;
+    const Vecs &dir = L.dir, &sel = L.sel;
     const int G = std::min(p.G_swz, m), np = (int)passes.size(), nout = n - m;
     FrameSchedule S;
     S.mode = mode;
@@ -532,7 +591,7 @@ FrameSchedule FrameBuilder::build(int mode, int path, const std::vector<int>& ti
     Rng rng;
     for (int step = 0; step < np; ++step) {
         const int pi = mode == 0 ? step : np - 1 - step;
-        PassPlan& ps = passes[pi];
+        const PassPlan& ps = passes[pi];
         const bool last = pi == np - 1, end = step == np - 1;
         FPass fp{};
         // the tile's addresses as read: a reduced echelon basis with the G low units first
@@ -973,6 +1032,8 @@ FrameSchedule FrameBuilder::build(int mode, int path, const std::vector<int>& ti
     }
     return S;
 }
+
+}  // namespace
 
 std::vector<uint8_t> export_frames(const HostPlan& p) {
     std::vector<uint8_t> out = {'V', 'Q', 'C', 'F'};

@@ -380,3 +380,65 @@ def test_layered_16_passes():
                 assert len(s["passes"]) <= 6
                 assert len(s["stages"]) * s["K"] <= 1.3 * len(s["ops"])
         B.vqc_free(plan)
+
+
+def narrow(kind, n, k):
+    """Circuits of many stages on few directions: every run behind the one before it
+    ("rx", "ry"), or next to no runs, CZ gates in changing frames ("signs")."""
+    rng = np.random.default_rng(n * k)
+    spec = wl.CircuitSpec(n, 1, 1).add("RY", (0,), [("x", 0)])
+    for _ in range(k):
+        if kind == "rx":
+            spec.add("RX", (0,), [("w", 0)]).add("CX", (0, 1))
+        elif kind == "ry":
+            spec.add("RY", (0,), [("x", 0)]).add("CX", (0, 1)).add("RY", (1,), [("w", 0)]).add("CX", (1, 0))
+        else:
+            spec.add(("CX", "CZ")[rng.integers(2)], tuple(int(q) for q in rng.permutation(n)[:2]))
+    return spec
+
+
+def launch_bytes(s, n, dtype, dfloat, phases):
+    """Shared memory of the launches of a schedule's passes, one tile per CTA: the parts
+    that plan_hbm places, each as large as the largest pass needs it."""
+    most = {k: max(int(p[k + "_end"] - p[k + "_begin"]) for p in s["passes"]) for k in ("stage", "op", "seg")}
+    most.update({k: max(int(p[k]) for p in s["passes"]) for k in ("ps_count", "sh_count", "acc_count", "ndg")})
+    rs = 8 if dtype else 4
+    ew, T = 20 if dfloat else 8 if dtype else 32, 1 << (s["m"] - s["K"])
+    wg, dim = max(1, T // 32), 1 << s["m"]
+    nk = -(-dim // (16 // (2 * rs)) // T)
+    tables = T >= 32 and dtype and (dfloat or phases)
+    parts = [dim * 2 * rs * (2 if s["mode"] else 1), most["sh_count"] * ew * rs, most["ps_count"] * ew * rs,
+             most["acc_count"] * wg * 8 * rs if s["mode"] else wg * n * rs, 16 * nk, 16 * T,
+             (most["ndg"] << s["K"]) * 2 * rs if tables else 0, 4 * T * most["stage"],
+             most["stage"] * FSTAGE.itemsize + FFINAL.itemsize + 8 * most["op"] +
+             most["stage"] * s["nout"] * FFLIP.itemsize + most["seg"] * FSEG.itemsize, 8 * (most["stage"] + 1)]
+    return sum((b + 15) // 16 * 16 for b in parts)
+
+
+@pytest.mark.parametrize("kind,k", [("rx", 60), ("rx", 100), ("rx", 400), ("ry", 60), ("ry", 100), ("signs", 2000),
+                                    ("signs", 20000)])
+@pytest.mark.parametrize("n", [13, 16, 20])
+def test_passes_fit_shared_memory(monkeypatch, kind, k, n):
+    # 227 KB a CTA; with all of its stages the one pass of most of these takes more
+    monkeypatch.setenv("VQC_FORCE_PATH", "hbm")
+    spec = narrow(kind, n, k)
+    for dtype in (0, 1):
+        plan = compile_spec(spec, dtype)
+        hbm = [s for s in frames(plan) if s["path"] == 1]
+        B.vqc_free(plan)
+        assert [s["mode"] for s in hbm] == [0, 1]
+        for s in hbm:
+            for dfloat in (False, True)[:dtype + 1]:
+                assert launch_bytes(s, n, dtype, dfloat, False) <= 232448
+            assert sum(p["op_end"] - p["op_begin"] for p in s["passes"]) == len(s["ops"])
+
+
+@pytest.mark.parametrize("kind,k", [("rx", 130), ("ry", 100), ("signs", 4000)])
+def test_split_passes(monkeypatch, kind, k):
+    # consecutive passes on one tile: the same result
+    monkeypatch.setenv("VQC_FORCE_PATH", "hbm")
+    spec = narrow(kind, 13, k)
+    rng = np.random.default_rng(17)
+    x, w, gE = rng.uniform(-3, 3, (1, 1)), rng.uniform(-3, 3, 1), rng.standard_normal((1, 13))
+    fr = check(spec, x, w, gE, None, 1)
+    assert any(len(s["passes"]) > 1 for s in fr if s["path"] == 1)

@@ -21,6 +21,7 @@ torch = pytest.importorskip("torch")
 from oracle import oracle as orc  # noqa: E402
 from paper_2607_11985_gb300 import binding as B  # noqa: E402
 from paper_2607_11985_gb300 import workloads as wl  # noqa: E402
+from tests.test_frames_cpu import narrow  # noqa: E402
 from tests.test_gpu_parity import C, dev, devc, maxerr, run_bwd, run_fwd  # noqa: E402
 
 pytestmark = pytest.mark.gpu
@@ -123,6 +124,18 @@ def test_full_warp_passes(monkeypatch, dtype, n, batch, kinds, num_w):
     c = C(spec, dtype)
     assert c.info(batch)["fwd_path"] == 1 and c.info(batch)["bwd_path"] == 1
     check(c, *draw(spec, batch, dtype, 7000 + n, psi0=batch == 3))
+
+
+# passes whose stages exceed a CTA's shared memory all at once: several on one tile
+@pytest.mark.parametrize("dtype,kind,n,k", [("c64", "signs", 15, 2000), ("c128", "rx", 14, 100), ("c128", "ry", 13, 100),
+                                            ("c128", "signs", 15, 2000), ("c128df", "rx", 13, 400),
+                                            ("c128df", "ry", 14, 60)])
+def test_passes_of_many_stages(monkeypatch, dtype, kind, n, k):
+    monkeypatch.setenv("VQC_FORCE_PATH", "hbm")
+    spec = narrow(kind, n, k)
+    c = C(spec, dtype)
+    assert c.info(2)["fwd_path"] == 1 and c.info(2)["bwd_path"] == 1
+    check(c, *draw(spec, 2, dtype, 7050 + n))
 
 
 # CZ only acts as a sign: a register circuit of one direction needs one pass
