@@ -200,7 +200,7 @@ cudaError_t launch(const void* fn, dim3 grid, dim3 block, void** args, size_t sm
 // and the fused call) found no smaller K faster than this choice: smaller
 // blocks add stages (shared-memory round trips and barriers) faster than the
 // extra warps hide latency.
-int choose_k(const HostPlan& p, int mode, int B, int sms) {
+int choose_k(const HostPlan& p, int mode, int B, int sms, bool any_size = false) {
     const int forced = mode == 0 ? t_env.k_fwd : t_env.k_bwd;
     if (forced > 0 && find_frame(p, mode, VQC_PATH_RESIDENT, forced)) return forced;
     int kmax = 0;
@@ -209,7 +209,8 @@ int choose_k(const HostPlan& p, int mode, int B, int sms) {
     if (kmax == 0) return 0;
     // Double-float circuits with CRZ / RZZ: blocks of 8 where threads allow (ph2_any; 11-qubit
     // QAOA x 1600, 8 layers, forward 1.57 ms, 2.40 with blocks of 16).
-    if (p.dfloat && p.has_ph2 && kmax > 3 && find_frame(p, mode, VQC_PATH_RESIDENT, 3)) kmax = 3;
+    // any_size: without that rule, where such a launch does not fit.
+    if (!any_size && p.dfloat && p.has_ph2 && kmax > 3 && find_frame(p, mode, VQC_PATH_RESIDENT, 3)) kmax = 3;
     const int kmin = std::min(kmax, 3);
     const double want = (double)sms * 4 * 32;
     int K = kmax;
@@ -230,15 +231,15 @@ bool factors_pay(const HostPlan& p, int mode, int B, const FrameSchedule& f, int
     return mode == 1 || f.passes[0].ndg == 0 || !small || f.stages.size() >= 12;
 }
 
-vqc_status plan_launch_uncached(const HostPlan& p, int launch_mode, int B, Launch& L) {
+// The resident launch with blocks of 2^K amplitudes; lean: double-float without the
+// runs' factors and diagonals.
+vqc_status plan_launch_as(const HostPlan& p, int launch_mode, int B, int K, bool lean, int dev, const DevInfo& di,
+                          Launch& L) {
     // mode 2 (fused) has the backward's schedule and layout, its own kernel
     const int mode = launch_mode == 2 ? 1 : launch_mode;
-    int dev = 0;
-    VQC_CUDA(cudaGetDevice(&dev));
-    DevInfo di;
-    vqc_status st = device_info(dev, di);
-    if (st != VQC_OK) return st;
-    L.K = choose_k(p, mode, B, di.sms);
+    vqc_status st;
+    L = Launch();
+    L.K = K;
     L.f = L.K ? find_frame(p, mode, VQC_PATH_RESIDENT, L.K) : nullptr;
     if (!L.f)
         return fail(VQC_ERR_UNSUPPORTED, "no resident schedule for this circuit (n = " +
@@ -249,9 +250,9 @@ vqc_status plan_launch_uncached(const HostPlan& p, int launch_mode, int B, Launc
     L.wg = L.T > 32 ? L.T / 32 : 1;
     // Shared memory: a fixed part per CTA and a part per resident sample.
     const size_t dim = (size_t)1 << p.n;
-    const bool factored = p.dfloat && L.T >= 32 && factors_pay(p, mode, B, *L.f, di.sms);
-    const size_t ew = entry_reals(dbl, factored) / (mode == 0 && !dbl ? 2 : 1);   // ResidentWords
     const size_t io = (size_t)8 << L.K;   // slot offsets of the state copies
+    const bool factored = p.dfloat && !lean && L.T >= 32 && factors_pay(p, mode, B, *L.f, di.sms);
+    const size_t ew = entry_reals(dbl, factored) / (mode == 0 && !dbl ? 2 : 1);   // ResidentWords
     const size_t fixed = align16((size_t)p.n_sh * ew * rs) + align16(mode == 1 ? (size_t)p.num_w * rs : 0) +
                          align16((size_t)p.num_w * rs) + io + 10 * 16;
     // diagonal tables: two-local phases, and double-float's own (complex128 schedules count both)
@@ -340,6 +341,25 @@ vqc_status plan_launch_uncached(const HostPlan& p, int launch_mode, int B, Launc
     if (per_sm < 1) return fail(VQC_ERR_UNSUPPORTED, "kernel cannot be resident with this geometry");
     L.grid = std::max(1, std::min(L.nunits, per_sm * di.sms));
     return VQC_OK;
+}
+
+// The launch of the chosen block size; where a double-float layout does not fit a CTA, the
+// lean one (12 qubits x 7 layers of RX RY RZ, backward: 245 KB factored, 230 with 2x2
+// updates), then blocks of 16, with fewer warps to keep partials for.
+vqc_status plan_launch_uncached(const HostPlan& p, int launch_mode, int B, Launch& L) {
+    const int mode = launch_mode == 2 ? 1 : launch_mode;
+    int dev = 0;
+    VQC_CUDA(cudaGetDevice(&dev));
+    DevInfo di;
+    vqc_status st = device_info(dev, di);
+    if (st != VQC_OK) return st;
+    const int K = choose_k(p, mode, B, di.sms);
+    st = plan_launch_as(p, launch_mode, B, K, false, dev, di, L);
+    if (st == VQC_OK || !p.dfloat || K == 0) return st;
+    const std::string why = g_err;   // of the layout that the choice asked for
+    for (int k : {K, choose_k(p, mode, B, di.sms, true)})
+        if (plan_launch_as(p, launch_mode, B, k, true, dev, di, L) == VQC_OK) return VQC_OK;
+    return fail(st, why);
 }
 
 std::mutex g_geo_mu;
@@ -1797,7 +1817,7 @@ vqc_status vqc_plan_info(const vqc_plan* plan, int32_t batch, vqc_plan_stats* ou
         int* tps = mode == 0 ? &out->fwd_threads_per_sample : &out->bwd_threads_per_sample;
         int* tq = mode == 0 ? &out->fwd_tile_qubits : &out->bwd_tile_qubits;
         double* hb = mode == 0 ? &out->fwd_hbm_bytes_per_eval : &out->bwd_hbm_bytes_per_eval;
-        const int K = choose_k(p, mode, B, sms);
+        int K = choose_k(p, mode, B, sms);
         const bool clu = use_cluster(p, mode, B);
         const bool hbm = !clu && (ndev > 0 ? use_hbm(p, mode, B)
                                            : (K == 0 && find_frame(p, mode, VQC_PATH_HBM) != nullptr));
@@ -1811,6 +1831,8 @@ vqc_status vqc_plan_info(const vqc_plan* plan, int32_t batch, vqc_plan_stats* ou
             *tps = 1 << (p.n - s->K);
             continue;
         }
+        Launch L;
+        if (!clu && !hbm && ndev > 0 && plan_launch(p, mode, B, L) == VQC_OK) K = L.K;
         const FrameSchedule* s = hbm ? find_frame(p, mode, VQC_PATH_HBM)
                                      : K ? find_frame(p, mode, VQC_PATH_RESIDENT, K) : nullptr;
         if (!s) {

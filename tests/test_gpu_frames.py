@@ -283,3 +283,23 @@ def test_diagonal_groups(dtype, kinds, n):
 def test_table_data_in_and_out_of_shared_memory(dtype, n, layers):
     spec = mixed(n, ("RX", "RY", "CX"), layers=layers)
     check(C(spec, dtype), *draw(spec, 4, dtype, 7600 + n))
+
+
+# double-float sweeps on either side of what fits one CTA: with the runs' factors, with
+# their matrices only, neither (passes); the built-in scratch takes the first two
+@pytest.mark.parametrize("n,layers,path", [(12, 6, 0), (12, 7, 0), (12, 8, 1), (11, 18, 0), (11, 23, 0), (11, 24, 1),
+                                           (9, 60, 0)])
+def test_double_float_around_the_resident_limit(n, layers, path):
+    spec = wl.layered(n, layers, ("RX", "RY", "RZ"), "CX")
+    c = C(spec, "c128df")
+    assert c.info(9)["bwd_path"] == path
+    w_, p0 = draw(spec, 9, "c128df", 7700 + n)
+    check(c, w_, p0)
+    if path == 0:
+        x, w, gE = (dev(a, "c128df") for a in (w_.x, w_.w, w_.gE))
+        dx_ref, dw_ref = c.backward(x, w, gE)
+        dx, dw = torch.empty_like(x), torch.empty_like(w)
+        B.vqc_backward_noalloc(c.plan, 9, x.data_ptr(), w.data_ptr(), None, None, gE.data_ptr(), dx.data_ptr(),
+                               dw.data_ptr(), torch.cuda.current_stream().cuda_stream)
+        torch.cuda.synchronize()
+        assert torch.equal(dx, dx_ref) and torch.equal(dw, dw_ref)
