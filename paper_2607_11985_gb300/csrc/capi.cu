@@ -97,8 +97,9 @@ vqc_status allow_max_smem(const void* fn, int dev, int smem_optin) {
 }
 
 // mode 2: the backward with the forward sweep and E inside (vqc_forward_backward)
+// factored: double-float stages of factored runs; rounds: native complex128 ones in rounds
 const void* kernel_ptr(int dtype, bool dfloat, int mode, int K, bool full, bool ph2,
-                       bool factored) {
+                       bool factored, bool rounds) {
     // complex64 sweeps of plans without CRZ / RZZ: the instantiations without
     // the phase cases (fewer spills)
     if (!dfloat && dtype == VQC_C64 && !ph2)
@@ -107,10 +108,11 @@ const void* kernel_ptr(int dtype, bool dfloat, int mode, int K, bool full, bool 
     if (dfloat)
         return mode == 2 ? sweep_ptr_dd_fused(K, full, factored)
              : mode == 0 ? sweep_ptr_dd_fwd(K, full, factored) : sweep_ptr_dd_bwd(K, full, factored);
-    if (mode == 2) return dtype == VQC_C64 ? sweep_ptr_f32_fused(K, full) : sweep_ptr_f64_fused(K, full);
+    if (mode == 2) return dtype == VQC_C64 ? sweep_ptr_f32_fused(K, full)
+                                           : sweep_ptr_f64_fused(K, full, rounds);
     if (full) {
         if (dtype == VQC_C64) return mode == 0 ? sweep_ptr_f32_fwd(K) : sweep_ptr_f32_bwd(K);
-        return mode == 0 ? sweep_ptr_f64_fwd(K) : sweep_ptr_f64_bwd(K);
+        return mode == 0 ? sweep_ptr_f64_fwd(K, rounds) : sweep_ptr_f64_bwd(K, rounds);
     }
     if (dtype == VQC_C64) return mode == 0 ? sweep_ptr_f32_fwd_small(K) : sweep_ptr_f32_bwd_small(K);
     return mode == 0 ? sweep_ptr_f64_fwd_small(K) : sweep_ptr_f64_bwd_small(K);
@@ -231,8 +233,8 @@ bool factors_pay(const HostPlan& p, int mode, int B, const FrameSchedule& f, int
     return mode == 1 || f.passes[0].ndg == 0 || !small || f.stages.size() >= 12;
 }
 
-// The resident launch with blocks of 2^K amplitudes; lean: double-float without the
-// runs' factors and diagonals.
+// The resident launch with blocks of 2^K amplitudes; lean: without diagonal tables, and
+// double-float without the runs' factors.
 vqc_status plan_launch_as(const HostPlan& p, int launch_mode, int B, int K, bool lean, int dev, const DevInfo& di,
                           Launch& L) {
     // mode 2 (fused) has the backward's schedule and layout, its own kernel
@@ -256,7 +258,7 @@ vqc_status plan_launch_as(const HostPlan& p, int launch_mode, int B, int K, bool
     const size_t fixed = align16((size_t)p.n_sh * ew * rs) + align16(mode == 1 ? (size_t)p.num_w * rs : 0) +
                          align16((size_t)p.num_w * rs) + io + 10 * 16;
     // diagonal tables: two-local phases, and double-float's own (complex128 schedules count both)
-    L.ndg = L.T >= 32 && dbl && (p.dfloat ? factored : p.has_ph2) ? L.f->passes[0].ndg : 0;
+    L.ndg = L.T >= 32 && dbl && !lean && (p.dfloat ? factored : p.has_ph2) ? L.f->passes[0].ndg : 0;
     const size_t dgb = ((size_t)L.ndg << L.K) * cs;
     const size_t per_sample = dgb + (size_t)p.n_ps * ew * rs + dim * cs * (mode == 1 ? 2 : 1) +
                               (size_t)(p.num_x + p.n) * rs +
@@ -299,7 +301,7 @@ vqc_status plan_launch_as(const HostPlan& p, int launch_mode, int B, int K, bool
     L.sm_red = take((size_t)L.S * L.wg * p.n * rs);   // <Z> partials (forward, or recompute with E)
     L.sm_w = take((size_t)p.num_w * rs);
     L.sm_xg = take((size_t)L.S * (p.num_x + p.n) * rs);
-    L.fn = kernel_ptr(p.dtype, p.dfloat, launch_mode, L.K, L.T >= 32, p.has_ph2, factored);
+    L.fn = kernel_ptr(p.dtype, p.dfloat, launch_mode, L.K, L.T >= 32, p.has_ph2, factored, !lean);
     if (!L.fn) return fail(VQC_ERR_UNSUPPORTED, "kernel not instantiated for this K");
     st = allow_max_smem(L.fn, dev, di.smem_optin);
     if (st != VQC_OK) return st;
@@ -343,9 +345,9 @@ vqc_status plan_launch_as(const HostPlan& p, int launch_mode, int B, int K, bool
     return VQC_OK;
 }
 
-// The launch of the chosen block size; where a double-float layout does not fit a CTA, the
-// lean one (12 qubits x 7 layers of RX RY RZ, backward: 245 KB factored, 230 with 2x2
-// updates), then blocks of 16, with fewer warps to keep partials for.
+// The launch of the chosen block size; where a complex128 layout does not fit a CTA, the
+// lean one (double-float, 12 qubits x 7 layers of RX RY RZ, backward: 245 KB factored, 230
+// with 2x2 updates), then double-float's blocks of 16, with fewer warps to keep partials for.
 vqc_status plan_launch_uncached(const HostPlan& p, int launch_mode, int B, Launch& L) {
     const int mode = launch_mode == 2 ? 1 : launch_mode;
     int dev = 0;
@@ -355,7 +357,7 @@ vqc_status plan_launch_uncached(const HostPlan& p, int launch_mode, int B, Launc
     if (st != VQC_OK) return st;
     const int K = choose_k(p, mode, B, di.sms);
     st = plan_launch_as(p, launch_mode, B, K, false, dev, di, L);
-    if (st == VQC_OK || !p.dfloat || K == 0) return st;
+    if (st == VQC_OK || p.dtype != VQC_C128 || K == 0) return st;
     const std::string why = g_err;   // of the layout that the choice asked for
     for (int k : {K, choose_k(p, mode, B, di.sms, true)})
         if (plan_launch_as(p, launch_mode, B, k, true, dev, di, L) == VQC_OK) return VQC_OK;

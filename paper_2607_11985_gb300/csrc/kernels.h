@@ -7,8 +7,8 @@ namespace vqc {
 
 const void* sweep_ptr_f32_fwd(int K);          // sample groups of >= 32 threads
 const void* sweep_ptr_f32_bwd(int K);
-const void* sweep_ptr_f64_fwd(int K);
-const void* sweep_ptr_f64_bwd(int K);
+const void* sweep_ptr_f64_fwd(int K, bool rounds);   // stages in rounds, or the op switch
+const void* sweep_ptr_f64_bwd(int K, bool rounds);
 const void* sweep_ptr_f32_fwd_small(int K);    // sample groups of < 32 threads
 const void* sweep_ptr_f32_bwd_small(int K);
 const void* sweep_ptr_f64_fwd_small(int K);
@@ -19,7 +19,7 @@ const void* sweep_ptr_f32_fwd_nph(int K, bool full);
 const void* sweep_ptr_f32_bwd_nph(int K, bool full);
 const void* sweep_ptr_f32_fused_nph(int K, bool full);
 const void* pass_ptr_f32_nph(int mode, int K, bool full);
-const void* sweep_ptr_f64_fused(int K, bool full);
+const void* sweep_ptr_f64_fused(int K, bool full, bool rounds);
 // double-float arithmetic on complex128 storage (VQC_C128_DF plans)
 const void* sweep_ptr_dd_fwd(int K, bool full, bool factored);
 const void* sweep_ptr_dd_bwd(int K, bool full, bool factored);

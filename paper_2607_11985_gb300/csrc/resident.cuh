@@ -14,7 +14,9 @@ namespace vqc {
 // plain backward kernel.
 // PH2: the schedule may hold CRZ / RZZ.  Double-float: 2x2 updates throughout (else
 // factored stages, in groups of whole warps).
-template <typename R, int K, int MODE, bool FULL, bool FUSED, bool PH2 = true>
+// RND: stages in rounds, where the type has them, else the op switch throughout (the
+// launch of a complex128 circuit whose diagonal tables do not fit a CTA).
+template <typename R, int K, int MODE, bool FULL, bool FUSED, bool PH2 = true, bool RND = true>
 __global__ void __launch_bounds__(512) sweep_kernel(const __grid_constant__ KArgs<St<R>> A) {
     if (geometry_bad(blockDim.x != (unsigned)(A.S * A.tpg) || A.tpg != (1 << A.tbits) ||
                          A.tbits != A.n - K || A.n > kMaxTileBits || A.nstages < 1,
@@ -31,7 +33,7 @@ __global__ void __launch_bounds__(512) sweep_kernel(const __grid_constant__ KArg
     R* red_all = reinterpret_cast<R*>(smem + A.sm_red);
 
     constexpr bool DF = std::is_same<R, dd>::value;
-    constexpr bool ROUNDS = FULL && (!DF || Factored<R, FULL, PH2>::value);
+    constexpr bool ROUNDS = RND && FULL && (!DF || Factored<R, FULL, PH2>::value);
     constexpr bool DG = sizeof(R) == 8 && ROUNDS;   // the stages may have diagonal tables
     constexpr int EW = ResidentWords<R, MODE, FULL, PH2>::value;
     const int n = A.n, G = A.G;

@@ -303,3 +303,21 @@ def test_double_float_around_the_resident_limit(n, layers, path):
                                dw.data_ptr(), torch.cuda.current_stream().cuda_stream)
         torch.cuda.synchronize()
         assert torch.equal(dx, dx_ref) and torch.equal(dw, dw_ref)
+
+
+# native complex128 rings of RZZ whose phase tables do not fit beside the state: the op
+# switch instead, on either side of both lines
+@pytest.mark.parametrize("n,layers,path", [(11, 11, 0), (11, 12, 0), (11, 13, 1), (10, 24, 0), (10, 28, 0), (10, 29, 1),
+                                           (8, 80, 0)])
+def test_phase_tables_around_the_resident_limit(n, layers, path):
+    spec = wl.CircuitSpec(n, n, 2 * n * layers)
+    for q in range(n):
+        spec.add("RY", (q,), [("x", q)])
+    for l in range(layers):
+        for q in range(n):
+            spec.add("RZZ", (q, (q + 1) % n), [("w", 2 * n * l + q)])
+        for q in range(n):
+            spec.add("RX", (q,), [("w", 2 * n * l + n + q)])
+    c = C(spec, "c128")
+    assert c.info(5)["bwd_path"] == path
+    check(c, *draw(spec, 5, "c128", 7800 + n))
