@@ -636,7 +636,7 @@ vqc_status plan_cluster(const HostPlan& p, int mode, int B, Launch& L) {
     vqc_status st = device_info(dev, di);
     if (st != VQC_OK) return st;
     const bool dbl = p.dtype == VQC_C128;
-    const size_t rs = dbl ? 8 : 4, cs = 2 * rs, ew = entry_reals(dbl, p.dfloat);
+    const size_t rs = dbl ? 8 : 4, cs = 2 * rs, ew = entry_reals(dbl, false);   // ClusterWords
     L.K = L.s->K;
     L.cl = p.n - L.K - L.s->cta_bits;
     L.T = 1 << (p.n - L.K);           // threads of a sample group, over the whole cluster

@@ -112,8 +112,15 @@ __device__ __forceinline__ void cl_block_store(const C2<R> (&a)[1 << K], uint32_
 // the cluster), nunits (= B), x, w, psi0, E, state_out, the shared-memory
 // carve-up (sm_psi holds this CTA's slice of 2^(n - cl) amplitudes, sm_red the
 // per-warp <Z> sums, sm_ecl rank 0's [2^cl][n] gather of per-CTA sums), cl.
+// Table entries of the cluster kernels: stages are 2x2 updates throughout, so double-float
+// ones hold no factors (14 qubits, 400 x [RY CX RY CX] forward: 260 KB with them, 183 without).
+template <typename R> struct ClusterWords {
+    static constexpr int value = entry_reals(sizeof(R) == 8, false);
+};
+
 template <typename R, int K>
 __global__ void __launch_bounds__(512) cluster_fwd_kernel(const __grid_constant__ KArgs<St<R>> A) {
+    constexpr int EW = ClusterWords<R>::value;
     // every CTA of every cluster takes the same branch, before any cluster barrier
     uint32_t nrank;
     asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(nrank));
@@ -181,8 +188,8 @@ __global__ void __launch_bounds__(512) cluster_fwd_kernel(const __grid_constant_
     __syncthreads();
     for (int i = threadIdx.x; i < A.n_sh; i += nthr) {
         const DEntry e = P.entries[vqc_ld(&P.sh_list[i])];
-        eval_entry<R>(e, P.consts, static_cast<const R*>(nullptr), w_sm, Pcang, Pcmat,
-                      sh_tab + EntryWords<R>::value * e.slot);
+        eval_entry<R, EW>(e, P.consts, static_cast<const R*>(nullptr), w_sm, Pcang, Pcmat,
+                      sh_tab + EW * e.slot);
     }
 
     const int ns = A.nstages;
@@ -198,7 +205,7 @@ __global__ void __launch_bounds__(512) cluster_fwd_kernel(const __grid_constant_
         __syncthreads();
         for (int i = threadIdx.x; i < A.n_ps; i += nthr) {
             const DEntry e = P.entries[vqc_ld(&P.ps_list[i])];
-            eval_entry<R>(e, P.consts, xrow, w_sm, Pcang, Pcmat, ps_tab + EntryWords<R>::value * e.slot);
+            eval_entry<R, EW>(e, P.consts, xrow, w_sm, Pcang, Pcmat, ps_tab + EW * e.slot);
         }
         cluster_sync();   // tables ready here, every slice loaded cluster-wide
 
@@ -221,7 +228,7 @@ __global__ void __launch_bounds__(512) cluster_fwd_kernel(const __grid_constant_
             } else {
                 cl_block_load<R, K>(a, psi_sa, slice, v.swb, sg);
             }
-            run_ops<R, K, 0, true>(P.ops, vqc_ld(&sp->op_begin), vqc_ld(&sp->op_end), v.pb, a, a,
+            run_ops<R, K, 0, true, true, EW>(P.ops, vqc_ld(&sp->op_begin), vqc_ld(&sp->op_end), v.pb, a, a,
                                          sh_tab, ps_tab, nullptr, q, lane, warp);
             if (last) {   // <Z_j> partials: one butterfly per warp (n <= 16 here)
                 R ez[16];
@@ -294,6 +301,7 @@ __global__ void __launch_bounds__(512) cluster_fwd_kernel(const __grid_constant_
 // sm_xg holding the sample's x row followed by its gE row.
 template <typename R, int K>
 __global__ void __launch_bounds__(512) cluster_bwd_kernel(const __grid_constant__ KArgs<St<R>> A) {
+    constexpr int EW = ClusterWords<R>::value;
     uint32_t nrank;
     asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(nrank));
     if (geometry_bad(((unsigned)blockDim.x << A.cl) != (unsigned)A.tpg || nrank != (1u << A.cl) ||
@@ -374,8 +382,8 @@ __global__ void __launch_bounds__(512) cluster_bwd_kernel(const __grid_constant_
     __syncthreads();
     for (int i = threadIdx.x; i < A.n_sh; i += nthr) {
         const DEntry e = P.entries[vqc_ld(&P.sh_list[i])];
-        eval_entry<R>(e, P.consts, static_cast<const R*>(nullptr), w_sm, Pcang, Pcmat,
-                      sh_tab + EntryWords<R>::value * e.slot);
+        eval_entry<R, EW>(e, P.consts, static_cast<const R*>(nullptr), w_sm, Pcang, Pcmat,
+                      sh_tab + EW * e.slot);
     }
 
     const int ns = A.nstages;
@@ -395,7 +403,7 @@ __global__ void __launch_bounds__(512) cluster_bwd_kernel(const __grid_constant_
         __syncthreads();
         for (int i = threadIdx.x; i < A.n_ps; i += nthr) {
             const DEntry e = P.entries[vqc_ld(&P.ps_list[i])];
-            eval_entry<R>(e, P.consts, xrow, w_sm, Pcang, Pcmat, ps_tab + EntryWords<R>::value * e.slot);
+            eval_entry<R, EW>(e, P.consts, xrow, w_sm, Pcang, Pcmat, ps_tab + EW * e.slot);
         }
         cluster_sync();   // tables ready, every slice loaded cluster-wide
 
@@ -416,7 +424,7 @@ __global__ void __launch_bounds__(512) cluster_bwd_kernel(const __grid_constant_
                 } else {
                     cl_block_load<R, K>(a, psi_sa, slice, v.swb, sg);
                 }
-                run_ops<R, K, 0, true>(P.ops, vqc_ld(&sp->op_begin), vqc_ld(&sp->op_end), v.pb, a, a,
+                run_ops<R, K, 0, true, true, EW>(P.ops, vqc_ld(&sp->op_begin), vqc_ld(&sp->op_end), v.pb, a, a,
                                              sh_tab, ps_tab, nullptr, q, lane, warp);
                 if (s + 1 == ns) break;
                 if (vqc_ld(&sp->nperm)) {
@@ -453,7 +461,7 @@ __global__ void __launch_bounds__(512) cluster_bwd_kernel(const __grid_constant_
                     cl_block_load<R, K>(l, lam_sa, slice, b2, s2);
                 }
             }
-            run_ops<R, K, 1, true>(P.ops, vqc_ld(&sp->op_begin), vqc_ld(&sp->op_end), v.pb, a, l,
+            run_ops<R, K, 1, true, true, EW>(P.ops, vqc_ld(&sp->op_begin), vqc_ld(&sp->op_end), v.pb, a, l,
                                          sh_tab, ps_tab, acc_w, qa, lane, warp_a);
             if (s > 0) {   // back to the stage's input layout (load map)
                 if (vqc_ld(&sp->nperm)) {

@@ -321,3 +321,12 @@ def test_phase_tables_around_the_resident_limit(n, layers, path):
     c = C(spec, "c128")
     assert c.info(5)["bwd_path"] == path
     check(c, *draw(spec, 5, "c128", 7800 + n))
+
+
+# the same on the cluster path: 14 qubits forward, 13 backward
+@pytest.mark.parametrize("n,mode,kind,k", [(14, 0, "ry", 400), (13, 1, "layers", 11)])
+def test_double_float_around_the_cluster_limit(n, mode, kind, k):
+    spec = narrow(kind, n, k) if kind == "ry" else wl.layered(n, k, ("RX", "RY", "RZ"), "CX")
+    c = C(spec, "c128df")
+    assert c.info(2)["bwd_path" if mode else "fwd_path"] == 2
+    check(c, *draw(spec, 2, "c128df", 7900 + n))
