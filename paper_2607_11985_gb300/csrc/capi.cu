@@ -252,11 +252,12 @@ vqc_status plan_launch_as(const HostPlan& p, int launch_mode, int B, int K, bool
     L.wg = L.T > 32 ? L.T / 32 : 1;
     // Shared memory: a fixed part per CTA and a part per resident sample.
     const size_t dim = (size_t)1 << p.n;
-    const size_t io = (size_t)8 << L.K;   // slot offsets of the state copies
+    const size_t io = (size_t)(mode == 0 ? 8 : 4) << L.K;   // slot offsets of the state copies
     const bool factored = p.dfloat && !lean && L.T >= 32 && factors_pay(p, mode, B, *L.f, di.sms);
     const size_t ew = entry_reals(dbl, factored) / (mode == 0 && !dbl ? 2 : 1);   // ResidentWords
     const size_t fixed = align16((size_t)p.n_sh * ew * rs) + align16(mode == 1 ? (size_t)p.num_w * rs : 0) +
-                         align16((size_t)p.num_w * rs) + io + 10 * 16;
+                         align16((size_t)p.num_w * rs) + io +
+                         (mode == 0 ? 2 : 3) * 16;   // rounding up: red, xg, the backward's terms
     // diagonal tables: two-local phases, and double-float's own (complex128 schedules count both)
     L.ndg = L.T >= 32 && dbl && !lean && (p.dfloat ? factored : p.has_ph2) ? L.f->passes[0].ndg : 0;
     const size_t dgb = ((size_t)L.ndg << L.K) * cs;

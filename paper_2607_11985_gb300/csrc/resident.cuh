@@ -63,9 +63,9 @@ __global__ void __launch_bounds__(512) sweep_kernel(const __grid_constant__ KArg
     const bool from_global = src != nullptr;
     const bool final_order = MODE == 1 && A.psi_final != nullptr;   // amplitude order of src
     // slot of amplitude t + i T of a given state: a per-thread part XOR a per-i
-    // part; the latter for the given and the returned states' order, 2^K each
+    // part; the latter for the given and (forward) the returned states' order, 2^K each
     uint32_t* ioff = reinterpret_cast<uint32_t*>(smem + A.sm_io);
-    for (int i = threadIdx.x; i < (2 << K); i += blockDim.x) {
+    for (int i = threadIdx.x; i < ((MODE == 0 ? 2 : 1) << K); i += blockDim.x) {
         const uint32_t u = (uint32_t)(i & ((1 << K) - 1)) << A.tbits;
         ioff[i] = (i >> K) || final_order ? xor_cols(A.sout, u) : xor_cols(A.sin, u);
     }

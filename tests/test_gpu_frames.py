@@ -307,9 +307,11 @@ def test_double_float_around_the_resident_limit(n, layers, path):
 
 # native complex128 rings of RZZ whose phase tables do not fit beside the state: the op
 # switch instead, on either side of both lines
-@pytest.mark.parametrize("n,layers,path", [(11, 11, 0), (11, 12, 0), (11, 13, 1), (10, 24, 0), (10, 28, 0), (10, 29, 1),
-                                           (8, 80, 0)])
-def test_phase_tables_around_the_resident_limit(n, layers, path):
+# (complex64, 12 qubits x 17 layers: the layout to its last 100 bytes)
+@pytest.mark.parametrize("dtype,n,layers,path", [
+    ("c128", 11, 11, 0), ("c128", 11, 12, 0), ("c128", 11, 13, 1), ("c128", 10, 24, 0), ("c128", 10, 28, 0),
+    ("c128", 10, 29, 1), ("c128", 8, 80, 0), ("c64", 12, 17, 0), ("c64", 12, 18, 1)])
+def test_phase_tables_around_the_resident_limit(dtype, n, layers, path):
     spec = wl.CircuitSpec(n, n, 2 * n * layers)
     for q in range(n):
         spec.add("RY", (q,), [("x", q)])
@@ -318,9 +320,10 @@ def test_phase_tables_around_the_resident_limit(n, layers, path):
             spec.add("RZZ", (q, (q + 1) % n), [("w", 2 * n * l + q)])
         for q in range(n):
             spec.add("RX", (q,), [("w", 2 * n * l + n + q)])
-    c = C(spec, "c128")
-    assert c.info(5)["bwd_path"] == path
-    check(c, *draw(spec, 5, "c128", 7800 + n))
+    c = C(spec, dtype)
+    batch = 5 if dtype == "c128" else 100   # (enough for blocks of 16 amplitudes)
+    assert c.info(batch)["bwd_path"] == path
+    check(c, *draw(spec, batch, dtype, 7800 + n))
 
 
 # the same on the cluster path: 14 qubits forward, 13 backward
