@@ -1293,13 +1293,23 @@ bool use_hbm(const HostPlan& p, int mode, int B) {
 // unless the forward takes a larger register block than the backward.  The
 // fused kernel sweeps forward with the backward's schedule, so then the
 // forward call (its own, larger blocks) followed by the backward from the saved
-// states is faster (12-qubit workload, batch 4096: 1.68 ms against 1.75 ms).
+// states is faster (12-qubit workload, batch 4096: 1.68 ms against 1.75 ms).  The same where
+// a double-float forward could have taken larger blocks but for its phases (choose_k), of
+// more than a CTA per SM (rings of RZZ, batch 1600, two calls / fused: 9 qubits x 4 layers
+// 1.02 / 1.45 ms, 10 x 4 2.20 / 3.16; 12 qubits x 2, batch 100: 427 / 402 us) and not a
+// wave of few stages (8 qubits x 2: 372 / 335 us, x 4 482 / 623).
 bool resident_two_calls(const HostPlan& p, int B) {
     Launch Lf, Lb;
     const std::string saved = g_err;
     const bool ok = plan_launch(p, 0, B, Lf) == VQC_OK && plan_launch(p, 1, B, Lb) == VQC_OK;
     g_err = saved;
-    return ok && Lf.K > Lb.K;
+    if (!ok) return false;
+    int dev = 0;
+    DevInfo di;
+    if (Lf.K > Lb.K) return true;
+    if (cudaGetDevice(&dev) != cudaSuccess || device_info(dev, di) != VQC_OK) return false;
+    return choose_k(p, 0, B, di.sms, true) > Lb.K && Lb.nunits > di.sms &&
+           (Lb.nunits > Lb.grid || Lb.f->stages.size() >= 8);
 }
 
 // Workspace of the two-call form: [backward workspace | final states].

@@ -333,3 +333,23 @@ def test_double_float_around_the_cluster_limit(n, mode, kind, k):
     c = C(spec, "c128df")
     assert c.info(2)["bwd_path" if mode else "fwd_path"] == 2
     check(c, *draw(spec, 2, "c128df", 7900 + n))
+
+
+# double-float circuits with phases: forward and backward as one launch or as two calls
+# (more than one wave of CTAs), which are those of forward and backward
+@pytest.mark.parametrize("n,batch", [(9, 3), (9, 1301), (10, 640)])
+def test_double_float_phase_steps(n, batch):
+    spec = mixed(n, ("RX", "CRZ", "RZZ"))
+    c = C(spec, "c128df")
+    w_, _ = draw(spec, batch, "c128df", 8000 + n)
+    x, w, gE = (dev(a, "c128df") for a in (w_.x, w_.w, w_.gE))
+    E, st = c.forward(x, w, want_state=True)
+    dx, dw = c.backward(x, w, gE, psi_final=st)
+    E2, dx2, dw2 = c.forward_backward(x, w, gE)
+    d = 8 * U["c128df"] * len(spec.gates)
+    row = np.abs(w_.gE).sum(1) * (4 * d + 32 * U["c128df"])
+    assert maxerr(E2.cpu().numpy(), E.cpu().numpy()) <= 4 * d + 64 * U["c128df"]   # each within one bound
+    assert np.all(np.abs(dx2.cpu().numpy() - dx.cpu().numpy()) <= 2 * row[:, None])
+    assert maxerr(dw2.cpu().numpy(), dw.cpu().numpy()) <= 2 * row.sum()
+    if batch > 3:
+        assert torch.equal(E, E2) and torch.equal(dx, dx2) and torch.equal(dw, dw2)
