@@ -130,6 +130,7 @@ struct Launch {
     int sm_sh = 0, sm_ps = 0, sm_psi = 0, sm_lam = 0, sm_acc = 0, sm_terms = 0, sm_dw = 0,
         sm_red = 0, sm_plan = 0, sm_w = 0, sm_xg = 0, sm_io = 0, sm_dg = 0, ndg = 0;
     int cl = 0, sm_ecl = 0;   // cluster path: log2 CTAs per sample, <Z> gather area
+    bool factored = false;    // double-float: stages of factored runs
     bool plan_smem = false, tab_smem = true;   // resident: the plan's schedule / table data in shared memory
     const void* fn = nullptr;
 };
@@ -225,12 +226,13 @@ int choose_k(const HostPlan& p, int mode, int B, int sms, bool any_size = false)
 // stages take 2x2 updates; 9-qubit QAOA x 1600, 8 layers, forward 1036 us with the
 // factors beside them, 442 without), except small forwards of few stages, where the
 // factors and diagonals of a call, a chain of FP64 operations, take longer than they
-// save (RX RY RZ layers, CX ring, forward, factored / not: 8 qubits x 100, 1 layer 25 /
-// 22 us, 8 layers 72 / 77; 11 qubits x 1600, 1 layer 185 / 214; 12 x 100, 1 layer 47 / 54).
+// save (RX RY RZ layers, CX ring, forward, factored / not: 8 qubits x 100, 1 layer 26 /
+// 20 us, 8 layers 74 / 67; 9 x 100, 8 layers 61 / 62; 11 x 100, 1 layer 45 / 36; 11 x 1600,
+// 1 layer 180 / 211; 12 x 100, 1 layer 46 / 53).
 bool factors_pay(const HostPlan& p, int mode, int B, const FrameSchedule& f, int sms) {
     if (p.has_ph2) return false;
     const bool small = p.n <= 11 && (double)B * std::ldexp(1.0, p.n) <= sms * 8192.0;
-    return mode == 1 || f.passes[0].ndg == 0 || !small || f.stages.size() >= 12;
+    return mode == 1 || f.passes[0].ndg == 0 || !small || (p.n > 8 && f.stages.size() >= 12);
 }
 
 // The resident launch with blocks of 2^K amplitudes; lean: without diagonal tables, and
@@ -253,7 +255,7 @@ vqc_status plan_launch_as(const HostPlan& p, int launch_mode, int B, int K, bool
     // Shared memory: a fixed part per CTA and a part per resident sample.
     const size_t dim = (size_t)1 << p.n;
     const size_t io = (size_t)(mode == 0 ? 8 : 4) << L.K;   // slot offsets of the state copies
-    const bool factored = p.dfloat && !lean && L.T >= 32 && factors_pay(p, mode, B, *L.f, di.sms);
+    const bool factored = L.factored = p.dfloat && !lean && L.T >= 32 && factors_pay(p, mode, B, *L.f, di.sms);
     const size_t ew = entry_reals(dbl, factored) / (mode == 0 && !dbl ? 2 : 1);   // ResidentWords
     const size_t fixed = align16((size_t)p.n_sh * ew * rs) + align16(mode == 1 ? (size_t)p.num_w * rs : 0) +
                          align16((size_t)p.num_w * rs) + io +
@@ -346,6 +348,22 @@ vqc_status plan_launch_as(const HostPlan& p, int launch_mode, int B, int K, bool
     return VQC_OK;
 }
 
+// Of a factored launch f that fits and its lean form l, whether l is the faster one.  At 8
+// and 9 qubits a sample's updates are few beside its factors and diagonals, FP64 work of
+// every per-sample run, and its larger tables.  So l where these cost f a wave of CTAs
+// (9 qubits x 1600, re-uploading, 8 layers, forward: 544 us factored, 338 lean; weights
+// only, 303 / 347: kept but at 8 qubits), and backward, few stages, beyond a CTA per SM,
+// where most runs depend on the sample (8 qubits x 1600, 2 layers 227 / 184, 4 layers 306 /
+// 388; 9 qubits, re-uploading, 2 layers 393 / 345; one layer 209 / 215, but 232 behind a
+// lean forward).  From 10 qubits on f was faster everywhere (1.06 to 1.6 times).
+bool lean_pays(const HostPlan& p, int mode, const Launch& f, const Launch& l, int sms) {
+    if (p.n > 9 || f.ndg == 0) return false;
+    auto waves = [](const Launch& x) { return (x.nunits + x.grid - 1) / x.grid; };
+    const bool sample = 2 * p.n_ps >= p.n_runs;
+    if (waves(l) < waves(f) && (p.n == 8 || sample)) return true;
+    return mode == 1 && f.nunits > sms && f.f->stages.size() < 8 && (p.n_ps == p.n_runs || (sample && f.S * p.n_ps >= 32));
+}
+
 // The launch of the chosen block size; where a complex128 layout does not fit a CTA, the
 // lean one (double-float, 12 qubits x 7 layers of RX RY RZ, backward: 245 KB factored, 230
 // with 2x2 updates), then double-float's blocks of 16, with fewer warps to keep partials for.
@@ -358,6 +376,10 @@ vqc_status plan_launch_uncached(const HostPlan& p, int launch_mode, int B, Launc
     if (st != VQC_OK) return st;
     const int K = choose_k(p, mode, B, di.sms);
     st = plan_launch_as(p, launch_mode, B, K, false, dev, di, L);
+    if (st == VQC_OK && L.factored) {
+        Launch l;
+        if (plan_launch_as(p, launch_mode, B, K, true, dev, di, l) == VQC_OK && lean_pays(p, mode, L, l, di.sms)) L = l;
+    }
     if (st == VQC_OK || p.dtype != VQC_C128 || K == 0) return st;
     const std::string why = g_err;   // of the layout that the choice asked for
     for (int k : {K, choose_k(p, mode, B, di.sms, true)})

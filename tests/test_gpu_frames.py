@@ -353,3 +353,12 @@ def test_double_float_phase_steps(n, batch):
     assert maxerr(dw2.cpu().numpy(), dw.cpu().numpy()) <= 2 * row.sum()
     if batch > 3:
         assert torch.equal(E, E2) and torch.equal(dx, dx2) and torch.equal(dw, dw2)
+
+
+# double-float batches of more CTAs than SMs at 8 and 9 qubits: factored or not by the
+# layers and by what depends on the sample
+@pytest.mark.parametrize("n,layers,reupload", [(8, 2, False), (8, 4, False), (8, 8, False), (9, 2, True), (9, 4, True),
+                                               (9, 8, True)])
+def test_double_float_large_batches(n, layers, reupload):
+    spec = wl.layered(n, layers, ("RX", "RY", "RZ"), "CX", reupload=reupload)
+    check(C(spec, "c128df"), *draw(spec, 1303, "c128df", 8100 + n + layers))
