@@ -60,7 +60,7 @@ vqc_status cuda_fail(cudaError_t e, const char* what) {
     } while (0)
 
 struct DevInfo {
-    int sms = 0, smem_optin = 0;
+    int sms = 0, smem_optin = 0, smem_sm = 0, smem_reserved = 0;
     bool ok = false;
 };
 
@@ -74,6 +74,8 @@ vqc_status device_info(int dev, DevInfo& out) {
         VQC_CUDA(cudaDeviceGetAttribute(&g_dev[dev].sms, cudaDevAttrMultiProcessorCount, dev));
         VQC_CUDA(cudaDeviceGetAttribute(&g_dev[dev].smem_optin,
                                         cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+        VQC_CUDA(cudaDeviceGetAttribute(&g_dev[dev].smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev));
+        VQC_CUDA(cudaDeviceGetAttribute(&g_dev[dev].smem_reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev));
         g_dev[dev].ok = true;
     }
     out = g_dev[dev];
@@ -143,6 +145,22 @@ int env_int(const char* name, int dflt) {
 int cta_threads() {
     const int t = env_int("VQC_CTA_THREADS", 128);
     return t >= 32 && t <= 512 ? t : 128;
+}
+
+// Shared memory to ask for so that a grid of one wave spreads over the SMs.  A kernel that
+// is scheduled while the one before it still runs (launch) finds free shared memory
+// unevenly, and SMs then take more CTAs than their share while others stay idle: 12 qubits
+// x 100, RY x 8 layers, backward after forward 171 us, 110 spread; native complex128, 16
+// qubits x 3, step, 980 / 745 us, 11 qubits x 100, 1.8 times.  So no SM can hold more than
+// ceil(grid / SMs), as far as that asks for at most twice the memory -- for several CTAs
+// an SM at most 1.3 times, since more keeps the next kernel's CTAs out (9 qubits x 1600,
+// complex128 step 0.8 times).
+size_t spread_smem(size_t smem, int grid, int per_sm, const DevInfo& di) {
+    const int share = (grid + di.sms - 1) / di.sms;
+    if (share >= per_sm || di.smem_sm <= 0) return smem;
+    const size_t pad = align16((size_t)di.smem_sm / (share + 1) - di.smem_reserved + 1);
+    const double most = (share == 1 ? 2.0 : 1.3) * (double)smem;
+    return pad > smem && (double)pad <= most && pad <= (size_t)di.smem_optin ? pad : smem;
 }
 
 // The environment switches, read once per call from outside (a call asks for some of
@@ -345,6 +363,7 @@ vqc_status plan_launch_as(const HostPlan& p, int launch_mode, int B, int K, bool
     }
     if (per_sm < 1) return fail(VQC_ERR_UNSUPPORTED, "kernel cannot be resident with this geometry");
     L.grid = std::max(1, std::min(L.nunits, per_sm * di.sms));
+    L.smem = spread_smem(L.smem, L.grid, per_sm, di);
     return VQC_OK;
 }
 
@@ -928,6 +947,7 @@ vqc_status plan_hbm_uncached(const HostPlan& p, int mode, int B, PassGeo& L) {
     if ((long long)B * L.ntiles > 0x3fffffffLL) return fail(VQC_ERR_UNSUPPORTED, "too many tiles");
     L.nunits = (int)nunits;
     L.grid = std::max(1, std::min(L.nunits, per_sm * di.sms));
+    L.smem = spread_smem(L.smem, L.grid, per_sm, di);
     return VQC_OK;
 }
 
