@@ -253,6 +253,12 @@ bool factors_pay(const HostPlan& p, int mode, int B, const FrameSchedule& f, int
     return mode == 1 || f.passes[0].ndg == 0 || !small || (p.n > 8 && f.stages.size() >= 12);
 }
 
+// Diagonal tables of a pass: of two-local phases, and double-float's own (complex128
+// schedules hold both).
+int diagonal_tables(const HostPlan& p, const FrameSchedule& s, size_t pass) {
+    return p.dfloat ? s.passes[pass].ndg : s.phase_tables[pass];
+}
+
 // The resident launch with blocks of 2^K amplitudes; lean: without diagonal tables, and
 // double-float without the runs' factors.
 vqc_status plan_launch_as(const HostPlan& p, int launch_mode, int B, int K, bool lean, int dev, const DevInfo& di,
@@ -278,8 +284,7 @@ vqc_status plan_launch_as(const HostPlan& p, int launch_mode, int B, int K, bool
     const size_t fixed = align16((size_t)p.n_sh * ew * rs) + align16(mode == 1 ? (size_t)p.num_w * rs : 0) +
                          align16((size_t)p.num_w * rs) + io +
                          (mode == 0 ? 2 : 3) * 16;   // rounding up: red, xg, the backward's terms
-    // diagonal tables: two-local phases, and double-float's own (complex128 schedules count both)
-    L.ndg = L.T >= 32 && dbl && !lean && (p.dfloat ? factored : p.has_ph2) ? L.f->passes[0].ndg : 0;
+    L.ndg = L.T >= 32 && dbl && !lean && (p.dfloat ? factored : p.has_ph2) ? diagonal_tables(p, *L.f, 0) : 0;
     const size_t dgb = ((size_t)L.ndg << L.K) * cs;
     const size_t per_sample = dgb + (size_t)p.n_ps * ew * rs + dim * cs * (mode == 1 ? 2 : 1) +
                               (size_t)(p.num_x + p.n) * rs +
@@ -898,7 +903,7 @@ vqc_status plan_hbm_uncached(const HostPlan& p, int mode, int B, PassGeo& L) {
     L.wg = L.T > 32 ? L.T / 32 : 1;
     L.ntiles = 1 << (p.n - m);
     PassNeeds c;
-    for (const FPass& ps : L.s->passes) c.cover(ps);
+    for (size_t i = 0; i < L.s->passes.size(); ++i) c.cover(L.s->passes[i], diagonal_tables(p, *L.s, i));
     const size_t tdim = (size_t)1 << m;
     const size_t ew = entry_reals(dbl, p.dfloat);
     const size_t apv = 16 / cs, nk = (tdim / apv + L.T - 1) / L.T;
@@ -1130,7 +1135,7 @@ void fill_pass_args(const HostPlan& p, const PassGeo& L, const FPass& ps, const 
     a.sm_plan = L.sm_plan; a.sm_tfl = L.sm_tfl; a.sm_toff = L.sm_toff;
     a.sm_tbase = L.sm_tbase;
     a.sm_dg = L.sm_dg;
-    a.ndg = L.tables ? ps.ndg : 0;
+    a.ndg = L.tables ? diagonal_tables(p, s, &ps - s.passes.data()) : 0;
 }
 
 // Makes a pass read tables of its own entries and write rho sums of its own accumulators.

@@ -111,7 +111,7 @@ constexpr size_t kCtaSharedMemory = 232448;
 // of a schedule (whose launches share one layout).
 struct PassNeeds {
     int ps = 0, sh = 0, acc = 0, stages = 0, ops = 0, segs = 0, ndg = 0;
-    void cover(const FPass& p) {
+    void cover(const FPass& p, int tables) {
         auto most = [](int& a, int b) { a = b > a ? b : a; };
         most(ps, p.ps_count);
         most(sh, p.sh_count);
@@ -119,7 +119,7 @@ struct PassNeeds {
         most(stages, p.stage_end - p.stage_begin);
         most(ops, p.op_end - p.op_begin);
         most(segs, p.seg_end - p.seg_begin);
-        most(ndg, p.ndg);
+        most(ndg, tables);
     }
     // the pass's program: copies of its stages, ops, flips, rounds and FFinal
     size_t program(int nout) const {

@@ -70,7 +70,7 @@ struct FSeg {
     uint8_t flags;
     uint8_t pmask;               // positions that have a run
     // diagonal tables of the pass (kNoDiagonal: none): the group's two-local phases and
-    // (complex128) the runs' q, the runs' p
+    // (double-float's, counted for complex128) the runs' q, the runs' p
     uint16_t dg[2];
     uint16_t pad;
 };
@@ -126,6 +126,8 @@ struct FrameSchedule {
     std::vector<FSeg> segs;
     std::vector<FFlip> flips;              // [stages][nout]
     std::vector<FPass> passes;             // one on the resident path
+    std::vector<int32_t> phase_tables;     // per pass: its tables of two-local phases, numbered first
+                                           // (all that a native complex128 launch needs)
     std::vector<int32_t> pass_entries, pass_accs;
     FFinal fin{};
     size_t dev_ops = 0, dev_stages = 0, dev_segs = 0, dev_flips = 0, dev_fin = 0, dev_pass_entries = 0, dev_pass_accs = 0;

@@ -490,7 +490,7 @@ bool split(std::vector<PassPlan>& passes, const FrameSchedule& S, const HostPlan
     size_t most = 0;
     for (size_t i = 0; i < passes.size(); ++i) {
         PassNeeds c;
-        c.cover(S.passes[i]);
+        c.cover(S.passes[i], S.passes[i].ndg);
         const bool dbl = p.dtype == VQC_C128;   // (double-float plans run the same schedules)
         const PassBytes b = pass_bytes(c, p.n, S.mode, p.dtype, dbl, dbl, S.m, S.K);
         bytes.push_back(passes[i].stages.size() > 1 ? b.fixed + b.tile : 0);
@@ -549,7 +549,7 @@ FrameSchedule FrameBuilder::build(int mode, int path, const std::vector<int>& ti
         FrameSchedule S = lay_out(p, L, mode, path, m, K, passes);
         if (!tiled) return S;
         PassNeeds c;
-        for (const FPass& ps : S.passes) c.cover(ps);
+        for (const FPass& ps : S.passes) c.cover(ps, ps.ndg);
         const bool dbl = p.dtype == VQC_C128;
         const PassBytes b = pass_bytes(c, n, mode, p.dtype, dbl, dbl, m, K);
         if (b.fixed + b.tile <= kCtaSharedMemory || !split(passes, S, p)) return S;
@@ -587,6 +587,7 @@ FrameSchedule lay_out(const HostPlan& p, const FrameOps& L, int mode, int path, 
         }
     }
     S.passes.resize(np);
+    S.phase_tables.resize(np);
     S.fin = FFinal{};
     Rng rng;
     for (int step = 0; step < np; ++step) {
@@ -972,7 +973,7 @@ FrameSchedule lay_out(const HostPlan& p, const FrameOps& L, int mode, int path, 
                 const bool factors = p.dtype == VQC_C128;
                 const bool has[2] = {(sg.flags & kSegL) || (factors && (sg.flags & kSegQ)),
                                      factors && (sg.flags & kSegP)};
-                for (int k = 0; k < 2; ++k) sg.dg[k] = has[k] ? (uint16_t)fp.ndg++ : kNoDiagonal;
+                for (int k = 0; k < 2; ++k) sg.dg[k] = has[k] ? 0 : kNoDiagonal;   // numbered below
                 S.segs.push_back(sg);
             }
             st.seg_end = (int32_t)S.segs.size();
@@ -1013,6 +1014,15 @@ FrameSchedule lay_out(const HostPlan& p, const FrameOps& L, int mode, int path, 
         fp.stage_end = (int32_t)S.stages.size();
         fp.op_end = (int32_t)S.ops.size();
         fp.seg_end = (int32_t)S.segs.size();
+        // the tables: those of two-local phases, then double-float's alone
+        for (int own = 0; own < 2; ++own) {
+            for (int i = fp.seg_begin; i < fp.seg_end; ++i)
+                for (int k = 0; k < 2; ++k) {
+                    FSeg& sg = S.segs[i];
+                    if (sg.dg[k] != kNoDiagonal && (k == 0 && (sg.flags & kSegL)) == !own) sg.dg[k] = (uint16_t)fp.ndg++;
+                }
+            if (!own) S.phase_tables[pi] = fp.ndg;
+        }
         S.passes[pi] = fp;
 
         // the frame after the pass: M' vout[i] = gin[i], M' = M on the outer vectors

@@ -442,3 +442,20 @@ def test_split_passes(monkeypatch, kind, k):
     x, w, gE = rng.uniform(-3, 3, (1, 1)), rng.uniform(-3, 3, 1), rng.standard_normal((1, 13))
     fr = check(spec, x, w, gE, None, 1)
     assert any(len(s["passes"]) > 1 for s in fr if s["path"] == 1)
+
+
+def test_phase_tables_come_first():
+    # native complex128 launches hold the tables of two-local phases only
+    spec = wl.CircuitSpec(14, 14, 0)
+    for l in range(3):
+        for q in range(14):
+            spec.add("RY", (q,), [("x", q)]).add("RZZ", (q, (q + 1) % 14), [("c", 0.4)])
+    plan = compile_spec(spec, 1)
+    for s in frames(plan):
+        for ps in s["passes"]:
+            sg = s["segs"][ps["seg_begin"]:ps["seg_end"]]
+            ll = sg[(sg["flags"] & LL) != 0]["dg"][:, 0]
+            assert sorted(ll) == list(range(len(ll)))
+            every = sg["dg"][sg["dg"] != NO_DIAGONAL]
+            assert sorted(every) == list(range(ps["ndg"]))
+    B.vqc_free(plan)
