@@ -154,10 +154,11 @@ int cta_threads() {
 // qubits x 3, step, 980 / 745 us, 11 qubits x 100, 1.8 times.  So no SM can hold more than
 // ceil(grid / SMs), as far as that asks for at most twice the memory -- for several CTAs
 // an SM at most 1.3 times, since more keeps the next kernel's CTAs out (9 qubits x 1600,
-// complex128 step 0.8 times).
+// complex128 step 0.8 times).  Grids of half the SMs find as many free ones, and the larger
+// request itself took time (double-float, 9 qubits x 3, step 316 -> 339 us).
 size_t spread_smem(size_t smem, int grid, int per_sm, const DevInfo& di) {
     const int share = (grid + di.sms - 1) / di.sms;
-    if (share >= per_sm || di.smem_sm <= 0) return smem;
+    if (share >= per_sm || 2 * grid <= di.sms || di.smem_sm <= 0) return smem;
     const size_t pad = align16((size_t)di.smem_sm / (share + 1) - di.smem_reserved + 1);
     const double most = (share == 1 ? 2.0 : 1.3) * (double)smem;
     return pad > smem && (double)pad <= most && pad <= (size_t)di.smem_optin ? pad : smem;
