@@ -359,11 +359,10 @@ __device__ __forceinline__ void apply_group(const uint2* b, const uint2* e, uint
             if (TWO) l[r] = cmul<R>(l[r], g);
         }
     } else if (__any_sync(0xffffffffu, neg)) {
-        const R s = neg ? R(-1) : R(1);
 #pragma unroll
         for (int r = 0; r < (1 << K); ++r) {
-            a[r] = cm<R>(s * a[r].x, s * a[r].y);
-            if (TWO) l[r] = cm<R>(s * l[r].x, s * l[r].y);
+            a[r] = negated<R>(a[r], neg);
+            if (TWO) l[r] = negated<R>(l[r], neg);
         }
     }
     for (; b < e; ++b) {   // both local: CZ here, phases in the table

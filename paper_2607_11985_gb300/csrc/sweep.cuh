@@ -601,6 +601,19 @@ __device__ __forceinline__ void m1_back(C2<R> (&a)[1 << K], C2<R> (&l)[1 << K], 
     }
 }
 
+// v, negated when p.  double: its sign bit, beside the FP64 pipe, which a product with -1
+// would take 16 cycles a warp of.
+template <typename R>
+__device__ __forceinline__ C2<R> negated(C2<R> v, bool p) {
+    if constexpr (std::is_same<R, double>::value) {
+        const int m = p ? (int)0x80000000 : 0;
+        return cm<R>(__hiloint2double(__double2hiint(v.x) ^ m, __double2loint(v.x)),
+                     __hiloint2double(__double2hiint(v.y) ^ m, __double2loint(v.y)));
+    } else {
+        const R s = p ? R(-1) : R(1);
+        return cm<R>(s * v.x, s * v.y);
+    }
+}
 // Negate amplitudes with local bits A and Bq set (when p) -- CZ inside the block.
 template <typename R, int K, int A, int Bq>
 __device__ __forceinline__ void z2_ll(C2<R> (&a)[1 << K]) {
@@ -610,10 +623,9 @@ __device__ __forceinline__ void z2_ll(C2<R> (&a)[1 << K]) {
 }
 template <typename R, int K, int A>
 __device__ __forceinline__ void z1_pred(C2<R> (&a)[1 << K], bool p) {
-    const R s = p ? R(-1) : R(1);
 #pragma unroll
     for (int r = 0; r < (1 << K); ++r)
-        if ((r >> A) & 1) a[r] = cm<R>(s * a[r].x, s * a[r].y);
+        if ((r >> A) & 1) a[r] = negated<R>(a[r], p);
 }
 
 // ---------------------------------------------------------------- reductions
@@ -1067,11 +1079,11 @@ __device__ __forceinline__ void apply_op(uint2 raw, uint32_t pb, C2<R> (&a)[1 <<
         VQC_CZPL(0) VQC_CZPL(1) VQC_CZPL(2) VQC_CZPL(3) VQC_CZPL(4)
 #undef VQC_CZPL
     case DC_CZ_PP: {
-        const R sgn = (physbit(pb, ra) && physbit(pb, rb)) ? R(-1) : R(1);
+        const bool neg = physbit(pb, ra) && physbit(pb, rb);
 #pragma unroll
         for (int r = 0; r < (1 << K); ++r) {
-            a[r] = cm<R>(sgn * a[r].x, sgn * a[r].y);
-            if (MODE == 1) l[r] = cm<R>(sgn * l[r].x, sgn * l[r].y);
+            a[r] = negated<R>(a[r], neg);
+            if (MODE == 1) l[r] = negated<R>(l[r], neg);
         }
         break;
     }
