@@ -260,8 +260,8 @@ int diagonal_tables(const HostPlan& p, const FrameSchedule& s, size_t pass) {
     return p.dfloat ? s.passes[pass].ndg : s.phase_tables[pass];
 }
 
-// The resident launch with blocks of 2^K amplitudes; lean: without diagonal tables, and
-// double-float without the runs' factors.
+// The resident launch with blocks of 2^K amplitudes; lean: without diagonal tables, native
+// complex128 by the op switch, double-float without the runs' factors.
 vqc_status plan_launch_as(const HostPlan& p, int launch_mode, int B, int K, bool lean, int dev, const DevInfo& di,
                           Launch& L) {
     // mode 2 (fused) has the backward's schedule and layout, its own kernel
@@ -373,6 +373,23 @@ vqc_status plan_launch_as(const HostPlan& p, int launch_mode, int B, int K, bool
     return VQC_OK;
 }
 
+// Native complex128 resident sweeps: whether stages in rounds are the faster ones.  They
+// are for circuits without diagonal ops, and where a round that has phases has two or
+// more of them to collect (RZZ rings, 2.5 to 4: 9 qubits x 1600, one layer, forward 0.75 of
+// the op switch's time, 8 to 13 qubits 0.9 to 1.0).  With fewer (random circuits, 1.3 to
+// 1.8; step, 9 qubits x 100, 500 gates: 1.92 ms, 1.76 by the switch) or signs only (CZ
+// rings, forward 1.02 to 1.08 of the switch's time) the walk over the groups costs more.
+bool rounds_pay(const FrameSchedule& f) {
+    int phases = 0, groups = 0, signs = 0;
+    for (const FSeg& s : f.segs) {
+        int here = 0;
+        for (int i = s.op_begin; i < s.run_begin; ++i) ++(f.ops[i].code >= DC_PH2_LL ? here : signs);
+        phases += here;
+        groups += here > 0;
+    }
+    return phases ? phases >= 2 * groups : signs == 0;
+}
+
 // Of a factored launch f that fits and its lean form l, whether l is the faster one.  At 8
 // and 9 qubits a sample's updates are few beside its factors and diagonals, FP64 work of
 // every per-sample run, and its larger tables.  So l where these cost f a wave of CTAs
@@ -400,12 +417,14 @@ vqc_status plan_launch_uncached(const HostPlan& p, int launch_mode, int B, Launc
     vqc_status st = device_info(dev, di);
     if (st != VQC_OK) return st;
     const int K = choose_k(p, mode, B, di.sms);
-    st = plan_launch_as(p, launch_mode, B, K, false, dev, di, L);
+    const FrameSchedule* f = K ? find_frame(p, mode, VQC_PATH_RESIDENT, K) : nullptr;
+    const bool by_switch = f && p.dtype == VQC_C128 && !p.dfloat && !rounds_pay(*f);
+    st = plan_launch_as(p, launch_mode, B, K, by_switch, dev, di, L);
     if (st == VQC_OK && L.factored) {
         Launch l;
         if (plan_launch_as(p, launch_mode, B, K, true, dev, di, l) == VQC_OK && lean_pays(p, mode, L, l, di.sms)) L = l;
     }
-    if (st == VQC_OK || p.dtype != VQC_C128 || K == 0) return st;
+    if (st == VQC_OK || p.dtype != VQC_C128 || K == 0 || by_switch) return st;
     const std::string why = g_err;   // of the layout that the choice asked for
     for (int k : {K, choose_k(p, mode, B, di.sms, true)})
         if (plan_launch_as(p, launch_mode, B, k, true, dev, di, L) == VQC_OK) return VQC_OK;

@@ -15,7 +15,7 @@ namespace vqc {
 // PH2: the schedule may hold CRZ / RZZ.  Double-float: 2x2 updates throughout (else
 // factored stages, in groups of whole warps).
 // RND: stages in rounds, where the type has them, else the op switch throughout (the
-// launch of a complex128 circuit whose diagonal tables do not fit a CTA).
+// launch of a complex128 circuit with few phases a round or no room for their tables).
 template <typename R, int K, int MODE, bool FULL, bool FUSED, bool PH2 = true, bool RND = true>
 __global__ void __launch_bounds__(512) sweep_kernel(const __grid_constant__ KArgs<St<R>> A) {
     if (geometry_bad(blockDim.x != (unsigned)(A.S * A.tpg) || A.tpg != (1 << A.tbits) ||
