@@ -27,8 +27,9 @@ namespace {
 // call does not repeat the attribute and occupancy queries.
 struct GeoKey {
     const void* plan;
-    int mode, batch, dev, hbm;
+    int mode, batch, dev, hbm, arith;
     bool operator<(const GeoKey& o) const {
+        if (arith != o.arith) return arith < o.arith;
         if (plan != o.plan) return plan < o.plan;
         if (mode != o.mode) return mode < o.mode;
         if (batch != o.batch) return batch < o.batch;
@@ -171,6 +172,18 @@ struct Env {
     bool plan_smem = true, force = false, hbm = false, cluster = false;
 };
 thread_local Env t_env;
+
+// The arithmetic that launch geometry is worked out for: the plan's own (-1), or native
+// (0) or double-float (1) for a complex128 plan.  A workspace holds either of them, so
+// that plans of the two types can share one (vqc_workspace_bytes).
+thread_local int t_arith = -1;
+struct ArithScope {
+    const int saved = t_arith;
+    explicit ArithScope(int a) { t_arith = a; }
+    ~ArithScope() { t_arith = saved; }
+};
+bool dfloat_of(const HostPlan& p) { return t_arith < 0 ? p.dfloat : p.dtype == VQC_C128 && t_arith == 1; }
+
 thread_local int t_env_depth = 0;
 struct EnvScope {
     EnvScope() {
@@ -232,7 +245,7 @@ int choose_k(const HostPlan& p, int mode, int B, int sms, bool any_size = false)
     // Double-float circuits with CRZ / RZZ: blocks of 8 where threads allow (ph2_any; 11-qubit
     // QAOA x 1600, 8 layers, forward 1.57 ms, 2.40 with blocks of 16).
     // any_size: without that rule, where such a launch does not fit.
-    if (!any_size && p.dfloat && p.has_ph2 && kmax > 3 && find_frame(p, mode, VQC_PATH_RESIDENT, 3)) kmax = 3;
+    if (!any_size && dfloat_of(p) && p.has_ph2 && kmax > 3 && find_frame(p, mode, VQC_PATH_RESIDENT, 3)) kmax = 3;
     const int kmin = std::min(kmax, 3);
     const double want = (double)sms * 4 * 32;
     int K = kmax;
@@ -257,7 +270,7 @@ bool factors_pay(const HostPlan& p, int mode, int B, const FrameSchedule& f, int
 // Diagonal tables of a pass: of two-local phases, and double-float's own (complex128
 // schedules hold both).
 int diagonal_tables(const HostPlan& p, const FrameSchedule& s, size_t pass) {
-    return p.dfloat ? s.passes[pass].ndg : s.phase_tables[pass];
+    return dfloat_of(p) ? s.passes[pass].ndg : s.phase_tables[pass];
 }
 
 // The resident launch with blocks of 2^K amplitudes; lean: without diagonal tables, native
@@ -280,12 +293,12 @@ vqc_status plan_launch_as(const HostPlan& p, int launch_mode, int B, int K, bool
     // Shared memory: a fixed part per CTA and a part per resident sample.
     const size_t dim = (size_t)1 << p.n;
     const size_t io = (size_t)(mode == 0 ? 8 : 4) << L.K;   // slot offsets of the state copies
-    const bool factored = L.factored = p.dfloat && !lean && L.T >= 32 && factors_pay(p, mode, B, *L.f, di.sms);
+    const bool factored = L.factored = dfloat_of(p) && !lean && L.T >= 32 && factors_pay(p, mode, B, *L.f, di.sms);
     const size_t ew = entry_reals(dbl, factored) / (mode == 0 && !dbl ? 2 : 1);   // ResidentWords
     const size_t fixed = align16((size_t)p.n_sh * ew * rs) + align16(mode == 1 ? (size_t)p.num_w * rs : 0) +
                          align16((size_t)p.num_w * rs) + io +
                          (mode == 0 ? 2 : 3) * 16;   // rounding up: red, xg, the backward's terms
-    L.ndg = L.T >= 32 && dbl && !lean && (p.dfloat ? factored : p.has_ph2) ? diagonal_tables(p, *L.f, 0) : 0;
+    L.ndg = L.T >= 32 && dbl && !lean && (dfloat_of(p) ? factored : p.has_ph2) ? diagonal_tables(p, *L.f, 0) : 0;
     const size_t dgb = ((size_t)L.ndg << L.K) * cs;
     const size_t per_sample = dgb + (size_t)p.n_ps * ew * rs + dim * cs * (mode == 1 ? 2 : 1) +
                               (size_t)(p.num_x + p.n) * rs +
@@ -328,7 +341,7 @@ vqc_status plan_launch_as(const HostPlan& p, int launch_mode, int B, int K, bool
     L.sm_red = take((size_t)L.S * L.wg * p.n * rs);   // <Z> partials (forward, or recompute with E)
     L.sm_w = take((size_t)p.num_w * rs);
     L.sm_xg = take((size_t)L.S * (p.num_x + p.n) * rs);
-    L.fn = kernel_ptr(p.dtype, p.dfloat, launch_mode, L.K, L.T >= 32, p.has_ph2, factored, !lean);
+    L.fn = kernel_ptr(p.dtype, dfloat_of(p), launch_mode, L.K, L.T >= 32, p.has_ph2, factored, !lean);
     if (!L.fn) return fail(VQC_ERR_UNSUPPORTED, "kernel not instantiated for this K");
     st = allow_max_smem(L.fn, dev, di.smem_optin);
     if (st != VQC_OK) return st;
@@ -418,7 +431,7 @@ vqc_status plan_launch_uncached(const HostPlan& p, int launch_mode, int B, Launc
     if (st != VQC_OK) return st;
     const int K = choose_k(p, mode, B, di.sms);
     const FrameSchedule* f = K ? find_frame(p, mode, VQC_PATH_RESIDENT, K) : nullptr;
-    const bool by_switch = f && p.dtype == VQC_C128 && !p.dfloat && !rounds_pay(*f);
+    const bool by_switch = f && p.dtype == VQC_C128 && !dfloat_of(p) && !rounds_pay(*f);
     st = plan_launch_as(p, launch_mode, B, K, by_switch, dev, di, L);
     if (st == VQC_OK && L.factored) {
         Launch l;
@@ -434,13 +447,14 @@ vqc_status plan_launch_uncached(const HostPlan& p, int launch_mode, int B, Launc
 std::mutex g_geo_mu;
 std::map<GeoKey, Launch> g_launch_cache;
 std::map<GeoKey, Launch> g_cluster_cache;   // cluster-path geometry (forget_plan clears it too)
+std::map<GeoKey, size_t> g_workspace_cache;  // complex128: of both arithmetics
 
 GeoKey geo_key(const HostPlan& p, int mode, int B, int hbm) {
     int dev = -1;
     cudaGetDevice(&dev);
     // environment switches that change the geometry are part of the key
     const int env = t_env.k_fwd * 1000 + t_env.k_bwd * 10 + (t_env.plan_smem ? 1 : 0) + t_env.cta * 1000000;
-    return GeoKey{&p, mode, B, dev, hbm * 100000 + env};
+    return GeoKey{&p, mode, B, dev, hbm * 100000 + env, t_arith};
 }
 
 vqc_status plan_launch(const HostPlan& p, int mode, int B, Launch& L) {
@@ -740,7 +754,7 @@ vqc_status plan_cluster(const HostPlan& p, int mode, int B, Launch& L) {
     L.smem = off;
     if (L.smem > (size_t)di.smem_optin)
         return fail(VQC_ERR_UNSUPPORTED, "cluster slice does not fit in shared memory");
-    L.fn = mode == 0 ? (p.dfloat ? cluster_ptr_dd() : cluster_ptr(dbl)) : cluster_bwd_ptr(dbl, p.dfloat);
+    L.fn = mode == 0 ? (dfloat_of(p) ? cluster_ptr_dd() : cluster_ptr(dbl)) : cluster_bwd_ptr(dbl, dfloat_of(p));
     st = allow_max_smem(L.fn, dev, di.smem_optin);
     if (st != VQC_OK) return st;
     cudaLaunchConfig_t cfg{};
@@ -793,7 +807,7 @@ bool use_cluster(const HostPlan& p, int mode, int B) {
     if (t_env.cluster) return cluster_fits(p, mode);
     if (t_env.hbm) return false;
     if (p.n - s->K - s->cta_bits != 1) return false;
-    if (!(p.dfloat && mode == 1) && find_frame(p, mode, VQC_PATH_HBM)) {
+    if (!(dfloat_of(p) && mode == 1) && find_frame(p, mode, VQC_PATH_HBM)) {
         int dev = 0, sms = 152;   // without a device: GB300's SM count
         DevInfo di;
         if (cudaGetDevice(&dev) == cudaSuccess && device_info(dev, di) == VQC_OK) sms = di.sms;
@@ -925,10 +939,10 @@ vqc_status plan_hbm_uncached(const HostPlan& p, int mode, int B, PassGeo& L) {
     PassNeeds c;
     for (size_t i = 0; i < L.s->passes.size(); ++i) c.cover(L.s->passes[i], diagonal_tables(p, *L.s, i));
     const size_t tdim = (size_t)1 << m;
-    const size_t ew = entry_reals(dbl, p.dfloat);
+    const size_t ew = entry_reals(dbl, dfloat_of(p));
     const size_t apv = 16 / cs, nk = (tdim / apv + L.T - 1) / L.T;
-    L.tables = L.T >= 32 && dbl && (p.dfloat || p.has_ph2);   // as on the resident path
-    const PassBytes pb = pass_bytes(c, p.n, mode, p.dtype, p.dfloat, L.tables, m, L.K);
+    L.tables = L.T >= 32 && dbl && (dfloat_of(p) || p.has_ph2);   // as on the resident path
+    const PassBytes pb = pass_bytes(c, p.n, mode, p.dtype, dfloat_of(p), L.tables, m, L.K);
     const size_t fixed = pb.fixed, per_tile = pb.tile;
     int S = std::max(1, 128 / L.T);
     if ((size_t)di.smem_optin <= fixed + per_tile)
@@ -959,7 +973,7 @@ vqc_status plan_hbm_uncached(const HostPlan& p, int mode, int B, PassGeo& L) {
     L.sm_plan = take(c.program(L.s->nout));
     L.sm_tfl = take((size_t)S * (c.stages + 1) * 8);
     L.smem = off;
-    L.fn = p.dfloat ? pass_ptr_dd(mode, L.K, L.T >= 32)
+    L.fn = dfloat_of(p) ? pass_ptr_dd(mode, L.K, L.T >= 32)
            : (!dbl && !p.has_ph2) ? pass_ptr_f32_nph(mode, L.K, L.T >= 32)   // no phase cases
                                   : pass_ptr(dbl, mode, L.K, L.T >= 32);
     if (!L.fn) return fail(VQC_ERR_UNSUPPORTED, "pass kernel not instantiated for this K");
@@ -1004,6 +1018,8 @@ void forget_plan(const HostPlan* p) {
         it = it->first.plan == p ? g_pass_cache.erase(it) : std::next(it);
     for (auto it = g_cluster_cache.begin(); it != g_cluster_cache.end();)
         it = it->first.plan == p ? g_cluster_cache.erase(it) : std::next(it);
+    for (auto it = g_workspace_cache.begin(); it != g_workspace_cache.end();)
+        it = it->first.plan == p ? g_workspace_cache.erase(it) : std::next(it);
 }
 
 // Workspace of the HBM path.  Forward: [control | working state | <Z> partials |
@@ -1020,7 +1036,7 @@ size_t hbm_state_bytes(const HostPlan& p, int B) {
 HbmWs hbm_layout(const HostPlan& p, int mode, int B, int ntiles) {
     const size_t rs = p.dtype == VQC_C128 ? 8 : 4;
     const size_t sbytes = hbm_state_bytes(p, B);
-    const size_t entry = entry_reals(p.dtype == VQC_C128, p.dfloat) * rs;
+    const size_t entry = entry_reals(p.dtype == VQC_C128, dfloat_of(p)) * rs;
     HbmWs w;
     w.state = 256;
     if (mode == 0) {
@@ -1042,7 +1058,7 @@ HbmWs hbm_layout(const HostPlan& p, int mode, int B, int ntiles) {
 // call's whole ones would exceed the built-in scratch of vqc_backward_noalloc.
 HbmWs hbm_layout_by_pass(const HostPlan& p, int B, int ntiles) {
     const size_t rs = p.dtype == VQC_C128 ? 8 : 4, sbytes = hbm_state_bytes(p, B);
-    const size_t entry = entry_reals(p.dtype == VQC_C128, p.dfloat) * rs;
+    const size_t entry = entry_reals(p.dtype == VQC_C128, dfloat_of(p)) * rs;
     size_t accs = 1, ps = 0, sh = 0;
     for (int mode = 0; mode < 2; ++mode)
         for (const auto& f : find_frame(p, mode, VQC_PATH_HBM)->passes) {
@@ -1528,6 +1544,61 @@ vqc_status backward_with_scratch(const vqc_plan* plan, int32_t batch, const void
                        grad_w, scratch, scratch_bytes, s, true);
 }
 
+namespace {
+
+// Workspace bytes of a call in the arithmetic of t_arith.
+size_t workspace_need(const vqc_plan* plan, int batch, int mode) {
+    if (mode == 3) {   // vqc_forward_backward: its one-launch form, or either call's workspace
+        size_t need = std::max(workspace_need(plan, batch, 0), workspace_need(plan, batch, 1));
+        const HostPlan& p = plan->hp;
+        Launch L;
+        const std::string saved = g_err;
+        if (batch > 0 && !use_cluster(p, 0, batch) && !use_hbm(p, 0, batch) && !use_hbm(p, 1, batch)) {
+            if (resident_two_calls(p, batch)) {
+                const size_t cs = p.dtype == VQC_C128 ? 16 : 8;
+                need = std::max(need, two_call_state_offset(p, batch) + align256(((size_t)batch << p.n) * cs));
+            } else if (plan_launch(p, 2, batch, L) == VQC_OK) {
+                need = std::max(need, bwd_workspace(p, L));
+            }
+        }
+        if (batch > 0 && !use_cluster(p, 1, batch) && use_hbm(p, 1, batch)) {
+            // the final states in the backward's psi region, the forward's workspace behind them
+            need = std::max(need, hbm_state_bytes(p, batch) + workspace_need(plan, batch, 0));
+        }
+        if (batch > 0 && use_cluster(p, 1, batch)) {   // [either call's workspace | final states]
+            const size_t cs = p.dtype == VQC_C128 ? 16 : 8;
+            need = align256(need) + align256(((size_t)batch << p.n) * cs);
+        }
+        g_err = saved;
+        return need;
+    }
+    if (mode == 2 && batch > 0) {   // vqc_probabilities: forward workspace + state + E
+        const HostPlan& p = plan->hp;
+        const size_t rs = p.dtype == VQC_C128 ? 8 : 4;
+        return align256(workspace_need(plan, batch, 0)) +
+               align256(((size_t)batch << p.n) * 2 * rs) + align256((size_t)batch * p.n * rs);
+    }
+    if ((mode != 0 && mode != 1) || batch <= 0) return 0;
+    const HostPlan& p = plan->hp;
+    if (use_cluster(p, mode, batch)) {
+        if (mode == 0) return 0;
+        Launch L;
+        if (plan_cluster(p, 1, batch, L) != VQC_OK) return 0;
+        return cluster_bwd_workspace(p, L);
+    }
+    if (use_hbm(p, mode, batch)) {
+        PassGeo L;
+        if (plan_hbm(p, mode, batch, L) != VQC_OK) return 0;
+        return hbm_layout(p, mode, batch, L.ntiles).total;
+    }
+    if (mode == 0) return 0;
+    Launch L;
+    if (plan_launch(p, 1, batch, L) != VQC_OK) return 0;
+    return bwd_workspace(p, L);
+}
+
+}  // namespace
+
 }  // namespace vqc
 
 using namespace vqc;
@@ -1595,54 +1666,27 @@ void vqc_free(vqc_plan* plan) {
 
 size_t vqc_workspace_bytes(const vqc_plan* plan, int32_t batch, int32_t mode) {
     if (!plan) return (size_t)-1;
-    const EnvScope env;
-    if (mode == 3) {   // vqc_forward_backward: its one-launch form, or either call's workspace
-        size_t need = std::max(vqc_workspace_bytes(plan, batch, 0), vqc_workspace_bytes(plan, batch, 1));
+    try {
+        const EnvScope env;
         const HostPlan& p = plan->hp;
-        Launch L;
-        const std::string saved = g_err;
-        if (batch > 0 && !use_cluster(p, 0, batch) && !use_hbm(p, 0, batch) && !use_hbm(p, 1, batch)) {
-            if (resident_two_calls(p, batch)) {
-                const size_t cs = p.dtype == VQC_C128 ? 16 : 8;
-                need = std::max(need, two_call_state_offset(p, batch) + align256(((size_t)batch << p.n) * cs));
-            } else if (plan_launch(p, 2, batch, L) == VQC_OK) {
-                need = std::max(need, bwd_workspace(p, L));
-            }
+        if (p.dtype != VQC_C128) return workspace_need(plan, batch, mode);
+        // either arithmetic's (t_arith), kept: the launches of both are worked out once
+        const GeoKey k = geo_key(p, mode, batch, 3 + (t_env.hbm ? 1 : 0) + (t_env.cluster ? 2 : 0));
+        {
+            std::lock_guard<std::mutex> lk(g_geo_mu);
+            auto it = g_workspace_cache.find(k);
+            if (it != g_workspace_cache.end()) return it->second;
         }
-        if (batch > 0 && !use_cluster(p, 1, batch) && use_hbm(p, 1, batch)) {
-            // the final states in the backward's psi region, the forward's workspace behind them
-            need = std::max(need, hbm_state_bytes(p, batch) + vqc_workspace_bytes(plan, batch, 0));
+        size_t need = 0;
+        for (int a : {0, 1}) {
+            const ArithScope as(a);
+            need = std::max(need, workspace_need(plan, batch, mode));
         }
-        if (batch > 0 && use_cluster(p, 1, batch)) {   // [either call's workspace | final states]
-            const size_t cs = p.dtype == VQC_C128 ? 16 : 8;
-            need = align256(need) + align256(((size_t)batch << p.n) * cs);
-        }
-        g_err = saved;
-        return need;
+        std::lock_guard<std::mutex> lk(g_geo_mu);
+        return g_workspace_cache[k] = need;
+    } catch (...) {
+        return (size_t)-1;
     }
-    if (mode == 2 && batch > 0) {   // vqc_probabilities: forward workspace + state + E
-        const HostPlan& p = plan->hp;
-        const size_t rs = p.dtype == VQC_C128 ? 8 : 4;
-        return align256(vqc_workspace_bytes(plan, batch, 0)) +
-               align256(((size_t)batch << p.n) * 2 * rs) + align256((size_t)batch * p.n * rs);
-    }
-    if ((mode != 0 && mode != 1) || batch <= 0) return 0;
-    const HostPlan& p = plan->hp;
-    if (use_cluster(p, mode, batch)) {
-        if (mode == 0) return 0;
-        Launch L;
-        if (plan_cluster(p, 1, batch, L) != VQC_OK) return 0;
-        return cluster_bwd_workspace(p, L);
-    }
-    if (use_hbm(p, mode, batch)) {
-        PassGeo L;
-        if (plan_hbm(p, mode, batch, L) != VQC_OK) return 0;
-        return hbm_layout(p, mode, batch, L.ntiles).total;
-    }
-    if (mode == 0) return 0;
-    Launch L;
-    if (plan_launch(p, 1, batch, L) != VQC_OK) return 0;
-    return bwd_workspace(p, L);
 }
 
 vqc_status vqc_probabilities(const vqc_plan* plan, int32_t batch, const void* x, const void* w,

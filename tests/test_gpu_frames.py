@@ -362,3 +362,31 @@ def test_double_float_phase_steps(n, batch):
 def test_double_float_large_batches(n, layers, reupload):
     spec = wl.layered(n, layers, ("RX", "RY", "RZ"), "CX", reupload=reupload)
     check(C(spec, "c128df"), *draw(spec, 1303, "c128df", 8100 + n + layers))
+
+
+# the two complex128 types take workspaces of one size, whichever of them sized it
+@pytest.mark.parametrize("n", [4, 8, 9, 10, 11, 12, 13, 14, 15, 16])
+@pytest.mark.parametrize("kinds,layers", [(("RX", "RY", "RZ", "CX"), 1), (("RX", "RY", "RZ", "CX"), 8), (("RX", "RZZ"), 2)])
+def test_complex128_workspaces(n, kinds, layers):
+    spec = mixed(n, kinds, layers=layers)
+    native, df = C(spec, "c128"), C(spec, "c128df")
+    for batch in (1, 7, 60, 77, 100, 333, 1600):
+        for mode in range(4):
+            assert B.vqc_workspace_bytes(native.plan, batch, mode) == B.vqc_workspace_bytes(df.plan, batch, mode)
+
+
+def test_complex128_workspace_of_the_other_type():
+    spec = mixed(13, ("RX", "RY", "CX"))
+    native = C(spec, "c128")
+    for batch in (3, 90):
+        w_, _ = draw(spec, batch, "c128df", 8200)
+        x, w, gE = (dev(a, "c128df") for a in (w_.x, w_.w, w_.gE))
+        c = C(spec, "c128df")
+        want = c.forward_backward(x, w, gE)
+        E, dx, dw = (torch.empty_like(t) for t in want)
+        nbytes = B.vqc_workspace_bytes(native.plan, batch, 3)
+        ws = torch.zeros(nbytes, dtype=torch.uint8, device="cuda")
+        B.vqc_forward_backward(c.plan, batch, x.data_ptr(), w.data_ptr(), None, gE.data_ptr(), E.data_ptr(), dx.data_ptr(),
+                               dw.data_ptr(), ws.data_ptr(), nbytes, torch.cuda.current_stream().cuda_stream)
+        torch.cuda.synchronize()
+        assert all(torch.equal(a, b) for a, b in zip(want, (E, dx, dw)))
