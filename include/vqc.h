@@ -120,10 +120,11 @@ typedef enum {
                                taken by default for 2-CTA clusters (forward: complex64 15
                                qubits, complex128 14; backward: complex64 14, complex128 13)
                                and batches of at most half as many samples as the device has
-                               SMs (the double-float backward: any batch; vqc_backward_noalloc:
-                               also where the passes' states exceed its scratch), otherwise
-                               only when the environment sets VQC_FORCE_PATH=cluster (measured
-                               slower than VQC_PATH_HBM); VQC_FORCE_PATH=hbm turns it off.  The backward's workspace is a
+                               SMs (the double-float backward: any batch; others also where the
+                               passes' states exceed 16 GiB, vqc_backward_noalloc: its scratch),
+                               otherwise only when the environment sets VQC_FORCE_PATH=cluster
+                               (measured slower than VQC_PATH_HBM); VQC_FORCE_PATH=hbm turns it
+                               off.  The backward's workspace is a
                                256-byte control block and one dw partial per cluster. */
 } vqc_path;
 

@@ -698,6 +698,11 @@ vqc_status run(const HostPlan& p, int mode, int B, const void* x, const void* w,
 
 // ---------------------------------------------------------------- cluster path
 
+// One state per sample of a batch, as the passes keep it in HBM.
+size_t hbm_state_bytes(const HostPlan& p, int B) {
+    return align256((size_t)B * ((size_t)1 << p.n) * (p.dtype == VQC_C128 ? 16 : 8));
+}
+
 vqc_status plan_cluster(const HostPlan& p, int mode, int B, Launch& L) {
     const GeoKey k = geo_key(p, mode, B, 2);
     {
@@ -799,8 +804,11 @@ bool cluster_fits(const HostPlan& p, int mode) {
 // 191 / 232 / 312 and 118 / 172 / 200 us; complex128 1.0 to 1.3 times.  (Within a wave
 // the passes are 1.0 to 2.2 times faster too; that choice is kept for its workspace,
 // which holds no states.)  The double-float backward stays on clusters: 762 / 1319 /
-// 1555 us at batch 152 against 770 / 2203 / 1558 by passes.  Larger clusters run only
+// 1555 us at batch 152 against 770 / 2203 / 1558 by passes.  Batches whose states between
+// passes exceed kPassStates (65536 samples of a 14-qubit backward) take clusters too,
+// which need none.  Larger clusters run only
 // when VQC_FORCE_PATH=cluster asks; VQC_FORCE_PATH=hbm turns them off.
+constexpr size_t kPassStates = (size_t)16 << 30;
 bool use_cluster(const HostPlan& p, int mode, int B) {
     const Schedule* s = find_cluster_schedule(p, mode);
     if (!s) return false;
@@ -812,7 +820,7 @@ bool use_cluster(const HostPlan& p, int mode, int B) {
         DevInfo di;
         if (cudaGetDevice(&dev) == cudaSuccess && device_info(dev, di) == VQC_OK) sms = di.sms;
         else (void)cudaGetLastError();
-        if (B > sms / 2) return false;
+        if (B > sms / 2 && (mode == 0 ? 1 : 2) * hbm_state_bytes(p, B) <= kPassStates) return false;
     }
     return cluster_fits(p, mode);
 }
@@ -1028,10 +1036,6 @@ struct HbmWs {
     size_t state = 0, lam = 0, part = 0, terms = 0, ps = 0, sh = 0, total = 0;
     bool by_pass = false;   // the rho sums and the table entries of one pass at a time
 };
-
-size_t hbm_state_bytes(const HostPlan& p, int B) {
-    return align256((size_t)B * ((size_t)1 << p.n) * (p.dtype == VQC_C128 ? 16 : 8));
-}
 
 HbmWs hbm_layout(const HostPlan& p, int mode, int B, int ntiles) {
     const size_t rs = p.dtype == VQC_C128 ? 8 : 4;

@@ -390,3 +390,18 @@ def test_complex128_workspace_of_the_other_type():
                                dw.data_ptr(), ws.data_ptr(), nbytes, torch.cuda.current_stream().cuda_stream)
         torch.cuda.synchronize()
         assert all(torch.equal(a, b) for a, b in zip(want, (E, dx, dw)))
+
+
+def test_clusters_where_pass_states_exceed_their_cap():
+    # 14 qubits, backward: two states of 128 KiB a sample reach 16 GiB at 65536 samples
+    spec = mixed(14, ("RX", "CX"))
+    c = C(spec, "c64")
+    assert c.info(65536)["bwd_path"] == 1 and c.info(65537)["bwd_path"] == 2
+    assert B.vqc_workspace_bytes(c.plan, 65537, 1) < 1 << 20
+    w_, _ = draw(spec, 65537, "c64", 8300)
+    rows = [0, 40000, 65536]
+    dx_ref, _ = orc.backward(spec, w_.x[rows], w_.w, w_.gE[rows])
+    dx, _ = run_bwd(c, w_)
+    d = 8 * U["c64"] * len(spec.gates)
+    row = np.abs(w_.gE[rows]).sum(1) * (4 * d + 32 * U["c64"])
+    assert np.all(np.abs(dx[rows] - dx_ref) <= row[:, None])
