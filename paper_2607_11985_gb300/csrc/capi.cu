@@ -468,7 +468,7 @@ vqc_status plan_launch(const HostPlan& p, int mode, int B, Launch& L) {
         }
     }
     vqc_status st = plan_launch_uncached(p, mode, B, L);
-    if (st == VQC_OK) {
+    if (st == VQC_OK && p.dbuf) {   // (without a device copy its layout is not known)
         std::lock_guard<std::mutex> lk(g_geo_mu);
         g_launch_cache[k] = L;
     }
@@ -615,13 +615,27 @@ vqc_status upload(HostPlan& p) {
     size_t err_off = put(nullptr, 16);
     blob.resize(align256(blob.size()), 0);
     VQC_CUDA(cudaGetDevice(&p.device));
+    // (a call uploads the plan of every schedule, and its stream may be in capture: a copy
+    // beside it, which the relaxed mode allows)
+    cudaStreamCaptureMode mode = p.every ? cudaStreamCaptureModeRelaxed : cudaStreamCaptureModeGlobal;
+    if (p.every) VQC_CUDA(cudaThreadExchangeStreamCaptureMode(&mode));
     void* d = nullptr;
+    cudaStream_t s = nullptr;
     cudaError_t e = cudaMalloc(&d, blob.size());
-    if (e != cudaSuccess) {
+    const bool room = e == cudaSuccess;
+    if (!p.every) {
+        if (room) e = cudaMemcpy(d, blob.data(), blob.size(), cudaMemcpyHostToDevice);
+    } else {
+        if (room) e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(d, blob.data(), blob.size(), cudaMemcpyHostToDevice, s);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        if (s) cudaStreamDestroy(s);
+        VQC_CUDA(cudaThreadExchangeStreamCaptureMode(&mode));
+    }
+    if (!room) {
         (void)cudaGetLastError();
         return fail(VQC_ERR_OUT_OF_MEMORY, "cudaMalloc of the plan failed");
     }
-    e = cudaMemcpy(d, blob.data(), blob.size(), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
         cudaFree(d);
         return cuda_fail(e, "cudaMemcpy(plan)");
@@ -778,8 +792,10 @@ vqc_status plan_cluster(const HostPlan& p, int mode, int B, Launch& L) {
     if (nclusters < 1) return fail(VQC_ERR_UNSUPPORTED, "cluster kernel cannot be resident");
     L.nunits = B;
     L.grid = std::min(B, nclusters) << L.cl;
-    std::lock_guard<std::mutex> lk(g_geo_mu);
-    g_cluster_cache[k] = L;
+    if (p.dbuf) {
+        std::lock_guard<std::mutex> lk(g_geo_mu);
+        g_cluster_cache[k] = L;
+    }
     return VQC_OK;
 }
 
@@ -1011,7 +1027,7 @@ vqc_status plan_hbm(const HostPlan& p, int mode, int B, PassGeo& L) {
         }
     }
     vqc_status st = plan_hbm_uncached(p, mode, B, L);
-    if (st == VQC_OK) {
+    if (st == VQC_OK && p.dbuf) {
         std::lock_guard<std::mutex> lk(g_geo_mu);
         g_pass_cache[k] = L;
     }
@@ -1410,23 +1426,55 @@ size_t two_call_state_offset(const HostPlan& p, int B) {
 
 std::mutex g_upload_mu;
 
-vqc_status check_common(const vqc_plan* plan, int32_t batch) {
+// The plan that a call runs: the compiled one, or the one with every schedule where the
+// environment asks for a path or block size that the first has none for.
+const HostPlan& plan_for(const vqc_plan* plan) {
+    const HostPlan& p = plan->hp;
+    auto lacks = [&](int mode, int K) { return K > 0 && !find_frame(p, mode, VQC_PATH_RESIDENT, K); };
+    if (!(t_env.hbm && !find_frame(p, 0, VQC_PATH_HBM)) && !lacks(0, t_env.k_fwd) && !lacks(1, t_env.k_bwd)) return p;
+    std::lock_guard<std::mutex> lk(g_upload_mu);
+    if (!plan->every) {
+        std::unique_ptr<HostPlan> e(new HostPlan());
+        e->every = true;
+        e->env_tile = p.env_tile;
+        std::string err;
+        if (compile_host(plan->gates.data(), (int32_t)plan->gates.size(), p.n, p.num_x, p.num_w, p.dtype, *e, err) !=
+            VQC_OK)
+            return p;
+        e->dfloat = p.dfloat;
+        if (p.dbuf) {   // (launch geometry is worked out from the device copy's layout)
+            const std::string saved = g_err;
+            int cur = -1;
+            if (cudaGetDevice(&cur) != cudaSuccess) return p;
+            if (cur != p.device) cudaSetDevice(p.device);
+            const vqc_status st = upload(*e);
+            if (cur != p.device) cudaSetDevice(cur);
+            g_err = saved;
+            if (st != VQC_OK) return p;
+        }
+        plan->every = std::move(e);
+    }
+    return *plan->every;
+}
+
+// p: the plan that the call runs.
+vqc_status check_common(const vqc_plan* plan, int32_t batch, const HostPlan*& p) {
     if (!plan) return fail(VQC_ERR_INVALID_ARG, "plan is NULL");
     if (batch < 0) return fail(VQC_ERR_INVALID_ARG, "batch must be >= 0");
     int dev = -1;
     VQC_CUDA(cudaGetDevice(&dev));
-    {
+    auto ready = [](const HostPlan& h) -> vqc_status {
         std::lock_guard<std::mutex> lk(g_upload_mu);
-        if (!plan->hp.dbuf) {
-            vqc_status st = upload(const_cast<vqc_plan*>(plan)->hp);
-            if (st != VQC_OK) return st;
-        }
-    }
+        return h.dbuf ? VQC_OK : upload(const_cast<HostPlan&>(h));
+    };
+    vqc_status st = ready(plan->hp);
+    if (st != VQC_OK) return st;
     if (dev != plan->hp.device)
         return fail(VQC_ERR_INVALID_ARG, "plan was compiled for device " +
                                              std::to_string(plan->hp.device) +
                                              " but the current device is " + std::to_string(dev));
-    return VQC_OK;
+    p = &plan_for(plan);
+    return p == &plan->hp ? VQC_OK : ready(*p);
 }
 
 // Real arrays (E, gE, dx, dw, probabilities) must be aligned to the real type,
@@ -1472,9 +1520,10 @@ vqc_status backward_with_scratch(const vqc_plan* plan, int32_t batch, const void
                                  const void* grad_expz, void* grad_x, void* grad_w, void* scratch,
                                  size_t scratch_bytes, void* stream, bool clear_control) {
     const EnvScope env;
-    vqc_status st = check_common(plan, batch);
+    const HostPlan* hp = nullptr;
+    vqc_status st = check_common(plan, batch, hp);
     if (st != VQC_OK) return st;
-    const HostPlan& p = plan->hp;
+    const HostPlan& p = *hp;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (batch == 0) {
         if (grad_w && p.num_w > 0)
@@ -1554,7 +1603,7 @@ namespace {
 size_t workspace_need(const vqc_plan* plan, int batch, int mode) {
     if (mode == 3) {   // vqc_forward_backward: its one-launch form, or either call's workspace
         size_t need = std::max(workspace_need(plan, batch, 0), workspace_need(plan, batch, 1));
-        const HostPlan& p = plan->hp;
+        const HostPlan& p = plan_for(plan);
         Launch L;
         const std::string saved = g_err;
         if (batch > 0 && !use_cluster(p, 0, batch) && !use_hbm(p, 0, batch) && !use_hbm(p, 1, batch)) {
@@ -1577,13 +1626,13 @@ size_t workspace_need(const vqc_plan* plan, int batch, int mode) {
         return need;
     }
     if (mode == 2 && batch > 0) {   // vqc_probabilities: forward workspace + state + E
-        const HostPlan& p = plan->hp;
+        const HostPlan& p = plan_for(plan);
         const size_t rs = p.dtype == VQC_C128 ? 8 : 4;
         return align256(workspace_need(plan, batch, 0)) +
                align256(((size_t)batch << p.n) * 2 * rs) + align256((size_t)batch * p.n * rs);
     }
     if ((mode != 0 && mode != 1) || batch <= 0) return 0;
-    const HostPlan& p = plan->hp;
+    const HostPlan& p = plan_for(plan);
     if (use_cluster(p, mode, batch)) {
         if (mode == 0) return 0;
         Launch L;
@@ -1629,6 +1678,7 @@ vqc_status vqc_compile(const vqc_gate* gates, int32_t num_gates, int32_t num_qub
         vqc_status st = compile_host(gates, num_gates, num_qubits, num_x, num_w, store, p->hp, err);
         if (st != VQC_OK) return fail(st, err);
         p->hp.dfloat = dtype == VQC_C128_DF;
+        p->gates.assign(gates, gates + num_gates);
         // Upload now when a CUDA device is present; a host-only plan (no device
         // in this process) still serves vqc_plan_export and vqc_plan_info, and
         // is uploaded by the first launching call.
@@ -1655,15 +1705,18 @@ void vqc_free(vqc_plan* plan) {
     {
         std::lock_guard<std::mutex> lk(g_plans_mu);
         g_plans.erase(&plan->hp);
+        g_plans.erase(plan->every.get());
     }
-    forget_plan(&plan->hp);
     release_host_arena(plan);
-    if (plan->hp.dbuf) {
+    for (const HostPlan* p : std::initializer_list<const HostPlan*>{&plan->hp, plan->every.get()}) {
+        if (!p) continue;
+        forget_plan(p);
+        if (!p->dbuf) continue;
         int cur = -1;
         cudaGetDevice(&cur);
-        if (cur != plan->hp.device) cudaSetDevice(plan->hp.device);
-        cudaFree(plan->hp.dbuf);
-        if (cur != plan->hp.device && cur >= 0) cudaSetDevice(cur);
+        if (cur != p->device) cudaSetDevice(p->device);
+        cudaFree(p->dbuf);
+        if (cur != p->device && cur >= 0) cudaSetDevice(cur);
     }
     delete plan;
 }
@@ -1672,7 +1725,7 @@ size_t vqc_workspace_bytes(const vqc_plan* plan, int32_t batch, int32_t mode) {
     if (!plan) return (size_t)-1;
     try {
         const EnvScope env;
-        const HostPlan& p = plan->hp;
+        const HostPlan& p = plan_for(plan);
         if (p.dtype != VQC_C128) return workspace_need(plan, batch, mode);
         // either arithmetic's (t_arith), kept: the launches of both are worked out once
         const GeoKey k = geo_key(p, mode, batch, 3 + (t_env.hbm ? 1 : 0) + (t_env.cluster ? 2 : 0));
@@ -1686,8 +1739,11 @@ size_t vqc_workspace_bytes(const vqc_plan* plan, int32_t batch, int32_t mode) {
             const ArithScope as(a);
             need = std::max(need, workspace_need(plan, batch, mode));
         }
-        std::lock_guard<std::mutex> lk(g_geo_mu);
-        return g_workspace_cache[k] = need;
+        if (p.dbuf) {
+            std::lock_guard<std::mutex> lk(g_geo_mu);
+            g_workspace_cache[k] = need;
+        }
+        return need;
     } catch (...) {
         return (size_t)-1;
     }
@@ -1698,10 +1754,11 @@ vqc_status vqc_probabilities(const vqc_plan* plan, int32_t batch, const void* x,
                              size_t workspace_bytes, void* stream) {
     try {
         const EnvScope env;
-        vqc_status st = check_common(plan, batch);
+        const HostPlan* hp = nullptr;
+        vqc_status st = check_common(plan, batch, hp);
         if (st != VQC_OK) return st;
         if (batch == 0) return VQC_OK;
-        const HostPlan& p = plan->hp;
+        const HostPlan& p = *hp;
         if (!probs_out) return fail(VQC_ERR_INVALID_ARG, "probs_out is NULL");
         st = check_out_ptrs(p, {probs_out}, {});
         if (st != VQC_OK) return st;
@@ -1741,10 +1798,11 @@ vqc_status vqc_forward(const vqc_plan* plan, int32_t batch, const void* x, const
                        size_t workspace_bytes, void* stream) {
     try {
         const EnvScope env;
-        vqc_status st = check_common(plan, batch);
+        const HostPlan* hp = nullptr;
+        vqc_status st = check_common(plan, batch, hp);
         if (st != VQC_OK) return st;
         if (batch == 0) return VQC_OK;
-        const HostPlan& p = plan->hp;
+        const HostPlan& p = *hp;
         st = check_ptrs(p, x, w, psi0, nullptr);
         if (st != VQC_OK) return st;
         if (!expz_out) return fail(VQC_ERR_INVALID_ARG, "expz_out is NULL");
@@ -1779,9 +1837,10 @@ vqc_status vqc_backward(const vqc_plan* plan, int32_t batch, const void* x, cons
                         void* stream) {
     try {
         const EnvScope env;
-        vqc_status st = check_common(plan, batch);
+        const HostPlan* hp = nullptr;
+        vqc_status st = check_common(plan, batch, hp);
         if (st != VQC_OK) return st;
-        const HostPlan& p = plan->hp;
+        const HostPlan& p = *hp;
         cudaStream_t s = static_cast<cudaStream_t>(stream);
         if (batch == 0) {
             if (grad_w && p.num_w > 0)
@@ -1822,9 +1881,10 @@ vqc_status vqc_forward_backward(const vqc_plan* plan, int32_t batch, const void*
                                 void* grad_w, void* workspace, size_t workspace_bytes, void* stream) {
     try {
         const EnvScope env;
-        vqc_status st = check_common(plan, batch);
+        const HostPlan* hp = nullptr;
+        vqc_status st = check_common(plan, batch, hp);
         if (st != VQC_OK) return st;
-        const HostPlan& p = plan->hp;
+        const HostPlan& p = *hp;
         cudaStream_t s = static_cast<cudaStream_t>(stream);
         if (batch == 0) {
             if (grad_w && p.num_w > 0)
@@ -1906,10 +1966,10 @@ vqc_status vqc_forward_backward(const vqc_plan* plan, int32_t batch, const void*
     }
 }
 
-vqc_status vqc_plan_info(const vqc_plan* plan, int32_t batch, vqc_plan_stats* out) {
+vqc_status vqc_plan_info(const vqc_plan* plan, int32_t batch, vqc_plan_stats* out) try {
     const EnvScope env;
     if (!plan || !out) return fail(VQC_ERR_INVALID_ARG, "NULL argument");
-    const HostPlan& p = plan->hp;
+    const HostPlan& p = plan_for(plan);
     std::memset(out, 0, sizeof(*out));
     out->num_qubits = p.n;
     out->num_x = p.num_x;
@@ -1981,6 +2041,8 @@ vqc_status vqc_plan_info(const vqc_plan* plan, int32_t batch, vqc_plan_stats* ou
     }
     g_err = saved;
     return VQC_OK;
+} catch (...) {
+    return fail(VQC_ERR_OUT_OF_MEMORY, "vqc_plan_info failed");
 }
 
 vqc_status vqc_plan_export(const vqc_plan* plan, void* buf, size_t* inout_bytes) {

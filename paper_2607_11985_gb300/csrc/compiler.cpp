@@ -668,7 +668,7 @@ vqc_status compile_host(const vqc_gate* gates, int32_t G, int32_t n, int32_t nx,
     p.recompute_flops = f * dim;
     p.fwd_flops = (f + 3 + n) * dim;
     p.bwd_flops = (fb + n + 2) * dim;
-    if (const char* t = std::getenv("VQC_HBM_TILE_QUBITS")) {
+    if (const char* t = p.every ? nullptr : std::getenv("VQC_HBM_TILE_QUBITS")) {
         const int env_m = std::atoi(t);
         if (env_m > p.G_swz && env_m < n) p.env_tile = env_m;
     }
@@ -714,10 +714,10 @@ vqc_status compile_host(const vqc_gate* gates, int32_t G, int32_t n, int32_t nx,
     }
     // Frame schedules on the resident path, one block per thread (at most 512 threads
     // per sample): the block sizes that a launch chooses from (choose_k: 3 and up where
-    // the circuit has them), and the smaller ones when the environment asks for a size
-    // at compile time; then the HBM passes.
+    // the circuit has them), and the smaller ones when the environment asks for a size;
+    // then the HBM passes.
     const FrameBuilder frames(p);
-    const bool all_k = std::getenv("VQC_FORCE_K_FWD") || std::getenv("VQC_FORCE_K_BWD");
+    const bool all_k = p.every || std::getenv("VQC_FORCE_K_FWD") || std::getenv("VQC_FORCE_K_BWD");
     for (int mode = 0; mode < 2; ++mode) {
         const int kmax = std::min(max_k(mode, dtype), n);
         for (int K = all_k ? 1 : std::min(kmax, 3); K <= kmax; ++K)
@@ -725,8 +725,8 @@ vqc_status compile_host(const vqc_gate* gates, int32_t G, int32_t n, int32_t nx,
                 p.frames.push_back(frames.build(mode, VQC_PATH_RESIDENT, {n}, K));
     }
     // (Circuits whose sweeps fit one CTA in both modes never take the passes, unless
-    // the environment asks for them at compile time.)
-    const bool want_hbm = std::getenv("VQC_FORCE_PATH") || p.env_tile || !resident_fits(p);
+    // the environment asks for them.)
+    const bool want_hbm = p.every || std::getenv("VQC_FORCE_PATH") || p.env_tile || !resident_fits(p);
     for (int mode = 0; mode < 2; ++mode) {
         int m, K;
         if (!hbm_shape(p, mode, m, K)) continue;

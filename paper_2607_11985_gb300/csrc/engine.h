@@ -4,6 +4,7 @@
 
 #include <cstddef>
 #include <cstdint>
+#include <memory>
 #include <string>
 #include <vector>
 
@@ -62,6 +63,7 @@ struct HostPlan {
     int n_ps = 0, n_sh = 0;                // per-sample / shared table sizes
     int n_runs = 0;
     int env_tile = 0;                      // VQC_HBM_TILE_QUBITS at compile time, 0: none
+    bool every = false;                    // all schedules: HBM passes and block sizes below 3 as well
     std::vector<Schedule> scheds;          // of the cluster path
     std::vector<FrameSchedule> frames;     // of the resident and HBM-tiled kernels
     double fwd_flops = 0, bwd_flops = 0, recompute_flops = 0;
@@ -165,4 +167,8 @@ std::vector<uint8_t> export_plan(const HostPlan& p);
 // The opaque handle of the C ABI: a compiled host plan (and its device copy).
 struct vqc_plan {
     vqc::HostPlan hp;
+    // The same circuit with the schedules that only environment switches ask for, compiled
+    // by the first call that finds one set (plan_for).
+    std::vector<vqc_gate> gates;
+    mutable std::unique_ptr<vqc::HostPlan> every;
 };

@@ -405,3 +405,44 @@ def test_clusters_where_pass_states_exceed_their_cap():
     d = 8 * U["c64"] * len(spec.gates)
     row = np.abs(w_.gE[rows]).sum(1) * (4 * d + 32 * U["c64"])
     assert np.all(np.abs(dx[rows] - dx_ref) <= row[:, None])
+
+
+# environment switches set after the circuit was compiled: paths and block sizes that its
+# plan was compiled without
+@pytest.mark.parametrize("dtype,n", [("c64", 8), ("c128", 9), ("c128df", 9)])
+def test_switches_after_compiling(monkeypatch, dtype, n):
+    spec = mixed(n, ("RX", "RY", "CX", "RZZ"))
+    c = C(spec, dtype)
+    data = draw(spec, 3, dtype, 8400 + n, psi0=True)
+    assert c.info(3)["fwd_path"] == 0 and c.info(3)["bwd_path"] == 0
+    monkeypatch.setenv("VQC_FORCE_PATH", "hbm")
+    assert c.info(3)["fwd_path"] == 1 and c.info(3)["bwd_path"] == 1
+    check(c, *data)
+    monkeypatch.delenv("VQC_FORCE_PATH")
+    monkeypatch.setenv("VQC_FORCE_K_FWD", "2")
+    monkeypatch.setenv("VQC_FORCE_K_BWD", "1")
+    assert c.info(3)["fwd_k"] == 2 and c.info(3)["bwd_k"] == 1
+    check(c, *data)
+    monkeypatch.delenv("VQC_FORCE_K_FWD")
+    monkeypatch.delenv("VQC_FORCE_K_BWD")
+    assert c.info(3)["fwd_path"] == 0
+    check(c, *data)
+
+
+def test_switch_in_capture(monkeypatch):
+    spec = mixed(8, ("RX", "CX"))
+    c = C(spec, "c64")
+    w_, _ = draw(spec, 5, "c64", 8500)
+    x, w = dev(w_.x, "c64"), dev(w_.w, "c64")
+    want = c.forward(x, w)
+    monkeypatch.setenv("VQC_FORCE_PATH", "hbm")
+    E = torch.empty_like(want)
+    nbytes = B.vqc_workspace_bytes(c.plan, 5, 0)
+    ws = torch.zeros(nbytes, dtype=torch.uint8, device="cuda")
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):   # (the first call that needs the passes' schedules)
+        B.vqc_forward(c.plan, 5, x.data_ptr(), w.data_ptr(), None, E.data_ptr(), None, ws.data_ptr(), nbytes,
+                      torch.cuda.current_stream().cuda_stream)
+    g.replay()
+    torch.cuda.synchronize()
+    assert maxerr(E.cpu().numpy(), want.cpu().numpy()) <= 4 * 8 * U["c64"] * len(spec.gates) + 64 * U["c64"]
