@@ -296,16 +296,18 @@ class CircuitBench:
 
     def launches(self):
         """Library kernels per step: resident forward 1, resident backward 2
-        (sweep + fixed-order dw sum); HBM-tiled: one launch per pass plus the
-        tables and the partial sums (E; the per-sample gradient terms, dx and dw,
-        which complex64 sums in one launch where a circuit has both); cluster
-        forward 1, cluster backward 2."""
+        (sweep + fixed-order dw sum); HBM-tiled: one launch per pass, the tables
+        of the circuit's runs and phases, and the partial sums (E; the per-sample
+        gradient terms, dx and dw, which complex64 sums in one launch where a
+        circuit has both); cluster forward 1, cluster backward 2."""
         inf, nx, nw = self.info, self.w_.spec.num_x > 0, self.w_.spec.num_w > 0
-        f = inf["fwd_passes"] + 1 + int(nx) if inf["fwd_path"] == 1 else 1
+        tables = int(nx or nw or inf.get("num_runs", 0) > 0)
+        f = inf["fwd_passes"] + 1 + tables if inf["fwd_path"] == 1 else 1
         if not self.w_.backward:
             return f
         if inf["bwd_path"] == 1:
-            b = inf["bwd_passes"] + int(nx or nw) + int(nx) + int(nw) + int(nx and self.w_.dtype != "c64")
+            sums = 1 if self.w_.dtype == "c64" and nx and nw else int(nx) + int(nw)
+            b = inf["bwd_passes"] + tables + int(nx or nw) + sums
         else:
             b = 1 + int(nw)
         return f + b

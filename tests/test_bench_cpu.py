@@ -68,3 +68,18 @@ def test_launch_count_per_step():
     assert b.launches() == 1 + 2
     b.info = {"fwd_path": 0, "bwd_path": 2, "fwd_passes": 1, "bwd_passes": 1}
     assert b.launches() == 1 + 2
+
+
+@pytest.mark.parametrize("num_x,num_w,dtype,sums", [(0, 4, "c64", 1), (4, 0, "c64", 1), (4, 4, "c64", 1),
+                                                    (0, 4, "c128", 1), (4, 0, "c128", 1), (4, 4, "c128", 2)])
+def test_launch_count_of_circuits_without_x_or_w(num_x, num_w, dtype, sums):
+    # HBM passes: the tables once per direction, whatever their angles come from
+    class W:
+        backward = True
+        spec = wl.CircuitSpec(16, num_x, num_w)
+
+    W.dtype = dtype
+    b = bench.CircuitBench.__new__(bench.CircuitBench)
+    b.w_ = W()
+    b.info = {"fwd_path": 1, "bwd_path": 1, "fwd_passes": 3, "bwd_passes": 4, "num_runs": 16}
+    assert b.launches() == (1 + 3 + 1) + (1 + 4 + 1 + sums)
