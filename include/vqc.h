@@ -285,7 +285,8 @@ vqc_status vqc_probabilities(const vqc_plan* plan, int32_t batch, const void* x,
  *   whose scratch need (vqc_workspace_bytes(plan, batch, 1); for HBM passes the
  *   states, the gradient terms, the per-sample matrices and one sum per gradient
  *   slot and tile) exceeds it is rejected with VQC_ERR_WORKSPACE and a message
- *   giving both sizes.
+ *   giving both sizes.  (Resident sweeps run on as few as half as many CTAs, where
+ *   their partial sums of dw then fit.)
  *   No cudaMalloc, cudaFree or allocating library call is made.  Each call
  *   clears the array's control block on `stream` before its launch; all calls
  *   on a device share the array, so calls that overlap on the GPU race and must

@@ -230,11 +230,12 @@ cudaError_t launch(const void* fn, dim3 grid, dim3 block, void** args, size_t sm
 
 // Pick the register-block size: the largest K that still gives the batch
 // enough threads to cover every SM's schedulers (SMs x 4 warps), but not below
-// 3 (a block of 8 amplitudes) where the circuit allows it.  A forced-K sweep on
-// GB300 (8-qubit batch 1024 and 8192, 12-qubit batch 4096; forward, backward
-// and the fused call) found no smaller K faster than this choice: smaller
-// blocks add stages (shared-memory round trips and barriers) faster than the
-// extra warps hide latency.
+// 3 (a block of 8 amplitudes) where the circuit allows it.  Of the forced sizes
+// (VQC_FORCE_K_*: RX RY RZ layers, CX ring, complex64; 8 qubits x 100, 1024 and 8192,
+// 10 x 251, 12 x 100 and 4096; forward, one call, saved) this choice was the fastest
+// everywhere but in the 8-qubit x 8192 one-call step (156 us, 136 with 3 / 3): smaller
+// blocks add stages (shared-memory round trips and barriers) faster than the extra warps
+// hide latency (12 x 4096 step 1.67 ms with 5 / 4, 1.73 with 4 / 4, 2.36 with 3 / 3).
 int choose_k(const HostPlan& p, int mode, int B, int sms, bool any_size = false) {
     const int forced = mode == 0 ? t_env.k_fwd : t_env.k_bwd;
     if (forced > 0 && find_frame(p, mode, VQC_PATH_RESIDENT, forced)) return forced;
@@ -586,9 +587,6 @@ vqc_status upload(HostPlan& p) {
         s.dev_region_begin = blob.size();
         s.dev_ops = put(s.ops.data(), s.ops.size() * sizeof(DOp));
         s.dev_stages = put(s.stages.data(), s.stages.size() * sizeof(DStage));
-        s.dev_passes = put(s.passes.data(), s.passes.size() * sizeof(DPass));
-        s.dev_pass_entries = put(s.pass_entries.data(), s.pass_entries.size() * 4);
-        s.dev_pass_accs = put(s.pass_accs.data(), s.pass_accs.size() * 4);
         s.dev_region_end = blob.size();
     }
     std::vector<int32_t> iota;   // 0, 1, ...: the indices of a pass's own tables (own_tables)
@@ -648,7 +646,7 @@ vqc_status upload(HostPlan& p) {
     return VQC_OK;
 }
 
-// Workspace of a backward call: [0, 256) control block (counter), then the
+// Workspace of a backward call: [0, 256) control block (reserved), then the
 // per-CTA dw partials [grid, num_w].
 size_t bwd_workspace(const HostPlan& p, const Launch& L) {
     const size_t rs = p.dtype == VQC_C128 ? 8 : 4;
@@ -694,7 +692,6 @@ vqc_status run(const HostPlan& p, int mode, int B, const void* x, const void* w,
         if (!ws || ws_bytes < need || misaligned(ws, 256))
             return fail(VQC_ERR_WORKSPACE, "backward workspace must be >= " + std::to_string(need) +
                                                " bytes and 256-byte aligned");
-        a.counter = static_cast<unsigned*>(ws);
         a.dw_part = reinterpret_cast<R*>(static_cast<char*>(ws) + 256);
     }
     void* args[] = {&a};
@@ -906,7 +903,6 @@ vqc_status run_cluster_backward(const HostPlan& p, int B, const void* x, const v
     a.gE = static_cast<const R*>(gE);
     a.dx = static_cast<R*>(dx);
     a.dw = static_cast<R*>(dw);
-    a.counter = static_cast<unsigned*>(ws);
     a.dw_part = reinterpret_cast<R*>(static_cast<char*>(ws) + 256);
     void* args[] = {&a};
     cudaLaunchAttribute attr[2];

@@ -24,7 +24,8 @@ struct HOp {
     uint8_t gen;       // OPF_GEN_* for PH2
 };
 
-// One register-block stage schedule for a (mode, K, tile) choice.
+// One register-block stage schedule for a (mode, K, tile) choice: the cluster path's, and
+// the axis-aligned ones that vqc_plan_export builds for itself.
 struct Schedule {
     int mode = 0;          // 0 forward, 1 backward
     int K = 0;             // register-block qubits
@@ -35,16 +36,16 @@ struct Schedule {
     int cta_bits = 0;           // cluster path: log2(threads per CTA); 2^(m-K-cta_bits) CTAs
     std::vector<DOp> ops;
     std::vector<DStage> stages;
-    std::vector<DPass> passes;            // HBM path: one record per pass
-    std::vector<int32_t> pass_entries;    // HBM path: table entries per pass (ps, then sh)
-    std::vector<int32_t> pass_accs;       // HBM path: accumulator ids per pass
+    // exported HBM schedules only: one record per pass, its table entries (per sample, then
+    // shared) and its accumulators
+    std::vector<DPass> passes;
+    std::vector<int32_t> pass_entries, pass_accs;
     // Per stage, kMaxK + kMaxThreadBits physical-index masks: the image under
     // the stage's absorbed permutation of each local bit, then of each thread
     // bit (exported for tests; the kernels use the swizzled store map).
     std::vector<uint32_t> store_masks;
     size_t dev_ops = 0, dev_stages = 0;   // byte offsets inside the device buffer
-    size_t dev_passes = 0, dev_pass_entries = 0, dev_pass_accs = 0;
-    size_t dev_region_begin = 0, dev_region_end = 0;   // [ops .. pass_accs] in the blob
+    size_t dev_region_begin = 0, dev_region_end = 0;   // [ops, stages] in the blob
 };
 
 struct HostPlan {
@@ -95,11 +96,11 @@ inline int hbm_k(int mode, int dtype) {
 }
 
 // Tile bits offered to the frame schedules of the HBM passes.  complex64: 32 KiB of
-// forward tile (18-qubit / batch-48 forward 468 us, 500 with 13 bits, 502 with 11),
+// forward tile (18-qubit / batch-48 forward 451 us, 485 with 13 bits, 488 with 11),
 // or one bit less where that costs no pass and no stage (16-qubit / batch-512 step
-// 6.39 ms against 6.66): a pass is bound by the latency of its stages, and smaller
+// 6.21 ms against 6.50): a pass is bound by the latency of its stages, and smaller
 // tiles mean more CTAs per SM, each waiting for fewer warps.  complex128: 64 KiB
-// (16-qubit double-float step 9.72 ms, 10.3 with 11 / 10 bits).
+// (16-qubit / batch-77 double-float step 7.79 ms, 8.03 with 11 bits both ways, 9.74 with 10).
 inline std::vector<int> frame_tile_qubits(int mode, int dtype, int n) {
     auto fit = [n](int m) { return m < n - 1 ? m : n - 1; };
     if (dtype == VQC_C64) return {fit(12), fit(11)};

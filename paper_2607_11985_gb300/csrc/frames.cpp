@@ -766,7 +766,7 @@ FrameSchedule lay_out(const HostPlan& p, const FrameOps& L, int mode, int path, 
             vout = vin;
         } else {
             gout = gin;
-            Vecs l = line, pickd;
+            Vecs l = line;
             Span bs;
             if (vbits) {   // the vector's own bit: the one whose bank the others can spare
                 for (size_t i = 0; i < l.size(); ++i) {

@@ -12,8 +12,7 @@
 // allocating library routine.
 //
 // All calls on a device share that one array, and it keeps the previous call's
-// contents: each call clears the control block (the CTA-completion counter)
-// before its launch.  Calls whose kernels overlap on the GPU race on the array,
+// contents: each call clears the control block (reserved) before its launch.  Calls whose kernels overlap on the GPU race on the array,
 // so callers must order them (e.g. on one stream).
 //
 // The device address of the array is looked up once per device, on the first

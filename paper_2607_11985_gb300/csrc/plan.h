@@ -16,7 +16,8 @@
 //     non-diagonal op of the stage acts on these only, diagonal ops may use any
 //     qubit.  Between stages the state goes through shared memory.
 //
-// Amplitude addressing in shared memory (per sample, tile-local index u):
+// Amplitude addressing in shared memory on the cluster path and in exported schedules (per
+// sample, tile-local index u; frame schedules search a fold of their own per pass):
 //   slot(u) = sw(u) ^ h_sample,   sw(u) = u ^ (fold_G(u >> G) & (2^G - 1))
 // with G = 4 for complex64 and 3 for complex128 (2^G amplitudes = 128 bytes).
 // sw is linear over GF(2), so the slot of amplitude r of a thread's block is
@@ -49,6 +50,7 @@ enum OpFlags : uint8_t {
 // branch per op, each case specialised for fixed local positions.
 enum DispatchCode : uint8_t {
     DC_M1 = 0,       // + t: 2x2 on local position t (0..4)
+    // (DC_CX_*: in exported HBM schedules only; no kernel has them)
     DC_CX_LL = 5,    // + 4c + (t < c ? t : t - 1): local control c, local target t
     DC_CX_PL = 25,   // + t: control outside the block (ref a), local target t
     DC_CZ_LL = 30,   // + cz_pair_index(lo, hi): both qubits local
@@ -152,8 +154,8 @@ VQC_HD inline int run_form(const DConst* c, int count) {
     return general ? 3 : (first > 0 ? 1 : 0) | (last + 1 < count ? 2 : 0);
 }
 
-// One pass of the HBM-tiled path: its stages act on tiles of m qubits; the
-// other n - m qubits index the tiles of a sample.
+// One pass of an exported HBM schedule (the pass kernels run FPass): its stages act on
+// tiles of m qubits; the other n - m qubits index the tiles of a sample.
 struct DPass {
     int32_t stage_begin, stage_end;
     int32_t m, nout;

@@ -241,7 +241,6 @@ struct KArgs {
     R* dx;
     R* dw;
     R* dw_part;          // [gridDim.x, Pw]
-    unsigned* counter;
     // shared-memory carve-up (byte offsets)
     int sm_sh, sm_ps, sm_psi, sm_lam, sm_acc, sm_terms, sm_dw, sm_red;
     int sm_w, sm_xg;   // shared copies of w [Pw] and of the unit's x / gE rows [S][Px + n]
@@ -971,28 +970,6 @@ __device__ __forceinline__ void ph2_any(int ra, int rb, uint32_t pb, const R* tp
 }
 
 // ---------------------------------------------------------------- op dispatch
-template <typename R> __device__ __forceinline__ M2<R> load_m2v(const R* p);
-template <> __device__ __forceinline__ M2<float> load_m2v<float>(const float* p) {
-    const float4 u = *reinterpret_cast<const float4*>(p);
-    const float4 v = *reinterpret_cast<const float4*>(p + 4);
-    M2<float> m;
-    m.a = make_float2(u.x, u.y); m.b = make_float2(u.z, u.w);
-    m.c = make_float2(v.x, v.y); m.d = make_float2(v.z, v.w);
-    return m;
-}
-template <> __device__ __forceinline__ M2<double> load_m2v<double>(const double* p) {
-    const double2* q = reinterpret_cast<const double2*>(p);
-    M2<double> m;
-    m.a = q[0]; m.b = q[1]; m.c = q[2]; m.d = q[3];
-    return m;
-}
-template <> __device__ __forceinline__ M2<dd> load_m2v<dd>(const dd* p) {
-    const dd2* q = reinterpret_cast<const dd2*>(p);
-    M2<dd> m;
-    m.a = q[0]; m.b = q[1]; m.c = q[2]; m.d = q[3];
-    return m;
-}
-
 __device__ __forceinline__ bool physbit(uint32_t pb, int ref) {
     return ((pb >> (ref - kRefPhys)) & 1u) != 0;
 }
