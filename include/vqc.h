@@ -379,6 +379,11 @@ vqc_status vqc_plan_info(const vqc_plan* plan, int32_t batch, vqc_plan_stats* ou
  * are a deterministic function of the vqc_compile arguments. */
 vqc_status vqc_plan_export(const vqc_plan* plan, void* buf, size_t* inout_bytes);
 
+/* The frame schedules of a compiled plan as the resident and HBM kernels read them
+ * (paper_2607_11985_gb300/csrc/frame.h), for tests and inspection; buf and inout_bytes as
+ * in vqc_plan_export.  The records are those of this build, not a stable format. */
+vqc_status vqc_frames_export(const vqc_plan* plan, void* buf, size_t* inout_bytes);
+
 /* Synchronise `stream` and report any CUDA error, then read (and clear) the
  * error word of every plan of this process on the current device: each kernel
  * checks its launch geometry against the plan before touching memory and, on

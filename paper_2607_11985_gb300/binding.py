@@ -72,6 +72,7 @@ SIGNATURES = [
     ("vqc_stage_apply", _I, [_I, _I, _I, ctypes.POINTER(ctypes.c_double), _P, _P, _I, _P]),
     ("vqc_plan_info", _I, [_P, _I, ctypes.POINTER(vqc_plan_stats)]),
     ("vqc_plan_export", _I, [_P, _P, ctypes.POINTER(_S)]),
+    ("vqc_frames_export", _I, [_P, _P, ctypes.POINTER(_S)]),
     ("vqc_sync_check", _I, [_P]),
     ("vqc_last_error", ctypes.c_char_p, []),
     ("vqc_abi_version", _I, []),

@@ -2088,7 +2088,6 @@ vqc_status vqc_sync_check(void* stream) {
     return stage_error_check();   // vqc_stage_apply's tensor-core waits
 }
 
-// The frame schedules' records (frame.h), for the CPU tests; like vqc_plan_export.
 vqc_status vqc_frames_export(const vqc_plan* plan, void* buf, size_t* inout_bytes) {
     if (!plan || !inout_bytes) return fail(VQC_ERR_INVALID_ARG, "NULL argument");
     try {

@@ -2,9 +2,11 @@
 
 This checks the host compiler (fusion, constant pre-multiplication, stage
 cutting, register-block addressing, gradient-term bookkeeping) without a GPU:
-each schedule is run stage by stage, thread block by thread block, exactly as
-the kernels address amplitudes, in numpy complex128, and the result is
+each schedule is run stage by stage, thread block by thread block, as its
+records address amplitudes, in numpy complex128, and the result is
 compared with the oracle.  The emulator reads only the exported plan bytes.
+(Of these schedules the cluster kernels run theirs; resident and HBM kernels
+run frame schedules, which tests/test_frames_cpu.py executes.)
 """
 from __future__ import annotations
 

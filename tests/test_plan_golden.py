@@ -9,6 +9,11 @@ workloads up to 14 qubits, random circuits over the whole gate set with
 constant, per-sample and shared angles, every gate in both qubit orders, and
 the degenerate circuits; complex64, complex128 and double-float plans (the
 last export the complex128 bytes); resident and HBM-tiled schedules.
+
+Every kernel runs the fused ops, entries, constants and gradient terms compared
+here.  Of the exported schedules, the cluster kernels run theirs; the resident
+and HBM ones are a format of the export alone: those kernels run frame schedules,
+which tests/test_frames_cpu.py executes from their own records.
 """
 import numpy as np
 import pytest
