@@ -927,27 +927,28 @@ FrameSchedule lay_out(const HostPlan& p, const FrameOps& L, int mode, int path, 
             // each op's round: a run follows the diagonal ops it does not commute with in
             // the same round or an earlier one, and the run before it on its position; a
             // diagonal op follows such runs by a round
-            std::vector<int> round(s.ops.size(), 0);
-            int rounds = 1;
-            for (size_t i = 0; i < s.ops.size(); ++i) {
-                const FOp& o = f[s.ops[i]];
-                for (size_t k = 0; k < i; ++k) {
-                    const FOp& q = f[s.ops[k]];
-                    if (!o.run && !q.run) continue;
-                    const bool clash = o.run && q.run ? q.d == o.d
-                                     : o.run ? odd(q.r & o.d) || odd(q.r2 & o.d) : odd(o.r & q.d) || odd(o.r2 & q.d);
-                    if (clash) round[i] = std::max(round[i], round[k] + (q.run ? 1 : 0));
+            std::vector<std::vector<int>> round(1);
+            int after_run[kMaxK] = {0}, after_diag[kMaxK] = {0};   // earliest rounds, by position
+            for (int x : s.ops) {
+                const FOp& o = f[x];
+                int rd = 0;
+                for (int k = 0; k < K; ++k) {
+                    const bool meets = o.run ? s.D[k] == o.d : odd(o.r & s.D[k]) || odd(o.r2 & s.D[k]);
+                    if (meets) rd = std::max({rd, after_run[k], o.run ? after_diag[k] : 0});
                 }
-                rounds = std::max(rounds, round[i] + 1);
+                for (int k = 0; k < K; ++k) {
+                    if (o.run && s.D[k] == o.d) after_run[k] = rd + 1;
+                    if (!o.run && (odd(o.r & s.D[k]) || odd(o.r2 & s.D[k]))) after_diag[k] = std::max(after_diag[k], rd);
+                }
+                if ((int)round.size() <= rd) round.resize(rd + 1);
+                round[rd].push_back(x);
             }
             st.op_begin = (int32_t)S.ops.size();
             st.seg_begin = (int32_t)S.segs.size();
-            for (int rd = 0; rd < rounds && !s.ops.empty(); ++rd) {
+            for (size_t rd = 0; rd < round.size() && !s.ops.empty(); ++rd) {
                 FSeg sg{};
                 std::vector<DOp> diag, runs;
-                for (size_t i = 0; i < s.ops.size(); ++i) {
-                    if (round[i] != rd) continue;
-                    const int x = s.ops[i];
+                for (int x : round[rd]) {
                     const DOp d = record(x);
                     if (f[x].run) {
                         sg.pmask |= (uint8_t)(1u << d.a);
