@@ -107,8 +107,9 @@ inline std::vector<int> frame_tile_qubits(int mode, int dtype, int n) {
     return {fit(mode == 0 ? 12 : 11)};
 }
 
-// Shared memory that a CTA can have on sm_103a (227 KB).
+// Shared memory that a CTA can have on sm_103a (227 KB), and each of two on one SM.
 constexpr size_t kCtaSharedMemory = 232448;
+constexpr size_t kHalfSharedMemory = 115712;
 
 // The largest of each count that sizes a launch of a pass: of one, or over all passes
 // of a schedule (whose launches share one layout).

@@ -77,7 +77,8 @@ struct FSeg {
 static_assert(sizeof(FSeg) == 20, "FSeg layout");
 enum : uint8_t {
     kSegPs = 1,             // a table depends on the sample
-    kSegQ = 2, kSegP = 4,   // some run needs its diagonal before / after the rotation (run_form)
+    kSegQ = 2, kSegP = 4,   // some run needs its diagonal before / after the rotation (run_form);
+                            // not in stages with phases, whose runs double-float does not factor
     kSegA = 8,              // the group has gradient terms
     kSegL = 16              // it has phases of two local positions
 };

@@ -354,7 +354,8 @@ FrameOps lower(const HostPlan& p) {
 
 // The passes over tiles of m bits (the resident path: one pass, m = n) and their
 // stages of K directions.
-std::vector<PassPlan> plan_passes(const HostPlan& p, const FrameOps& L, int mode, bool tiled, int m, int K) {
+std::vector<PassPlan> plan_passes(const HostPlan& p, const FrameOps& L, int mode, bool tiled, int m, int K,
+                                  int max_entries = kMaxPassEntries) {
     const int n = p.n, G = std::min(p.G_swz, m);
     const std::vector<FOp>& f = L.f;
     const Vecs& dir = L.dir;
@@ -406,7 +407,7 @@ std::vector<PassPlan> plan_passes(const HostPlan& p, const FrameOps& L, int mode
                     bool ok = w.passes(o);
                     const int e = p.ops[o.hop].entry;
                     const bool newe = e >= 0 && !have[e];
-                    if (ok && newe) ok = entries < kMaxPassEntries;
+                    if (ok && newe) ok = entries < max_entries;
                     if (ok && o.run) ok = t.add(o.d, m, room);
                     if (ok && newe) {
                         have[e] = 1;
@@ -545,15 +546,27 @@ FrameSchedule FrameBuilder::build(int mode, int path, const std::vector<int>& ti
         nst = c;
         passes = std::move(q);
     }
-    for (;;) {
-        FrameSchedule S = lay_out(p, L, mode, path, m, K, passes);
-        if (!tiled) return S;
+    FrameSchedule S = lay_out(p, L, mode, path, m, K, passes);
+    if (!tiled) return S;
+    const bool dbl = p.dtype == VQC_C128;
+    auto bytes = [&](const FrameSchedule& s) {
         PassNeeds c;
-        for (const FPass& ps : S.passes) c.cover(ps, ps.ndg);
-        const bool dbl = p.dtype == VQC_C128;
+        for (const FPass& ps : s.passes) c.cover(ps, ps.ndg);
         const PassBytes b = pass_bytes(c, n, mode, p.dtype, dbl, dbl, m, K);
-        if (b.fixed + b.tile <= kCtaSharedMemory || !split(passes, S, p)) return S;
-    }
+        return b.fixed + b.tile;
+    };
+    // complex128: two CTAs an SM, where passes of fewer table entries, at most twice as many,
+    // give them (double-float rings of RZZ, 15 qubits x 57, 5 layers, step: 4.58 ms with one CTA
+    // an SM, 3.81 with two)
+    if (dbl && bytes(S) > kHalfSharedMemory)
+        for (int entries : {72, 56, 40}) {
+            std::vector<PassPlan> q = plan_passes(p, L, mode, tiled, m, K, entries);
+            if (q.size() > 2 * passes.size()) break;
+            FrameSchedule T = lay_out(p, L, mode, path, m, K, q);
+            if (bytes(T) <= kHalfSharedMemory) return T;
+        }
+    while (bytes(S) > kCtaSharedMemory && split(passes, S, p)) S = lay_out(p, L, mode, path, m, K, passes);
+    return S;
 }
 
 namespace {
@@ -945,6 +958,8 @@ FrameSchedule lay_out(const HostPlan& p, const FrameOps& L, int mode, int path, 
             }
             st.op_begin = (int32_t)S.ops.size();
             st.seg_begin = (int32_t)S.segs.size();
+            bool phases = false;
+            for (int x : s.ops) phases = phases || p.ops[f[x].hop].type == OP_PH2;
             for (size_t rd = 0; rd < round.size() && !s.ops.empty(); ++rd) {
                 FSeg sg{};
                 std::vector<DOp> diag, runs;
@@ -954,7 +969,7 @@ FrameSchedule lay_out(const HostPlan& p, const FrameOps& L, int mode, int path, 
                         sg.pmask |= (uint8_t)(1u << d.a);
                         if (d.flags & OPF_PER_SAMPLE) sg.flags |= kSegPs;
                         const DEntry& e = p.entries[p.ops[f[x].hop].entry];
-                        const int form = run_form(&p.consts[e.cfirst], e.ccount);
+                        const int form = phases ? 0 : run_form(&p.consts[e.cfirst], e.ccount);
                         sg.flags |= (uint8_t)((form & 1 ? kSegQ : 0) | (form & 2 ? kSegP : 0));
                         runs.push_back(d);
                     } else {
@@ -983,8 +998,7 @@ FrameSchedule lay_out(const HostPlan& p, const FrameOps& L, int mode, int path, 
                 st.kind = kStagePure;
                 st.pmask = st.seg_begin < st.seg_end ? S.segs.back().pmask : 0;
             }
-            for (int x : s.ops)
-                if (p.ops[f[x].hop].type == OP_PH2) st.kind |= kStagePhases;
+            if (phases) st.kind |= kStagePhases;
             st.op_end = (int32_t)S.ops.size();
             st.nsel = (uint8_t)outside.size();
             auto word = [&](uint32_t v) {

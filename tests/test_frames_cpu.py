@@ -459,3 +459,20 @@ def test_phase_tables_come_first():
             every = sg["dg"][sg["dg"] != NO_DIAGONAL]
             assert sorted(every) == list(range(ps["ndg"]))
     B.vqc_free(plan)
+
+
+@pytest.mark.parametrize("n", [13, 15, 18])
+def test_complex128_passes_leave_room_for_two_ctas(n):
+    # many gradient slots a pass: fewer entries a pass instead of one CTA per SM
+    spec = wl.CircuitSpec(n, n, 12 * n)
+    for q in range(n):
+        spec.add("RY", (q,), [("x", q)])
+    for l in range(6):
+        for q in range(n):
+            spec.add("RZZ", (q, (q + 1) % n), [("w", 2 * n * l + q)])
+        for q in range(n):
+            spec.add("RX", (q,), [("w", 2 * n * l + n + q)])
+    plan = compile_spec(spec, 1)
+    hbm = [s for s in frames(plan) if s["path"] == 1]
+    B.vqc_free(plan)
+    assert hbm and all(launch_bytes(s, n, 1, True, True) <= 115712 for s in hbm)
