@@ -416,7 +416,7 @@ bool lean_pays(const HostPlan& p, int mode, const Launch& f, const Launch& l, in
     if (p.n > 9 || f.ndg == 0) return false;
     auto waves = [](const Launch& x) { return (x.nunits + x.grid - 1) / x.grid; };
     const bool sample = 2 * p.n_ps >= p.n_runs;
-    if (waves(l) < waves(f) && (p.n == 8 || sample)) return true;
+    if (waves(l) < waves(f) && (sample || (p.n == 8 && waves(f) >= 2 * waves(l)))) return true;
     return mode == 1 && f.nunits > sms && f.f->stages.size() < 8 && (p.n_ps == p.n_runs || (sample && f.S * p.n_ps >= 32));
 }
 
@@ -1393,10 +1393,12 @@ bool use_hbm(const HostPlan& p, int mode, int B) {
 // fused kernel sweeps forward with the backward's schedule, so then the
 // forward call (its own, larger blocks) followed by the backward from the saved
 // states is faster (12-qubit workload, batch 4096: 1.68 ms against 1.75 ms).  The same where
-// a double-float forward could have taken larger blocks but for its phases (choose_k), of
-// more than a CTA per SM (rings of RZZ, batch 1600, two calls / fused: 9 qubits x 4 layers
-// 1.02 / 1.45 ms, 10 x 4 2.20 / 3.16; 12 qubits x 2, batch 100: 427 / 402 us) and not a
-// wave of few stages (8 qubits x 2: 372 / 335 us, x 4 482 / 623).
+// a double-float forward could have taken larger blocks but for its phases (choose_k), up
+// to 11 qubits, beyond three CTAs an SM, or two where there are stages enough (rings of
+// RZZ, two calls / fused, us: 9 qubits x 4 layers, batch 700 489 / 503, 1000 758 / 1027; 10
+// x 1, 320 217 / 197, 500 292 / 310; 10 x 4, 1000 1480 / 2029; 11 x 1, 800 775 / 741; 12 x 1,
+// 600 1106 / 1023; random circuits, 11 qubits, 800 1488 / 1642): the fused kernel holds the
+// code of both sweeps, two calls a second launch and the states' way through HBM.
 bool resident_two_calls(const HostPlan& p, int B) {
     Launch Lf, Lb;
     const std::string saved = g_err;
@@ -1407,8 +1409,9 @@ bool resident_two_calls(const HostPlan& p, int B) {
     DevInfo di;
     if (Lf.K > Lb.K) return true;
     if (cudaGetDevice(&dev) != cudaSuccess || device_info(dev, di) != VQC_OK) return false;
-    return choose_k(p, 0, B, di.sms, true) > Lb.K && Lb.nunits > di.sms &&
-           (Lb.nunits > Lb.grid || Lb.f->stages.size() >= 8);
+    const bool deep = Lb.f->stages.size() >= 8;
+    return p.n <= 11 && choose_k(p, 0, B, di.sms, true) > Lb.K && Lb.nunits > (deep && p.n < 11 ? 2 : 3) * di.sms &&
+           (p.n < 11 || deep);
 }
 
 // Workspace of the two-call form: [backward workspace | final states].
