@@ -130,6 +130,7 @@ struct Launch {
     const FrameSchedule* f = nullptr;   // resident path
     int K = 0, T = 0, S = 0, block = 0, grid = 0, nunits = 0, wg = 1;
     size_t smem = 0;
+    size_t smem_states = 0;   // resident: the same of a launch that writes final states
     int sm_sh = 0, sm_ps = 0, sm_psi = 0, sm_lam = 0, sm_acc = 0, sm_terms = 0, sm_dw = 0,
         sm_red = 0, sm_plan = 0, sm_w = 0, sm_xg = 0, sm_io = 0, sm_dg = 0, ndg = 0;
     int cl = 0, sm_ecl = 0;   // cluster path: log2 CTAs per sample, <Z> gather area
@@ -155,7 +156,8 @@ int cta_threads() {
 // qubits x 3, step, 980 / 745 us, 11 qubits x 100, 1.8 times.  So no SM can hold more than
 // ceil(grid / SMs), as far as that asks for at most twice the memory -- for several CTAs
 // an SM at most 1.3 times, since more keeps the next kernel's CTAs out (9 qubits x 1600,
-// complex128 step 0.8 times).  Grids of half the SMs find as many free ones, and the larger
+// complex128 step 0.8 times), and not where a forward writes states, whose backward
+// comes next (10 qubits x 1600, re-uploading x 4, saved, 145 us spread, 120 not).  Grids of half the SMs find as many free ones, and the larger
 // request itself took time (double-float, 9 qubits x 3, step 316 -> 339 us).
 size_t spread_smem(size_t smem, int grid, int per_sm, const DevInfo& di) {
     const int share = (grid + di.sms - 1) / di.sms;
@@ -383,7 +385,9 @@ vqc_status plan_launch_as(const HostPlan& p, int launch_mode, int B, int K, bool
     }
     if (per_sm < 1) return fail(VQC_ERR_UNSUPPORTED, "kernel cannot be resident with this geometry");
     L.grid = std::max(1, std::min(L.nunits, per_sm * di.sms));
+    L.smem_states = L.smem;
     L.smem = spread_smem(L.smem, L.grid, per_sm, di);
+    if (L.grid <= di.sms) L.smem_states = L.smem;
     return VQC_OK;
 }
 
@@ -695,7 +699,7 @@ vqc_status run(const HostPlan& p, int mode, int B, const void* x, const void* w,
         a.dw_part = reinterpret_cast<R*>(static_cast<char*>(ws) + 256);
     }
     void* args[] = {&a};
-    VQC_CUDA(launch(L.fn, dim3(L.grid), dim3(L.block), args, L.smem, stream));
+    VQC_CUDA(launch(L.fn, dim3(L.grid), dim3(L.block), args, state_out ? L.smem_states : L.smem, stream));
     if (mode >= 1 && dw && p.num_w > 0) {
         const R* part = a.dw_part;
         int rows = L.grid, cols = p.num_w;
@@ -1404,13 +1408,13 @@ bool resident_two_calls(const HostPlan& p, int B) {
     const std::string saved = g_err;
     const bool ok = plan_launch(p, 0, B, Lf) == VQC_OK && plan_launch(p, 1, B, Lb) == VQC_OK;
     g_err = saved;
-    if (!ok) return false;
+    if (!ok || Lf.K > Lb.K) return ok;
+    if (!dfloat_of(p) || !p.has_ph2 || p.n > 11) return false;
     int dev = 0;
     DevInfo di;
-    if (Lf.K > Lb.K) return true;
     if (cudaGetDevice(&dev) != cudaSuccess || device_info(dev, di) != VQC_OK) return false;
     const bool deep = Lb.f->stages.size() >= 8;
-    return p.n <= 11 && choose_k(p, 0, B, di.sms, true) > Lb.K && Lb.nunits > (deep && p.n < 11 ? 2 : 3) * di.sms &&
+    return choose_k(p, 0, B, di.sms, true) > Lb.K && Lb.nunits > (deep && p.n < 11 ? 2 : 3) * di.sms &&
            (p.n < 11 || deep);
 }
 

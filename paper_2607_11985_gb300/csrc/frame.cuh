@@ -189,7 +189,8 @@ __device__ __forceinline__ void lambda_frame(const uint8_t* lmask, uint32_t pbf,
 // 18-qubit RZZ rings, not kept; resident kernels of such circuits take 2x2 updates in
 // every stage), and complex64 ones with diagonal ops, where a
 // multiplication is cheap beside the walk over the group (scalar phases: 13-qubit random circuit 216
-// us, 247 in rounds; 15-qubit RZZ rings 797 us against 835).
+// us, 247 in rounds; 15-qubit RZZ rings 797 us against 835).  Native complex128 resident
+// launches of circuits with few phases a round take it throughout (rounds_pay).
 template <typename R, bool PH2>
 __device__ __forceinline__ bool op_switch(unsigned kind) {
     return std::is_same<R, float>::value ? !(kind & kStagePure)
